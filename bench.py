@@ -52,11 +52,11 @@ CAPTURED_TRAFFIC = {
 
 
 def kernel_source_digest():
-    """sha256 over the sources of the analysis kernel (gcaps_rta.cu and the header it shares)."""
+    """sha256 over the sources of the analysis kernel (gcaps_rta.cu and the headers it shares)."""
     import hashlib
     h = hashlib.sha256()
     try:
-        for name in ("gcaps_rta.cu", "rta_common.cuh"):
+        for name in ("gcaps_rta.cu", "rta_device.cuh", "rta_common.cuh"):
             with open(os.path.join(ROOT, "paper_2406_05221_b200", "csrc", name), "rb") as fh:
                 h.update(fh.read())
     except OSError:

@@ -233,6 +233,9 @@ int enqueue_plan(KParams &p, void *workspace, size_t workspace_bytes, cudaStream
 // One launch over all size bins for analysis `mode` (0 GCAPS self-suspension, 1 GCAPS
 // busy-waiting, 2 RR self-suspension, 3 RR busy-waiting); defined in gcaps_rta_any.cu.
 cudaError_t launch_any_bins(int mode, const KParams &p, int sm_count, cudaStream_t st);
+// Launches over all size bins for the analyses sw.enabled names (bit m = mode m; one of 1, 2, 4, 8,
+// 5, 10) under every pair of `sw`; defined in gcaps_rta_sweep.cu.
+cudaError_t launch_sweep_set(const KParams &p, const SweepArgs &sw, int sm_count, cudaStream_t st);
 
 }  // namespace gcaps_detail
 #endif  // GCAPS_RTA_COMMON_CUH_

@@ -1,0 +1,1296 @@
+// rta_device.cuh -- device code of the analysis kernels, shared by the translation units that
+// instantiate them: gcaps_rta.cu (one analysis per launch), gcaps_rta_any.cu (all size bins in one
+// launch), gcaps_rta_sweep.cu (several analyses per launch).  Internal.
+//
+// One warp analyses one taskset at a time:
+//   stage      coalesced loads of the taskset's per-task slices into registers (lane = task)
+//   aggregate  coalesced loads of the segment arrays, warp prefix sums into shared memory; the
+//              per-task sums C_i, G^m_i, G^e_i and the RR slice count of Eq. 3 are differences of
+//              two prefix values
+//   order      rank of every task by (priority desc, position asc); the per-task values move
+//              through shared memory to the lane that owns the task's rank
+//   iterate    for each task in rank order the recurrence of Eq. 1 with the lemma set of the
+//              chosen analysis: lanes over the higher-priority interferers, each evaluating
+//              ceil((R+J)/T_h)*W terms (division by the invariant T_h is a multiply-high by a
+//              per-task reciprocal), summed across the warp
+//   publish    the lane that owns the converged task keeps R_i and forms its jitters J^c, J^g
+//   early exit the first deadline miss ends the taskset
+//   write      out_wcrt (one value per task), out_sched (one byte per taskset)
+// The fast path holds every time in 32 bits and is taken when all values of a taskset are below
+// 2^26 us; any other taskset goes through an exact 64-bit path with saturating arithmetic.
+// Tasksets are binned by size (a small plan pass writes a permutation into the workspace) so that
+// the warps of a launch hold the same number of tasks per lane; inside a launch warps pull chunks
+// of tasksets from a counter, because iteration counts differ widely.
+//
+// A "one warp" above is a group of 8 or 16 lanes for tasksets of up to 32 tasks (two or four
+// tasksets per warp).  gcaps_rta_multi_batch / gcaps_rta_sweep_batch use the same code with one
+// staging, ordering and aggregation per taskset and one recurrence per requested analysis and
+// (timeslice, overhead) pair.
+#ifndef GCAPS_RTA_DEVICE_CUH_
+#define GCAPS_RTA_DEVICE_CUH_
+
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include "rta_common.cuh"
+
+namespace {
+
+using namespace gcaps_detail;
+
+// Shared-memory image of one taskset, indexed by priority rank unless noted.
+template <int MAXN>
+struct GroupSmem {
+  u64 T[MAXN];     // period
+  u64 D[MAXN];     // deadline
+  u64 A[MAXN];     // C + G^m
+  u64 Ge[MAXN];    // G^e
+  u64 Star[MAXN];  // 2 * eps * eta^g   (GCAPS)   /   (L + theta) * slices, clamped   (RR)
+  u64 R[MAXN];     // converged response time
+  i64 prio_out[MAXN];  // by position: priority while ranking, then the output value
+  int core[MAXN];
+  int eta[MAXN];
+  unsigned short ord[MAXN];  // rank -> position
+};
+
+// ---------------------------------------------------------------------------------------------
+// the analysis of one taskset by a group of LPT lanes (exact 64-bit arithmetic)
+// ---------------------------------------------------------------------------------------------
+template <int LPT, int MAXN>
+__device__ void analyse_taskset(const KParams &p, i64 t, GroupSmem<MAXN> &s, int lane,
+                                unsigned int mask) {
+  const int policy = p.policy & 0xff;
+  const bool busy = (p.policy & GCAPS_RTA_BUSY) != 0;
+  const bool literal = (p.policy & GCAPS_RTA_LITERAL) != 0;
+  const bool best_effort = (p.policy & GCAPS_RTA_BEST_EFFORT) != 0;
+  const u64 L = (u64)p.L, ovh = (u64)p.ovh;
+
+  const i64 a = p.task_off[t] - p.task_base, b = p.task_off[t + 1] - p.task_base;
+  if (a < 0 || b < a || b > p.n_tasks || b - a > MAXN) {
+    // a range this launch cannot hold is a broken or oversized taskset: nothing is addressable
+    if (lane == 0) p.out_sched[t] = GCAPS_SCHED_INVALID;
+    return;
+  }
+  const int n = (int)(b - a);
+
+  // ---- stage: priorities by position, domain check of the per-task scalars -------------------
+  int bad = 0;
+  for (int i = lane; i < n; i += LPT) {
+    const i64 k = a + i;
+    s.prio_out[i] = p.priority[k];
+    const i64 T = p.period[k], D = p.deadline[k], c = p.core[k];
+    if (T < 1 || T > GCAPS_RTA_MAX_TIME) bad |= GCAPS_BAD_PERIOD;
+    if (D < 1 || D > T) bad |= GCAPS_BAD_DEADLINE;
+    if (c < 0 || c > GCAPS_RTA_MAX_CORE) bad |= GCAPS_BAD_CORE;
+  }
+  __syncwarp(mask);
+
+  // ---- order + aggregate: each lane ranks its tasks, sums their segments, stores by rank ------
+  int n_gpu_lane = 0;
+  for (int i = lane; i < n; i += LPT) {
+    const i64 k = a + i;
+    const i64 pi = s.prio_out[i];
+    int rank = 0;
+    for (int q = 0; q < n; ++q) {
+      const i64 pq = s.prio_out[q];
+      rank += (pq > pi || (pq == pi && q < i)) ? 1 : 0;
+    }
+    const i64 c0 = p.cseg_off[k] - p.cseg_base, c1 = p.cseg_off[k + 1] - p.cseg_base;
+    const i64 g0 = p.gseg_off[k] - p.gseg_base, g1 = p.gseg_off[k + 1] - p.gseg_base;
+    bool seg_ok = !(c0 < 0 || c1 < c0 || c1 > p.n_csegs || c1 - c0 > GCAPS_RTA_MAX_SEGMENTS ||
+                    g0 < 0 || g1 < g0 || g1 > p.n_gsegs || g1 - g0 > GCAPS_RTA_MAX_SEGMENTS);
+    u64 C = 0, Gm = 0, Ge = 0, slices = 0;
+    if (seg_ok) {
+      for (i64 j = c0; j < c1; ++j) {
+        const i64 w = p.cseg_wcet[j];
+        if (w < 0 || w > GCAPS_RTA_MAX_TIME) bad |= GCAPS_BAD_WCET;
+        C += (u64)w;
+      }
+      for (i64 j = g0; j < g1; ++j) {
+        const i64 m = p.gseg_misc[j], e = p.gseg_exec[j];
+        if (m < 0 || m > GCAPS_RTA_MAX_TIME || e < 0 || e > GCAPS_RTA_MAX_TIME)
+          bad |= GCAPS_BAD_WCET;
+        Gm += (u64)m;
+        Ge += (u64)e;
+        if (policy == GCAPS_POLICY_RR && e > 0) slices += ceil_div64((u64)e, L);  // Eq. 3
+      }
+    } else {
+      bad |= GCAPS_BAD_SEG_RANGE;
+    }
+    const int eta = seg_ok ? (int)(g1 - g0) : 0;
+    n_gpu_lane += eta > 0 ? 1 : 0;
+    s.T[rank] = (u64)p.period[k];
+    s.D[rank] = (u64)p.deadline[k];
+    s.A[rank] = C + Gm;
+    s.Ge[rank] = Ge;
+    s.Star[rank] = policy == GCAPS_POLICY_GCAPS ? 2 * ovh * (u64)eta : sat_mul(L + ovh, slices);
+    s.core[rank] = (int)p.core[k];
+    s.eta[rank] = eta;
+    // a best-effort task (flag set, priority <= 0) ranks behind every real-time task; bit 15
+    s.ord[rank] = (unsigned short)(i | ((best_effort && pi <= 0) ? 0x8000 : 0));
+  }
+  bad = group_or<LPT>(bad, mask);
+  const int n_gpu = group_sum_int<LPT>(n_gpu_lane, mask);  // N_g
+  __syncwarp(mask);
+  if (bad) {
+    if (p.out_wcrt)
+      for (int i = lane; i < n; i += LPT) p.out_wcrt[a + i] = GCAPS_WCRT_INVALID;
+    if (lane == 0) p.out_sched[t] = GCAPS_SCHED_INVALID;
+    return;
+  }
+  for (int i = lane; i < n; i += LPT)
+    s.prio_out[i] = (best_effort && s.prio_out[i] <= 0) ? GCAPS_WCRT_BEST_EFFORT : GCAPS_WCRT_SKIPPED;
+  __syncwarp(mask);
+
+  // ---- iterate: tasks in decreasing priority ---------------------------------------------------
+  int sched = GCAPS_SCHED_YES;
+  for (int pos = 0; pos < n; ++pos) {
+    if (s.ord[pos] & 0x8000) break;  // only best-effort tasks from here on: nothing to bound
+    const u64 Di = s.D[pos];
+    const int core_i = s.core[pos];
+    const bool gi = s.eta[pos] > 0;
+    u64 base;
+    u64 nu = 0;  // Lemma 4's interleaving-set size
+    if (policy == GCAPS_POLICY_GCAPS) {
+      // C_i + G*_i + B^C_i  (Sec. 6.3, Lemma 8); Star = 2*eps*eta
+      base = s.A[pos] + s.Ge[pos] + s.Star[pos] + ((u64)s.eta[pos] + 1) * ovh;
+    } else {
+      // C_i + G_i + I^ie_i  (Lemma 1); Star = (L+theta)*slices
+      base = s.A[pos] + s.Ge[pos] + (gi ? sat_mul(s.Star[pos], (u64)(n_gpu - 1)) : 0);
+      if (busy) {
+        int c = 0;
+        for (int h = lane; h < pos; h += LPT) c += (s.core[h] == core_i && s.eta[h] > 0) ? 1 : 0;
+        nu = (u64)(n_gpu - group_sum_int<LPT>(c, mask) + 1);
+      }
+    }
+    u64 R = base;
+    i64 verdict = 0;
+    i64 sweeps = 0;
+    for (;;) {
+      if (R > Di) {
+        verdict = GCAPS_WCRT_MISS;
+        break;
+      }
+      if (sweeps >= GCAPS_RTA_ITER_CAP) {
+        verdict = GCAPS_WCRT_ITER_LIMIT;
+        break;
+      }
+      sweeps += 1;
+      u64 part = 0;
+      for (int h = lane; h < pos; h += LPT) {
+        const u64 Th = s.T[h];
+        const bool same = s.core[h] == core_i;
+        const bool gh = s.eta[h] > 0;
+        const u64 Rh = s.R[h];
+        const u64 Jc = Rh - s.A[h], Jg = Rh - s.Ge[h];
+        u64 term = 0;
+        if (policy == GCAPS_POLICY_GCAPS && !busy) {
+          if (same && !gh) term = sat_mul(ceil_div64(R, Th), s.A[h]);  // Lemma 15 (G^m_h = 0)
+          if (same && gh) term = sat_mul(ceil_div64(R + Jc, Th), s.A[h] + s.Star[h]);
+          if (same && gh && gi) term += sat_mul(ceil_div64(R + Jg, Th), s.Ge[h]);   // Lemma 13
+          if (!same && gh && gi) term = sat_mul(ceil_div64(R + Jg, Th), s.Ge[h] + s.Star[h]);
+        } else if (policy == GCAPS_POLICY_GCAPS) {
+          if (same) {
+            u64 W = s.A[h];                                                        // Lemma 12
+            if (gh && (gi || !literal)) W += s.Ge[h] + s.Star[h];                  // Lemma 10
+            term = sat_mul(ceil_div64(R, Th), W);
+          } else if (gh) {
+            term = sat_mul(ceil_div64(R + Jg, Th), s.Ge[h] + s.Star[h]);           // Lemma 10/11
+          }
+        } else if (!busy) {
+          if (same) term = sat_mul(ceil_div64(R + ((gh || literal) ? Jc : 0), Th), s.A[h]);  // L7
+        } else {
+          if (same) {
+            u64 W = s.A[h];                                                        // Lemma 5
+            if (gh) W += sat_mul(s.Star[h], nu);                                   // Lemma 4
+            term = sat_mul(ceil_div64(R, Th), W);
+          }
+        }
+        part += term;  // each term <= 2^51, at most 8 per lane: no overflow
+      }
+      const u64 next = base + group_sum<LPT>(part, mask);
+      if (next == R) break;
+      R = next;
+    }
+    if (verdict == 0) {
+      if (lane == 0) {
+        s.R[pos] = R;
+        s.prio_out[s.ord[pos] & 0x7fff] = (i64)R;
+      }
+      __syncwarp(mask);
+    } else {
+      if (lane == 0) s.prio_out[s.ord[pos] & 0x7fff] = verdict;
+      sched = GCAPS_SCHED_NO;
+      break;
+    }
+  }
+  __syncwarp(mask);
+  if (p.out_wcrt)
+    for (int i = lane; i < n; i += LPT) p.out_wcrt[a + i] = s.prio_out[i];
+  if (lane == 0) p.out_sched[t] = (uint8_t)sched;
+  __syncwarp(mask);
+}
+
+// ---------------------------------------------------------------------------------------------
+// 32-bit fast path
+// ---------------------------------------------------------------------------------------------
+// ---- running sums of a segment array, 128 elements per step ------------------------------------
+// Lane l takes four consecutive elements (two 16-byte loads), so a warp reads 1 KB contiguous.
+// Loads must start on a 16-byte boundary: when the slice starts on an odd element the step begins
+// one element early (`par` = 1).  Q[x] receives the sum (modulo 2^32) of elements -par .. x - par;
+// Q[-1] is a guard word holding 0.  For 0 <= lo <= hi <= N the sum of elements [lo, hi) is
+// Q[hi - 1 + par] - Q[lo - 1 + par]: a borrowed element in front only shifts every entry by the
+// same amount, and elements behind the slice only reach entries that are never read.
+struct Quad {
+  i64 v[4];
+};
+
+// Elements e .. e+3 of X, for a slice whose 16-byte pairs all lie inside the array (the common
+// case, checked once per taskset by the caller).  Pairs that start at or behind N are not read.
+__device__ __forceinline__ void load_quad_inside(const i64 *__restrict__ X, int e, int N, Quad &q) {
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    longlong2 w = make_longlong2(0, 0);
+    if (e + 2 * h < N) w = __ldg(reinterpret_cast<const longlong2 *>(X + e + 2 * h));
+    q.v[2 * h] = w.x, q.v[2 * h + 1] = w.y;
+  }
+}
+
+// The same for a slice at the very edge of its array: only wanted elements inside [lo, hi) are
+// touched, everything else reads as 0.
+__device__ __noinline__ Quad load_quad_edge(const i64 *__restrict__ X, int e, int N, const i64 *lo,
+                                            const i64 *hi) {
+  Quad q;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const i64 *ptr = X + e + j;
+    q.v[j] = (e + j >= 0 && e + j < N && ptr >= lo && ptr < hi) ? __ldg(ptr) : 0;
+  }
+  return q;
+}
+
+// Narrows a quad to 32 bits, leaves the lane's own running sums in x[0..3] and records in `bad`
+// whether a wanted element lies outside [0, 2^26).
+__device__ __forceinline__ void narrow_quad(const Quad &q, int e, int N, u32 (&x)[4], u32 &bad) {
+  const u32 hi_or = (u32)((u64)q.v[0] >> 32) | (u32)((u64)q.v[1] >> 32) | (u32)((u64)q.v[2] >> 32) |
+                    (u32)((u64)q.v[3] >> 32);
+  const u32 lo_or = (u32)q.v[0] | (u32)q.v[1] | (u32)q.v[2] | (u32)q.v[3];
+  if (hi_or | (lo_or >> 26)) {  // rare: look again, this time only at the elements of this slice
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if ((u32)(e + j) < (u32)N) bad |= (u32)((u64)q.v[j] >> 32) | ((u32)q.v[j] >> 26);
+  }
+  x[0] = (u32)q.v[0];
+  x[1] = x[0] + (u32)q.v[1];
+  x[2] = x[1] + (u32)q.v[2];
+  x[3] = x[2] + (u32)q.v[3];
+}
+
+// True if every 16-byte pair that load_quad_inside would read for this slice is inside the array.
+__device__ __forceinline__ bool slice_is_inside(i64 first, int N, int par, i64 total) {
+  return (par == 0 || first >= 1) && ((((N + par) & 1) == 0) || first + N < total);
+}
+
+template <int LPT, int SLOTS>
+struct FastLayout {
+  static constexpr int MAXN = LPT * SLOTS;
+  static constexpr int kStep = 4 * LPT;  // elements one prefix step of the group covers
+  // a prefix array takes slices of up to CAP-1 elements and is written kStep words at a time
+  static constexpr int CAP = (6 * MAXN + kStep - 1) / kStep * kStep;
+  static constexpr int kInfo = 0;  // uint4 per rank: deadline, core, base, position | GPU flag
+  static constexpr int kQ0 = 4 * MAXN + 4;
+  static constexpr int kQ1 = kQ0 + CAP + 4;
+  static constexpr int kFastWords = kQ1 + CAP;
+  static constexpr int kExactWords = (17 * MAXN + 3) / 4 * 4;  // the exact path: 66 B per task
+  static constexpr int kWords = kFastWords > kExactWords ? kFastWords : kExactWords;
+  static_assert(kWords % 4 == 0 && CAP % kStep == 0 && 4 * MAXN <= CAP, "16-byte aligned rows");
+};
+
+// One step (NB blocks of 4*LPT elements) of the running sums of up to two arrays that share their
+// offsets, by a group of LPT lanes (`gmask`).
+template <int LPT, int NB, bool TWO>
+__device__ __forceinline__ void prefix_step(const i64 *__restrict__ X0, const i64 *__restrict__ X1,
+                                            int e0, int N, int par0, int par1, bool inside,
+                                            const i64 *lo0, const i64 *hi0, const i64 *lo1,
+                                            const i64 *hi1, u32 *Q0, u32 *Q1, u32 &carry0,
+                                            u32 &carry1, u32 &bad, int lane, unsigned int gmask) {
+  Quad q0[NB], q1[NB];
+  u32 x0[NB][4], x1[NB][4], i0[NB], i1[NB];
+  if (inside) {
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+      load_quad_inside(X0, e0 + 4 * LPT * b + 4 * lane - par0, N, q0[b]);
+      if (TWO) load_quad_inside(X1, e0 + 4 * LPT * b + 4 * lane - par1, N, q1[b]);
+    }
+  } else {
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+      q0[b] = load_quad_edge(X0, e0 + 4 * LPT * b + 4 * lane - par0, N, lo0, hi0);
+      if (TWO) q1[b] = load_quad_edge(X1, e0 + 4 * LPT * b + 4 * lane - par1, N, lo1, hi1);
+    }
+  }
+#pragma unroll
+  for (int b = 0; b < NB; ++b) {
+    narrow_quad(q0[b], e0 + 4 * LPT * b + 4 * lane - par0, N, x0[b], bad);
+    i0[b] = x0[b][3];
+    if (TWO) {
+      narrow_quad(q1[b], e0 + 4 * LPT * b + 4 * lane - par1, N, x1[b], bad);
+      i1[b] = x1[b][3];
+    }
+  }
+#pragma unroll
+  for (int d = 1; d < LPT; d <<= 1) {  // the warp scans of all blocks side by side
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+      const u32 y0 = __shfl_up_sync(gmask, i0[b], d, LPT);
+      if (lane >= d) i0[b] += y0;
+      if (TWO) {
+        const u32 y1 = __shfl_up_sync(gmask, i1[b], d, LPT);
+        if (lane >= d) i1[b] += y1;
+      }
+    }
+  }
+#pragma unroll
+  for (int b = 0; b < NB; ++b) {
+    if (e0 + 4 * LPT * b < N + 1) {
+      const u32 b0 = i0[b] - x0[b][3] + carry0;
+      *reinterpret_cast<uint4 *>(Q0 + e0 + 4 * LPT * b + 4 * lane) =
+          make_uint4(x0[b][0] + b0, x0[b][1] + b0, x0[b][2] + b0, x0[b][3] + b0);
+      carry0 += __shfl_sync(gmask, i0[b], LPT - 1, LPT);
+      if (TWO) {
+        const u32 b1 = i1[b] - x1[b][3] + carry1;
+        *reinterpret_cast<uint4 *>(Q1 + e0 + 4 * LPT * b + 4 * lane) =
+            make_uint4(x1[b][0] + b1, x1[b][1] + b1, x1[b][2] + b1, x1[b][3] + b1);
+        carry1 += __shfl_sync(gmask, i1[b], LPT - 1, LPT);
+      }
+    }
+  }
+}
+
+// Range check of segment slices without running sums: `bad` collects whether a wanted element lies
+// outside [0, 2^26), and the elements, narrowed to 32 bits, go to shared memory as they are
+// (D[w] = element w - par; same loads and store pattern as prefix_step).  NB blocks of 128
+// elements per array in flight together (TWO: two arrays that share their offsets).
+template <int NB, bool TWO>
+__device__ __forceinline__ void check_slices(const i64 *__restrict__ X0, const i64 *__restrict__ X1, int N,
+                                             int par0, int par1, bool inside, const i64 *lo0,
+                                             const i64 *hi0, const i64 *lo1, const i64 *hi1, u32 *D0,
+                                             u32 *D1, int lane, u32 &bad) {
+  for (int e0 = 0; e0 < N + (par0 > par1 ? par0 : par1); e0 += 128 * NB) {
+    Quad q0[NB], q1[NB];
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+      if (inside) {
+        load_quad_inside(X0, e0 + 128 * b + 4 * lane - par0, N, q0[b]);
+        if (TWO) load_quad_inside(X1, e0 + 128 * b + 4 * lane - par1, N, q1[b]);
+      } else {
+        q0[b] = load_quad_edge(X0, e0 + 128 * b + 4 * lane - par0, N, lo0, hi0);
+        if (TWO) q1[b] = load_quad_edge(X1, e0 + 128 * b + 4 * lane - par1, N, lo1, hi1);
+      }
+    }
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+      if (e0 + 128 * b < N + 1) {
+        u32 x[4];
+        narrow_quad(q0[b], e0 + 128 * b + 4 * lane - par0, N, x, bad);
+        *reinterpret_cast<uint4 *>(D0 + e0 + 128 * b + 4 * lane) =
+            make_uint4((u32)q0[b].v[0], (u32)q0[b].v[1], (u32)q0[b].v[2], (u32)q0[b].v[3]);
+        if (TWO) {
+          narrow_quad(q1[b], e0 + 128 * b + 4 * lane - par1, N, x, bad);
+          *reinterpret_cast<uint4 *>(D1 + e0 + 128 * b + 4 * lane) =
+              make_uint4((u32)q1[b].v[0], (u32)q1[b].v[1], (u32)q1[b].v[2], (u32)q1[b].v[3]);
+        }
+      }
+    }
+  }
+}
+
+// The first kFirstRanks tasks of the priority order, analysed before anything is summed for the
+// rest of the taskset (a warp per taskset).  Where tasksets are far from schedulable the first
+// deadline miss comes within a handful of ranks, and the per-task sums of all the other tasks
+// would never be used: here every segment value is still read and range-checked (a value outside
+// the 32-bit path's range sends the taskset to the exact path, as always), but sums are formed
+// only for these ranks: four lanes per rank add up the rank's own few segments, all ranks at once
+// (one trip to memory), and lane r then holds everything about rank r, as the task under analysis
+// and as an interferer of the ranks behind it.  The recurrence over these ranks needs registers
+// and warp collectives only.  Same arithmetic, same sequence of iterates, same sentinels as the
+// full pass.  `first8[r]` = (first, end) of rank r's CPU segments and of its GPU segments within
+// the taskset's slices; info[r] = (deadline, core, period, position).
+// Returns 1: the taskset is finished (a miss among these ranks, or no other real-time task), its
+// outputs are written; 0: all these ranks converged, the caller runs the full pass (which repeats
+// them); -1: a value does not fit the 32-bit path.
+constexpr int kFirstRanks = 8;
+template <int SLOTS, int MODE>
+__device__ __forceinline__ int first_ranks(const KParams &p, i64 t, i64 a, int n, const uint4 *info,
+                                           const uint4 *first8, u32 *Q0, u32 *Q1, int n_rt,
+                                           const int (&rank)[SLOTS], const int (&g0)[SLOTS],
+                                           const int (&g1)[SLOTS], const i64 *__restrict__ Xc,
+                                           const i64 *__restrict__ Xm, const i64 *__restrict__ Xe, int Nc,
+                                           int Ng, int parc, int parm, int pare, i64 cfirst, i64 gfirst,
+                                           int lane, bool literal) {
+  const int limit = n_rt < kFirstRanks ? n_rt : kFirstRanks;
+  // lanes 4r .. 4r+3 add up the segments of rank r
+  const int r4 = lane >> 2, sub = lane & 3;
+  uint4 seg = make_uint4(0u, 0u, 0u, 0u);
+  if (r4 < limit) seg = first8[r4];
+  u32 bad = 0, sum_c = 0, sum_m = 0, sum_e = 0, sum_s = 0;
+  // every segment value of the taskset must be in [0, 2^26); on the way the values stop over in
+  // shared memory, where the eight ranks find their own
+  check_slices<(SLOTS < 3 ? SLOTS : 3), false>(Xc, Xc, Nc, parc, parc, slice_is_inside(cfirst, Nc, parc, p.n_csegs),
+                                               p.cseg_wcet, p.cseg_wcet + p.n_csegs, p.cseg_wcet, p.cseg_wcet,
+                                               Q0, Q0, lane, bad);
+  __syncwarp();
+  for (int j = (int)seg.x + parc + sub; j < (int)seg.y + parc; j += 4) sum_c += Q0[j];
+  __syncwarp();
+  check_slices<2, true>(Xm, Xe, Ng, parm, pare,
+                        slice_is_inside(gfirst, Ng, parm, p.n_gsegs) && slice_is_inside(gfirst, Ng, pare, p.n_gsegs),
+                        p.gseg_misc, p.gseg_misc + p.n_gsegs, p.gseg_exec, p.gseg_exec + p.n_gsegs, Q1, Q0,
+                        lane, bad);
+  __syncwarp();
+  for (int j = (int)seg.z + sub; j < (int)seg.w; j += 4) {
+    sum_m += Q1[j + parm];
+    const u32 e = Q0[j + pare] & (kFastLimit - 1);  // (checked above; keeps the division exact)
+    sum_e += e;
+    if (MODE >= 2) {  // Eq. 3: slices of the pure GPU part
+      if (p.l_mode == 0) sum_s += __umulhi(e + (u32)p.L - 1u, p.l_magic) >> p.l_shift;
+      else if (p.l_mode == 1) sum_s += e;
+      else sum_s += e > 0 ? 1u : 0u;
+    }
+  }
+  int n_gpu = 0;  // N_g
+#pragma unroll
+  for (int s = 0; s < SLOTS; ++s) n_gpu += __popc(__ballot_sync(kFull, g1[s] > g0[s]));
+#pragma unroll
+  for (int d = 1; d <= 2; d <<= 1) {
+    sum_c += __shfl_xor_sync(kFull, sum_c, d), sum_m += __shfl_xor_sync(kFull, sum_m, d);
+    sum_e += __shfl_xor_sync(kFull, sum_e, d);
+    if (MODE >= 2) sum_s += __shfl_xor_sync(kFull, sum_s, d);
+  }
+  // lane r takes rank r from lane 4r (a task has fewer than 64 segments of a kind, every value is
+  // below 2^26: no overflow)
+  const int src = (4 * lane) & 31;
+  sum_c = __shfl_sync(kFull, sum_c, src), sum_m = __shfl_sync(kFull, sum_m, src);
+  sum_e = __shfl_sync(kFull, sum_e, src);
+  if (MODE >= 2) sum_s = __shfl_sync(kFull, sum_s, src);
+  const u32 eta_r = __shfl_sync(kFull, seg.w - seg.z, src);
+  const bool mine = lane < limit;
+  const uint4 f = mine ? info[lane] : make_uint4(1u, 0xffffffffu, 2u, 0u);  // deadline, core, period, position
+  const u32 ovh = (u32)p.ovh;  // below 2^20 on this path
+  const u32 D_r = f.x, core_r = f.y, Tm1 = f.z - 1, A_r = sum_c + sum_m, Ge_r = sum_e;
+  const bool gpu_r = eta_r > 0;
+  u32 S_r, base_r;
+  if (MODE < 2) {
+    S_r = 2 * ovh * eta_r;                               // eta < 64: below 2^27
+    base_r = A_r + Ge_r + S_r + (eta_r + 1) * ovh;       // C_i + G*_i + B^C_i, below 2^29
+    if (mine) bad |= S_r >> 26;
+  } else {
+    const u64 lt = (u64)p.L + ovh;                       // <= 2^41
+    u64 B = sum_s == 0 ? 0 : (lt >= kFastClamp ? kFastClamp : lt * (u64)sum_s);
+    if (B > kFastClamp) B = kFastClamp;
+    S_r = (u32)B;
+    const u64 b64 = (u64)A_r + Ge_r + (gpu_r ? B * (u64)(n_gpu - 1) : 0);  // Lemma 1
+    base_r = b64 > (u64)(2 * kFastClamp) ? 2 * kFastClamp : (u32)b64;
+  }
+  base_r = base_r > 2 * kFastClamp ? 2 * kFastClamp : base_r;
+  if (mine) bad |= (sum_c | sum_m | A_r | Ge_r) >> 26;
+  if (__any_sync(kFull, bad != 0)) return -1;
+  u32 magic, shift;
+  make_reciprocal(f.z, magic, shift);
+  // what rank r contributes as an interferer (the jitters follow when it has converged)
+  u32 Wa, Wb;
+  if (MODE == 0) {
+    Wa = A_r + (gpu_r ? S_r : 0u);    // Lemma 15: C_h, or C_h + G^{m*}_h
+    Wb = gpu_r ? Ge_r + S_r : 0u;     // Lemma 13, other cores: G^{e*}_h
+  } else if (MODE == 1) {
+    Wa = A_r;                         // Lemma 12
+    Wb = gpu_r ? Ge_r + S_r : 0u;     // Lemmas 10, 11: G^{e*}_h
+  } else {
+    Wa = A_r;                         // Lemmas 5, 7
+    Wb = gpu_r ? S_r : 0u;            // Lemma 4: (L+theta) * slices
+  }
+  u32 Jc = Tm1, Jg = Tm1;
+  // ---- the recurrence of Eq. 1 over these ranks -----------------------------------------------------
+  int verdict = 0, pos = 0;
+  for (; pos < limit; ++pos) {
+    const u32 Di = __shfl_sync(kFull, D_r, pos), core_i = __shfl_sync(kFull, core_r, pos);
+    const u32 base_i = __shfl_sync(kFull, base_r, pos);
+    const bool gi = __shfl_sync(kFull, (int)gpu_r, pos) != 0;
+    const bool act = lane < pos, same = core_r == core_i;
+    u32 j1, w1, w2 = 0;
+    if (MODE == 0) {
+      w1 = same ? Wa : (gi ? Wb : 0u);            // Lemma 15 / Lemma 13 (other cores)
+      j1 = same ? Jc : Jg;
+      w2 = (same && gi && gpu_r) ? Ge_r : 0u;     // Lemma 13 (same core), jitter J^g
+    } else if (MODE == 1) {
+      w1 = same ? Wa + ((gi || !literal) ? Wb : 0u) : Wb;  // Lemmas 12+10 / 10, 11
+      j1 = same ? Tm1 : Jg;
+    } else if (MODE == 2) {
+      w1 = same ? Wa : 0u;                        // Lemma 7
+      j1 = Jc;
+    } else {
+      // Lemma 4: N_g - |{h in hpp(i): GPU-using}| + 1
+      const u32 nu = (u32)(n_gpu - __popc(__ballot_sync(kFull, act && same && gpu_r)) + 1);
+      const u64 w = (u64)Wa + (u64)Wb * nu;       // Lemmas 5 and 4
+      w1 = same ? (w > kFastClamp ? kFastClamp : (u32)w) : 0u;
+      j1 = Tm1;
+    }
+    if (!act) w1 = 0, w2 = 0;
+    u32 R = base_i;
+    int sweeps = 0;
+    for (;;) {
+      if (R > Di) {
+        verdict = GCAPS_WCRT_MISS;
+        break;
+      }
+      if (sweeps >= (int)GCAPS_RTA_ITER_CAP) {
+        verdict = GCAPS_WCRT_ITER_LIMIT;
+        break;
+      }
+      sweeps += 1;
+      u32 next = base_i;
+      if (pos > 0) {
+        u64 acc = (u64)(__umulhi(R + j1, magic) >> shift) * w1;
+        if (MODE == 0) acc += (u64)(__umulhi(R + Jg, magic) >> shift) * w2;
+        const u32 part = acc > (u64)kFastClamp ? kFastClamp : (u32)acc;
+        next += __reduce_add_sync(kFull, part);
+      }
+      if (next == R) break;
+      R = next;
+    }
+    if (verdict != 0) break;
+    // publish: R_i goes out; lane `pos` forms the jitters J^c = R - (C+G^m), J^g = R - G^e (a
+    // CPU-only task has no J^c unless the printed form of Lemma 7 is asked for)
+    if (lane == pos) {
+      if (p.out_wcrt) p.out_wcrt[a + f.w] = (i64)R;
+      if (MODE == 0 ? gpu_r : (MODE == 2 ? (gpu_r || literal) : false)) Jc = R - A_r + Tm1;
+      Jg = R - Ge_r + Tm1;
+    }
+  }
+  if (verdict == 0 && limit < n_rt) return 0;  // undecided: the full pass takes over
+  const int n_done = pos;  // ranks that converged (= n_rt without a verdict)
+  if (p.out_wcrt) {
+#pragma unroll
+    for (int s = 0; s < SLOTS; ++s) {
+      const int r = rank[s];
+      if (lane + 32 * s < n && r >= n_done)
+        p.out_wcrt[a + lane + 32 * s] = r >= n_rt ? (i64)GCAPS_WCRT_BEST_EFFORT
+                                                  : (r == n_done ? (i64)verdict : (i64)GCAPS_WCRT_SKIPPED);
+    }
+  }
+  if (lane == 0) p.out_sched[t] = verdict == 0 ? GCAPS_SCHED_YES : GCAPS_SCHED_NO;
+  return 1;
+}
+
+// An analysis mode known at compile time (converts to int like a run-time mode does).
+template <int V>
+struct ModeTag {
+  __host__ __device__ constexpr operator int() const { return V; }
+};
+
+// MODE: 0 GCAPS self-suspension, 1 GCAPS busy-waiting, 2 RR self-suspension, 3 RR busy-waiting.
+// Returns false, having written nothing, if the taskset is not eligible for 32-bit arithmetic
+// (or is invalid): the caller then runs the exact 64-bit path, which also does the validation.
+//
+// A group of LPT lanes (8, 16 or a whole warp) works on one taskset.  Until the per-task sums are
+// known lane l of the group holds the tasks at positions l, l+LPT, ... ("slots").
+// Then every task's values move through shared memory to the lane that owns its rank, so that the
+// interferers of the task of rank `pos` sit in lanes (pos-1) % LPT downwards of slots up to
+// (pos-1) / LPT and higher slots can be skipped.
+//
+// MASK: bit m set = analysis MODE m is compiled in.  SWEEP: the taskset is staged, ordered and
+// aggregated once and then analysed under every (timeslice, overhead) pair q of `sw` and every
+// mode m of MASK that sw->enabled names; that analysis writes result block
+// q * sw->block_stride + sw->block_of_mode[m] (out_wcrt + block * n_tasks, skipped when out_wcrt
+// is null; out_sched + block * n_tasksets).  Without SWEEP, MASK has one bit and the analysis
+// takes its constants and outputs from `p`.
+//
+// Returns kFastDone (outputs written), kFastDeclined (nothing written that matters: the caller runs
+// the exact path) or, with FIRST_ONLY, kFastUndecided.  FIRST_ONLY (one analysis, a warp per
+// taskset): only the first ranks of the priority order are analysed (first_ranks below); if they
+// all converge and more ranks follow, nothing is decided and the caller runs the full pass.
+constexpr int kFastDeclined = 0, kFastDone = 1, kFastUndecided = 2;
+template <int LPT, int SLOTS, int MASK, bool SWEEP = false, bool FIRST_ONLY = false>
+__device__ __forceinline__ int analyse_fast(const KParams &p, i64 t, i64 a, int n, u32 *buf, int lane,
+                                            unsigned int gmask, const SweepArgs *sw = nullptr) {
+  static_assert(!FIRST_ONLY || (LPT == 32 && !SWEEP), "the first ranks' own pass: a warp per taskset");
+  typedef FastLayout<LPT, SLOTS> Lay;
+  constexpr int kLog = LPT == 32 ? 5 : LPT == 16 ? 4 : 3;  // log2 of the lanes per taskset
+  constexpr int MAXN = Lay::MAXN, CAP = Lay::CAP;
+  // prefix blocks of the CPU segments whose loads are issued together.  Tasksets of 65..96 tasks
+  // with a few GPU segments per task have 200..400 CPU segments: three blocks of 128 cover them
+  // in one step where two need a second, mostly empty one (80-task tasksets: -4 % for a GCAPS
+  // kernel; the RR kernels, which carry the slice sums too, lose as much to the registers it takes)
+  constexpr int BC = SLOTS <= 2 ? SLOTS : ((SLOTS == 3 && (MASK & 12) == 0 && !SWEEP) ? 3 : 2);
+  constexpr int BG = 1;
+  constexpr bool kAnyGcaps = (MASK & 3) != 0;
+  constexpr bool kMulti = (MASK & (MASK - 1)) != 0;
+  static_assert(!kMulti || SWEEP, "several analyses per taskset use the sweep loop");
+  const bool literal = (p.policy & GCAPS_RTA_LITERAL) != 0;
+  const bool best_effort = (p.policy & GCAPS_RTA_BEST_EFFORT) != 0;
+  uint4 *info = reinterpret_cast<uint4 *>(buf + Lay::kInfo);
+  u32 *Q0 = buf + Lay::kQ0, *Q1 = buf + Lay::kQ1;
+
+  // ---- stage: per-task scalars, lane = position; rank ----------------------------------------
+  u32 T[SLOTS];
+  int rank[SLOTS], c0[SLOTS], g0[SLOTS];
+  bool ok = true;
+  int Nc, Ng;
+  i64 cfirst, gfirst;
+  {
+    i64 t64[SLOTS], d64[SLOTS], pr[SLOTS], c64[SLOTS], co[SLOTS], go[SLOTS];
+#pragma unroll
+    for (int s = 0; s < SLOTS; ++s) {  // all loads of the taskset's per-task arrays in flight
+      const i64 k = a + (lane + LPT * s < n ? lane + LPT * s : 0);
+      t64[s] = p.period[k], d64[s] = p.deadline[k], pr[s] = p.priority[k], c64[s] = p.core[k];
+      co[s] = p.cseg_off[k], go[s] = p.gseg_off[k];
+    }
+    const i64 cend = p.cseg_off[a + n] - p.cseg_base, gend = p.gseg_off[a + n] - p.gseg_base;
+    cfirst = __shfl_sync(gmask, co[0], 0, LPT) - p.cseg_base;
+    gfirst = __shfl_sync(gmask, go[0], 0, LPT) - p.gseg_base;
+    const i64 Nc64 = cend - cfirst, Ng64 = gend - gfirst;
+    if (cfirst < 0 || Nc64 < 0 || cend > p.n_csegs || Nc64 >= CAP || gfirst < 0 || Ng64 < 0 ||
+        gend > p.n_gsegs || Ng64 >= CAP)
+      return kFastDeclined;
+    Nc = (int)Nc64, Ng = (int)Ng64;
+    u32 high = 0;  // any set bit: some value does not fit the 32-bit path
+    u32 D[SLOTS], core[SLOTS];
+    int prio[SLOTS];
+#pragma unroll
+    for (int s = 0; s < SLOTS; ++s) {
+      const bool v = lane + LPT * s < n;
+      const i64 rc = co[s] - p.cseg_base - cfirst, rg = go[s] - p.gseg_base - gfirst;
+      const u32 h = (u32)((u64)t64[s] >> 32) | (u32)((u64)d64[s] >> 32) | (u32)((u64)c64[s] >> 32) |
+                    (u32)((u64)rc >> 32) | (u32)((u64)rg >> 32) |
+                    (u32)(((u64)pr[s] + 0x80000000ull) >> 32);
+      T[s] = v ? (u32)t64[s] : 2u;
+      D[s] = (u32)d64[s];
+      core[s] = (u32)c64[s];
+      prio[s] = v ? (int)pr[s] : (int)0x80000000;
+      c0[s] = v ? (int)rc : Nc;
+      g0[s] = v ? (int)rg : Ng;
+      high |= v ? h : 0u;
+      // 2 <= T < 2^26, 1 <= D <= T, core < 2^31, offsets inside the slice
+      ok &= T[s] - 2u < kFastLimit - 2u && (!v || (D[s] - 1u < T[s] && (int)core[s] >= 0)) &&
+            (u32)c0[s] <= (u32)Nc && (u32)g0[s] <= (u32)Ng;
+    }
+    if (__any_sync(gmask, high != 0 || !ok)) return kFastDeclined;  // (a wide priority also lands here)
+    // order: rank by (priority desc, position asc)
+    int m = prio[0];
+#pragma unroll
+    for (int s = 1; s < SLOTS; ++s) m = prio[s] > m ? prio[s] : m;
+    const int pmax = __reduce_max_sync(gmask, m);
+    bool dense = true;  // distinct priorities max-n+1 .. max: the rank is max - priority
+#pragma unroll
+    for (int s = 0; s < SLOTS; ++s) {
+      const u32 r = (u32)pmax - (u32)prio[s];
+      const bool v = lane + LPT * s < n;
+      dense &= !v || r < (u32)n;
+      rank[s] = v ? (int)r : MAXN;
+    }
+    dense = __all_sync(gmask, dense);
+    if (dense) {
+#pragma unroll
+      for (int s = 0; s < SLOTS; ++s)
+        if (lane + LPT * s < n) Q0[rank[s]] = (u32)(lane + LPT * s);
+      __syncwarp(gmask);
+      bool uniq = true;
+#pragma unroll
+      for (int s = 0; s < SLOTS; ++s)
+        if (lane + LPT * s < n) uniq &= Q0[rank[s]] == (u32)(lane + LPT * s);
+      dense = __all_sync(gmask, uniq);
+      __syncwarp(gmask);
+    }
+    if (!dense) {  // any priorities: count the tasks that come before
+#pragma unroll
+      for (int s = 0; s < SLOTS; ++s) {
+        const int i = lane + LPT * s;
+        int r = 0;
+        for (int q = 0; q < n; ++q) {
+          const int pq = (int)p.priority[a + q];
+          r += (pq > prio[s] || (pq == prio[s] && q < i)) ? 1 : 0;
+        }
+        rank[s] = i < n ? r : MAXN;
+      }
+    }
+    // best-effort tasks (flag set, priority <= 0) rank behind every real-time task: the ranks
+    // from n_rt on are theirs
+    // (kept in a spare word in front of Q0's guard entry until the recurrence starts)
+    {
+      int n_rt = n;
+      if (best_effort) {
+#pragma unroll
+        for (int s = 0; s < SLOTS; ++s)
+          n_rt -= __popc(__ballot_sync(gmask, lane + LPT * s < n && prio[s] <= 0));
+      }
+      if (lane == 0) Q0[-2] = (u32)n_rt;
+    }
+    // what every lane must know about the task of a given rank (base and GPU flag follow; the
+    // first ranks' own pass keeps the period and the position there instead)
+#pragma unroll
+    for (int s = 0; s < SLOTS; ++s) {
+      if constexpr (FIRST_ONLY) {
+        if (rank[s] < kFirstRanks) info[rank[s]] = make_uint4(D[s], core[s], T[s], (u32)(lane + LPT * s));
+      } else {
+        if (lane + LPT * s < n) *reinterpret_cast<uint2 *>(&info[rank[s]]) = make_uint2(D[s], core[s]);
+      }
+    }
+  }
+  // end offsets: the next task's start (positions beyond n hold the total)
+  int c1[SLOTS], g1[SLOTS];
+#pragma unroll
+  for (int s = 0; s < SLOTS; ++s) {
+    const int cn = __shfl_down_sync(gmask, c0[s], 1, LPT), gn = __shfl_down_sync(gmask, g0[s], 1, LPT);
+    const int ch = __shfl_sync(gmask, s + 1 < SLOTS ? c0[s + 1 < SLOTS ? s + 1 : s] : Nc, 0, LPT);
+    const int gh = __shfl_sync(gmask, s + 1 < SLOTS ? g0[s + 1 < SLOTS ? s + 1 : s] : Ng, 0, LPT);
+    c1[s] = lane == LPT - 1 ? ch : cn;
+    g1[s] = lane == LPT - 1 ? gh : gn;
+    ok &= (u32)(c1[s] - c0[s]) < 64u && (u32)(g1[s] - g0[s]) < 64u;
+  }
+  if (!__all_sync(gmask, ok)) return kFastDeclined;
+
+  // ---- aggregate: running sums of the segment arrays; per-task sums are differences --------
+  u32 A[SLOTS], Ge[SLOTS], S[SLOTS];  // C+G^m, G^e, and 2*eps*eta (GCAPS) or (L+theta)*slices (RR)
+  u32 bad = 0;
+  const i64 *__restrict__ Xc = p.cseg_wcet + cfirst;
+  const i64 *__restrict__ Xm = p.gseg_misc + gfirst, *__restrict__ Xe = p.gseg_exec + gfirst;
+  const int parc = (int)(((uintptr_t)Xc >> 3) & 1), parm = (int)(((uintptr_t)Xm >> 3) & 1);
+  const int pare = (int)(((uintptr_t)Xe >> 3) & 1);
+  if constexpr (FIRST_ONLY) {
+    constexpr int MODE = (MASK & 1) ? 0 : (MASK & 2) ? 1 : (MASK & 4) ? 2 : 3;
+    uint4 *first8 = info + kFirstRanks;  // (only the first ranks' rows of `info` are used here)
+#pragma unroll
+    for (int s = 0; s < SLOTS; ++s)
+      if (rank[s] < kFirstRanks) first8[rank[s]] = make_uint4((u32)c0[s], (u32)c1[s], (u32)g0[s], (u32)g1[s]);
+    __syncwarp(gmask);
+    const int r = first_ranks<SLOTS, MODE>(p, t, a, n, info, first8, Q0, Q1, (int)Q0[-2], rank, g0, g1, Xc, Xm, Xe,
+                                           Nc, Ng, parc, parm, pare, cfirst, gfirst, lane, literal);
+    __syncwarp(gmask);
+    return r > 0 ? kFastDone : (r == 0 ? kFastUndecided : kFastDeclined);
+  }
+  if (lane == 0) Q0[-1] = 0, Q1[-1] = 0;
+  {  // CPU segments -> Q0
+    const bool inside = slice_is_inside(cfirst, Nc, parc, p.n_csegs);
+    u32 carry = 0, unused = 0;
+    for (int e0 = 0; e0 < Nc + parc; e0 += Lay::kStep * BC)
+      prefix_step<LPT, BC, false>(Xc, Xc, e0, Nc, parc, parc, inside, p.cseg_wcet, p.cseg_wcet + p.n_csegs,
+                             p.cseg_wcet, p.cseg_wcet, Q0, Q0, carry, unused, bad, lane, gmask);
+  }
+  __syncwarp(gmask);
+#pragma unroll
+  for (int s = 0; s < SLOTS; ++s) A[s] = Q0[c1[s] - 1 + parc] - Q0[c0[s] - 1 + parc];
+  __syncwarp(gmask);
+  {  // G^m -> Q0, G^e -> Q1
+    const bool inside = slice_is_inside(gfirst, Ng, parm, p.n_gsegs) &&
+                        slice_is_inside(gfirst, Ng, pare, p.n_gsegs);
+    u32 cm = 0, ce = 0;
+    for (int e0 = 0; e0 < Ng + 1; e0 += Lay::kStep * BG)
+      prefix_step<LPT, BG, true>(Xm, Xe, e0, Ng, parm, pare, inside, p.gseg_misc, p.gseg_misc + p.n_gsegs,
+                            p.gseg_exec, p.gseg_exec + p.n_gsegs, Q0, Q1, cm, ce, bad, lane, gmask);
+  }
+  __syncwarp(gmask);
+  u32 eta[SLOTS];
+#pragma unroll
+  for (int s = 0; s < SLOTS; ++s) {
+    const u32 Gm = Q0[g1[s] - 1 + parm] - Q0[g0[s] - 1 + parm];
+    Ge[s] = Q1[g1[s] - 1 + pare] - Q1[g0[s] - 1 + pare];
+    eta[s] = (u32)(g1[s] - g0[s]);
+    bad |= (A[s] | Gm | Ge[s]) >> 26;
+    A[s] += Gm;
+    bad |= A[s] >> 26;
+  }
+  __syncwarp(gmask);
+  // ---- what does not depend on the timeslice or the overhead ---------------------------------
+  int n_gpu = 0;  // N_g
+#pragma unroll
+  for (int s = 0; s < SLOTS; ++s) n_gpu += __popc(__ballot_sync(gmask, eta[s] > 0));
+  if (kAnyGcaps) {  // 2 * eps * eta must stay below 2^26 (eta < 64, eps < 2^20: no overflow here)
+    const u32 ovh_max = SWEEP ? (u32)sw->max_ovh : (u32)p.ovh;
+#pragma unroll
+    for (int s = 0; s < SLOTS; ++s) bad |= (2 * ovh_max * eta[s]) >> 26;
+  }
+  if (__any_sync(gmask, bad != 0)) return kFastDeclined;
+  const int n_rt_all = (int)Q0[-2];  // real-time tasks: the ranks that are analysed
+  uint4 *xch = reinterpret_cast<uint4 *>(Q0);  // by rank: T, C+G^m, G^e, S  (Q0 is dead by now)
+
+  // Eq. 3: running sums of the slices of every pure GPU part for timeslice L (values already
+  // checked) into Ps
+  auto slice_sums = [&](u32 *Ps, i64 L64, u32 l_mode, u32 l_magic, u32 l_shift) {
+    // Eq. 3: slices of every pure GPU part, summed per task (values already checked)
+    const bool inside = slice_is_inside(gfirst, Ng, pare, p.n_gsegs);
+    u32 carry = 0;
+    if (lane == 0) Ps[-1] = 0;
+    for (int e0 = 0; e0 < Ng + 1; e0 += Lay::kStep * BG) {
+      Quad qe[BG];
+      u32 x[BG][4], incl[BG];
+#pragma unroll
+      for (int b = 0; b < BG; ++b) {
+        if (inside) load_quad_inside(Xe, e0 + 4 * LPT * b + 4 * lane - pare, Ng, qe[b]);
+        else qe[b] = load_quad_edge(Xe, e0 + 4 * LPT * b + 4 * lane - pare, Ng, p.gseg_exec, p.gseg_exec + p.n_gsegs);
+      }
+#pragma unroll
+      for (int b = 0; b < BG; ++b) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          // a neighbour's element may be large: keep it below 2^26 so the division stays exact
+          const u32 w = (u32)qe[b].v[j] & (kFastLimit - 1);
+          u32 sq;
+          if (l_mode == 0) sq = __umulhi(w + (u32)L64 - 1u, l_magic) >> l_shift;
+          else if (l_mode == 1) sq = w;
+          else sq = w > 0 ? 1u : 0u;
+          x[b][j] = sq + (j > 0 ? x[b][j - 1] : 0u);
+        }
+        incl[b] = x[b][3];
+      }
+#pragma unroll
+      for (int d = 1; d < LPT; d <<= 1) {
+#pragma unroll
+        for (int b = 0; b < BG; ++b) {
+          const u32 y = __shfl_up_sync(gmask, incl[b], d, LPT);
+          if (lane >= d) incl[b] += y;
+        }
+      }
+#pragma unroll
+      for (int b = 0; b < BG; ++b) {
+        if (e0 + 4 * LPT * b < Ng + 1) {
+          const u32 before = incl[b] - x[b][3] + carry;
+          *reinterpret_cast<uint4 *>(Ps + e0 + 4 * LPT * b + 4 * lane) =
+              make_uint4(x[b][0] + before, x[b][1] + before, x[b][2] + before, x[b][3] + before);
+          carry += __shfl_sync(gmask, incl[b], LPT - 1, LPT);
+        }
+      }
+    }
+    __syncwarp(gmask);
+  };
+
+  // The recurrence of Eq. 1 for every real-time task in rank order under analysis MODE, once the
+  // tasks sit in the lanes of their ranks: Sr = 2*eps*eta (GCAPS) or (L+theta)*slices (RR) of this
+  // lane's tasks, info[rank].z = base.  Writes out_wcrt (unless null in a sweep) and out_sched.
+  auto recurrence = [&](auto mode_tag, i64 *out_wcrt, uint8_t *out_sched) {
+  constexpr int MODE = mode_tag;  // a ModeTag: every analysis of a kernel gets its own copy
+  const int n_rt = n_rt_all;
+  // by rank from here on: period - 1, C+G^m, G^e, core, position, GPU-using, and the two weights
+  // of the analysis' pairs
+  u32 Tm1[SLOTS], Ar[SLOTS], Ger[SLOTS], pos_of[SLOTS], core[SLOTS], Wa[SLOTS], Wb[SLOTS];
+  bool gpu[SLOTS];
+  u32 magic[SLOTS], shift[SLOTS];  // reciprocal of T_h, made when the slot is first needed
+  int slots_made = 0;
+#pragma unroll
+  for (int s = 0; s < SLOTS; ++s) {
+    const int r = lane + LPT * s;
+    const uint4 x = r < n ? xch[r] : make_uint4(2u, 0u, 0u, 0u);
+    const uint4 f = r < n ? info[r] : make_uint4(0u, 0xffffffffu, 0u, 0u);
+    const u32 Sr = x.w;  // 2*eps*eta (GCAPS) or (L+theta)*slices (RR) of this rank's task
+    Tm1[s] = x.x - 1, Ar[s] = x.y, Ger[s] = x.z;
+    core[s] = f.y, pos_of[s] = f.w & 0xffffu, gpu[s] = (f.w & 0x10000u) != 0;
+    magic[s] = 0, shift[s] = 0;
+    if (MODE == 0) {
+      Wa[s] = Ar[s] + (gpu[s] ? Sr : 0u);    // Lemma 15: C_h, or C_h + G^{m*}_h
+      Wb[s] = gpu[s] ? Ger[s] + Sr : 0u;     // Lemma 13, other cores: G^{e*}_h
+    } else if (MODE == 1) {
+      Wa[s] = Ar[s];                            // Lemma 12
+      Wb[s] = gpu[s] ? Ger[s] + Sr : 0u;     // Lemmas 10, 11: G^{e*}_h
+    } else {
+      Wa[s] = Ar[s];                            // Lemmas 5, 7
+      Wb[s] = gpu[s] ? Sr : 0u;              // Lemma 4: (L+theta) * slices
+    }
+  }
+
+  // ---- iterate in rank order ------------------------------------------------------------------
+  u32 Jc[SLOTS], Jg[SLOTS];               // jitters with T_h - 1 folded in (ceiling)
+#pragma unroll
+  for (int s = 0; s < SLOTS; ++s) Jc[s] = Jg[s] = Tm1[s];
+  int n_done = n_rt;
+  int verdict = 0;
+  for (int pos = 0; pos < n_rt; ++pos) {
+    const uint4 f = info[pos];
+    const u32 Di = f.x, core_i = f.y, base_i = f.z;
+    const bool gi = (f.w & 0x10000u) != 0;
+    const int smax = (pos - 1) >> kLog;  // -1 for the first task: nothing interferes
+    if (smax >= slots_made) {              // the first task that looks at slot smax
+#pragma unroll
+      for (int s = 0; s < SLOTS; ++s)
+        if (s == smax) make_reciprocal(Tm1[s] + 1, magic[s], shift[s]);
+      slots_made = smax + 1;
+    }
+    u32 nu = 0;
+    if (MODE == 3) {  // Lemma 4: N_g - |{h in hpp(i): GPU-using}| + 1
+      int c = 0;
+#pragma unroll
+      for (int s = 0; s < SLOTS; ++s)
+        if (s <= smax) c += __popc(__ballot_sync(gmask, lane + LPT * s < pos && core[s] == core_i && gpu[s]));
+      nu = (u32)(n_gpu - c + 1);
+    }
+    // the (J, W) pairs of this task's interferers; W = 0 where a pair does not apply
+    u32 J1[SLOTS], W1[SLOTS], W2[SLOTS];
+#pragma unroll
+    for (int s = 0; s < SLOTS; ++s) {
+      J1[s] = 0, W1[s] = 0, W2[s] = 0;
+      if (s <= smax) {
+        const bool act = lane + LPT * s < pos;
+        const bool same = core[s] == core_i;
+        u32 w1, w2 = 0, j1;
+        if (MODE == 0) {
+          w1 = same ? Wa[s] : (gi ? Wb[s] : 0u);           // Lemma 15 / Lemma 13 (other cores)
+          j1 = same ? Jc[s] : Jg[s];
+          w2 = (same && gi && gpu[s]) ? Ger[s] : 0u;       // Lemma 13 (same core), jitter J^g
+        } else if (MODE == 1) {
+          w1 = same ? Wa[s] + ((gi || !literal) ? Wb[s] : 0u) : Wb[s];  // Lemmas 12+10 / 10, 11
+          j1 = same ? Tm1[s] : Jg[s];
+        } else if (MODE == 2) {
+          w1 = same ? Wa[s] : 0u;                          // Lemma 7
+          j1 = Jc[s];
+        } else {
+          const u64 w = (u64)Wa[s] + (u64)Wb[s] * nu;      // Lemmas 5 and 4
+          w1 = same ? (w > kFastClamp ? kFastClamp : (u32)w) : 0u;
+          j1 = Tm1[s];
+        }
+        J1[s] = j1, W1[s] = act ? w1 : 0u, W2[s] = act ? w2 : 0u;
+      }
+    }
+    u32 R = base_i;
+    int v = 0;
+    int sweeps = 0;
+    for (;;) {
+      if (R > Di) {
+        v = GCAPS_WCRT_MISS;
+        break;
+      }
+      if (sweeps >= (int)GCAPS_RTA_ITER_CAP) {
+        v = GCAPS_WCRT_ITER_LIMIT;
+        break;
+      }
+      sweeps += 1;
+      u32 next = base_i;
+      if (smax >= 0) {
+        u64 acc = 0;
+#pragma unroll
+        for (int s = 0; s < SLOTS; ++s) {
+          if (s <= smax) {
+            acc += (u64)(__umulhi(R + J1[s], magic[s]) >> shift[s]) * W1[s];
+            if (MODE == 0) acc += (u64)(__umulhi(R + Jg[s], magic[s]) >> shift[s]) * W2[s];
+          }
+        }
+        const u32 part = acc > (u64)kFastClamp ? kFastClamp : (u32)acc;
+        next += __reduce_add_sync(gmask, part);
+      }
+      if (next == R) break;
+      R = next;
+    }
+    if (v != 0) {
+      n_done = pos;
+      verdict = v;
+      break;
+    }
+    // publish: the owner writes R_i and forms its jitters J^c = R - (C+G^m), J^g = R - G^e (a
+    // CPU-only task has no J^c unless the printed form of Lemma 7 is asked for)
+#pragma unroll
+    for (int s = 0; s < SLOTS; ++s) {
+      if (lane + LPT * s == pos) {
+        if (!SWEEP || out_wcrt) out_wcrt[a + pos_of[s]] = (i64)R;
+        if (MODE == 0 ? gpu[s] : (MODE == 2 ? (gpu[s] || literal) : false)) Jc[s] = R - Ar[s] + Tm1[s];
+        Jg[s] = R - Ger[s] + Tm1[s];
+      }
+    }
+  }
+  // ---- write the sentinels of the tasks that did not converge ---------------------------------
+  if (!SWEEP || out_wcrt) {
+#pragma unroll
+    for (int s = 0; s < SLOTS; ++s) {
+      const int r = lane + LPT * s;
+      if (r < n && r >= n_done)
+        out_wcrt[a + pos_of[s]] = r >= n_rt ? (i64)GCAPS_WCRT_BEST_EFFORT
+                                          : (r == n_done ? (i64)verdict : (i64)GCAPS_WCRT_SKIPPED);
+    }
+  }
+  if (lane == 0) out_sched[t] = verdict == 0 ? GCAPS_SCHED_YES : GCAPS_SCHED_NO;
+  __syncwarp(gmask);
+  };  // recurrence
+
+  if constexpr (!SWEEP) {
+    // ---- one analysis: constants by position, then everything moves to the rank's lane ---------
+    constexpr int MODE = (MASK & 1) ? 0 : (MASK & 2) ? 1 : (MASK & 4) ? 2 : 3;
+    constexpr bool kGcaps = MODE < 2;
+    const u32 ovh = (u32)p.ovh;  // the fast path needs eps, theta < 2^20
+    u32 sl[SLOTS];               // RR: slices of the task's pure GPU parts (Eq. 3)
+#pragma unroll
+    for (int s = 0; s < SLOTS; ++s) sl[s] = 0;
+    if (!kGcaps) {
+      slice_sums(Q0, p.L, p.l_mode, p.l_magic, p.l_shift);
+      __syncwarp(gmask);
+#pragma unroll
+      for (int s = 0; s < SLOTS; ++s) sl[s] = Q0[g1[s] - 1 + pare] - Q0[g0[s] - 1 + pare];
+      __syncwarp(gmask);
+    }
+    u32 base[SLOTS];
+#pragma unroll
+    for (int s = 0; s < SLOTS; ++s) {
+      if (kGcaps) {
+        S[s] = 2 * ovh * eta[s];                                 // eta < 64: below 2^27
+        base[s] = A[s] + Ge[s] + S[s] + (eta[s] + 1) * ovh;        // C_i + G*_i + B^C_i, below 2^29
+      } else {
+        const u64 slices = sl[s];
+        const u64 lt = (u64)p.L + ovh;  // <= 2^41
+        u64 B = slices == 0 ? 0 : (lt >= kFastClamp ? kFastClamp : lt * slices);  // < 2^26 * 2^32
+        if (B > kFastClamp) B = kFastClamp;
+        S[s] = (u32)B;
+        const u64 b64 = (u64)A[s] + Ge[s] + (eta[s] > 0 ? B * (u64)(n_gpu - 1) : 0);  // Lemma 1
+        base[s] = b64 > (u64)(2 * kFastClamp) ? 2 * kFastClamp : (u32)b64;
+      }
+      base[s] = base[s] > 2 * kFastClamp ? 2 * kFastClamp : base[s];
+    }
+    __syncwarp(gmask);
+#pragma unroll
+    for (int s = 0; s < SLOTS; ++s) {
+      if (lane + LPT * s < n) {
+        *(reinterpret_cast<uint2 *>(&info[rank[s]]) + 1) =
+            make_uint2(base[s], (u32)(lane + LPT * s) | (eta[s] > 0 ? 0x10000u : 0u));
+        xch[rank[s]] = make_uint4(T[s], A[s], Ge[s], S[s]);
+      }
+    }
+    __syncwarp(gmask);
+    recurrence(ModeTag<MODE>(), p.out_wcrt, p.out_sched);
+  } else {
+    // ---- several analyses: the tasks move to the rows of their ranks once; for every analysis
+    // the lane of a rank then makes that task's S and base from the row and the recurrence
+    // starts from the rows again, so nothing per task is held in registers across analyses ------
+    // second row by rank: GPU segment range (11 bits each) and number of GPU segments (6 bits)
+    // packed in .x, slices of Eq. 3 for the timeslice sl_L in .y
+    uint2 *xch2 = reinterpret_cast<uint2 *>(Q0 + 4 * MAXN);
+    static_assert(Lay::CAP <= 2048 && Lay::CAP >= 6 * MAXN, "packed segment range, room for the second row");
+#pragma unroll
+    for (int s = 0; s < SLOTS; ++s) {
+      if (lane + LPT * s < n) {
+        info[rank[s]].w = (u32)(lane + LPT * s) | (eta[s] > 0 ? 0x10000u : 0u);
+        xch[rank[s]] = make_uint4(T[s], A[s], Ge[s], 0u);
+        xch2[rank[s]] = make_uint2((u32)g0[s] | ((u32)g1[s] << 11) | (eta[s] << 22), 0u);
+      }
+    }
+    __syncwarp(gmask);
+    i64 sl_L = -1;
+    constexpr bool kMultiModes = (MASK & (MASK - 1)) != 0;
+    const int enabled = kMultiModes ? sw->enabled : MASK;
+    for (int q = 0; q < sw->n; ++q) {
+      const i64 L64 = sw->q[q].L;
+      const u32 ovh = (u32)sw->q[q].ovh;  // the fast path needs eps, theta < 2^20
+      auto analyse_as = [&](auto mode_tag) {
+        constexpr int MODE = mode_tag;
+        constexpr bool kGcaps = MODE < 2;
+        const int block = q * sw->block_stride + sw->block_of_mode[MODE];
+        i64 *const out_wcrt = p.out_wcrt ? p.out_wcrt + (i64)block * p.n_tasks : nullptr;
+        uint8_t *const out_sched = p.out_sched + (i64)block * p.n_tasksets;
+        if (!kGcaps && L64 != sl_L) {
+          sl_L = L64;
+          slice_sums(Q1, L64, sw->q[q].l_mode, sw->q[q].l_magic, sw->q[q].l_shift);
+          __syncwarp(gmask);
+#pragma unroll
+          for (int s = 0; s < SLOTS; ++s) {
+            const int r = lane + LPT * s;
+            if (r < n) {
+              const u32 g = xch2[r].x;
+              xch2[r].y = Q1[(int)((g >> 11) & 0x7ffu) - 1 + pare] - Q1[(int)(g & 0x7ffu) - 1 + pare];
+            }
+          }
+        }
+#pragma unroll
+        for (int s = 0; s < SLOTS; ++s) {
+          const int r = lane + LPT * s;
+          if (r < n) {
+            const uint4 x = xch[r];
+            const uint2 g = xch2[r];
+            const u32 eta_r = g.x >> 22;
+            u32 Sr, base;
+            if (kGcaps) {
+              Sr = 2 * ovh * eta_r;                                 // eta < 64: below 2^27
+              base = x.y + x.z + Sr + (eta_r + 1) * ovh;             // C_i + G*_i + B^C_i, below 2^29
+            } else {
+              const u64 slices = g.y;
+              const u64 lt = (u64)L64 + ovh;  // <= 2^41
+              u64 B = slices == 0 ? 0 : (lt >= kFastClamp ? kFastClamp : lt * slices);
+              if (B > kFastClamp) B = kFastClamp;
+              Sr = (u32)B;
+              const u64 b64 = (u64)x.y + x.z + (eta_r > 0 ? B * (u64)(n_gpu - 1) : 0);  // Lemma 1
+              base = b64 > (u64)(2 * kFastClamp) ? 2 * kFastClamp : (u32)b64;
+            }
+            base = base > 2 * kFastClamp ? 2 * kFastClamp : base;
+            xch[r].w = Sr;
+            info[r].z = base;
+          }
+        }
+        __syncwarp(gmask);
+        recurrence(mode_tag, out_wcrt, out_sched);
+      };
+      if ((MASK & 1) && (enabled & 1)) analyse_as(ModeTag<0>());
+      if ((MASK & 2) && (enabled & 2)) analyse_as(ModeTag<1>());
+      if ((MASK & 4) && (enabled & 4)) analyse_as(ModeTag<2>());
+      if ((MASK & 8) && (enabled & 8)) analyse_as(ModeTag<3>());
+    }
+  }
+  return kFastDone;
+}
+
+__device__ __forceinline__ void prefetch_l2(const void *ptr) {
+  asm volatile("prefetch.global.L2 [%0];" ::"l"(ptr));
+}
+
+// What a warp knows in advance about one taskset of a chunk (kept in shared memory).
+struct Ahead {
+  i64 a;           // first task
+  i64 c_lo, g_lo;  // first CPU segment, first GPU segment
+  u32 t;           // taskset index
+  u32 packed;      // tasks (bits 0-8) | CPU segments (9-19) | GPU segments (20-30) | fast (31)
+};
+static_assert(sizeof(Ahead) == 32, "two 16-byte rows");
+constexpr int kMaxAhead = 16;  // tasksets of one pull
+constexpr int kAheadWords = 2 * kMaxAhead * (int)(sizeof(Ahead) / sizeof(u32));  // two chunks
+
+// blocks per SM the register allocation aims at: more warps in flight matter more here than a
+// few spilled values, because every phase is a chain of dependent instructions and the loads of
+// a taskset can only be hidden behind the work of other warps
+__host__ __device__ constexpr int min_blocks(int slots) {
+  return slots <= 3 ? 6 : slots == 4 ? 4 : slots == 6 ? 3 : 2;
+}
+
+// One size bin, worked through by all warps of a persistent launch.  A warp is 32/LPT groups of
+// LPT lanes; every group analyses one taskset at a time.  Warps pull chunks of taskset indices
+// from the bin's counter; the index, task range and first segment offsets of the next chunk are
+// fetched while the current one is analysed.
+template <int LPT, int SLOTS, int MASK, bool SWEEP = false>
+__device__ __forceinline__ void run_bin(const KParams &p, int bin, u32 *warp_buf, Ahead *ahead,
+                                        const SweepArgs *sw = nullptr) {
+  typedef FastLayout<LPT, SLOTS> Lay;
+  constexpr int MAXN = LPT * SLOTS;
+  constexpr int G = 32 / LPT;  // groups per warp
+  static_assert(sizeof(GroupSmem<MAXN>) <= sizeof(u32) * Lay::kWords, "exact path fits");
+  const int lane32 = threadIdx.x & 31, group = lane32 / LPT, lane = lane32 % LPT;
+  const unsigned int gmask = LPT == 32 ? kFull : (((1u << LPT) - 1u) << (group * LPT));
+  u32 *buf = warp_buf + group * Lay::kWords;
+  const unsigned int start = p.hdr->bin_start[bin], count = p.hdr->bin_count[bin];
+  if (count == 0) return;
+  // keeps 2*eps*eta and (eta+1)*eps in 32 bits
+  const bool fast_call = (SWEEP ? sw->max_ovh : p.ovh) < (1 << 20);
+  // tasksets per pull: up to 8 per group when the bin is large, fewer when that would leave warps
+  // without work
+  const unsigned int n_groups = gridDim.x * (kBlockThreads / 32) * G;
+  const int rounds = count >= 32 * n_groups ? (G == 1 ? 8 : kMaxAhead / G)
+                                            : (count >= 8 * n_groups ? 4 / (G > 2 ? 2 : 1) : 1);
+  const int chunk = rounds * G;  // <= kMaxAhead
+
+  // lanes 0..chunk-1 each look up one taskset of a chunk and leave what they found in `slot`
+  auto look_up = [&](unsigned int first, Ahead *slot) {
+    if (lane32 < chunk) {
+      Ahead me;
+      me.a = 0, me.c_lo = me.g_lo = 0, me.t = 0, me.packed = 0;
+      if (first < count && first + lane32 < count) {
+        me.t = p.perm[start + first + lane32];
+        me.a = p.task_off[me.t] - p.task_base;
+        const i64 b = p.task_off[(i64)me.t + 1] - p.task_base;
+        if (me.a >= 0 && b > me.a && b <= p.n_tasks && b - me.a <= MAXN) {
+          u32 nc = 0, ng = 0;
+          me.c_lo = p.cseg_off[me.a] - p.cseg_base, me.g_lo = p.gseg_off[me.a] - p.gseg_base;
+          const i64 c_hi = p.cseg_off[b] - p.cseg_base, g_hi = p.gseg_off[b] - p.gseg_base;
+          if (me.c_lo >= 0 && c_hi <= p.n_csegs && c_hi - me.c_lo < Lay::CAP && c_hi > me.c_lo)
+            nc = (u32)(c_hi - me.c_lo);
+          if (me.g_lo >= 0 && g_hi <= p.n_gsegs && g_hi - me.g_lo < Lay::CAP && g_hi > me.g_lo)
+            ng = (u32)(g_hi - me.g_lo);
+          me.packed = (u32)(b - me.a) | (nc << 9) | (ng << 20) | 0x80000000u;
+        }
+      }
+      slot[lane32] = me;
+    }
+    __syncwarp();
+  };
+  static_assert(MAXN <= 256 && Lay::CAP <= 2048, "fields of Ahead::packed");
+
+  int undecided_run = 0, tried_since = 0;  // (the first ranks' own pass, see below)
+  unsigned int first = 0;
+  if (lane32 == 0) first = atomicAdd(&p.hdr->next[bin], (unsigned int)chunk);
+  first = __shfl_sync(kFull, first, 0);
+  int which = 0;
+  look_up(first, ahead);
+  while (first < count) {
+    unsigned int nfirst = 0;
+    if (lane32 == 0) nfirst = atomicAdd(&p.hdr->next[bin], (unsigned int)chunk);
+    const Ahead *cur = ahead + which * kMaxAhead;
+    Ahead *nxt = ahead + (which ^ 1) * kMaxAhead;
+    const int in_chunk = count - first < (unsigned int)chunk ? (int)(count - first) : chunk;
+    const int in_rounds = (in_chunk + G - 1) / G;
+    for (int c = 0; c < in_rounds; ++c) {
+      if (c == 1 || in_rounds == 1) {  // the next chunk's index has arrived by now
+        nfirst = __shfl_sync(kFull, nfirst, 0);
+        look_up(nfirst, nxt);
+      }
+      const int mine = c * G + group;
+      if (mine < in_chunk) {
+        const Ahead me = cur[mine];
+        const i64 t = (i64)me.t;
+        const int n = (int)(me.packed & 0x1ffu), nc = (int)((me.packed >> 9) & 0x7ffu);
+        const int ng = (int)((me.packed >> 20) & 0x7ffu);
+        // the segment slices start their way into L2 now; the per-task loads follow at once, so
+        // that the running sums later wait for L2 rather than for DRAM (16 elements per line,
+        // only addresses inside the arrays)
+        for (int e = 16 * lane; e < nc; e += 16 * LPT) prefetch_l2(p.cseg_wcet + me.c_lo + e);
+        for (int e = 16 * lane; e < ng; e += 16 * LPT)
+          prefetch_l2(p.gseg_misc + me.g_lo + e), prefetch_l2(p.gseg_exec + me.g_lo + e);
+        bool done = false;
+        if (fast_call && (me.packed >> 31) != 0) {
+          int how = kFastUndecided;
+          if constexpr (LPT == 32 && !SWEEP && (MASK & 12) != 0) {
+            // Far from schedulable, a taskset ends with a miss among its first ranks; nearly
+            // schedulable, looking at them first is wasted.  Tasksets of a batch tend to be alike:
+            // after four undecided ones in a row only every sixteenth taskset is tried that way.
+            // (Round robin only: with tens of GPU-using tasks taking turns on the GPU the first or
+            // second rank already misses, and the pass pays; under GCAPS the first miss comes a few
+            // ranks later and the pass was measured slower than the full one.)
+            if (undecided_run < 4 || (tried_since & 15) == 0) {
+              how = analyse_fast<LPT, SLOTS, MASK, false, true>(p, t, me.a, n, buf, lane, gmask);
+              undecided_run = how == kFastUndecided ? undecided_run + 1 : 0;
+              __syncwarp(gmask);
+            }
+            tried_since += 1;
+          }
+          if (how == kFastUndecided) how = analyse_fast<LPT, SLOTS, MASK, SWEEP>(p, t, me.a, n, buf, lane, gmask, sw);
+          done = how == kFastDone;
+        }
+        __syncwarp(gmask);
+        if (!done && !SWEEP) {
+          // the exact path reads task_off again and validates everything itself
+          analyse_taskset<LPT, MAXN>(p, t, *reinterpret_cast<GroupSmem<MAXN> *>(buf), lane, gmask);
+        }
+        if (!done && SWEEP) {  // the exact path once per (timeslice, overhead) pair
+          constexpr bool kMulti = (MASK & (MASK - 1)) != 0;
+          const int enabled = kMulti ? sw->enabled : MASK;
+          for (int q = 0; q < sw->n; ++q) {
+            for (int m = 0; m < 4; ++m) {
+              if (!((MASK & enabled) >> m & 1)) continue;
+              const int block = q * sw->block_stride + sw->block_of_mode[m];
+              KParams pq = p;
+              pq.policy = (p.policy & ~(0xff | GCAPS_RTA_BUSY)) | (m >= 2 ? GCAPS_POLICY_RR : GCAPS_POLICY_GCAPS) |
+                          ((m & 1) ? GCAPS_RTA_BUSY : 0);
+              pq.L = sw->q[q].L, pq.ovh = sw->q[q].ovh;
+              pq.out_wcrt = p.out_wcrt ? p.out_wcrt + (i64)block * p.n_tasks : nullptr;
+              pq.out_sched = p.out_sched + (i64)block * p.n_tasksets;
+              analyse_taskset<LPT, MAXN>(pq, t, *reinterpret_cast<GroupSmem<MAXN> *>(buf), lane, gmask);
+              __syncwarp(gmask);
+            }
+          }
+        }
+      }
+      __syncwarp();
+    }
+    first = nfirst;
+    which ^= 1;
+  }
+}
+
+// shared memory of one warp for the bins a kernel covers
+template <int LPT, int SLOTS>
+__host__ __device__ constexpr int bin_warp_words() {
+  return (32 / LPT) * FastLayout<LPT, SLOTS>::kWords;
+}
+__host__ __device__ constexpr int cmax(int a, int b) { return a > b ? a : b; }
+constexpr int kSmallWarpWords =
+    cmax(cmax(bin_warp_words<8, 1>(), bin_warp_words<8, 2>()),
+         cmax(bin_warp_words<8, 3>(), bin_warp_words<16, 2>())) + kAheadWords;
+
+}  // namespace
+#endif  // GCAPS_RTA_DEVICE_CUH_
