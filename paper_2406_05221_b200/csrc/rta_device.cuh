@@ -33,6 +33,7 @@
 #include <stdint.h>
 
 #include "rta_common.cuh"
+#include "rta_recurrence.cuh"
 
 namespace {
 
@@ -291,29 +292,15 @@ __device__ __forceinline__ bool slice_is_inside(i64 first, int N, int par, i64 t
   return (par == 0 || first >= 1) && ((((N + par) & 1) == 0) || first + N < total);
 }
 
-template <int LPT, int SLOTS>
-struct FastLayout {
-  static constexpr int MAXN = LPT * SLOTS;
-  static constexpr int kStep = 4 * LPT;  // elements one prefix step of the group covers
-  // a prefix array takes slices of up to CAP-1 elements and is written kStep words at a time
-  static constexpr int CAP = (6 * MAXN + kStep - 1) / kStep * kStep;
-  static constexpr int kInfo = 0;  // uint4 per rank: deadline, core, base, position | GPU flag
-  static constexpr int kQ0 = 4 * MAXN + 4;
-  static constexpr int kQ1 = kQ0 + CAP + 4;
-  static constexpr int kFastWords = kQ1 + CAP;
-  static constexpr int kExactWords = (17 * MAXN + 3) / 4 * 4;  // the exact path: 66 B per task
-  static constexpr int kWords = kFastWords > kExactWords ? kFastWords : kExactWords;
-  static_assert(kWords % 4 == 0 && CAP % kStep == 0 && 4 * MAXN <= CAP, "16-byte aligned rows");
-};
-
 // One step (NB blocks of 4*LPT elements) of the running sums of up to two arrays that share their
-// offsets, by a group of LPT lanes (`gmask`).
+// offsets, by a group of LPT lanes.  Called by the whole warp (its groups step side by side; a
+// group whose slice has ended reads nothing and stores nothing).
 template <int LPT, int NB, bool TWO>
 __device__ __forceinline__ void prefix_step(const i64 *__restrict__ X0, const i64 *__restrict__ X1,
                                             int e0, int N, int par0, int par1, bool inside,
                                             const i64 *lo0, const i64 *hi0, const i64 *lo1,
                                             const i64 *hi1, u32 *Q0, u32 *Q1, u32 &carry0,
-                                            u32 &carry1, u32 &bad, int lane, unsigned int gmask) {
+                                            u32 &carry1, u32 &bad, int lane) {
   Quad q0[NB], q1[NB];
   u32 x0[NB][4], x1[NB][4], i0[NB], i1[NB];
   if (inside) {
@@ -339,32 +326,42 @@ __device__ __forceinline__ void prefix_step(const i64 *__restrict__ X0, const i6
     }
   }
 #pragma unroll
-  for (int d = 1; d < LPT; d <<= 1) {  // the warp scans of all blocks side by side
+  for (int d = 1; d < LPT; d <<= 1) {  // the scans of all blocks side by side
 #pragma unroll
     for (int b = 0; b < NB; ++b) {
-      const u32 y0 = __shfl_up_sync(gmask, i0[b], d, LPT);
+      const u32 y0 = __shfl_up_sync(kFull, i0[b], d, LPT);
       if (lane >= d) i0[b] += y0;
       if (TWO) {
-        const u32 y1 = __shfl_up_sync(gmask, i1[b], d, LPT);
+        const u32 y1 = __shfl_up_sync(kFull, i1[b], d, LPT);
         if (lane >= d) i1[b] += y1;
       }
     }
   }
 #pragma unroll
   for (int b = 0; b < NB; ++b) {
-    if (e0 + 4 * LPT * b < N + 1) {
-      const u32 b0 = i0[b] - x0[b][3] + carry0;
+    const bool wanted = e0 + 4 * LPT * b < N + 1;
+    if (LPT == 32 && !wanted) break;  // (the same in every lane)
+    const u32 b0 = i0[b] - x0[b][3] + carry0;
+    if (wanted)
       *reinterpret_cast<uint4 *>(Q0 + e0 + 4 * LPT * b + 4 * lane) =
           make_uint4(x0[b][0] + b0, x0[b][1] + b0, x0[b][2] + b0, x0[b][3] + b0);
-      carry0 += __shfl_sync(gmask, i0[b], LPT - 1, LPT);
-      if (TWO) {
-        const u32 b1 = i1[b] - x1[b][3] + carry1;
+    carry0 += __shfl_sync(kFull, i0[b], LPT - 1, LPT);
+    if (TWO) {
+      const u32 b1 = i1[b] - x1[b][3] + carry1;
+      if (wanted)
         *reinterpret_cast<uint4 *>(Q1 + e0 + 4 * LPT * b + 4 * lane) =
             make_uint4(x1[b][0] + b1, x1[b][1] + b1, x1[b][2] + b1, x1[b][3] + b1);
-        carry1 += __shfl_sync(gmask, i1[b], LPT - 1, LPT);
-      }
+      carry1 += __shfl_sync(kFull, i1[b], LPT - 1, LPT);
     }
   }
+}
+
+// True while the group's slice of N elements has elements at or behind e0 (a warp per taskset), or
+// while any group of the warp does.
+template <int LPT>
+__device__ __forceinline__ bool more_steps(int e0, int N) {
+  if constexpr (LPT == 32) return e0 < N;
+  return __any_sync(kFull, e0 < N);
 }
 
 // Range check of segment slices without running sums: `bad` collects whether a wanted element lies
@@ -588,14 +585,12 @@ struct ModeTag {
 };
 
 // MODE: 0 GCAPS self-suspension, 1 GCAPS busy-waiting, 2 RR self-suspension, 3 RR busy-waiting.
-// Returns false, having written nothing, if the taskset is not eligible for 32-bit arithmetic
-// (or is invalid): the caller then runs the exact 64-bit path, which also does the validation.
 //
-// A group of LPT lanes (8, 16 or a whole warp) works on one taskset.  Until the per-task sums are
-// known lane l of the group holds the tasks at positions l, l+LPT, ... ("slots").
-// Then every task's values move through shared memory to the lane that owns its rank, so that the
-// interferers of the task of rank `pos` sit in lanes (pos-1) % LPT downwards of slots up to
-// (pos-1) / LPT and higher slots can be skipped.
+// A group of LPT lanes (8, 16 or a whole warp) works on one taskset; the whole warp calls this and
+// its groups go through every step side by side (`live`: the group has a taskset), so that each
+// shuffle, vote and reduction is one instruction for all of them.  Until the per-task sums are
+// known lane l of a group holds the tasks at positions l, l+LPT, ... ("slots"); then every task's
+// values go to the row of its rank in shared memory, where the recurrence finds them.
 //
 // MASK: bit m set = analysis MODE m is compiled in.  SWEEP: the taskset is staged, ordered and
 // aggregated once and then analysed under every (timeslice, overhead) pair q of `sw` and every
@@ -604,17 +599,17 @@ struct ModeTag {
 // is null; out_sched + block * n_tasksets).  Without SWEEP, MASK has one bit and the analysis
 // takes its constants and outputs from `p`.
 //
-// Returns kFastDone (outputs written), kFastDeclined (nothing written that matters: the caller runs
-// the exact path) or, with FIRST_ONLY, kFastUndecided.  FIRST_ONLY (one analysis, a warp per
-// taskset): only the first ranks of the priority order are analysed (first_ranks below); if they
-// all converge and more ranks follow, nothing is decided and the caller runs the full pass.
+// Returns, per group, kFastDone (outputs written), kFastDeclined (some value does not fit the
+// 32-bit path or the taskset is invalid; nothing written: the caller runs the exact path) or, with
+// FIRST_ONLY, kFastUndecided.  FIRST_ONLY (one analysis, a warp per taskset): only the first ranks
+// of the priority order are analysed (first_ranks below); if they all converge and more ranks
+// follow, nothing is decided and the caller runs the full pass.
 constexpr int kFastDeclined = 0, kFastDone = 1, kFastUndecided = 2;
 template <int LPT, int SLOTS, int MASK, bool SWEEP = false, bool FIRST_ONLY = false>
-__device__ __forceinline__ int analyse_fast(const KParams &p, i64 t, i64 a, int n, u32 *buf, int lane,
+__device__ __forceinline__ int analyse_fast(const KParams &p, bool live, i64 t, i64 a, int n, u32 *buf, int lane,
                                             unsigned int gmask, const SweepArgs *sw = nullptr) {
   static_assert(!FIRST_ONLY || (LPT == 32 && !SWEEP), "the first ranks' own pass: a warp per taskset");
   typedef FastLayout<LPT, SLOTS> Lay;
-  constexpr int kLog = LPT == 32 ? 5 : LPT == 16 ? 4 : 3;  // log2 of the lanes per taskset
   constexpr int MAXN = Lay::MAXN, CAP = Lay::CAP;
   // prefix blocks of the CPU segments whose loads are issued together.  Tasksets of 65..96 tasks
   // with a few GPU segments per task have 200..400 CPU segments: three blocks of 128 cover them
@@ -627,32 +622,47 @@ __device__ __forceinline__ int analyse_fast(const KParams &p, i64 t, i64 a, int 
   static_assert(!kMulti || SWEEP, "several analyses per taskset use the sweep loop");
   const bool literal = (p.policy & GCAPS_RTA_LITERAL) != 0;
   const bool best_effort = (p.policy & GCAPS_RTA_BEST_EFFORT) != 0;
-  uint4 *info = reinterpret_cast<uint4 *>(buf + Lay::kInfo);
+  const Rows<LPT, SLOTS, SWEEP> rows{buf};
   u32 *Q0 = buf + Lay::kQ0, *Q1 = buf + Lay::kQ1;
+  // A group that has no taskset, or declines it, goes on as one with an empty taskset.
+#define GCAPS_LEAVE_IF_NONE_LIVE()                       \
+  do {                                                   \
+    if (LPT == 32 ? !live : !__any_sync(kFull, live)) return kFastDeclined; \
+    if (!live) n = 0, Nc = 0, Ng = 0;                    \
+  } while (0)
 
   // ---- stage: per-task scalars, lane = position; rank ----------------------------------------
   u32 T[SLOTS];
   int rank[SLOTS], c0[SLOTS], g0[SLOTS];
-  bool ok = true;
-  int Nc, Ng;
+  int Nc = 0, Ng = 0;
   i64 cfirst, gfirst;
   {
-    i64 t64[SLOTS], d64[SLOTS], pr[SLOTS], c64[SLOTS], co[SLOTS], go[SLOTS];
+    i64 t64[SLOTS], d64[SLOTS], pr[SLOTS], c64[SLOTS], co[SLOTS], go[SLOTS], cend = 0, gend = 0;
+    if (!live) n = 0;
+    {
+      const i64 k = a + lane;
+      const i64 *pT = p.period + k, *pD = p.deadline + k, *pP = p.priority + k, *pK = p.core + k;
+      const i64 *pc = p.cseg_off + k, *pg = p.gseg_off + k;
 #pragma unroll
-    for (int s = 0; s < SLOTS; ++s) {  // all loads of the taskset's per-task arrays in flight
-      const i64 k = a + (lane + LPT * s < n ? lane + LPT * s : 0);
-      t64[s] = p.period[k], d64[s] = p.deadline[k], pr[s] = p.priority[k], c64[s] = p.core[k];
-      co[s] = p.cseg_off[k], go[s] = p.gseg_off[k];
+      for (int s = 0; s < SLOTS; ++s) {  // all loads of the taskset's per-task arrays in flight
+        t64[s] = 2, d64[s] = 1, pr[s] = 0, c64[s] = 0, co[s] = 0, go[s] = 0;
+        if (lane + LPT * s < n) {
+          t64[s] = pT[LPT * s], d64[s] = pD[LPT * s], pr[s] = pP[LPT * s], c64[s] = pK[LPT * s];
+          co[s] = pc[LPT * s], go[s] = pg[LPT * s];
+        }
+      }
     }
-    const i64 cend = p.cseg_off[a + n] - p.cseg_base, gend = p.gseg_off[a + n] - p.gseg_base;
-    cfirst = __shfl_sync(gmask, co[0], 0, LPT) - p.cseg_base;
-    gfirst = __shfl_sync(gmask, go[0], 0, LPT) - p.gseg_base;
+    if (n > 0) cend = p.cseg_off[a + n] - p.cseg_base, gend = p.gseg_off[a + n] - p.gseg_base;
+    cfirst = __shfl_sync(kFull, co[0], 0, LPT) - p.cseg_base;
+    gfirst = __shfl_sync(kFull, go[0], 0, LPT) - p.gseg_base;
     const i64 Nc64 = cend - cfirst, Ng64 = gend - gfirst;
     if (cfirst < 0 || Nc64 < 0 || cend > p.n_csegs || Nc64 >= CAP || gfirst < 0 || Ng64 < 0 ||
         gend > p.n_gsegs || Ng64 >= CAP)
-      return kFastDeclined;
+      live = false;
     Nc = (int)Nc64, Ng = (int)Ng64;
+    GCAPS_LEAVE_IF_NONE_LIVE();
     u32 high = 0;  // any set bit: some value does not fit the 32-bit path
+    bool ok = true, any_wide = false;
     u32 D[SLOTS], core[SLOTS];
     int prio[SLOTS];
 #pragma unroll
@@ -662,7 +672,7 @@ __device__ __forceinline__ int analyse_fast(const KParams &p, i64 t, i64 a, int 
       const u32 h = (u32)((u64)t64[s] >> 32) | (u32)((u64)d64[s] >> 32) | (u32)((u64)c64[s] >> 32) |
                     (u32)((u64)rc >> 32) | (u32)((u64)rg >> 32) |
                     (u32)(((u64)pr[s] + 0x80000000ull) >> 32);
-      T[s] = v ? (u32)t64[s] : 2u;
+      T[s] = (u32)t64[s];
       D[s] = (u32)d64[s];
       core[s] = (u32)c64[s];
       prio[s] = v ? (int)pr[s] : (int)0x80000000;
@@ -670,15 +680,30 @@ __device__ __forceinline__ int analyse_fast(const KParams &p, i64 t, i64 a, int 
       g0[s] = v ? (int)rg : Ng;
       high |= v ? h : 0u;
       // 2 <= T < 2^26, 1 <= D <= T, core < 2^31, offsets inside the slice
-      ok &= T[s] - 2u < kFastLimit - 2u && (!v || (D[s] - 1u < T[s] && (int)core[s] >= 0)) &&
-            (u32)c0[s] <= (u32)Nc && (u32)g0[s] <= (u32)Ng;
+      ok &= !v || (T[s] - 2u < kFastLimit - 2u && D[s] - 1u < T[s] && (int)core[s] >= 0 && (u32)c0[s] <= (u32)Nc &&
+                   (u32)g0[s] <= (u32)Ng);
+      any_wide |= v && T[s] >= kNarrowLimit;
     }
-    if (__any_sync(gmask, high != 0 || !ok)) return kFastDeclined;  // (a wide priority also lands here)
+    live = group_all<LPT>(high == 0 && ok, gmask) && live;  // (a wide priority also lands here)
+    GCAPS_LEAVE_IF_NONE_LIVE();
+    if (LPT != 32 && !live) {
+#pragma unroll
+      for (int s = 0; s < SLOTS; ++s) c0[s] = g0[s] = 0, prio[s] = (int)0x80000000;
+    }
     // order: rank by (priority desc, position asc)
     int m = prio[0];
 #pragma unroll
     for (int s = 1; s < SLOTS; ++s) m = prio[s] > m ? prio[s] : m;
-    const int pmax = __reduce_max_sync(gmask, m);
+    int pmax = m;
+    if constexpr (LPT == 32) {
+      pmax = __reduce_max_sync(kFull, m);
+    } else {
+#pragma unroll
+      for (int d = 1; d < LPT; d <<= 1) {
+        const int o = __shfl_xor_sync(kFull, pmax, d);
+        pmax = o > pmax ? o : pmax;
+      }
+    }
     bool dense = true;  // distinct priorities max-n+1 .. max: the rank is max - priority
 #pragma unroll
     for (int s = 0; s < SLOTS; ++s) {
@@ -687,19 +712,20 @@ __device__ __forceinline__ int analyse_fast(const KParams &p, i64 t, i64 a, int 
       dense &= !v || r < (u32)n;
       rank[s] = v ? (int)r : MAXN;
     }
-    dense = __all_sync(gmask, dense);
+    dense = group_all<LPT>(dense, gmask);
     if (dense) {
 #pragma unroll
       for (int s = 0; s < SLOTS; ++s)
         if (lane + LPT * s < n) Q0[rank[s]] = (u32)(lane + LPT * s);
-      __syncwarp(gmask);
-      bool uniq = true;
+    }
+    __syncwarp();
+    bool uniq = true;
+    if (dense) {
 #pragma unroll
       for (int s = 0; s < SLOTS; ++s)
         if (lane + LPT * s < n) uniq &= Q0[rank[s]] == (u32)(lane + LPT * s);
-      dense = __all_sync(gmask, uniq);
-      __syncwarp(gmask);
     }
+    dense = group_all<LPT>(dense && uniq, gmask);
     if (!dense) {  // any priorities: count the tasks that come before
 #pragma unroll
       for (int s = 0; s < SLOTS; ++s) {
@@ -712,44 +738,61 @@ __device__ __forceinline__ int analyse_fast(const KParams &p, i64 t, i64 a, int 
         rank[s] = i < n ? r : MAXN;
       }
     }
+    __syncwarp();
     // best-effort tasks (flag set, priority <= 0) rank behind every real-time task: the ranks
-    // from n_rt on are theirs
-    // (kept in a spare word in front of Q0's guard entry until the recurrence starts)
+    // from n_rt on are theirs.  n_narrow: the ranks in front of the first period of kNarrowLimit or
+    // more.  (Both are kept in spare words in front of Q0's guard entry until the recurrence
+    // starts.)
     {
       int n_rt = n;
       if (best_effort) {
 #pragma unroll
         for (int s = 0; s < SLOTS; ++s)
-          n_rt -= __popc(__ballot_sync(gmask, lane + LPT * s < n && prio[s] <= 0));
+          n_rt -= __popc(__ballot_sync(kFull, lane + LPT * s < n && prio[s] <= 0) & gmask);
       }
-      if (lane == 0) Q0[-2] = (u32)n_rt;
+      int n_narrow = n_rt;
+      if (!FIRST_ONLY && __any_sync(kFull, any_wide)) {
+#pragma unroll
+        for (int s = 0; s < SLOTS; ++s)
+          if (lane + LPT * s < n && T[s] >= kNarrowLimit && rank[s] < n_narrow) n_narrow = rank[s];
+#pragma unroll
+        for (int d = 1; d < LPT; d <<= 1) {
+          const int o = __shfl_xor_sync(kFull, n_narrow, d);
+          n_narrow = o < n_narrow ? o : n_narrow;
+        }
+      }
+      if (lane == 0) Q0[-2] = (u32)n_rt, Q0[-3] = (u32)n_narrow;
     }
-    // what every lane must know about the task of a given rank (base and GPU flag follow; the
-    // first ranks' own pass keeps the period and the position there instead)
+    // what the row of a rank says about the task itself (the first ranks' own pass keeps the
+    // period and the position there instead)
 #pragma unroll
     for (int s = 0; s < SLOTS; ++s) {
       if constexpr (FIRST_ONLY) {
-        if (rank[s] < kFirstRanks) info[rank[s]] = make_uint4(D[s], core[s], T[s], (u32)(lane + LPT * s));
+        if (rank[s] < kFirstRanks) rows.a(rank[s]) = make_uint4(D[s], core[s], T[s], (u32)(lane + LPT * s));
       } else {
-        if (lane + LPT * s < n) *reinterpret_cast<uint2 *>(&info[rank[s]]) = make_uint2(D[s], core[s]);
+        if (lane + LPT * s < n) *reinterpret_cast<uint2 *>(&rows.a(rank[s])) = make_uint2(D[s], core[s]);
       }
     }
   }
   // end offsets: the next task's start (positions beyond n hold the total)
   int c1[SLOTS], g1[SLOTS];
+  {
+    bool ok = true;
 #pragma unroll
-  for (int s = 0; s < SLOTS; ++s) {
-    const int cn = __shfl_down_sync(gmask, c0[s], 1, LPT), gn = __shfl_down_sync(gmask, g0[s], 1, LPT);
-    const int ch = __shfl_sync(gmask, s + 1 < SLOTS ? c0[s + 1 < SLOTS ? s + 1 : s] : Nc, 0, LPT);
-    const int gh = __shfl_sync(gmask, s + 1 < SLOTS ? g0[s + 1 < SLOTS ? s + 1 : s] : Ng, 0, LPT);
-    c1[s] = lane == LPT - 1 ? ch : cn;
-    g1[s] = lane == LPT - 1 ? gh : gn;
-    ok &= (u32)(c1[s] - c0[s]) < 64u && (u32)(g1[s] - g0[s]) < 64u;
+    for (int s = 0; s < SLOTS; ++s) {
+      const int cn = __shfl_down_sync(kFull, c0[s], 1, LPT), gn = __shfl_down_sync(kFull, g0[s], 1, LPT);
+      const int ch = s + 1 < SLOTS ? __shfl_sync(kFull, c0[s + 1 < SLOTS ? s + 1 : s], 0, LPT) : Nc;
+      const int gh = s + 1 < SLOTS ? __shfl_sync(kFull, g0[s + 1 < SLOTS ? s + 1 : s], 0, LPT) : Ng;
+      c1[s] = lane == LPT - 1 ? ch : cn;
+      g1[s] = lane == LPT - 1 ? gh : gn;
+      ok &= (u32)(c1[s] - c0[s]) < 64u && (u32)(g1[s] - g0[s]) < 64u;
+    }
+    live = group_all<LPT>(ok, gmask) && live;
+    GCAPS_LEAVE_IF_NONE_LIVE();
   }
-  if (!__all_sync(gmask, ok)) return kFastDeclined;
 
   // ---- aggregate: running sums of the segment arrays; per-task sums are differences --------
-  u32 A[SLOTS], Ge[SLOTS], S[SLOTS];  // C+G^m, G^e, and 2*eps*eta (GCAPS) or (L+theta)*slices (RR)
+  u32 A[SLOTS], Ge[SLOTS];  // C+G^m, G^e
   u32 bad = 0;
   const i64 *__restrict__ Xc = p.cseg_wcet + cfirst;
   const i64 *__restrict__ Xm = p.gseg_misc + gfirst, *__restrict__ Xe = p.gseg_exec + gfirst;
@@ -757,37 +800,38 @@ __device__ __forceinline__ int analyse_fast(const KParams &p, i64 t, i64 a, int 
   const int pare = (int)(((uintptr_t)Xe >> 3) & 1);
   if constexpr (FIRST_ONLY) {
     constexpr int MODE = (MASK & 1) ? 0 : (MASK & 2) ? 1 : (MASK & 4) ? 2 : 3;
+    uint4 *info = reinterpret_cast<uint4 *>(buf + Lay::kInfo);
     uint4 *first8 = info + kFirstRanks;  // (only the first ranks' rows of `info` are used here)
 #pragma unroll
     for (int s = 0; s < SLOTS; ++s)
       if (rank[s] < kFirstRanks) first8[rank[s]] = make_uint4((u32)c0[s], (u32)c1[s], (u32)g0[s], (u32)g1[s]);
-    __syncwarp(gmask);
+    __syncwarp();
     const int r = first_ranks<SLOTS, MODE>(p, t, a, n, info, first8, Q0, Q1, (int)Q0[-2], rank, g0, g1, Xc, Xm, Xe,
                                            Nc, Ng, parc, parm, pare, cfirst, gfirst, lane, literal);
-    __syncwarp(gmask);
+    __syncwarp();
     return r > 0 ? kFastDone : (r == 0 ? kFastUndecided : kFastDeclined);
   }
   if (lane == 0) Q0[-1] = 0, Q1[-1] = 0;
   {  // CPU segments -> Q0
     const bool inside = slice_is_inside(cfirst, Nc, parc, p.n_csegs);
     u32 carry = 0, unused = 0;
-    for (int e0 = 0; e0 < Nc + parc; e0 += Lay::kStep * BC)
+    for (int e0 = 0; more_steps<LPT>(e0, Nc + parc); e0 += Lay::kStep * BC)
       prefix_step<LPT, BC, false>(Xc, Xc, e0, Nc, parc, parc, inside, p.cseg_wcet, p.cseg_wcet + p.n_csegs,
-                             p.cseg_wcet, p.cseg_wcet, Q0, Q0, carry, unused, bad, lane, gmask);
+                             p.cseg_wcet, p.cseg_wcet, Q0, Q0, carry, unused, bad, lane);
   }
-  __syncwarp(gmask);
+  __syncwarp();
 #pragma unroll
   for (int s = 0; s < SLOTS; ++s) A[s] = Q0[c1[s] - 1 + parc] - Q0[c0[s] - 1 + parc];
-  __syncwarp(gmask);
+  __syncwarp();
   {  // G^m -> Q0, G^e -> Q1
     const bool inside = slice_is_inside(gfirst, Ng, parm, p.n_gsegs) &&
                         slice_is_inside(gfirst, Ng, pare, p.n_gsegs);
     u32 cm = 0, ce = 0;
-    for (int e0 = 0; e0 < Ng + 1; e0 += Lay::kStep * BG)
+    for (int e0 = 0; more_steps<LPT>(e0, Ng + 1); e0 += Lay::kStep * BG)
       prefix_step<LPT, BG, true>(Xm, Xe, e0, Ng, parm, pare, inside, p.gseg_misc, p.gseg_misc + p.n_gsegs,
-                            p.gseg_exec, p.gseg_exec + p.n_gsegs, Q0, Q1, cm, ce, bad, lane, gmask);
+                            p.gseg_exec, p.gseg_exec + p.n_gsegs, Q0, Q1, cm, ce, bad, lane);
   }
-  __syncwarp(gmask);
+  __syncwarp();
   u32 eta[SLOTS];
 #pragma unroll
   for (int s = 0; s < SLOTS; ++s) {
@@ -798,28 +842,29 @@ __device__ __forceinline__ int analyse_fast(const KParams &p, i64 t, i64 a, int 
     A[s] += Gm;
     bad |= A[s] >> 26;
   }
-  __syncwarp(gmask);
+  __syncwarp();
   // ---- what does not depend on the timeslice or the overhead ---------------------------------
   int n_gpu = 0;  // N_g
 #pragma unroll
-  for (int s = 0; s < SLOTS; ++s) n_gpu += __popc(__ballot_sync(gmask, eta[s] > 0));
+  for (int s = 0; s < SLOTS; ++s) n_gpu += __popc(__ballot_sync(kFull, eta[s] > 0) & gmask);
   if (kAnyGcaps) {  // 2 * eps * eta must stay below 2^26 (eta < 64, eps < 2^20: no overflow here)
     const u32 ovh_max = SWEEP ? (u32)sw->max_ovh : (u32)p.ovh;
 #pragma unroll
     for (int s = 0; s < SLOTS; ++s) bad |= (2 * ovh_max * eta[s]) >> 26;
   }
-  if (__any_sync(gmask, bad != 0)) return kFastDeclined;
-  const int n_rt_all = (int)Q0[-2];  // real-time tasks: the ranks that are analysed
-  uint4 *xch = reinterpret_cast<uint4 *>(Q0);  // by rank: T, C+G^m, G^e, S  (Q0 is dead by now)
+  live = group_all<LPT>(bad == 0, gmask) && live;
+  if (LPT == 32 ? !live : !__any_sync(kFull, live)) return kFastDeclined;
+  if (!live) n = 0;
+  const int n_rt = live ? (int)Q0[-2] : 0;      // real-time tasks: the ranks that are analysed
+  const int n_narrow = live ? (int)Q0[-3] : 0;  // ... of which so many in single precision
 
   // Eq. 3: running sums of the slices of every pure GPU part for timeslice L (values already
   // checked) into Ps
   auto slice_sums = [&](u32 *Ps, i64 L64, u32 l_mode, u32 l_magic, u32 l_shift) {
-    // Eq. 3: slices of every pure GPU part, summed per task (values already checked)
     const bool inside = slice_is_inside(gfirst, Ng, pare, p.n_gsegs);
     u32 carry = 0;
     if (lane == 0) Ps[-1] = 0;
-    for (int e0 = 0; e0 < Ng + 1; e0 += Lay::kStep * BG) {
+    for (int e0 = 0; more_steps<LPT>(e0, Ng + 1); e0 += Lay::kStep * BG) {
       Quad qe[BG];
       u32 x[BG][4], incl[BG];
 #pragma unroll
@@ -845,233 +890,99 @@ __device__ __forceinline__ int analyse_fast(const KParams &p, i64 t, i64 a, int 
       for (int d = 1; d < LPT; d <<= 1) {
 #pragma unroll
         for (int b = 0; b < BG; ++b) {
-          const u32 y = __shfl_up_sync(gmask, incl[b], d, LPT);
+          const u32 y = __shfl_up_sync(kFull, incl[b], d, LPT);
           if (lane >= d) incl[b] += y;
         }
       }
 #pragma unroll
       for (int b = 0; b < BG; ++b) {
-        if (e0 + 4 * LPT * b < Ng + 1) {
-          const u32 before = incl[b] - x[b][3] + carry;
+        const u32 before = incl[b] - x[b][3] + carry;
+        if (e0 + 4 * LPT * b < Ng + 1)
           *reinterpret_cast<uint4 *>(Ps + e0 + 4 * LPT * b + 4 * lane) =
               make_uint4(x[b][0] + before, x[b][1] + before, x[b][2] + before, x[b][3] + before);
-          carry += __shfl_sync(gmask, incl[b], LPT - 1, LPT);
-        }
+        carry += __shfl_sync(kFull, incl[b], LPT - 1, LPT);
       }
     }
-    __syncwarp(gmask);
+    __syncwarp();
   };
 
-  // The recurrence of Eq. 1 for every real-time task in rank order under analysis MODE, once the
-  // tasks sit in the lanes of their ranks: Sr = 2*eps*eta (GCAPS) or (L+theta)*slices (RR) of this
-  // lane's tasks, info[rank].z = base.  Writes out_wcrt (unless null in a sweep) and out_sched.
-  auto recurrence = [&](auto mode_tag, i64 *out_wcrt, uint8_t *out_sched) {
-  constexpr int MODE = mode_tag;  // a ModeTag: every analysis of a kernel gets its own copy
-  const int n_rt = n_rt_all;
-  // by rank from here on: period - 1, C+G^m, G^e, core, position, GPU-using, and the two weights
-  // of the analysis' pairs
-  u32 Tm1[SLOTS], Ar[SLOTS], Ger[SLOTS], pos_of[SLOTS], core[SLOTS], Wa[SLOTS], Wb[SLOTS];
-  bool gpu[SLOTS];
-  u32 magic[SLOTS], shift[SLOTS];  // reciprocal of T_h, made when the slot is first needed
-  int slots_made = 0;
-#pragma unroll
-  for (int s = 0; s < SLOTS; ++s) {
-    const int r = lane + LPT * s;
-    const uint4 x = r < n ? xch[r] : make_uint4(2u, 0u, 0u, 0u);
-    const uint4 f = r < n ? info[r] : make_uint4(0u, 0xffffffffu, 0u, 0u);
-    const u32 Sr = x.w;  // 2*eps*eta (GCAPS) or (L+theta)*slices (RR) of this rank's task
-    Tm1[s] = x.x - 1, Ar[s] = x.y, Ger[s] = x.z;
-    core[s] = f.y, pos_of[s] = f.w & 0xffffu, gpu[s] = (f.w & 0x10000u) != 0;
-    magic[s] = 0, shift[s] = 0;
-    if (MODE == 0) {
-      Wa[s] = Ar[s] + (gpu[s] ? Sr : 0u);    // Lemma 15: C_h, or C_h + G^{m*}_h
-      Wb[s] = gpu[s] ? Ger[s] + Sr : 0u;     // Lemma 13, other cores: G^{e*}_h
-    } else if (MODE == 1) {
-      Wa[s] = Ar[s];                            // Lemma 12
-      Wb[s] = gpu[s] ? Ger[s] + Sr : 0u;     // Lemmas 10, 11: G^{e*}_h
-    } else {
-      Wa[s] = Ar[s];                            // Lemmas 5, 7
-      Wb[s] = gpu[s] ? Sr : 0u;              // Lemma 4: (L+theta) * slices
+  int blocks_made = 0;
+  // The recurrence under analysis MODE once the rows are complete, and its outputs, written by
+  // position: out_wcrt (unless null in a sweep) and out_sched.
+  auto analyse = [&](auto mode_tag, const PairConsts &pc, i64 *out_wcrt, uint8_t *out_sched) {
+    constexpr int MODE = mode_tag;  // a ModeTag: every analysis of a kernel gets its own copy
+    Outcome o = recurrence_narrow<LPT, SLOTS, MODE, SWEEP>(rows, n_narrow, n_gpu, pc, literal, lane, gmask, blocks_made);
+    if (o.verdict == 0 && n_narrow < n_rt) {
+      __syncwarp(gmask);
+      o = recurrence_wide<LPT, SLOTS, MODE, SWEEP>(buf, n, n_rt, n_narrow, n_gpu, pc, literal, lane, gmask);
     }
-  }
-
-  // ---- iterate in rank order ------------------------------------------------------------------
-  u32 Jc[SLOTS], Jg[SLOTS];               // jitters with T_h - 1 folded in (ceiling)
+    __syncwarp();
+    if (!SWEEP || out_wcrt) {
+      i64 *const out = out_wcrt + a + lane;
 #pragma unroll
-  for (int s = 0; s < SLOTS; ++s) Jc[s] = Jg[s] = Tm1[s];
-  int n_done = n_rt;
-  int verdict = 0;
-  for (int pos = 0; pos < n_rt; ++pos) {
-    const uint4 f = info[pos];
-    const u32 Di = f.x, core_i = f.y, base_i = f.z;
-    const bool gi = (f.w & 0x10000u) != 0;
-    const int smax = (pos - 1) >> kLog;  // -1 for the first task: nothing interferes
-    if (smax >= slots_made) {              // the first task that looks at slot smax
-#pragma unroll
-      for (int s = 0; s < SLOTS; ++s)
-        if (s == smax) make_reciprocal(Tm1[s] + 1, magic[s], shift[s]);
-      slots_made = smax + 1;
-    }
-    u32 nu = 0;
-    if (MODE == 3) {  // Lemma 4: N_g - |{h in hpp(i): GPU-using}| + 1
-      int c = 0;
-#pragma unroll
-      for (int s = 0; s < SLOTS; ++s)
-        if (s <= smax) c += __popc(__ballot_sync(gmask, lane + LPT * s < pos && core[s] == core_i && gpu[s]));
-      nu = (u32)(n_gpu - c + 1);
-    }
-    // the (J, W) pairs of this task's interferers; W = 0 where a pair does not apply
-    u32 J1[SLOTS], W1[SLOTS], W2[SLOTS];
-#pragma unroll
-    for (int s = 0; s < SLOTS; ++s) {
-      J1[s] = 0, W1[s] = 0, W2[s] = 0;
-      if (s <= smax) {
-        const bool act = lane + LPT * s < pos;
-        const bool same = core[s] == core_i;
-        u32 w1, w2 = 0, j1;
-        if (MODE == 0) {
-          w1 = same ? Wa[s] : (gi ? Wb[s] : 0u);           // Lemma 15 / Lemma 13 (other cores)
-          j1 = same ? Jc[s] : Jg[s];
-          w2 = (same && gi && gpu[s]) ? Ger[s] : 0u;       // Lemma 13 (same core), jitter J^g
-        } else if (MODE == 1) {
-          w1 = same ? Wa[s] + ((gi || !literal) ? Wb[s] : 0u) : Wb[s];  // Lemmas 12+10 / 10, 11
-          j1 = same ? Tm1[s] : Jg[s];
-        } else if (MODE == 2) {
-          w1 = same ? Wa[s] : 0u;                          // Lemma 7
-          j1 = Jc[s];
-        } else {
-          const u64 w = (u64)Wa[s] + (u64)Wb[s] * nu;      // Lemmas 5 and 4
-          w1 = same ? (w > kFastClamp ? kFastClamp : (u32)w) : 0u;
-          j1 = Tm1[s];
+      for (int s = 0; s < SLOTS; ++s) {
+        if (lane + LPT * s < n) {
+          const int r = rank[s];
+          i64 value = r >= n_rt ? (i64)GCAPS_WCRT_BEST_EFFORT
+                                : (r == o.n_done ? (i64)o.verdict : (i64)GCAPS_WCRT_SKIPPED);
+          if (r < o.n_done) value = (i64)rows.R(r);
+          out[LPT * s] = value;
         }
-        J1[s] = j1, W1[s] = act ? w1 : 0u, W2[s] = act ? w2 : 0u;
       }
     }
-    u32 R = base_i;
-    int v = 0;
-    int sweeps = 0;
-    for (;;) {
-      if (R > Di) {
-        v = GCAPS_WCRT_MISS;
-        break;
-      }
-      if (sweeps >= (int)GCAPS_RTA_ITER_CAP) {
-        v = GCAPS_WCRT_ITER_LIMIT;
-        break;
-      }
-      sweeps += 1;
-      u32 next = base_i;
-      if (smax >= 0) {
-        u64 acc = 0;
-#pragma unroll
-        for (int s = 0; s < SLOTS; ++s) {
-          if (s <= smax) {
-            acc += (u64)(__umulhi(R + J1[s], magic[s]) >> shift[s]) * W1[s];
-            if (MODE == 0) acc += (u64)(__umulhi(R + Jg[s], magic[s]) >> shift[s]) * W2[s];
-          }
-        }
-        const u32 part = acc > (u64)kFastClamp ? kFastClamp : (u32)acc;
-        next += __reduce_add_sync(gmask, part);
-      }
-      if (next == R) break;
-      R = next;
-    }
-    if (v != 0) {
-      n_done = pos;
-      verdict = v;
-      break;
-    }
-    // publish: the owner writes R_i and forms its jitters J^c = R - (C+G^m), J^g = R - G^e (a
-    // CPU-only task has no J^c unless the printed form of Lemma 7 is asked for)
-#pragma unroll
-    for (int s = 0; s < SLOTS; ++s) {
-      if (lane + LPT * s == pos) {
-        if (!SWEEP || out_wcrt) out_wcrt[a + pos_of[s]] = (i64)R;
-        if (MODE == 0 ? gpu[s] : (MODE == 2 ? (gpu[s] || literal) : false)) Jc[s] = R - Ar[s] + Tm1[s];
-        Jg[s] = R - Ger[s] + Tm1[s];
-      }
-    }
-  }
-  // ---- write the sentinels of the tasks that did not converge ---------------------------------
-  if (!SWEEP || out_wcrt) {
-#pragma unroll
-    for (int s = 0; s < SLOTS; ++s) {
-      const int r = lane + LPT * s;
-      if (r < n && r >= n_done)
-        out_wcrt[a + pos_of[s]] = r >= n_rt ? (i64)GCAPS_WCRT_BEST_EFFORT
-                                          : (r == n_done ? (i64)verdict : (i64)GCAPS_WCRT_SKIPPED);
-    }
-  }
-  if (lane == 0) out_sched[t] = verdict == 0 ? GCAPS_SCHED_YES : GCAPS_SCHED_NO;
-  __syncwarp(gmask);
-  };  // recurrence
+    if (live && lane == 0) out_sched[t] = o.verdict == 0 ? GCAPS_SCHED_YES : GCAPS_SCHED_NO;
+    __syncwarp();
+  };
 
   if constexpr (!SWEEP) {
-    // ---- one analysis: constants by position, then everything moves to the rank's lane ---------
+    // ---- one analysis: constants by position, then everything goes to the rank's rows -----------
     constexpr int MODE = (MASK & 1) ? 0 : (MASK & 2) ? 1 : (MASK & 4) ? 2 : 3;
     constexpr bool kGcaps = MODE < 2;
-    const u32 ovh = (u32)p.ovh;  // the fast path needs eps, theta < 2^20
+    PairConsts pc;
+    pc.ovh = (u32)p.ovh;  // the fast path needs eps, theta < 2^20
+    pc.slot_cost = (u64)p.L + pc.ovh;  // <= 2^41
     u32 sl[SLOTS];               // RR: slices of the task's pure GPU parts (Eq. 3)
 #pragma unroll
     for (int s = 0; s < SLOTS; ++s) sl[s] = 0;
     if (!kGcaps) {
       slice_sums(Q0, p.L, p.l_mode, p.l_magic, p.l_shift);
-      __syncwarp(gmask);
 #pragma unroll
       for (int s = 0; s < SLOTS; ++s) sl[s] = Q0[g1[s] - 1 + pare] - Q0[g0[s] - 1 + pare];
-      __syncwarp(gmask);
+      __syncwarp();
     }
-    u32 base[SLOTS];
 #pragma unroll
     for (int s = 0; s < SLOTS; ++s) {
-      if (kGcaps) {
-        S[s] = 2 * ovh * eta[s];                                 // eta < 64: below 2^27
-        base[s] = A[s] + Ge[s] + S[s] + (eta[s] + 1) * ovh;        // C_i + G*_i + B^C_i, below 2^29
-      } else {
-        const u64 slices = sl[s];
-        const u64 lt = (u64)p.L + ovh;  // <= 2^41
-        u64 B = slices == 0 ? 0 : (lt >= kFastClamp ? kFastClamp : lt * slices);  // < 2^26 * 2^32
-        if (B > kFastClamp) B = kFastClamp;
-        S[s] = (u32)B;
-        const u64 b64 = (u64)A[s] + Ge[s] + (eta[s] > 0 ? B * (u64)(n_gpu - 1) : 0);  // Lemma 1
-        base[s] = b64 > (u64)(2 * kFastClamp) ? 2 * kFastClamp : (u32)b64;
-      }
-      base[s] = base[s] > 2 * kFastClamp ? 2 * kFastClamp : base[s];
-    }
-    __syncwarp(gmask);
-#pragma unroll
-    for (int s = 0; s < SLOTS; ++s) {
+      u32 S, base;
+      own_cost<kGcaps>(pc, A[s], Ge[s], eta[s], sl[s], n_gpu, S, base);
       if (lane + LPT * s < n) {
-        *(reinterpret_cast<uint2 *>(&info[rank[s]]) + 1) =
-            make_uint2(base[s], (u32)(lane + LPT * s) | (eta[s] > 0 ? 0x10000u : 0u));
-        xch[rank[s]] = make_uint4(T[s], A[s], Ge[s], S[s]);
+        const u32 flag = eta[s] > 0 ? kRowGpu : 0u;
+        rows.b(rank[s]) = make_uint4(T[s], A[s], Ge[s] | flag, S);
+        rows.base(rank[s]) = base;
       }
     }
-    __syncwarp(gmask);
-    recurrence(ModeTag<MODE>(), p.out_wcrt, p.out_sched);
+    __syncwarp();
+    analyse(ModeTag<MODE>(), pc, p.out_wcrt, p.out_sched);
   } else {
-    // ---- several analyses: the tasks move to the rows of their ranks once; for every analysis
-    // the lane of a rank then makes that task's S and base from the row and the recurrence
-    // starts from the rows again, so nothing per task is held in registers across analyses ------
-    // second row by rank: GPU segment range (11 bits each) and number of GPU segments (6 bits)
-    // packed in .x, slices of Eq. 3 for the timeslice sl_L in .y
-    uint2 *xch2 = reinterpret_cast<uint2 *>(Q0 + 4 * MAXN);
+    // ---- several analyses: the tasks go to the rows of their ranks once; S and base of a task are
+    // made from the rows when an analysis reaches it (most stop early) ------------------------------
     static_assert(Lay::CAP <= 2048 && Lay::CAP >= 6 * MAXN, "packed segment range, room for the second row");
 #pragma unroll
     for (int s = 0; s < SLOTS; ++s) {
       if (lane + LPT * s < n) {
-        info[rank[s]].w = (u32)(lane + LPT * s) | (eta[s] > 0 ? 0x10000u : 0u);
-        xch[rank[s]] = make_uint4(T[s], A[s], Ge[s], 0u);
-        xch2[rank[s]] = make_uint2((u32)g0[s] | ((u32)g1[s] << 11) | (eta[s] << 22), 0u);
+        const u32 flag = eta[s] > 0 ? kRowGpu : 0u;
+        rows.b(rank[s]) = make_uint4(T[s], A[s], Ge[s] | flag, 0u);
+        // GPU segment range (11 bits each) and number of GPU segments (6 bits), slices
+        rows.second(rank[s]) = make_uint2((u32)g0[s] | ((u32)g1[s] << 11) | (eta[s] << 22), 0u);
       }
     }
-    __syncwarp(gmask);
+    __syncwarp();
     i64 sl_L = -1;
-    constexpr bool kMultiModes = (MASK & (MASK - 1)) != 0;
-    const int enabled = kMultiModes ? sw->enabled : MASK;
+    const int enabled = kMulti ? sw->enabled : MASK;
     for (int q = 0; q < sw->n; ++q) {
       const i64 L64 = sw->q[q].L;
-      const u32 ovh = (u32)sw->q[q].ovh;  // the fast path needs eps, theta < 2^20
+      PairConsts pc;
+      pc.ovh = (u32)sw->q[q].ovh;  // the fast path needs eps, theta < 2^20
+      pc.slot_cost = (u64)L64 + pc.ovh;
       auto analyse_as = [&](auto mode_tag) {
         constexpr int MODE = mode_tag;
         constexpr bool kGcaps = MODE < 2;
@@ -1081,43 +992,17 @@ __device__ __forceinline__ int analyse_fast(const KParams &p, i64 t, i64 a, int 
         if (!kGcaps && L64 != sl_L) {
           sl_L = L64;
           slice_sums(Q1, L64, sw->q[q].l_mode, sw->q[q].l_magic, sw->q[q].l_shift);
-          __syncwarp(gmask);
 #pragma unroll
           for (int s = 0; s < SLOTS; ++s) {
             const int r = lane + LPT * s;
             if (r < n) {
-              const u32 g = xch2[r].x;
-              xch2[r].y = Q1[(int)((g >> 11) & 0x7ffu) - 1 + pare] - Q1[(int)(g & 0x7ffu) - 1 + pare];
+              const u32 g = rows.second(r).x;
+              rows.second(r).y = Q1[(int)((g >> 11) & 0x7ffu) - 1 + pare] - Q1[(int)(g & 0x7ffu) - 1 + pare];
             }
           }
+          __syncwarp();
         }
-#pragma unroll
-        for (int s = 0; s < SLOTS; ++s) {
-          const int r = lane + LPT * s;
-          if (r < n) {
-            const uint4 x = xch[r];
-            const uint2 g = xch2[r];
-            const u32 eta_r = g.x >> 22;
-            u32 Sr, base;
-            if (kGcaps) {
-              Sr = 2 * ovh * eta_r;                                 // eta < 64: below 2^27
-              base = x.y + x.z + Sr + (eta_r + 1) * ovh;             // C_i + G*_i + B^C_i, below 2^29
-            } else {
-              const u64 slices = g.y;
-              const u64 lt = (u64)L64 + ovh;  // <= 2^41
-              u64 B = slices == 0 ? 0 : (lt >= kFastClamp ? kFastClamp : lt * slices);
-              if (B > kFastClamp) B = kFastClamp;
-              Sr = (u32)B;
-              const u64 b64 = (u64)x.y + x.z + (eta_r > 0 ? B * (u64)(n_gpu - 1) : 0);  // Lemma 1
-              base = b64 > (u64)(2 * kFastClamp) ? 2 * kFastClamp : (u32)b64;
-            }
-            base = base > 2 * kFastClamp ? 2 * kFastClamp : base;
-            xch[r].w = Sr;
-            info[r].z = base;
-          }
-        }
-        __syncwarp(gmask);
-        recurrence(mode_tag, out_wcrt, out_sched);
+        analyse(mode_tag, pc, out_wcrt, out_sched);
       };
       if ((MASK & 1) && (enabled & 1)) analyse_as(ModeTag<0>());
       if ((MASK & 2) && (enabled & 2)) analyse_as(ModeTag<1>());
@@ -1125,7 +1010,8 @@ __device__ __forceinline__ int analyse_fast(const KParams &p, i64 t, i64 a, int 
       if ((MASK & 8) && (enabled & 8)) analyse_as(ModeTag<3>());
     }
   }
-  return kFastDone;
+#undef GCAPS_LEAVE_IF_NONE_LIVE
+  return live ? kFastDone : kFastDeclined;
 }
 
 __device__ __forceinline__ void prefetch_l2(const void *ptr) {
@@ -1220,43 +1106,47 @@ __device__ __forceinline__ void run_bin(const KParams &p, int bin, u32 *warp_buf
         look_up(nfirst, nxt);
       }
       const int mine = c * G + group;
-      if (mine < in_chunk) {
-        const Ahead me = cur[mine];
-        const i64 t = (i64)me.t;
-        const int n = (int)(me.packed & 0x1ffu), nc = (int)((me.packed >> 9) & 0x7ffu);
-        const int ng = (int)((me.packed >> 20) & 0x7ffu);
-        // the segment slices start their way into L2 now; the per-task loads follow at once, so
-        // that the running sums later wait for L2 rather than for DRAM (16 elements per line,
-        // only addresses inside the arrays)
+      const bool have = mine < in_chunk;
+      const Ahead me = cur[have ? mine : 0];
+      const i64 t = (i64)me.t;
+      const int n = (int)(me.packed & 0x1ffu), nc = (int)((me.packed >> 9) & 0x7ffu);
+      const int ng = (int)((me.packed >> 20) & 0x7ffu);
+      const bool fast = have && fast_call && (me.packed >> 31) != 0;
+      // the segment slices start their way into L2 now; the per-task loads follow at once, so
+      // that the running sums later wait for L2 rather than for DRAM (16 elements per line,
+      // only addresses inside the arrays)
+      if (have) {
         for (int e = 16 * lane; e < nc; e += 16 * LPT) prefetch_l2(p.cseg_wcet + me.c_lo + e);
         for (int e = 16 * lane; e < ng; e += 16 * LPT)
           prefetch_l2(p.gseg_misc + me.g_lo + e), prefetch_l2(p.gseg_exec + me.g_lo + e);
-        bool done = false;
-        if (fast_call && (me.packed >> 31) != 0) {
-          int how = kFastUndecided;
-          if constexpr (LPT == 32 && !SWEEP && (MASK & 12) != 0) {
-            // Far from schedulable, a taskset ends with a miss among its first ranks; nearly
-            // schedulable, looking at them first is wasted.  Tasksets of a batch tend to be alike:
-            // after four undecided ones in a row only every sixteenth taskset is tried that way.
-            // (Round robin only: with tens of GPU-using tasks taking turns on the GPU the first or
-            // second rank already misses, and the pass pays; under GCAPS the first miss comes a few
-            // ranks later and the pass was measured slower than the full one.)
-            if (undecided_run < 4 || (tried_since & 15) == 0) {
-              how = analyse_fast<LPT, SLOTS, MASK, false, true>(p, t, me.a, n, buf, lane, gmask);
-              undecided_run = how == kFastUndecided ? undecided_run + 1 : 0;
-              __syncwarp(gmask);
-            }
-            tried_since += 1;
+      }
+      int how = kFastDeclined;
+      if constexpr (LPT == 32 && !SWEEP && (MASK & 12) != 0) {
+        // Far from schedulable, a taskset ends with a miss among its first ranks; nearly
+        // schedulable, looking at them first is wasted.  Tasksets of a batch tend to be alike:
+        // after four undecided ones in a row only every sixteenth taskset is tried that way.
+        // (Round robin only: with tens of GPU-using tasks taking turns on the GPU the first or
+        // second rank already misses, and the pass pays; under GCAPS the first miss comes a few
+        // ranks later and the pass was measured slower than the full one.)
+        if (fast) {
+          how = kFastUndecided;
+          if (undecided_run < 4 || (tried_since & 15) == 0) {
+            how = analyse_fast<LPT, SLOTS, MASK, false, true>(p, true, t, me.a, n, buf, lane, gmask);
+            undecided_run = how == kFastUndecided ? undecided_run + 1 : 0;
+            __syncwarp();
           }
-          if (how == kFastUndecided) how = analyse_fast<LPT, SLOTS, MASK, SWEEP>(p, t, me.a, n, buf, lane, gmask, sw);
-          done = how == kFastDone;
+          tried_since += 1;
         }
-        __syncwarp(gmask);
-        if (!done && !SWEEP) {
+        if (how == kFastUndecided) how = analyse_fast<LPT, SLOTS, MASK, SWEEP>(p, true, t, me.a, n, buf, lane, gmask, sw);
+      } else if (fast_call) {
+        how = analyse_fast<LPT, SLOTS, MASK, SWEEP>(p, fast, t, me.a, n, buf, lane, gmask, sw);
+      }
+      __syncwarp();
+      if (have && how != kFastDone) {
+        if (!SWEEP) {
           // the exact path reads task_off again and validates everything itself
           analyse_taskset<LPT, MAXN>(p, t, *reinterpret_cast<GroupSmem<MAXN> *>(buf), lane, gmask);
-        }
-        if (!done && SWEEP) {  // the exact path once per (timeslice, overhead) pair
+        } else {  // the exact path once per (timeslice, overhead) pair
           constexpr bool kMulti = (MASK & (MASK - 1)) != 0;
           const int enabled = kMulti ? sw->enabled : MASK;
           for (int q = 0; q < sw->n; ++q) {
