@@ -37,8 +37,9 @@ ALU_PEAK_DERIVED = 148 * 128 * 1.965e9
 MAX_TASKSETS_PER_GPU = 1_000_000
 K_TERM, K_SETUP = 6, 16   # algorithmic integer lane-operations per interference term / per task
 # kernels launched by one gcaps_rta_batch call: 3 plan kernels, one analysis kernel for the bins
-# of up to 32 tasks and one each for the 64-, 96-, 128-, 192- and 256-task bins
-LAUNCHES_PER_CALL = 9        # three plan kernels + one kernel per group of size bins
+# of up to 32 tasks, one each for the 64-, 96-, 128-, 192- and 256-task bins and two for the larger
+# tasksets that those left over
+LAUNCHES_PER_CALL = 11       # three plan kernels + one kernel per group of size bins + two
 LAUNCHES_PER_SMALL_CALL = 2  # batches of up to 8,192 tasksets: one plan kernel, one kernel for all bins
 # DRAM bytes (read + write) per taskset of the analysis kernel on the 'large' workload, from an
 # ncu capture of a 131,072-taskset launch (traffic grows in proportion to the tasksets of a

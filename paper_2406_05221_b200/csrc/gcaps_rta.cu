@@ -14,6 +14,7 @@
 #include <mutex>
 
 #include "rta_device.cuh"
+#include "rta_staged.cuh"
 
 using namespace gcaps_detail;
 
@@ -65,6 +66,7 @@ __global__ void plan_scan_kernel(KParams p, unsigned int n_blocks) {
       p.hdr->bin_start[k] = s;
       p.hdr->bin_count[k] = c;
       p.hdr->next[k] = 0;
+      if (k < kNumBins) p.hdr->next2[k] = 0, p.hdr->deferred[k] = 0, p.hdr->first_tries[k] = 0;
       s += c;
     }
   }
@@ -101,6 +103,7 @@ __global__ void __launch_bounds__(1024) plan_small_kernel(KParams p) {
       p.hdr->bin_start[k] = s;
       p.hdr->bin_count[k] = c;
       p.hdr->next[k] = 0;
+      if (k < kNumBins) p.hdr->next2[k] = 0, p.hdr->deferred[k] = 0, p.hdr->first_tries[k] = 0;
       start[k] = s;
       cnt[k] = 0;  // from here on the write cursor of the bin
       s += c;
@@ -115,7 +118,8 @@ __global__ void __launch_bounds__(1024) plan_small_kernel(KParams p) {
 
 // The bins of up to 32 tasks in one persistent launch, largest tasksets first: (lanes per
 // taskset, tasks per lane) = (16,2) (8,3) (8,2) (8,1) for at most 32, 24, 16, 8 tasks, i.e. two or
-// four tasksets per warp.
+// four tasksets per warp.  (A look at the first ranks out of a stage, a warp per taskset, was slower
+// here in every form tried: 100,000 24-task tasksets under round robin 163 us against 128.)
 template <int MODE>
 __global__ void __launch_bounds__(kBlockThreads, min_blocks(3)) rta_small_kernel(KParams p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -129,16 +133,49 @@ __global__ void __launch_bounds__(kBlockThreads, min_blocks(3)) rta_small_kernel
   wait_for_previous_grid();
 }
 
-// One bin of larger tasksets (a warp per taskset, 2, 3, 4, 6 or 8 tasks per lane) per launch.
+// First launch of a bin of larger tasksets: a warp per taskset, SLOTS tasks per lane.
 template <int SLOTS, int MODE>
-__global__ void __launch_bounds__(kBlockThreads, min_blocks(SLOTS)) rta_big_kernel(KParams p, int bin) {
+__global__ void __launch_bounds__(kStagedThreads, staged_min_blocks(SLOTS))
+rta_big_kernel(KParams p, int bin, u32 stage_bytes) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ SliceTable tab;
   let_dependents_start();  // the kernel of the next size bin shares no data with this one
-  constexpr int kWarpWords = bin_warp_words<32, SLOTS>() + kAheadWords;
-  u32 *warp_buf = reinterpret_cast<u32 *>(smem_raw) + (threadIdx.x >> 5) * kWarpWords;
-  Ahead *ahead = reinterpret_cast<Ahead *>(warp_buf + kWarpWords - kAheadWords);
-  run_bin<32, SLOTS, 1 << MODE>(p, bin, warp_buf, ahead);
+  if (threadIdx.x == 0) {
+    tab.ptr[0] = p.period, tab.ptr[1] = p.deadline, tab.ptr[2] = p.priority, tab.ptr[3] = p.core;
+    tab.ptr[4] = p.cseg_off, tab.ptr[5] = p.gseg_off;
+    tab.ptr[6] = p.cseg_wcet, tab.ptr[7] = p.gseg_misc, tab.ptr[8] = p.gseg_exec;
+#pragma unroll
+    for (int k = 0; k < kArrays; ++k)
+      tab.len[k] = k < 4 ? p.n_tasks : (k < 6 ? p.n_tasks + 1 : (k == 6 ? p.n_csegs : p.n_gsegs));
+  }
+  __syncthreads();
+  unsigned char *mine = smem_raw + (threadIdx.x >> 5) * (sizeof(StagedWarp<SLOTS>) + stage_bytes);
+  run_staged_bin<SLOTS, MODE>(p, bin, stage_bytes, *reinterpret_cast<StagedWarp<SLOTS> *>(mine),
+                              mine + sizeof(StagedWarp<SLOTS>), tab);
   wait_for_previous_grid();
+}
+
+// Second launches: what the first ones marked, largest tasksets first.  LARGE: the bins of more than 96
+// tasks, which need twice the registers.
+template <bool LARGE>
+__host__ __device__ constexpr int deferred_warp_words() {
+  return bin_warp_words<32, LARGE ? 8 : 3>() + kAheadWords;
+}
+template <bool LARGE, int MODE>
+__global__ void __launch_bounds__(kBlockThreads, min_blocks(LARGE ? 6 : 3)) rta_deferred_kernel(KParams p) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  wait_for_previous_grid();  // the marks in the permutation are complete from here on
+  let_dependents_start();
+  u32 *buf = reinterpret_cast<u32 *>(smem_raw) + (threadIdx.x >> 5) * deferred_warp_words<LARGE>();
+  Ahead *ahead = reinterpret_cast<Ahead *>(buf + deferred_warp_words<LARGE>() - kAheadWords);
+  if constexpr (LARGE) {
+    run_deferred_bin<8, MODE>(p, 8, buf, ahead);
+    run_deferred_bin<6, MODE>(p, 7, buf, ahead);
+    run_deferred_bin<4, MODE>(p, 6, buf, ahead);
+  } else {
+    run_deferred_bin<3, MODE>(p, 5, buf, ahead);
+    run_deferred_bin<2, MODE>(p, 4, buf, ahead);
+  }
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -291,13 +328,44 @@ int enqueue_plan(KParams &p, void *workspace, size_t workspace_bytes, cudaStream
 
 namespace {
 
+// The stage of a bin: room for a taskset of the bin's largest size with a tenth more segments per task
+// than the batch has on average, as long as an SM then still holds kMinStages of them.  Where the
+// batch's mean size lies in the bin its tasksets are probably alike, and 5 % above the mean (but no
+// less than the middle of the bin) has to do: more stages, i.e. more warps, per SM count for more
+// than the few tasksets left over (80-task tasksets: 18 instead of 16 warps, 1.53 instead of 1.64 ms
+// per 1,000,000).
+constexpr size_t kSmemPerSm = 228 * 1024, kSmemPerBlockReserved = 1024 + 256;
+constexpr int kMinStages = 8;
+
 template <int SLOTS, int MODE>
 cudaError_t launch_big(const KParams &p, int bin, int sm_count, cudaStream_t st) {
+  constexpr int kWarps = kStagedThreads / 32;
+  constexpr size_t kFixed = sizeof(StagedWarp<SLOTS>);
+  constexpr size_t kLeast = sizeof(u32) * FastLayout<32, SLOTS>::kWords;  // the full pass works in a stage too
+  constexpr size_t kMost = (kSmemPerSm / kMinStages - kSmemPerBlockReserved - kFixed) / 16 * 16;
+  static_assert(kFixed % 16 == 0 && kLeast <= kMost, "stages are 16-byte aligned");
+  static int blocks_by_registers[64] = {0};
+  const double per_task = 48.0 + 8.8 * ((double)p.n_csegs + 2.0 * (double)p.n_gsegs) / (double)(p.n_tasks > 0 ? p.n_tasks : 1);
+  constexpr double kTasksLo = SLOTS <= 4 ? 32 * (SLOTS - 1) : 32 * (SLOTS - 2), kTasksHi = 32 * SLOTS;
+  const double mean = (double)p.n_tasks / (double)p.n_tasksets;
+  double tasks = kTasksHi;
+  if (mean > kTasksLo && 1.05 * mean < kTasksHi) tasks = 1.05 * mean > (kTasksLo + kTasksHi) / 2 ? 1.05 * mean : (kTasksLo + kTasksHi) / 2;
+  const double want = per_task * tasks + 9 * 24;
+  size_t stage = want > (double)kMost ? kMost : ((size_t)want + 15) / 16 * 16;
+  if (stage < kLeast) stage = (kLeast + 15) / 16 * 16;
+  const size_t smem = kWarps * (kFixed + stage);
+  return launch_staged(rta_big_kernel<SLOTS, MODE>, blocks_by_registers, kWarps * (kFixed + kMost), smem,
+                       kSmemPerSm / (smem + kSmemPerBlockReserved), (p.n_tasksets + kWarps - 1) / kWarps, sm_count, st, p,
+                       bin, (u32)stage);
+}
+
+template <bool LARGE, int MODE>
+cudaError_t launch_deferred(const KParams &p, int sm_count, cudaStream_t st) {
   constexpr int kWarps = kBlockThreads / 32;
   static int blocks_per_sm[64] = {0};
-  const size_t smem = sizeof(u32) * (bin_warp_words<32, SLOTS>() + kAheadWords) * kWarps;
-  return launch_persistent_ex(true, rta_big_kernel<SLOTS, MODE>, blocks_per_sm, smem,
-                           (p.n_tasksets + kWarps - 1) / kWarps, sm_count, st, p, bin);
+  const size_t smem = sizeof(u32) * deferred_warp_words<LARGE>() * kWarps;
+  return launch_persistent_ex(true, rta_deferred_kernel<LARGE, MODE>, blocks_per_sm, smem,
+                              (p.n_tasksets + kWarps - 1) / kWarps, sm_count, st, p);
 }
 
 template <int MODE>
@@ -313,6 +381,8 @@ cudaError_t launch_all_bins(const KParams &p, int sm_count, cudaStream_t st) {
   if (e == cudaSuccess) e = launch_big<4, MODE>(p, 6, sm_count, st);
   if (e == cudaSuccess) e = launch_big<6, MODE>(p, 7, sm_count, st);
   if (e == cudaSuccess) e = launch_big<8, MODE>(p, 8, sm_count, st);
+  if (e == cudaSuccess) e = launch_deferred<false, MODE>(p, sm_count, st);
+  if (e == cudaSuccess) e = launch_deferred<true, MODE>(p, sm_count, st);
   return e;
 }
 

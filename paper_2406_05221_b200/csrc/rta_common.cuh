@@ -23,6 +23,7 @@ typedef unsigned int u32;
 constexpr u32 kFastLimit = 1u << 26;  // fast path: every time of the taskset is below this
 constexpr u32 kFastClamp = 1u << 26;  // ... so a sum clamped here still exceeds every deadline
 constexpr int kBlockThreads = 128;
+constexpr int kStagedBlockThreads = 64;  // kernels that stage tasksets by bulk copies
 constexpr int kPlanItems = 1024;  // tasksets per plan block
 constexpr int kPlanSmall = 8192;  // batches up to this size are planned by one block in one launch
 constexpr u64 kClamp = 1ull << 50;  // any quantity >= 2^50 exceeds every deadline (<= 2^40)
@@ -30,8 +31,14 @@ constexpr u64 kClamp = 1ull << 50;  // any quantity >= 2^50 exceeds every deadli
 struct PlanHeader {
   unsigned int bin_start[kBinStride];
   unsigned int bin_count[kBinStride];
-  unsigned int next[kBinStride];  // work counters of the analysis launches
+  unsigned int next[kBinStride];      // work counters of the analysis launches
+  unsigned int next2[kNumBins];     // ... of the second launches over the deferred tasksets
+  unsigned int deferred[kNumBins];  // tasksets the first launch left to the second
+  // of each warp's first taskset in the first launch: how many there were (low half) and how many
+  // the first ranks did not decide (high half)
+  unsigned int first_tries[kNumBins];
 };
+constexpr unsigned int kDeferred = 0x80000000u;  // in a permutation entry: left to the second launch
 static_assert(sizeof(PlanHeader) <= 256, "header layout");
 
 struct KParams {
@@ -201,6 +208,42 @@ cudaError_t launch_persistent_ex(bool overlap_previous, void (*kernel)(Args...),
   }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned int)grid), cfg.blockDim = dim3(kBlockThreads);
+  cfg.dynamicSmemBytes = smem, cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr, cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+// The same for a kernel whose shared memory varies from call to call (at most `most_smem`):
+// `by_smem` blocks fit an SM by shared memory, the limit by registers is looked up once.
+template <typename... Args>
+cudaError_t launch_staged(void (*kernel)(Args...), int *by_registers, size_t most_smem, size_t smem, size_t by_smem,
+                          long long want, int sm_count, cudaStream_t st, Args... args) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  dev &= 63;
+  int resident = __atomic_load_n(&by_registers[dev], __ATOMIC_ACQUIRE);
+  if (resident == 0) {
+    std::lock_guard<std::mutex> lock(g_init_mutex);
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most_smem);
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    if (e != cudaSuccess) return e;
+    int per_sm = 1;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kStagedBlockThreads, 0);
+    if (e != cudaSuccess) return e;
+    resident = per_sm < 1 ? 1 : per_sm;
+    __atomic_store_n(&by_registers[dev], resident, __ATOMIC_RELEASE);
+  }
+  if ((size_t)resident > by_smem) resident = by_smem < 1 ? 1 : (int)by_smem;
+  long long grid = (long long)sm_count * resident;
+  if (grid > want) grid = want;
+  if (grid < 1) grid = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned int)grid), cfg.blockDim = dim3(kStagedBlockThreads);
   cfg.dynamicSmemBytes = smem, cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

@@ -364,220 +364,6 @@ __device__ __forceinline__ bool more_steps(int e0, int N) {
   return __any_sync(kFull, e0 < N);
 }
 
-// Range check of segment slices without running sums: `bad` collects whether a wanted element lies
-// outside [0, 2^26), and the elements, narrowed to 32 bits, go to shared memory as they are
-// (D[w] = element w - par; same loads and store pattern as prefix_step).  NB blocks of 128
-// elements per array in flight together (TWO: two arrays that share their offsets).
-template <int NB, bool TWO>
-__device__ __forceinline__ void check_slices(const i64 *__restrict__ X0, const i64 *__restrict__ X1, int N,
-                                             int par0, int par1, bool inside, const i64 *lo0,
-                                             const i64 *hi0, const i64 *lo1, const i64 *hi1, u32 *D0,
-                                             u32 *D1, int lane, u32 &bad) {
-  for (int e0 = 0; e0 < N + (par0 > par1 ? par0 : par1); e0 += 128 * NB) {
-    Quad q0[NB], q1[NB];
-#pragma unroll
-    for (int b = 0; b < NB; ++b) {
-      if (inside) {
-        load_quad_inside(X0, e0 + 128 * b + 4 * lane - par0, N, q0[b]);
-        if (TWO) load_quad_inside(X1, e0 + 128 * b + 4 * lane - par1, N, q1[b]);
-      } else {
-        q0[b] = load_quad_edge(X0, e0 + 128 * b + 4 * lane - par0, N, lo0, hi0);
-        if (TWO) q1[b] = load_quad_edge(X1, e0 + 128 * b + 4 * lane - par1, N, lo1, hi1);
-      }
-    }
-#pragma unroll
-    for (int b = 0; b < NB; ++b) {
-      if (e0 + 128 * b < N + 1) {
-        u32 x[4];
-        narrow_quad(q0[b], e0 + 128 * b + 4 * lane - par0, N, x, bad);
-        *reinterpret_cast<uint4 *>(D0 + e0 + 128 * b + 4 * lane) =
-            make_uint4((u32)q0[b].v[0], (u32)q0[b].v[1], (u32)q0[b].v[2], (u32)q0[b].v[3]);
-        if (TWO) {
-          narrow_quad(q1[b], e0 + 128 * b + 4 * lane - par1, N, x, bad);
-          *reinterpret_cast<uint4 *>(D1 + e0 + 128 * b + 4 * lane) =
-              make_uint4((u32)q1[b].v[0], (u32)q1[b].v[1], (u32)q1[b].v[2], (u32)q1[b].v[3]);
-        }
-      }
-    }
-  }
-}
-
-// The first kFirstRanks tasks of the priority order, analysed before anything is summed for the
-// rest of the taskset (a warp per taskset).  Where tasksets are far from schedulable the first
-// deadline miss comes within a handful of ranks, and the per-task sums of all the other tasks
-// would never be used: here every segment value is still read and range-checked (a value outside
-// the 32-bit path's range sends the taskset to the exact path, as always), but sums are formed
-// only for these ranks: four lanes per rank add up the rank's own few segments, all ranks at once
-// (one trip to memory), and lane r then holds everything about rank r, as the task under analysis
-// and as an interferer of the ranks behind it.  The recurrence over these ranks needs registers
-// and warp collectives only.  Same arithmetic, same sequence of iterates, same sentinels as the
-// full pass.  `first8[r]` = (first, end) of rank r's CPU segments and of its GPU segments within
-// the taskset's slices; info[r] = (deadline, core, period, position).
-// Returns 1: the taskset is finished (a miss among these ranks, or no other real-time task), its
-// outputs are written; 0: all these ranks converged, the caller runs the full pass (which repeats
-// them); -1: a value does not fit the 32-bit path.
-constexpr int kFirstRanks = 8;
-template <int SLOTS, int MODE>
-__device__ __forceinline__ int first_ranks(const KParams &p, i64 t, i64 a, int n, const uint4 *info,
-                                           const uint4 *first8, u32 *Q0, u32 *Q1, int n_rt,
-                                           const int (&rank)[SLOTS], const int (&g0)[SLOTS],
-                                           const int (&g1)[SLOTS], const i64 *__restrict__ Xc,
-                                           const i64 *__restrict__ Xm, const i64 *__restrict__ Xe, int Nc,
-                                           int Ng, int parc, int parm, int pare, i64 cfirst, i64 gfirst,
-                                           int lane, bool literal) {
-  const int limit = n_rt < kFirstRanks ? n_rt : kFirstRanks;
-  // lanes 4r .. 4r+3 add up the segments of rank r
-  const int r4 = lane >> 2, sub = lane & 3;
-  uint4 seg = make_uint4(0u, 0u, 0u, 0u);
-  if (r4 < limit) seg = first8[r4];
-  u32 bad = 0, sum_c = 0, sum_m = 0, sum_e = 0, sum_s = 0;
-  // every segment value of the taskset must be in [0, 2^26); on the way the values stop over in
-  // shared memory, where the eight ranks find their own
-  check_slices<(SLOTS < 3 ? SLOTS : 3), false>(Xc, Xc, Nc, parc, parc, slice_is_inside(cfirst, Nc, parc, p.n_csegs),
-                                               p.cseg_wcet, p.cseg_wcet + p.n_csegs, p.cseg_wcet, p.cseg_wcet,
-                                               Q0, Q0, lane, bad);
-  __syncwarp();
-  for (int j = (int)seg.x + parc + sub; j < (int)seg.y + parc; j += 4) sum_c += Q0[j];
-  __syncwarp();
-  check_slices<2, true>(Xm, Xe, Ng, parm, pare,
-                        slice_is_inside(gfirst, Ng, parm, p.n_gsegs) && slice_is_inside(gfirst, Ng, pare, p.n_gsegs),
-                        p.gseg_misc, p.gseg_misc + p.n_gsegs, p.gseg_exec, p.gseg_exec + p.n_gsegs, Q1, Q0,
-                        lane, bad);
-  __syncwarp();
-  for (int j = (int)seg.z + sub; j < (int)seg.w; j += 4) {
-    sum_m += Q1[j + parm];
-    const u32 e = Q0[j + pare] & (kFastLimit - 1);  // (checked above; keeps the division exact)
-    sum_e += e;
-    if (MODE >= 2) {  // Eq. 3: slices of the pure GPU part
-      if (p.l_mode == 0) sum_s += __umulhi(e + (u32)p.L - 1u, p.l_magic) >> p.l_shift;
-      else if (p.l_mode == 1) sum_s += e;
-      else sum_s += e > 0 ? 1u : 0u;
-    }
-  }
-  int n_gpu = 0;  // N_g
-#pragma unroll
-  for (int s = 0; s < SLOTS; ++s) n_gpu += __popc(__ballot_sync(kFull, g1[s] > g0[s]));
-#pragma unroll
-  for (int d = 1; d <= 2; d <<= 1) {
-    sum_c += __shfl_xor_sync(kFull, sum_c, d), sum_m += __shfl_xor_sync(kFull, sum_m, d);
-    sum_e += __shfl_xor_sync(kFull, sum_e, d);
-    if (MODE >= 2) sum_s += __shfl_xor_sync(kFull, sum_s, d);
-  }
-  // lane r takes rank r from lane 4r (a task has fewer than 64 segments of a kind, every value is
-  // below 2^26: no overflow)
-  const int src = (4 * lane) & 31;
-  sum_c = __shfl_sync(kFull, sum_c, src), sum_m = __shfl_sync(kFull, sum_m, src);
-  sum_e = __shfl_sync(kFull, sum_e, src);
-  if (MODE >= 2) sum_s = __shfl_sync(kFull, sum_s, src);
-  const u32 eta_r = __shfl_sync(kFull, seg.w - seg.z, src);
-  const bool mine = lane < limit;
-  const uint4 f = mine ? info[lane] : make_uint4(1u, 0xffffffffu, 2u, 0u);  // deadline, core, period, position
-  const u32 ovh = (u32)p.ovh;  // below 2^20 on this path
-  const u32 D_r = f.x, core_r = f.y, Tm1 = f.z - 1, A_r = sum_c + sum_m, Ge_r = sum_e;
-  const bool gpu_r = eta_r > 0;
-  u32 S_r, base_r;
-  if (MODE < 2) {
-    S_r = 2 * ovh * eta_r;                               // eta < 64: below 2^27
-    base_r = A_r + Ge_r + S_r + (eta_r + 1) * ovh;       // C_i + G*_i + B^C_i, below 2^29
-    if (mine) bad |= S_r >> 26;
-  } else {
-    const u64 lt = (u64)p.L + ovh;                       // <= 2^41
-    u64 B = sum_s == 0 ? 0 : (lt >= kFastClamp ? kFastClamp : lt * (u64)sum_s);
-    if (B > kFastClamp) B = kFastClamp;
-    S_r = (u32)B;
-    const u64 b64 = (u64)A_r + Ge_r + (gpu_r ? B * (u64)(n_gpu - 1) : 0);  // Lemma 1
-    base_r = b64 > (u64)(2 * kFastClamp) ? 2 * kFastClamp : (u32)b64;
-  }
-  base_r = base_r > 2 * kFastClamp ? 2 * kFastClamp : base_r;
-  if (mine) bad |= (sum_c | sum_m | A_r | Ge_r) >> 26;
-  if (__any_sync(kFull, bad != 0)) return -1;
-  u32 magic, shift;
-  make_reciprocal(f.z, magic, shift);
-  // what rank r contributes as an interferer (the jitters follow when it has converged)
-  u32 Wa, Wb;
-  if (MODE == 0) {
-    Wa = A_r + (gpu_r ? S_r : 0u);    // Lemma 15: C_h, or C_h + G^{m*}_h
-    Wb = gpu_r ? Ge_r + S_r : 0u;     // Lemma 13, other cores: G^{e*}_h
-  } else if (MODE == 1) {
-    Wa = A_r;                         // Lemma 12
-    Wb = gpu_r ? Ge_r + S_r : 0u;     // Lemmas 10, 11: G^{e*}_h
-  } else {
-    Wa = A_r;                         // Lemmas 5, 7
-    Wb = gpu_r ? S_r : 0u;            // Lemma 4: (L+theta) * slices
-  }
-  u32 Jc = Tm1, Jg = Tm1;
-  // ---- the recurrence of Eq. 1 over these ranks -----------------------------------------------------
-  int verdict = 0, pos = 0;
-  for (; pos < limit; ++pos) {
-    const u32 Di = __shfl_sync(kFull, D_r, pos), core_i = __shfl_sync(kFull, core_r, pos);
-    const u32 base_i = __shfl_sync(kFull, base_r, pos);
-    const bool gi = __shfl_sync(kFull, (int)gpu_r, pos) != 0;
-    const bool act = lane < pos, same = core_r == core_i;
-    u32 j1, w1, w2 = 0;
-    if (MODE == 0) {
-      w1 = same ? Wa : (gi ? Wb : 0u);            // Lemma 15 / Lemma 13 (other cores)
-      j1 = same ? Jc : Jg;
-      w2 = (same && gi && gpu_r) ? Ge_r : 0u;     // Lemma 13 (same core), jitter J^g
-    } else if (MODE == 1) {
-      w1 = same ? Wa + ((gi || !literal) ? Wb : 0u) : Wb;  // Lemmas 12+10 / 10, 11
-      j1 = same ? Tm1 : Jg;
-    } else if (MODE == 2) {
-      w1 = same ? Wa : 0u;                        // Lemma 7
-      j1 = Jc;
-    } else {
-      // Lemma 4: N_g - |{h in hpp(i): GPU-using}| + 1
-      const u32 nu = (u32)(n_gpu - __popc(__ballot_sync(kFull, act && same && gpu_r)) + 1);
-      const u64 w = (u64)Wa + (u64)Wb * nu;       // Lemmas 5 and 4
-      w1 = same ? (w > kFastClamp ? kFastClamp : (u32)w) : 0u;
-      j1 = Tm1;
-    }
-    if (!act) w1 = 0, w2 = 0;
-    u32 R = base_i;
-    int sweeps = 0;
-    for (;;) {
-      if (R > Di) {
-        verdict = GCAPS_WCRT_MISS;
-        break;
-      }
-      if (sweeps >= (int)GCAPS_RTA_ITER_CAP) {
-        verdict = GCAPS_WCRT_ITER_LIMIT;
-        break;
-      }
-      sweeps += 1;
-      u32 next = base_i;
-      if (pos > 0) {
-        u64 acc = (u64)(__umulhi(R + j1, magic) >> shift) * w1;
-        if (MODE == 0) acc += (u64)(__umulhi(R + Jg, magic) >> shift) * w2;
-        const u32 part = acc > (u64)kFastClamp ? kFastClamp : (u32)acc;
-        next += __reduce_add_sync(kFull, part);
-      }
-      if (next == R) break;
-      R = next;
-    }
-    if (verdict != 0) break;
-    // publish: R_i goes out; lane `pos` forms the jitters J^c = R - (C+G^m), J^g = R - G^e (a
-    // CPU-only task has no J^c unless the printed form of Lemma 7 is asked for)
-    if (lane == pos) {
-      if (p.out_wcrt) p.out_wcrt[a + f.w] = (i64)R;
-      if (MODE == 0 ? gpu_r : (MODE == 2 ? (gpu_r || literal) : false)) Jc = R - A_r + Tm1;
-      Jg = R - Ge_r + Tm1;
-    }
-  }
-  if (verdict == 0 && limit < n_rt) return 0;  // undecided: the full pass takes over
-  const int n_done = pos;  // ranks that converged (= n_rt without a verdict)
-  if (p.out_wcrt) {
-#pragma unroll
-    for (int s = 0; s < SLOTS; ++s) {
-      const int r = rank[s];
-      if (lane + 32 * s < n && r >= n_done)
-        p.out_wcrt[a + lane + 32 * s] = r >= n_rt ? (i64)GCAPS_WCRT_BEST_EFFORT
-                                                  : (r == n_done ? (i64)verdict : (i64)GCAPS_WCRT_SKIPPED);
-    }
-  }
-  if (lane == 0) p.out_sched[t] = verdict == 0 ? GCAPS_SCHED_YES : GCAPS_SCHED_NO;
-  return 1;
-}
-
 // An analysis mode known at compile time (converts to int like a run-time mode does).
 template <int V>
 struct ModeTag {
@@ -599,16 +385,12 @@ struct ModeTag {
 // is null; out_sched + block * n_tasksets).  Without SWEEP, MASK has one bit and the analysis
 // takes its constants and outputs from `p`.
 //
-// Returns, per group, kFastDone (outputs written), kFastDeclined (some value does not fit the
-// 32-bit path or the taskset is invalid; nothing written: the caller runs the exact path) or, with
-// FIRST_ONLY, kFastUndecided.  FIRST_ONLY (one analysis, a warp per taskset): only the first ranks
-// of the priority order are analysed (first_ranks below); if they all converge and more ranks
-// follow, nothing is decided and the caller runs the full pass.
-constexpr int kFastDeclined = 0, kFastDone = 1, kFastUndecided = 2;
-template <int LPT, int SLOTS, int MASK, bool SWEEP = false, bool FIRST_ONLY = false>
+// Returns, per group, kFastDone (outputs written) or kFastDeclined (some value does not fit the
+// 32-bit path or the taskset is invalid; nothing written: the caller runs the exact path).
+constexpr int kFastDeclined = 0, kFastDone = 1;
+template <int LPT, int SLOTS, int MASK, bool SWEEP = false>
 __device__ __forceinline__ int analyse_fast(const KParams &p, bool live, i64 t, i64 a, int n, u32 *buf, int lane,
                                             unsigned int gmask, const SweepArgs *sw = nullptr) {
-  static_assert(!FIRST_ONLY || (LPT == 32 && !SWEEP), "the first ranks' own pass: a warp per taskset");
   typedef FastLayout<LPT, SLOTS> Lay;
   constexpr int MAXN = Lay::MAXN, CAP = Lay::CAP;
   // prefix blocks of the CPU segments whose loads are issued together.  Tasksets of 65..96 tasks
@@ -751,7 +533,7 @@ __device__ __forceinline__ int analyse_fast(const KParams &p, bool live, i64 t, 
           n_rt -= __popc(__ballot_sync(kFull, lane + LPT * s < n && prio[s] <= 0) & gmask);
       }
       int n_narrow = n_rt;
-      if (!FIRST_ONLY && __any_sync(kFull, any_wide)) {
+      if (__any_sync(kFull, any_wide)) {
 #pragma unroll
         for (int s = 0; s < SLOTS; ++s)
           if (lane + LPT * s < n && T[s] >= kNarrowLimit && rank[s] < n_narrow) n_narrow = rank[s];
@@ -763,16 +545,10 @@ __device__ __forceinline__ int analyse_fast(const KParams &p, bool live, i64 t, 
       }
       if (lane == 0) Q0[-2] = (u32)n_rt, Q0[-3] = (u32)n_narrow;
     }
-    // what the row of a rank says about the task itself (the first ranks' own pass keeps the
-    // period and the position there instead)
+    // what the row of a rank says about the task itself
 #pragma unroll
-    for (int s = 0; s < SLOTS; ++s) {
-      if constexpr (FIRST_ONLY) {
-        if (rank[s] < kFirstRanks) rows.a(rank[s]) = make_uint4(D[s], core[s], T[s], (u32)(lane + LPT * s));
-      } else {
-        if (lane + LPT * s < n) *reinterpret_cast<uint2 *>(&rows.a(rank[s])) = make_uint2(D[s], core[s]);
-      }
-    }
+    for (int s = 0; s < SLOTS; ++s)
+      if (lane + LPT * s < n) *reinterpret_cast<uint2 *>(&rows.a(rank[s])) = make_uint2(D[s], core[s]);
   }
   // end offsets: the next task's start (positions beyond n hold the total)
   int c1[SLOTS], g1[SLOTS];
@@ -798,19 +574,6 @@ __device__ __forceinline__ int analyse_fast(const KParams &p, bool live, i64 t, 
   const i64 *__restrict__ Xm = p.gseg_misc + gfirst, *__restrict__ Xe = p.gseg_exec + gfirst;
   const int parc = (int)(((uintptr_t)Xc >> 3) & 1), parm = (int)(((uintptr_t)Xm >> 3) & 1);
   const int pare = (int)(((uintptr_t)Xe >> 3) & 1);
-  if constexpr (FIRST_ONLY) {
-    constexpr int MODE = (MASK & 1) ? 0 : (MASK & 2) ? 1 : (MASK & 4) ? 2 : 3;
-    uint4 *info = reinterpret_cast<uint4 *>(buf + Lay::kInfo);
-    uint4 *first8 = info + kFirstRanks;  // (only the first ranks' rows of `info` are used here)
-#pragma unroll
-    for (int s = 0; s < SLOTS; ++s)
-      if (rank[s] < kFirstRanks) first8[rank[s]] = make_uint4((u32)c0[s], (u32)c1[s], (u32)g0[s], (u32)g1[s]);
-    __syncwarp();
-    const int r = first_ranks<SLOTS, MODE>(p, t, a, n, info, first8, Q0, Q1, (int)Q0[-2], rank, g0, g1, Xc, Xm, Xe,
-                                           Nc, Ng, parc, parm, pare, cfirst, gfirst, lane, literal);
-    __syncwarp();
-    return r > 0 ? kFastDone : (r == 0 ? kFastUndecided : kFastDeclined);
-  }
   if (lane == 0) Q0[-1] = 0, Q1[-1] = 0;
   {  // CPU segments -> Q0
     const bool inside = slice_is_inside(cfirst, Nc, parc, p.n_csegs);
@@ -1029,6 +792,40 @@ static_assert(sizeof(Ahead) == 32, "two 16-byte rows");
 constexpr int kMaxAhead = 16;  // tasksets of one pull
 constexpr int kAheadWords = 2 * kMaxAhead * (int)(sizeof(Ahead) / sizeof(u32));  // two chunks
 
+constexpr u32 kNoTaskset = 0xffffffffu;
+
+// Looks up one taskset (or none) of a bin for at most MAXN tasks and CAP-1 segments of a kind.
+template <int MAXN, int CAP>
+__device__ __forceinline__ Ahead look_up_taskset(const KParams &p, u32 t) {
+  static_assert(MAXN <= 256 && CAP <= 2048, "fields of Ahead::packed");
+  Ahead me;
+  me.a = 0, me.c_lo = me.g_lo = 0, me.t = t, me.packed = 0;
+  if (t != kNoTaskset) {
+    me.a = p.task_off[t] - p.task_base;
+    const i64 b = p.task_off[(i64)t + 1] - p.task_base;
+    if (me.a >= 0 && b > me.a && b <= p.n_tasks && b - me.a <= MAXN) {
+      u32 nc = 0, ng = 0;
+      me.c_lo = p.cseg_off[me.a] - p.cseg_base, me.g_lo = p.gseg_off[me.a] - p.gseg_base;
+      const i64 c_hi = p.cseg_off[b] - p.cseg_base, g_hi = p.gseg_off[b] - p.gseg_base;
+      if (me.c_lo >= 0 && c_hi <= p.n_csegs && c_hi - me.c_lo < CAP && c_hi > me.c_lo) nc = (u32)(c_hi - me.c_lo);
+      if (me.g_lo >= 0 && g_hi <= p.n_gsegs && g_hi - me.g_lo < CAP && g_hi > me.g_lo) ng = (u32)(g_hi - me.g_lo);
+      me.packed = (u32)(b - me.a) | (nc << 9) | (ng << 20) | 0x80000000u;
+    }
+  }
+  return me;
+}
+
+// The segment slices start their way into L2 (16 elements per line, only addresses inside the
+// arrays); the per-task loads follow at once, so that the running sums later wait for L2 rather
+// than for DRAM.
+template <int LPT>
+__device__ __forceinline__ void prefetch_segments(const KParams &p, const Ahead &me, int lane) {
+  const int nc = (int)((me.packed >> 9) & 0x7ffu), ng = (int)((me.packed >> 20) & 0x7ffu);
+  for (int e = 16 * lane; e < nc; e += 16 * LPT) prefetch_l2(p.cseg_wcet + me.c_lo + e);
+  for (int e = 16 * lane; e < ng; e += 16 * LPT)
+    prefetch_l2(p.gseg_misc + me.g_lo + e), prefetch_l2(p.gseg_exec + me.g_lo + e);
+}
+
 // blocks per SM the register allocation aims at: more warps in flight matter more here than a
 // few spilled values, because every phase is a chain of dependent instructions and the loads of
 // a taskset can only be hidden behind the work of other warps
@@ -1058,36 +855,19 @@ __device__ __forceinline__ void run_bin(const KParams &p, int bin, u32 *warp_buf
   // without work
   const unsigned int n_groups = gridDim.x * (kBlockThreads / 32) * G;
   const int rounds = count >= 32 * n_groups ? (G == 1 ? 8 : kMaxAhead / G)
-                                            : (count >= 8 * n_groups ? 4 / (G > 2 ? 2 : 1) : 1);
+                                      : (count >= 8 * n_groups ? 4 / (G > 2 ? 2 : 1) : 1);
   const int chunk = rounds * G;  // <= kMaxAhead
 
   // lanes 0..chunk-1 each look up one taskset of a chunk and leave what they found in `slot`
   auto look_up = [&](unsigned int first, Ahead *slot) {
     if (lane32 < chunk) {
-      Ahead me;
-      me.a = 0, me.c_lo = me.g_lo = 0, me.t = 0, me.packed = 0;
-      if (first < count && first + lane32 < count) {
-        me.t = p.perm[start + first + lane32];
-        me.a = p.task_off[me.t] - p.task_base;
-        const i64 b = p.task_off[(i64)me.t + 1] - p.task_base;
-        if (me.a >= 0 && b > me.a && b <= p.n_tasks && b - me.a <= MAXN) {
-          u32 nc = 0, ng = 0;
-          me.c_lo = p.cseg_off[me.a] - p.cseg_base, me.g_lo = p.gseg_off[me.a] - p.gseg_base;
-          const i64 c_hi = p.cseg_off[b] - p.cseg_base, g_hi = p.gseg_off[b] - p.gseg_base;
-          if (me.c_lo >= 0 && c_hi <= p.n_csegs && c_hi - me.c_lo < Lay::CAP && c_hi > me.c_lo)
-            nc = (u32)(c_hi - me.c_lo);
-          if (me.g_lo >= 0 && g_hi <= p.n_gsegs && g_hi - me.g_lo < Lay::CAP && g_hi > me.g_lo)
-            ng = (u32)(g_hi - me.g_lo);
-          me.packed = (u32)(b - me.a) | (nc << 9) | (ng << 20) | 0x80000000u;
-        }
-      }
-      slot[lane32] = me;
+      u32 t = kNoTaskset;
+      if (first < count && first + lane32 < count) t = p.perm[start + first + lane32];
+      slot[lane32] = look_up_taskset<MAXN, Lay::CAP>(p, t);
     }
     __syncwarp();
   };
-  static_assert(MAXN <= 256 && Lay::CAP <= 2048, "fields of Ahead::packed");
 
-  int undecided_run = 0, tried_since = 0;  // (the first ranks' own pass, see below)
   unsigned int first = 0;
   if (lane32 == 0) first = atomicAdd(&p.hdr->next[bin], (unsigned int)chunk);
   first = __shfl_sync(kFull, first, 0);
@@ -1106,41 +886,14 @@ __device__ __forceinline__ void run_bin(const KParams &p, int bin, u32 *warp_buf
         look_up(nfirst, nxt);
       }
       const int mine = c * G + group;
+      const Ahead me = cur[mine < in_chunk ? mine : 0];
       const bool have = mine < in_chunk;
-      const Ahead me = cur[have ? mine : 0];
       const i64 t = (i64)me.t;
-      const int n = (int)(me.packed & 0x1ffu), nc = (int)((me.packed >> 9) & 0x7ffu);
-      const int ng = (int)((me.packed >> 20) & 0x7ffu);
+      const int n = (int)(me.packed & 0x1ffu);
       const bool fast = have && fast_call && (me.packed >> 31) != 0;
-      // the segment slices start their way into L2 now; the per-task loads follow at once, so
-      // that the running sums later wait for L2 rather than for DRAM (16 elements per line,
-      // only addresses inside the arrays)
-      if (have) {
-        for (int e = 16 * lane; e < nc; e += 16 * LPT) prefetch_l2(p.cseg_wcet + me.c_lo + e);
-        for (int e = 16 * lane; e < ng; e += 16 * LPT)
-          prefetch_l2(p.gseg_misc + me.g_lo + e), prefetch_l2(p.gseg_exec + me.g_lo + e);
-      }
+      if (have) prefetch_segments<LPT>(p, me, lane);
       int how = kFastDeclined;
-      if constexpr (LPT == 32 && !SWEEP && (MASK & 12) != 0) {
-        // Far from schedulable, a taskset ends with a miss among its first ranks; nearly
-        // schedulable, looking at them first is wasted.  Tasksets of a batch tend to be alike:
-        // after four undecided ones in a row only every sixteenth taskset is tried that way.
-        // (Round robin only: with tens of GPU-using tasks taking turns on the GPU the first or
-        // second rank already misses, and the pass pays; under GCAPS the first miss comes a few
-        // ranks later and the pass was measured slower than the full one.)
-        if (fast) {
-          how = kFastUndecided;
-          if (undecided_run < 4 || (tried_since & 15) == 0) {
-            how = analyse_fast<LPT, SLOTS, MASK, false, true>(p, true, t, me.a, n, buf, lane, gmask);
-            undecided_run = how == kFastUndecided ? undecided_run + 1 : 0;
-            __syncwarp();
-          }
-          tried_since += 1;
-        }
-        if (how == kFastUndecided) how = analyse_fast<LPT, SLOTS, MASK, SWEEP>(p, true, t, me.a, n, buf, lane, gmask, sw);
-      } else if (fast_call) {
-        how = analyse_fast<LPT, SLOTS, MASK, SWEEP>(p, fast, t, me.a, n, buf, lane, gmask, sw);
-      }
+      if (fast_call) how = analyse_fast<LPT, SLOTS, MASK, SWEEP>(p, fast, t, me.a, n, buf, lane, gmask, sw);
       __syncwarp();
       if (have && how != kFastDone) {
         if (!SWEEP) {

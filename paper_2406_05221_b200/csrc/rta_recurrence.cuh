@@ -152,8 +152,8 @@ struct Outcome {
 // GCAPS_RTA_ITER_CAP: a longer climb from base_i could run into the sweep limit, which is part of
 // the result.
 // `blocks_made`: blocks of ranks already in single precision (kept across the analyses of a sweep).
-template <int LPT, int SLOTS, int MODE, bool SWEEP>
-__device__ __forceinline__ Outcome recurrence_narrow(const Rows<LPT, SLOTS, SWEEP> rows, int n_f, int n_gpu,
+template <int LPT, int SLOTS, int MODE, bool SWEEP, class RowsT>
+__device__ __forceinline__ Outcome recurrence_narrow(const RowsT rows, int n_f, int n_gpu,
                                                      const PairConsts &pc, bool literal, int lane,
                                                      unsigned int gmask, int &blocks_made) {
   constexpr bool kGcaps = MODE < 2;
