@@ -6,16 +6,20 @@
 // constant of the taskset and the tasks of a taskset can be bounded in any order.  A group of 8,
 // 16 or 32 lanes works on one taskset (tasksets are binned by size with the same plan as the
 // default analysis); lane l of the group keeps, in registers, what its tasks (positions l,
-// l + lanes, ...) contribute as interferers: the reciprocal of T_h, the same-core pairs
-// (J^c_h, C_h + G^{m*}_h) and (J^g_h, G^e_h), and the other-core pair (J^g_h, G^{e*}_h).
-// Bounding one task is then: a per-lane choice of which pairs apply (same core and higher CPU
-// priority; or higher GPU priority, which during the search means "still without a level"), and
-// sweeps of multiply-high / shift / multiply-add summed across the group.  All values of a
-// taskset below 2^26 us: 32-bit arithmetic; otherwise the same loop in saturating 64-bit.
+// l + lanes, ...) contribute as interferers: 1/T_h, the same-core pairs (J^c_h, C_h + G^{m*}_h) and
+// (J^g_h, G^e_h), and the other-core pair (J^g_h, G^{e*}_h).  Bounding one task is then: a per-lane
+// choice of which pairs apply (same core and higher CPU priority; or "still without a level"), and
+// sweeps summed across the group.
+//
+// search_narrow does the search for tasksets whose periods all lie below kNarrowLimit: staged and
+// aggregated like the default analysis (stage_fast), bounded in packed single precision with exact
+// integer results (see rta_recurrence.cuh).  analyse_gpu_priority takes all others, and given
+// priorities: 32-bit integers while all values of a taskset are below 2^26 us, else the same loop in
+// saturating 64-bit.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include "rta_common.cuh"
+#include "rta_device.cuh"
 
 using namespace gcaps_detail;
 
@@ -136,7 +140,7 @@ __device__ __forceinline__ i64 bound_of(const GpLane<S> &me, int lane, unsigned 
 }
 
 template <int LPT, int S>
-__device__ void analyse_gpu_priority(const GpParams &g, i64 t, GpSmem<LPT * S> &sm, int lane,
+__device__ __noinline__ void analyse_gpu_priority(const GpParams &g, i64 t, GpSmem<LPT * S> &sm, int lane,
                                      unsigned int gmask) {
   constexpr int MAXN = LPT * S;
   const KParams &p = g.k;
@@ -402,67 +406,306 @@ __device__ void analyse_gpu_priority(const GpParams &g, i64 t, GpSmem<LPT * S> &
   __syncwarp(gmask);
 }
 
-// The tasksets of one size bin, pulled from the bin's counter by the warps of the launch.
-// `warp_smem` is this warp's own shared memory (the same stride for every bin a kernel covers:
-// the warps of a block may be working on different bins at the same time).
-template <int LPT, int S>
-__device__ __forceinline__ void run_bin(const GpParams &g, int bin, unsigned char *warp_smem) {
-  constexpr int G = 32 / LPT;  // tasksets per warp
-  typedef GpSmem<LPT * S> Sm;
+// The search of Sec. 5.3 in single precision.  Called by the whole warp; its groups step from bound to
+// bound side by side and sweep until the last of them has settled.  Returns, per group, whether its
+// taskset is done (outputs written); the others are analyse_gpu_priority's.
+//
+// Bound by instruction issue (4,420 warp instructions per 80-task taskset of `large`, 60 % of the issue
+// slots; about 15 bounds and 43 sweeps each).  100,000 of them 1.19 -> 0.77 ms: what went are per-lane
+// loops over global memory for the sums, a quadratic loop for every core's lowest task, 64-bit state
+// and the integer form of the terms (7,230 instructions).
+template <int LPT, int S, bool BUSY>
+__device__ __forceinline__ bool search_narrow(const GpParams &g, bool live, i64 t, i64 a, int n, u32 *buf, int lane,
+                                              unsigned int gmask) {
+  const KParams &p = g.k;
+  const bool literal = (p.policy & GCAPS_RTA_LITERAL) != 0;
+  const u32 eps = (u32)p.ovh;
+  const Rows<LPT, S, false> rows{buf};
+  TaskValues<S> o;
+  if (!stage_fast<LPT, S, (S <= 3 ? S : 2), true>(p, live, a, n, buf, rows, lane, gmask, false, eps, o)) return false;
+  live = o.live && o.n_narrow == o.n;
+  if (LPT == 32 ? !live : !__any_sync(kFull, live)) return false;
+  n = live ? o.n : 0;
+  // what this lane's tasks contribute as interferers; inv = 0 where there is no task
+  float inv[S], Kc[S], Kg[S], Wc[S], We[S], Wes[S];
+  u32 core[S], found[S];  // found: level << 23 | bound, 0 without a level
+  PairConsts pc;
+  pc.ovh = eps, pc.slot_cost = 0;
+  u32 unplaced = 0;  // bit s: the task of slot s has no level yet
+#pragma unroll
+  for (int s = 0; s < S; ++s) {
+    inv[s] = Kc[s] = Kg[s] = Wc[s] = We[s] = Wes[s] = 0.0f, core[s] = 0xffffffffu, found[s] = 0;
+    if (lane + LPT * s < n) {
+      uint4 row = rows.a(o.rank[s]);
+      const float T = (float)o.T[s], D = (float)row.x, A = (float)o.A[s], Ge = (float)o.Ge[s];
+      const bool gpu = o.eta[s] > 0;
+      u32 star, base;
+      own_cost<true>(pc, o.A[s], o.Ge[s], o.eta[s], 0, 0, star, base);
+      // Sec. 6.4: J^c_h = D_h - (C_h + G^m_h), J^g_h = D_h - G^e_h (a task whose own execution exceeds
+      // its deadline has no such slack: 0); a CPU-only tau_h has no J^c (Lemma 15), and none matters
+      // in busy-waiting mode.  As J + T - 1/2 - 2^23, like in the recurrence.
+      const float k = (T - 0.5f) - kTwo23, St = (float)star;
+      inv[s] = __frcp_rn(T), core[s] = row.y;
+      Kc[s] = (!BUSY && gpu) ? k + fmaxf(D - A, 0.0f) : k;
+      Kg[s] = k + fmaxf(D - Ge, 0.0f);
+      We[s] = Ge, Wes[s] = gpu ? Ge + St : 0.0f;
+      Wc[s] = BUSY ? A : A + St;  // Lemma 12: C_h + G^m_h; Lemma 15: C_h + G^{m*}_h (star = 0 without segments)
+      unplaced |= 1u << s;
+      row.x += kOne23;
+      row.z = kOne23 + (base < 0x7fffffu ? base : 0x7fffffu);
+      row.w = (u32)(lane + LPT * s) | (gpu ? 0x10000u : 0u);
+      rows.a(o.rank[s]) = row;
+    }
+  }
+  __syncwarp();
+  auto group_max = [&](int v) -> int {
+    if constexpr (LPT == 32) {
+      return __reduce_max_sync(kFull, v);
+    } else {
+#pragma unroll
+      for (int d = 1; d < LPT; d <<= 1) {
+        const int y = __shfl_xor_sync(kFull, v, d);
+        v = y > v ? y : v;
+      }
+      return v;
+    }
+  };
+  // cand: bit r set = the task of CPU rank r has no level yet and no task of lower CPU priority on its
+  // core is without one, i.e. it may take the next level (the same-core rule of Sec. 5.3).  To start
+  // with, the lowest task of every core.
+  constexpr int kWords = LPT * S > 32 ? LPT * S / 32 : 1;
+  u32 cand[kWords];
+#pragma unroll
+  for (int k = 0; k < kWords; ++k) cand[k] = 0;
+  auto flip = [&](int r) {
+#pragma unroll
+    for (int k = 0; k < kWords; ++k)
+      if (r >= 0 && (r >> 5) == k) cand[k] ^= 1u << (r & 31);
+  };
+  {
+    u32 rest = unplaced;
+    for (;;) {
+      int low = -1;
+#pragma unroll
+      for (int s = 0; s < S; ++s)
+        if ((rest >> s & 1u) && o.rank[s] > low) low = o.rank[s];
+      low = group_max(low);
+      if (LPT == 32 ? low < 0 : !__any_sync(kFull, low >= 0)) break;
+      flip(low);
+      const u32 its_core = rows.a(low < 0 ? 0 : low).y;
+#pragma unroll
+      for (int s = 0; s < S; ++s)
+        if (core[s] == its_core) rest &= ~(1u << s);
+      if (low < 0) rest = 0;
+    }
+  }
+  bool active = live && n > 0;
+  int sched = GCAPS_SCHED_YES, level = 1, want = n;
+  for (;;) {
+    // ---- the next candidate, from the lowest CPU priority upwards ---------------------------------
+    int next = -1;
+#pragma unroll
+    for (int k = 0; k < kWords; ++k) {
+      const int below = want - 32 * k;  // ranks 32 k .. 32 k + 31 that count: those below `want`
+      const u32 m = below >= 32 ? cand[k] : (below <= 0 ? 0u : cand[k] & ((1u << below) - 1u));
+      if (m) next = 32 * k + 31 - __clz((int)m);
+    }
+    want = next;
+    if (active && want < 0) sched = GCAPS_SCHED_NO, active = false;
+    if (LPT == 32 ? !active : !__any_sync(kFull, active)) break;
+    const uint4 row = rows.a(want < 0 ? 0 : want);
+    const u32 core_i = row.y;
+    const float Db = __uint_as_float(row.x), base_b = __uint_as_float(row.z);
+    const int c = (int)(row.w & 0xffffu);
+    const bool gi = (row.w & 0x10000u) != 0;
+    // ---- the (J, W) pairs; W = 0 where a pair does not apply ----------------------------------------
+    f32x2 I2[S], J2[S], W2[S];
+#pragma unroll
+    for (int s = 0; s < S; ++s) {
+      const bool hpp = core[s] == core_i && o.rank[s] < want;
+      const bool hpg = (unplaced >> s & 1u) && !hpp && lane + LPT * s != c;  // hp(tau_i) of Sec. 6.4 minus hpp
+      float w1 = 0.0f, w2 = 0.0f;
+      if (BUSY) {
+        if (hpp) w1 = Wc[s] + ((gi || !literal) ? Wes[s] : 0.0f);  // Lemmas 12, 10
+        if (hpg) w2 = Wes[s];                                      // Lemmas 10, 11
+      } else {
+        if (hpp) w1 = Wc[s];                                       // Lemma 15
+        if (gi) w2 = hpp ? We[s] : (hpg ? Wes[s] : 0.0f);          // Lemma 13: same core, other cores
+      }
+      I2[s] = pack2(inv[s], inv[s]), J2[s] = pack2(Kc[s], Kg[s]), W2[s] = pack2(w1, w2);
+    }
+    const f32x2 two23 = pack2(kTwo23, kTwo23), minus23 = pack2(-kTwo23, -kTwo23);
+    const u32 base_bits = __float_as_uint(base_b) - 32u * kOne23;
+    const f32x2 acc0 = LPT == 32 ? pack2(kTwo23, 0.0f) : pack2(0.0f, 0.0f);
+    auto total = [&](f32x2 acc) -> float {  // base + the group's sum, as 2^23 + value
+      float f = sum2(acc);
+      if constexpr (LPT == 32) {
+        f = fminf(f, kTwo23 + 4194304.0f);
+        return __uint_as_float(__reduce_add_sync(kFull, __float_as_uint(f)) + base_bits);
+      } else {
+#pragma unroll
+        for (int d = 1; d < LPT; d <<= 1) f += __shfl_xor_sync(kFull, f, d);
+        return base_b + f;
+      }
+    };
+    f32x2 acc = acc0;
+#pragma unroll
+    for (int s = 0; s < S; ++s) acc = add2(acc, W2[s]);
+    const float all_once = total(acc);  // (a first iterate as in recurrence_narrow)
+    float R = (Db - base_b < (float)GCAPS_RTA_ITER_CAP && base_b > kTwo23) ? all_once : base_b;
+    bool go = active && !(R > Db);
+    int left = (int)GCAPS_RTA_ITER_CAP;
+    while ((LPT == 32 ? go : __any_sync(kFull, go)) && left > 0) {
+      left -= 1;
+      const f32x2 RR = pack2(R, R);
+      acc = acc0;
+#pragma unroll
+      for (int s = 0; s < S; ++s) {
+        const f32x2 q = fma2_down(add2(RR, J2[s]), I2[s], two23);
+        acc = fma2(add2(q, minus23), W2[s], acc);
+      }
+      const float to = total(acc);
+      const bool moved = go && to != R;
+      R = moved ? to : R;
+      go = moved && !(R > Db);
+    }
+    // ---- a bound within the deadline takes the level -------------------------------------------------
+    const bool placed = active && !go && !(R > Db);
+    if (LPT == 32 ? placed : __any_sync(kFull, placed)) {
+      int up = -1;  // the task of the core that becomes a candidate now
+#pragma unroll
+      for (int s = 0; s < S; ++s) {
+        if (placed && lane + LPT * s == c) {
+          unplaced &= ~(1u << s);
+          found[s] = ((u32)level << 23) | (__float_as_uint(R) - kOne23);
+        }
+        if ((unplaced >> s & 1u) && core[s] == core_i && o.rank[s] < want && o.rank[s] > up) up = o.rank[s];
+      }
+      up = group_max(up);
+      if (placed) {
+        flip(want);
+        flip(up);
+        level += 1, want = n;
+        if (level > n) active = false;
+      }
+    }
+  }
+  // ---- results ------------------------------------------------------------------------------------------
+#pragma unroll
+  for (int s = 0; s < S; ++s) {
+    if (lane + LPT * s < n) {
+      const u32 lv = found[s] >> 23;
+      p.out_wcrt[a + lane + LPT * s] = lv > 0 ? (i64)(found[s] & 0x7fffffu) : (i64)GCAPS_WCRT_MISS;
+      g.gpu_prio_out[a + lane + LPT * s] = (i64)lv;
+    }
+  }
+  if (live && lane == 0) p.out_sched[t] = (uint8_t)sched;
+  __syncwarp();
+  return live;
+}
+
+// The tasksets of one size bin, pulled in chunks from the bin's counter by the warps of the launch; the
+// next chunk is looked up while the current one is worked on.  `warp_buf` is this warp's own shared
+// memory (the same stride for every bin a kernel covers: the warps of a block may be working on
+// different bins at the same time).
+template <int LPT, int S, bool BUSY>
+__device__ __forceinline__ void run_gp_bin(const GpParams &g, int bin, u32 *warp_buf, Ahead *ahead) {
+  constexpr int G = 32 / LPT, MAXN = LPT * S;  // tasksets per warp
+  typedef FastLayout<LPT, S> Lay;
+  typedef GpSmem<MAXN> Sm;
+  static_assert(sizeof(Sm) <= sizeof(u32) * Lay::kWords && sizeof(u32) * Lay::kWords % 16 == 0, "the other path fits");
   const KParams &p = g.k;
   const int lane32 = threadIdx.x & 31, group = lane32 / LPT, lane = lane32 % LPT;
   const unsigned int gmask = LPT == 32 ? kFull : (((1u << LPT) - 1u) << (group * LPT));
-  Sm &sm = reinterpret_cast<Sm *>(warp_smem)[group];
+  u32 *const buf = warp_buf + group * Lay::kWords;
   const unsigned int start = p.hdr->bin_start[bin], count = p.hdr->bin_count[bin];
-  for (;;) {
-    unsigned int first = 0;
-    if (lane32 == 0) first = atomicAdd(&p.hdr->next[bin], (unsigned int)G);
-    first = __shfl_sync(kFull, first, 0);
-    if (first >= count) break;
-    if (first + group < count)
-      analyse_gpu_priority<LPT, S>(g, (i64)p.perm[start + first + group], sm, lane, gmask);
+  if (count == 0) return;
+  const bool fast_call = g.assign && p.ovh < (1 << 20);
+  const unsigned int n_groups = gridDim.x * (kBlockThreads / 32) * G;
+  const int chunk = G * (count >= 32 * n_groups ? (G == 1 ? 8 : kMaxAhead / G) : (count >= 8 * n_groups ? 2 : 1));
+  auto look_up = [&](unsigned int first, Ahead *slot) {
+    if (lane32 < chunk)
+      slot[lane32] = look_up_taskset<MAXN, Lay::CAP>(p, (first < count && first + lane32 < count) ? p.perm[start + first + lane32] : kNoTaskset);
     __syncwarp();
+  };
+  auto pull = [&]() {
+    unsigned int first = 0;
+    if (lane32 == 0) first = atomicAdd(&p.hdr->next[bin], (unsigned int)chunk);
+    return __shfl_sync(kFull, first, 0);
+  };
+  unsigned int first = pull();
+  int which = 0;
+  look_up(first, ahead);
+  while (first < count) {
+    const unsigned int nfirst = pull();
+    look_up(nfirst, ahead + (which ^ 1) * kMaxAhead);
+    const Ahead *cur = ahead + which * kMaxAhead;
+    const int in_chunk = count - first < (unsigned int)chunk ? (int)(count - first) : chunk;
+    for (int c = 0; c < in_chunk; c += G) {
+      const bool have = c + group < in_chunk;
+      const Ahead me = cur[have ? c + group : 0];
+      const bool fast = have && fast_call && (me.packed >> 31) != 0;
+      bool done = false;
+      if (fast_call) {
+        if (fast) prefetch_segments<LPT>(p, me, lane);
+        done = search_narrow<LPT, S, BUSY>(g, fast, (i64)me.t, me.a, (int)(me.packed & 0x1ffu), buf, lane, gmask);
+      }
+      __syncwarp();
+      if (have && !done) analyse_gpu_priority<LPT, S>(g, (i64)me.t, *reinterpret_cast<Sm *>(buf), lane, gmask);
+      __syncwarp();
+    }
+    first = nfirst;
+    which ^= 1;
   }
 }
 
-template <int LPT, int S>
-__host__ __device__ constexpr size_t warp_bytes() {
-  return (size_t)(32 / LPT) * sizeof(GpSmem<LPT * S>);
-}
-constexpr size_t cmax(size_t x, size_t y) { return x > y ? x : y; }
-constexpr size_t kSmallWarpBytes =
-    cmax(cmax(warp_bytes<16, 2>(), warp_bytes<8, 3>()), cmax(warp_bytes<8, 2>(), warp_bytes<8, 1>()));
-static_assert(kSmallWarpBytes % 16 == 0, "every warp's area starts 16-byte aligned");
-
 // the four bins of up to 32 tasks: (lanes per taskset, tasks per lane) as in the default analysis
-__global__ void __launch_bounds__(kBlockThreads) gpu_priority_small_kernel(GpParams g) {
+template <bool BUSY>
+__global__ void __launch_bounds__(kBlockThreads, 5) gpu_priority_small_kernel(GpParams g) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   let_dependents_start();  // the kernel of the next size bin shares no data with this one
-  unsigned char *mine = smem_raw + (threadIdx.x >> 5) * kSmallWarpBytes;
-  run_bin<16, 2>(g, 3, mine);
-  run_bin<8, 3>(g, 2, mine);
-  run_bin<8, 2>(g, 1, mine);
-  run_bin<8, 1>(g, 0, mine);
+  u32 *mine = reinterpret_cast<u32 *>(smem_raw) + (threadIdx.x >> 5) * kSmallWarpWords;
+  Ahead *ahead = reinterpret_cast<Ahead *>(mine + kSmallWarpWords - kAheadWords);
+  run_gp_bin<16, 2, BUSY>(g, 3, mine, ahead);
+  run_gp_bin<8, 3, BUSY>(g, 2, mine, ahead);
+  run_gp_bin<8, 2, BUSY>(g, 1, mine, ahead);
+  run_gp_bin<8, 1, BUSY>(g, 0, mine, ahead);
   wait_for_previous_grid();
 }
 
-// one bin of larger tasksets, a warp per taskset.  Five blocks per SM (96 registers): the search is
-// bound by instruction issue and dependent latency, and 20 warps hide more of it than the 16 that
-// the unbounded 127 registers allow, spills included (-7 % on 80-task tasksets).
-template <int S>
-__global__ void __launch_bounds__(kBlockThreads, 5) gpu_priority_big_kernel(GpParams g, int bin) {
+// one bin of larger tasksets, a warp per taskset
+__host__ __device__ constexpr int gp_min_blocks(int slots) { return slots <= 3 ? 5 : slots == 4 ? 4 : 2; }
+template <int S, bool BUSY>
+__global__ void __launch_bounds__(kBlockThreads, gp_min_blocks(S)) gpu_priority_big_kernel(GpParams g, int bin) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   let_dependents_start();
-  run_bin<32, S>(g, bin, smem_raw + (threadIdx.x >> 5) * warp_bytes<32, S>());
+  constexpr int kWarpWords = bin_warp_words<32, S>() + kAheadWords;
+  u32 *mine = reinterpret_cast<u32 *>(smem_raw) + (threadIdx.x >> 5) * kWarpWords;
+  run_gp_bin<32, S, BUSY>(g, bin, mine, reinterpret_cast<Ahead *>(mine + kWarpWords - kAheadWords));
   wait_for_previous_grid();
 }
 
-template <int S>
+template <int S, bool BUSY>
 cudaError_t launch_big(const GpParams &g, int bin, int sm_count, cudaStream_t st) {
   constexpr int kWarps = kBlockThreads / 32;
   static int blocks_per_sm[64] = {0};
-  return launch_persistent_ex(true, gpu_priority_big_kernel<S>, blocks_per_sm, warp_bytes<32, S>() * kWarps,
-                           (g.k.n_tasksets + kWarps - 1) / kWarps, sm_count, st, g, bin);
+  return launch_persistent_ex(true, gpu_priority_big_kernel<S, BUSY>, blocks_per_sm,
+                              sizeof(u32) * (bin_warp_words<32, S>() + kAheadWords) * kWarps,
+                              (g.k.n_tasksets + kWarps - 1) / kWarps, sm_count, st, g, bin);
+}
+
+template <bool BUSY>
+cudaError_t launch_gp_bins(const GpParams &g, int sm_count, cudaStream_t st) {
+  constexpr int kWarps = kBlockThreads / 32;
+  static int blocks_per_sm[64] = {0};
+  cudaError_t e = launch_persistent(gpu_priority_small_kernel<BUSY>, blocks_per_sm, sizeof(u32) * kSmallWarpWords * kWarps,
+                                    (g.k.n_tasksets + kWarps - 1) / kWarps, sm_count, st, g);
+  if (e == cudaSuccess) e = launch_big<2, BUSY>(g, 4, sm_count, st);
+  if (e == cudaSuccess) e = launch_big<3, BUSY>(g, 5, sm_count, st);
+  if (e == cudaSuccess) e = launch_big<4, BUSY>(g, 6, sm_count, st);
+  if (e == cudaSuccess) e = launch_big<6, BUSY>(g, 7, sm_count, st);
+  if (e == cudaSuccess) e = launch_big<8, BUSY>(g, 8, sm_count, st);
+  return e;
 }
 
 }  // namespace
@@ -492,17 +735,8 @@ extern "C" int gcaps_rta_gpu_priority_batch(const gcaps_tasksets_t *ts, int64_t 
   rc = enqueue_plan(g.k, workspace, workspace_bytes, st);
   if (rc != GCAPS_OK) return rc;
   cudaError_t e = cudaGetLastError();
-  if (e == cudaSuccess) {
-    constexpr int kWarps = kBlockThreads / 32;
-    static int blocks_per_sm[64] = {0};
-    e = launch_persistent(gpu_priority_small_kernel, blocks_per_sm, kSmallWarpBytes * kWarps,
-                          (n_tasksets + kWarps - 1) / kWarps, di.sm_count, st, g);
-  }
-  if (e == cudaSuccess) e = launch_big<2>(g, 4, di.sm_count, st);
-  if (e == cudaSuccess) e = launch_big<3>(g, 5, di.sm_count, st);
-  if (e == cudaSuccess) e = launch_big<4>(g, 6, di.sm_count, st);
-  if (e == cudaSuccess) e = launch_big<6>(g, 7, di.sm_count, st);
-  if (e == cudaSuccess) e = launch_big<8>(g, 8, di.sm_count, st);
+  if (e == cudaSuccess)
+    e = (flags & GCAPS_RTA_BUSY) ? launch_gp_bins<true>(g, di.sm_count, st) : launch_gp_bins<false>(g, di.sm_count, st);
   if (e != cudaSuccess) {
     g_last_cuda_error = (int)e;
     return GCAPS_ERR_CUDA;

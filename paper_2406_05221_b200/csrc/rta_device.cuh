@@ -370,52 +370,40 @@ struct ModeTag {
   __host__ __device__ constexpr operator int() const { return V; }
 };
 
-// MODE: 0 GCAPS self-suspension, 1 GCAPS busy-waiting, 2 RR self-suspension, 3 RR busy-waiting.
-//
-// A group of LPT lanes (8, 16 or a whole warp) works on one taskset; the whole warp calls this and
-// its groups go through every step side by side (`live`: the group has a taskset), so that each
-// shuffle, vote and reduction is one instruction for all of them.  Until the per-task sums are
-// known lane l of a group holds the tasks at positions l, l+LPT, ... ("slots"); then every task's
-// values go to the row of its rank in shared memory, where the recurrence finds them.
-//
-// MASK: bit m set = analysis MODE m is compiled in.  SWEEP: the taskset is staged, ordered and
-// aggregated once and then analysed under every (timeslice, overhead) pair q of `sw` and every
-// mode m of MASK that sw->enabled names; that analysis writes result block
-// q * sw->block_stride + sw->block_of_mode[m] (out_wcrt + block * n_tasks, skipped when out_wcrt
-// is null; out_sched + block * n_tasksets).  Without SWEEP, MASK has one bit and the analysis
-// takes its constants and outputs from `p`.
-//
-// Returns, per group, kFastDone (outputs written) or kFastDeclined (some value does not fit the
-// 32-bit path or the taskset is invalid; nothing written: the caller runs the exact path).
-constexpr int kFastDeclined = 0, kFastDone = 1;
-template <int LPT, int SLOTS, int MASK, bool SWEEP = false>
-__device__ __forceinline__ int analyse_fast(const KParams &p, bool live, i64 t, i64 a, int n, u32 *buf, int lane,
-                                            unsigned int gmask, const SweepArgs *sw = nullptr) {
+// What a taskset's staging, ordering and aggregation leave in a lane (slot s: position lane + LPT * s);
+// info rows (deadline, core) by rank are in shared memory.
+template <int SLOTS>
+struct TaskValues {
+  u32 T[SLOTS], A[SLOTS], Ge[SLOTS], eta[SLOTS];  // period, C+G^m, G^e, GPU segments
+  int rank[SLOTS], g0[SLOTS], g1[SLOTS];          // GPU segments of the task within the taskset's slice
+  int n, n_gpu, n_rt, n_narrow;  // tasks, GPU-using ones, real-time ones, ranks in single precision
+  int Ng, pare;                  // the taskset's G^e slice: elements, odd start
+  i64 gfirst;
+  bool live;
+};
+
+// Stage, order and aggregate, by a group of LPT lanes (8, 16 or a whole warp) per taskset; the whole
+// warp calls this and its groups go through every step side by side (`live`: the group has a taskset),
+// so that each shuffle, vote and reduction is one instruction for all of them.  False if no group of
+// the warp has a taskset that fits the 32-bit path; else o.live says which do.  BC: prefix blocks of
+// the CPU segments whose loads are issued together.  ovh_max: the largest epsilon of a GCAPS analysis.
+template <int LPT, int SLOTS, int BC, bool kAnyGcaps, class RowsT>
+__device__ __forceinline__ bool stage_fast(const KParams &p, bool live, i64 a, int n, u32 *buf, const RowsT rows, int lane,
+                                           unsigned int gmask, bool best_effort, u32 ovh_max, TaskValues<SLOTS> &o) {
   typedef FastLayout<LPT, SLOTS> Lay;
   constexpr int MAXN = Lay::MAXN, CAP = Lay::CAP;
-  // prefix blocks of the CPU segments whose loads are issued together.  Tasksets of 65..96 tasks
-  // with a few GPU segments per task have 200..400 CPU segments: three blocks of 128 cover them
-  // in one step where two need a second, mostly empty one (80-task tasksets: -4 % for a GCAPS
-  // kernel; the RR kernels, which carry the slice sums too, lose as much to the registers it takes)
-  constexpr int BC = SLOTS <= 2 ? SLOTS : ((SLOTS == 3 && (MASK & 12) == 0 && !SWEEP) ? 3 : 2);
   constexpr int BG = 1;
-  constexpr bool kAnyGcaps = (MASK & 3) != 0;
-  constexpr bool kMulti = (MASK & (MASK - 1)) != 0;
-  static_assert(!kMulti || SWEEP, "several analyses per taskset use the sweep loop");
-  const bool literal = (p.policy & GCAPS_RTA_LITERAL) != 0;
-  const bool best_effort = (p.policy & GCAPS_RTA_BEST_EFFORT) != 0;
-  const Rows<LPT, SLOTS, SWEEP> rows{buf};
   u32 *Q0 = buf + Lay::kQ0, *Q1 = buf + Lay::kQ1;
   // A group that has no taskset, or declines it, goes on as one with an empty taskset.
-#define GCAPS_LEAVE_IF_NONE_LIVE()                       \
-  do {                                                   \
-    if (LPT == 32 ? !live : !__any_sync(kFull, live)) return kFastDeclined; \
-    if (!live) n = 0, Nc = 0, Ng = 0;                    \
+#define GCAPS_LEAVE_IF_NONE_LIVE()                                    \
+  do {                                                                \
+    if (LPT == 32 ? !live : !__any_sync(kFull, live)) return false;   \
+    if (!live) n = 0, Nc = 0, Ng = 0;                                 \
   } while (0)
 
   // ---- stage: per-task scalars, lane = position; rank ----------------------------------------
-  u32 T[SLOTS];
-  int rank[SLOTS], c0[SLOTS], g0[SLOTS];
+  u32 (&T)[SLOTS] = o.T, (&A)[SLOTS] = o.A, (&Ge)[SLOTS] = o.Ge, (&eta)[SLOTS] = o.eta;
+  int (&rank)[SLOTS] = o.rank, (&g0)[SLOTS] = o.g0, (&g1)[SLOTS] = o.g1, c0[SLOTS], c1[SLOTS];
   int Nc = 0, Ng = 0;
   i64 cfirst, gfirst;
   {
@@ -551,7 +539,6 @@ __device__ __forceinline__ int analyse_fast(const KParams &p, bool live, i64 t, 
       if (lane + LPT * s < n) *reinterpret_cast<uint2 *>(&rows.a(rank[s])) = make_uint2(D[s], core[s]);
   }
   // end offsets: the next task's start (positions beyond n hold the total)
-  int c1[SLOTS], g1[SLOTS];
   {
     bool ok = true;
 #pragma unroll
@@ -568,7 +555,6 @@ __device__ __forceinline__ int analyse_fast(const KParams &p, bool live, i64 t, 
   }
 
   // ---- aggregate: running sums of the segment arrays; per-task sums are differences --------
-  u32 A[SLOTS], Ge[SLOTS];  // C+G^m, G^e
   u32 bad = 0;
   const i64 *__restrict__ Xc = p.cseg_wcet + cfirst;
   const i64 *__restrict__ Xm = p.gseg_misc + gfirst, *__restrict__ Xe = p.gseg_exec + gfirst;
@@ -595,7 +581,6 @@ __device__ __forceinline__ int analyse_fast(const KParams &p, bool live, i64 t, 
                             p.gseg_exec, p.gseg_exec + p.n_gsegs, Q0, Q1, cm, ce, bad, lane);
   }
   __syncwarp();
-  u32 eta[SLOTS];
 #pragma unroll
   for (int s = 0; s < SLOTS; ++s) {
     const u32 Gm = Q0[g1[s] - 1 + parm] - Q0[g0[s] - 1 + parm];
@@ -611,15 +596,64 @@ __device__ __forceinline__ int analyse_fast(const KParams &p, bool live, i64 t, 
 #pragma unroll
   for (int s = 0; s < SLOTS; ++s) n_gpu += __popc(__ballot_sync(kFull, eta[s] > 0) & gmask);
   if (kAnyGcaps) {  // 2 * eps * eta must stay below 2^26 (eta < 64, eps < 2^20: no overflow here)
-    const u32 ovh_max = SWEEP ? (u32)sw->max_ovh : (u32)p.ovh;
-#pragma unroll
+    #pragma unroll
     for (int s = 0; s < SLOTS; ++s) bad |= (2 * ovh_max * eta[s]) >> 26;
   }
   live = group_all<LPT>(bad == 0, gmask) && live;
-  if (LPT == 32 ? !live : !__any_sync(kFull, live)) return kFastDeclined;
-  if (!live) n = 0;
-  const int n_rt = live ? (int)Q0[-2] : 0;      // real-time tasks: the ranks that are analysed
-  const int n_narrow = live ? (int)Q0[-3] : 0;  // ... of which so many in single precision
+  if (LPT == 32 ? !live : !__any_sync(kFull, live)) return false;
+  o.live = live, o.n = live ? n : 0, o.n_gpu = n_gpu;
+  o.n_rt = live ? (int)Q0[-2] : 0, o.n_narrow = live ? (int)Q0[-3] : 0;
+  o.Ng = Ng, o.pare = pare, o.gfirst = gfirst;
+#undef GCAPS_LEAVE_IF_NONE_LIVE
+  return true;
+}
+
+// MODE: 0 GCAPS self-suspension, 1 GCAPS busy-waiting, 2 RR self-suspension, 3 RR busy-waiting.
+//
+// A group of LPT lanes works on one taskset, side by side with the other groups of its warp.  Until the
+// per-task sums are known lane l of a group holds the tasks at positions l, l+LPT, ... ("slots"); then
+// every task's values go to the row of its rank in shared memory, where the recurrence finds them.
+//
+// MASK: bit m set = analysis MODE m is compiled in.  SWEEP: the taskset is staged, ordered and
+// aggregated once and then analysed under every (timeslice, overhead) pair q of `sw` and every
+// mode m of MASK that sw->enabled names; that analysis writes result block
+// q * sw->block_stride + sw->block_of_mode[m] (out_wcrt + block * n_tasks, skipped when out_wcrt
+// is null; out_sched + block * n_tasksets).  Without SWEEP, MASK has one bit and the analysis
+// takes its constants and outputs from `p`.
+//
+// Returns, per group, kFastDone (outputs written) or kFastDeclined (some value does not fit the
+// 32-bit path or the taskset is invalid; nothing written: the caller runs the exact path).
+constexpr int kFastDeclined = 0, kFastDone = 1;
+template <int LPT, int SLOTS, int MASK, bool SWEEP = false>
+__device__ __forceinline__ int analyse_fast(const KParams &p, bool live, i64 t, i64 a, int n, u32 *buf, int lane,
+                                            unsigned int gmask, const SweepArgs *sw = nullptr) {
+  typedef FastLayout<LPT, SLOTS> Lay;
+  constexpr int MAXN = Lay::MAXN, CAP = Lay::CAP;
+  // prefix blocks of the CPU segments whose loads are issued together.  Tasksets of 65..96 tasks
+  // with a few GPU segments per task have 200..400 CPU segments: three blocks of 128 cover them
+  // in one step where two need a second, mostly empty one (80-task tasksets: -4 % for a GCAPS
+  // kernel; the RR kernels, which carry the slice sums too, lose as much to the registers it takes)
+  constexpr int BC = SLOTS <= 2 ? SLOTS : ((SLOTS == 3 && (MASK & 12) == 0 && !SWEEP) ? 3 : 2);
+  constexpr int BG = 1;
+  constexpr bool kAnyGcaps = (MASK & 3) != 0;
+  constexpr bool kMulti = (MASK & (MASK - 1)) != 0;
+  static_assert(!kMulti || SWEEP, "several analyses per taskset use the sweep loop");
+  const bool literal = (p.policy & GCAPS_RTA_LITERAL) != 0;
+  const bool best_effort = (p.policy & GCAPS_RTA_BEST_EFFORT) != 0;
+  const Rows<LPT, SLOTS, SWEEP> rows{buf};
+  u32 *Q0 = buf + Lay::kQ0, *Q1 = buf + Lay::kQ1;
+  TaskValues<SLOTS> o;
+  if (!stage_fast<LPT, SLOTS, BC, kAnyGcaps>(p, live, a, n, buf, rows, lane, gmask, best_effort,
+                                             SWEEP ? (u32)sw->max_ovh : (u32)p.ovh, o))
+    return kFastDeclined;
+  live = o.live, n = o.n;
+  u32 (&T)[SLOTS] = o.T, (&A)[SLOTS] = o.A, (&Ge)[SLOTS] = o.Ge, (&eta)[SLOTS] = o.eta;
+  int (&rank)[SLOTS] = o.rank, (&g0)[SLOTS] = o.g0, (&g1)[SLOTS] = o.g1;
+  const int n_gpu = o.n_gpu, Ng = o.Ng, pare = o.pare;
+  const i64 gfirst = o.gfirst;
+  const i64 *__restrict__ Xe = p.gseg_exec + gfirst;
+  const int n_rt = o.n_rt;          // real-time tasks: the ranks that are analysed
+  const int n_narrow = o.n_narrow;  // ... of which so many in single precision
 
   // Eq. 3: running sums of the slices of every pure GPU part for timeslice L (values already
   // checked) into Ps
@@ -674,10 +708,10 @@ __device__ __forceinline__ int analyse_fast(const KParams &p, bool live, i64 t, 
   // position: out_wcrt (unless null in a sweep) and out_sched.
   auto analyse = [&](auto mode_tag, const PairConsts &pc, i64 *out_wcrt, uint8_t *out_sched) {
     constexpr int MODE = mode_tag;  // a ModeTag: every analysis of a kernel gets its own copy
-    Outcome o = recurrence_narrow<LPT, SLOTS, MODE, SWEEP>(rows, n_narrow, n_gpu, pc, literal, lane, gmask, blocks_made);
-    if (o.verdict == 0 && n_narrow < n_rt) {
+    Outcome out_of = recurrence_narrow<LPT, SLOTS, MODE, SWEEP>(rows, n_narrow, n_gpu, pc, literal, lane, gmask, blocks_made);
+    if (out_of.verdict == 0 && n_narrow < n_rt) {
       __syncwarp(gmask);
-      o = recurrence_wide<LPT, SLOTS, MODE, SWEEP>(buf, n, n_rt, n_narrow, n_gpu, pc, literal, lane, gmask);
+      out_of = recurrence_wide<LPT, SLOTS, MODE, SWEEP>(buf, n, n_rt, n_narrow, n_gpu, pc, literal, lane, gmask);
     }
     __syncwarp();
     if (!SWEEP || out_wcrt) {
@@ -687,13 +721,13 @@ __device__ __forceinline__ int analyse_fast(const KParams &p, bool live, i64 t, 
         if (lane + LPT * s < n) {
           const int r = rank[s];
           i64 value = r >= n_rt ? (i64)GCAPS_WCRT_BEST_EFFORT
-                                : (r == o.n_done ? (i64)o.verdict : (i64)GCAPS_WCRT_SKIPPED);
-          if (r < o.n_done) value = (i64)rows.R(r);
+                                : (r == out_of.n_done ? (i64)out_of.verdict : (i64)GCAPS_WCRT_SKIPPED);
+          if (r < out_of.n_done) value = (i64)rows.R(r);
           out[LPT * s] = value;
         }
       }
     }
-    if (live && lane == 0) out_sched[t] = o.verdict == 0 ? GCAPS_SCHED_YES : GCAPS_SCHED_NO;
+    if (live && lane == 0) out_sched[t] = out_of.verdict == 0 ? GCAPS_SCHED_YES : GCAPS_SCHED_NO;
     __syncwarp();
   };
 
@@ -773,7 +807,6 @@ __device__ __forceinline__ int analyse_fast(const KParams &p, bool live, i64 t, 
       if ((MASK & 8) && (enabled & 8)) analyse_as(ModeTag<3>());
     }
   }
-#undef GCAPS_LEAVE_IF_NONE_LIVE
   return live ? kFastDone : kFastDeclined;
 }
 
