@@ -484,6 +484,7 @@ __device__ __forceinline__ bool search_narrow(const GpParams &g, bool live, i64 
   };
   {
     u32 rest = unplaced;
+#pragma unroll 1
     for (;;) {
       int low = -1;
 #pragma unroll
@@ -501,6 +502,7 @@ __device__ __forceinline__ bool search_narrow(const GpParams &g, bool live, i64 
   }
   bool active = live && n > 0;
   int sched = GCAPS_SCHED_YES, level = 1, want = n;
+#pragma unroll 1
   for (;;) {
     // ---- the next candidate, from the lowest CPU priority upwards ---------------------------------
     int next = -1;
@@ -555,6 +557,7 @@ __device__ __forceinline__ bool search_narrow(const GpParams &g, bool live, i64 
     float R = (Db - base_b < (float)GCAPS_RTA_ITER_CAP && base_b > kTwo23) ? all_once : base_b;
     bool go = active && !(R > Db);
     int left = (int)GCAPS_RTA_ITER_CAP;
+#pragma unroll 1
     while ((LPT == 32 ? go : __any_sync(kFull, go)) && left > 0) {
       left -= 1;
       const f32x2 RR = pack2(R, R);
@@ -641,6 +644,7 @@ __device__ __forceinline__ void run_gp_bin(const GpParams &g, int bin, u32 *warp
     look_up(nfirst, ahead + (which ^ 1) * kMaxAhead);
     const Ahead *cur = ahead + which * kMaxAhead;
     const int in_chunk = count - first < (unsigned int)chunk ? (int)(count - first) : chunk;
+#pragma unroll 1
     for (int c = 0; c < in_chunk; c += G) {
       const bool have = c + group < in_chunk;
       const Ahead me = cur[have ? c + group : 0];

@@ -37,8 +37,10 @@ template <int LPT, int SLOTS>
 struct FastLayout {
   static constexpr int MAXN = LPT * SLOTS;
   static constexpr int kStep = 4 * LPT;  // elements one prefix step of the group covers
-  // a prefix array takes slices of up to CAP-1 elements and is written kStep words at a time
-  static constexpr int CAP = (6 * MAXN + kStep - 1) / kStep * kStep;
+  // a prefix array takes slices of up to CAP-1 elements (a taskset with more goes through the 64-bit
+  // path) and is written kStep words at a time.  Small tasksets vary more: 8 per task (200,000 tasksets
+  // of `divergence` under GCAPS 480 -> 455 us against 6 per task)
+  static constexpr int CAP = ((LPT == 32 ? 6 : 8) * MAXN + kStep - 1) / kStep * kStep;
   static constexpr int kInfo = 0;  // row A by rank
   static constexpr int kQ0 = 4 * MAXN + 4;
   static constexpr int kQ1 = kQ0 + CAP + 4;
@@ -190,6 +192,7 @@ __device__ __forceinline__ Outcome recurrence_narrow(const RowsT rows, int n_f, 
       }
       __syncwarp();
     }
+#pragma unroll 1
     for (int pos = LPT * blk; pos < LPT * (blk + 1); ++pos) {
       const bool active = alive && pos < n_f;
       if constexpr (LPT == 32) {
@@ -321,6 +324,7 @@ __device__ __forceinline__ Outcome recurrence_narrow(const RowsT rows, int n_f, 
         }
       } else {
         bool go = active && !(R > Db);
+#pragma unroll 1
         while (__any_sync(kFull, go) && left > 0) {
           left -= 1;
           const float next = sweep(R);

@@ -251,7 +251,9 @@ __device__ __forceinline__ int staged_head(const KParams &p, const Ahead &me, St
     const i64 *const sC = reinterpret_cast<const i64 *>(stage + off1.z);
     const i64 *const sM = reinterpret_cast<const i64 *>(stage + off1.w);
     const i64 *const sE = reinterpret_cast<const i64 *>(stage + off2.x);
+#pragma unroll 1
     for (u32 j = c0 + sub; j < cn; j += 2) A += (u32)sC[j];
+#pragma unroll 1
     for (u32 j = g0 + sub; j < gn; j += 2) {
       const u32 e = (u32)sE[j];
       A += (u32)sM[j], Ge += e;
@@ -375,6 +377,7 @@ __device__ __forceinline__ void run_staged_bin(const KParams &p, int bin, u32 st
     const Ahead *cur = w.ahead + which * kStagedChunk;
     Ahead *nxt = w.ahead + (which ^ 1) * kStagedChunk;
     const int in_chunk = count - first < (unsigned int)chunk ? (int)(count - first) : chunk;
+#pragma unroll 1
     for (int c = 0; c < in_chunk; ++c) {
       if (c == 1 || in_chunk == 1) {  // the next chunk's index has arrived by now
         nfirst = __shfl_sync(kFull, nfirst, 0);
@@ -442,6 +445,7 @@ __device__ __forceinline__ void run_staged_bin(const KParams &p, int bin, u32 st
   }
   if (deferred > 0 && lane == 0) atomicAdd(&p.hdr->deferred[bin], deferred);
   u32 *const buf = reinterpret_cast<u32 *>(stage);
+#pragma unroll 1
   for (int k = 0; k < n_left; ++k)
     full_pass<SLOTS, MODE>(p, look_up_taskset<MAXN, Lay::CAP>(p, w.left[k]), fast_call, buf, lane);
 }
@@ -480,6 +484,7 @@ __device__ __forceinline__ void run_deferred_bin(const KParams &p, int bin, u32 
     if (t & kDeferred)
       ahead[(which ^ 1) * kMaxAhead + __popc(found & ((1u << lane) - 1u))] = look_up_taskset<MAXN, Lay::CAP>(p, t & ~kDeferred);
     __syncwarp();
+#pragma unroll 1
     for (int c = 0; c < in_chunk; ++c) full_pass<SLOTS, MODE>(p, ahead[which * kMaxAhead + c], fast_call, buf, lane);
     if (first >= count) break;
     in_chunk = __popc(found);
