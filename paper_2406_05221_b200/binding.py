@@ -59,18 +59,24 @@ class GcapsError(RuntimeError):
 
 
 _lib = None
+_raw_stream = None   # torch's accessor of the current stream's handle, where it has one
 
 
 def load_library(path: Optional[str] = None):
     """Loads libgcaps_rta.so (never builds it implicitly on a machine without the source
     being newer: a missing library is an error, not a reason to fall back)."""
-    global _lib
+    global _lib, _raw_stream
     if _lib is None or path is not None:
         path = path or _build.CUDA_LIB
         if not os.path.exists(path):
             raise FileNotFoundError(
                 "%s is missing: run `python -m paper_2406_05221_b200.build` (needs nvcc)" % path)
         lib = ctypes.CDLL(path)
+        try:
+            import torch
+            _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        except ImportError:
+            pass
         lib.gcaps_rta_batch.argtypes = [
             ctypes.POINTER(CTasksets), ctypes.c_int64, ctypes.c_int, ctypes.c_int64, ctypes.c_int64,
             ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_size_t, ctypes.c_void_p]
@@ -131,17 +137,36 @@ def load_library(path: Optional[str] = None):
     return _lib
 
 
-@contextlib.contextmanager
-def _device_and_stream(dev, stream):
+class _device_and_stream:
     """Makes ``dev`` the current device and ``stream`` (default: torch's current one) the current
-    stream.  Tensors the wrappers create inside (outputs, workspace) then belong to the stream the
-    kernels run on, so torch's allocator cannot hand their memory to someone else while those
-    kernels are still in flight."""
-    import torch
-    with torch.cuda.device(dev):
-        st = stream if stream is not None else torch.cuda.current_stream(dev)
-        with torch.cuda.stream(st):
-            yield st
+    stream, and yields the stream's handle.  Tensors the wrappers create inside (outputs, workspace)
+    then belong to the stream the kernels run on, so torch's allocator cannot hand their memory to
+    someone else while those kernels are still in flight.
+
+    With ``dev`` current already and no stream given there is nothing to switch: only the handle is
+    looked up (entering torch's two context managers took 13 us, half of a call of 1,000 small
+    tasksets)."""
+    __slots__ = ("dev", "stream", "inside")
+
+    def __init__(self, dev, stream):
+        self.dev, self.stream, self.inside = dev, stream, None
+
+    def __enter__(self) -> int:
+        import torch
+        index = self.dev.index
+        here = torch.cuda.current_device()
+        if self.stream is None and (index is None or index == here):
+            return torch.cuda.current_stream(here).cuda_stream if _raw_stream is None else _raw_stream(here)
+        self.inside = contextlib.ExitStack()
+        self.inside.enter_context(torch.cuda.device(self.dev))
+        st = self.stream if self.stream is not None else torch.cuda.current_stream(self.dev)
+        self.inside.enter_context(torch.cuda.stream(st))
+        return st.cuda_stream
+
+    def __exit__(self, *exc):
+        if self.inside is not None:
+            self.inside.close()
+        return False
 
 
 def _check(rc: int):
@@ -191,12 +216,11 @@ def rta_batch(ts: DeviceTasksets, policy: int, timeslice_us: int = 1024, overhea
             out_wcrt = torch.empty(ts.n_tasks, dtype=torch.int64, device=dev)
         if out_sched is None:
             out_sched = torch.empty(max(ts.n_tasksets, 0), dtype=torch.uint8, device=dev)
-        need = workspace_bytes(ts.n_tasksets)
         if workspace is None:
-            workspace = torch.empty(max(need, 256), dtype=torch.uint8, device=dev)
+            workspace = torch.empty(max(workspace_bytes(ts.n_tasksets), 256), dtype=torch.uint8, device=dev)
         rc = lib.gcaps_rta_batch(ctypes.byref(ts.c), ts.n_tasksets, policy, timeslice_us, overhead_us,
                                  out_wcrt.data_ptr(), out_sched.data_ptr(), workspace.data_ptr(),
-                                 workspace.numel(), st.cuda_stream)
+                                 workspace.numel(), st)
     _check(rc)
     return out_wcrt, out_sched
 
@@ -217,13 +241,12 @@ def rta_sweep(ts: DeviceTasksets, policy: int, timeslices_us, overheads_us, want
             out_wcrt = torch.empty((k, ts.n_tasks), dtype=torch.int64, device=dev)
         if out_sched is None:
             out_sched = torch.empty((k, max(ts.n_tasksets, 0)), dtype=torch.uint8, device=dev)
-        need = workspace_bytes(ts.n_tasksets)
         if workspace is None:
-            workspace = torch.empty(max(need, 256), dtype=torch.uint8, device=dev)
+            workspace = torch.empty(max(workspace_bytes(ts.n_tasksets), 256), dtype=torch.uint8, device=dev)
         rc = lib.gcaps_rta_sweep_batch(ctypes.byref(ts.c), ts.n_tasksets, policy, k, Ls, ov,
                                        out_wcrt.data_ptr() if out_wcrt is not None else None,
                                        out_sched.data_ptr(), workspace.data_ptr(), workspace.numel(),
-                                       st.cuda_stream)
+                                       st)
     _check(rc)
     return out_wcrt, out_sched
 
@@ -251,7 +274,7 @@ def rta_multi(ts: DeviceTasksets, analyses: int, timeslices_us=(1024,), overhead
         rc = lib.gcaps_rta_multi_batch(ctypes.byref(ts.c), ts.n_tasksets, analyses, flags, n_pts, Ls, ov,
                                        out_wcrt.data_ptr() if out_wcrt is not None else None,
                                        out_sched.data_ptr(), workspace.data_ptr(), workspace.numel(),
-                                       st.cuda_stream)
+                                       st)
     _check(rc)
     return out_wcrt, out_sched
 
@@ -275,7 +298,7 @@ def rta_batch_static(ts: DeviceTasksets, policy: int, timeslice_us: int = 1024, 
             out_sched = torch.empty(max(ts.n_tasksets, 0), dtype=torch.uint8, device=dev)
         rc = lib.gcaps_rta_batch_static(ctypes.byref(ts.c), ts.n_tasksets, policy, timeslice_us,
                                         overhead_us, out_wcrt.data_ptr(), out_sched.data_ptr(),
-                                        st.cuda_stream)
+                                        st)
     _check(rc)
     return out_wcrt, out_sched
 
@@ -298,7 +321,7 @@ def rta_gpu_priority(ts: DeviceTasksets, flags: int = 0, overhead_us: int = 0, g
             ctypes.byref(ts.c), ts.n_tasksets, flags, overhead_us,
             gpu_priority.data_ptr() if gpu_priority is not None else None, out_gp.data_ptr(),
             out_wcrt.data_ptr(), out_sched.data_ptr(), workspace.data_ptr(), workspace.numel(),
-            st.cuda_stream)
+            st)
     _check(rc)
     return out_wcrt, out_sched, out_gp
 
@@ -320,11 +343,11 @@ def generate_device(params: GenParams, first: int, count: int, device="cuda:0", 
         totals = torch.zeros(3, dtype=torch.int64, device=dev)
         ev = [torch.cuda.Event(enable_timing=True) for _ in range(4)] if timing is not None else None
         if ev:
-            ev[0].record(st)
+            ev[0].record()
         _check(lib.gcaps_gen_count(ctypes.byref(cp), first, count, totals.data_ptr(), ws.data_ptr(),
-                                   ws.numel(), st.cuda_stream))
+                                   ws.numel(), st))
         if ev:
-            ev[1].record(st)
+            ev[1].record()
         n_tasks, n_c, n_g = (int(x) for x in totals.cpu().tolist())
         sizes = {"task_off": max(count, 0) + 1, "period": n_tasks, "deadline": n_tasks,
                  "priority": n_tasks, "core": n_tasks, "cseg_off": n_tasks + 1, "cseg_wcet": n_c,
@@ -332,11 +355,11 @@ def generate_device(params: GenParams, first: int, count: int, device="cuda:0", 
         t = {f: torch.zeros(sizes[f], dtype=torch.int64, device=dev) for f in ARRAY_FIELDS}
         ts = DeviceTasksets(t)
         if ev:
-            ev[2].record(st)
+            ev[2].record()
         _check(lib.gcaps_gen_fill(ctypes.byref(cp), first, count, ctypes.byref(ts.c), ws.data_ptr(),
-                                  ws.numel(), st.cuda_stream))
+                                  ws.numel(), st))
         if ev:
-            ev[3].record(st)
+            ev[3].record()
             torch.cuda.synchronize(dev)
             timing["count_ms"] = ev[0].elapsed_time(ev[1])
             timing["fill_ms"] = ev[2].elapsed_time(ev[3])
@@ -350,7 +373,7 @@ def rta_plan(ts: DeviceTasksets, workspace, stream=None):
     dev = ts.t["task_off"].device
     with _device_and_stream(dev, stream) as st:
         rc = lib.gcaps_rta_plan_batch(ctypes.byref(ts.c), ts.n_tasksets, workspace.data_ptr(),
-                                      workspace.numel(), st.cuda_stream)
+                                      workspace.numel(), st)
     _check(rc)
 
 
@@ -385,7 +408,7 @@ def rta_validate(ts: DeviceTasksets, stream=None):
     dev = ts.t["task_off"].device
     with _device_and_stream(dev, stream) as st:
         out = torch.empty(max(ts.n_tasksets, 0), dtype=torch.int32, device=dev)
-        rc = lib.gcaps_rta_validate(ctypes.byref(ts.c), ts.n_tasksets, out.data_ptr(), st.cuda_stream)
+        rc = lib.gcaps_rta_validate(ctypes.byref(ts.c), ts.n_tasksets, out.data_ptr(), st)
     _check(rc)
     return out
 
