@@ -40,7 +40,7 @@ K_TERM, K_SETUP = 6, 16   # algorithmic integer lane-operations per interference
 # of up to 32 tasks, one each for the 64-, 96-, 128-, 192- and 256-task bins and two for the larger
 # tasksets that those left over
 LAUNCHES_PER_CALL = 11       # three plan kernels + one kernel per group of size bins + two
-LAUNCHES_PER_SMALL_CALL = 2  # batches of up to 8,192 tasksets: one plan kernel, one kernel for all bins
+LAUNCHES_PER_SMALL_CALL = 1  # batches of up to 12,288 tasksets: a warp per taskset, no plan
 # DRAM bytes (read + write) per taskset of the analysis kernel on the 'large' workload, from an
 # ncu capture of a 131,072-taskset launch (traffic grows in proportion to the tasksets of a
 # launch).  Only reported while the kernel source is the one the counters were taken from.
@@ -595,7 +595,7 @@ def main():
             "clocks": clocks, "e2e": e2e,
             "gpu_launches": args.steps * (len(policies) if args.mode == "policies"
                                           else (1 + len(pairs)) if args.mode == "sweep" else 2)
-                            * (LAUNCHES_PER_SMALL_CALL if count <= 8192 else LAUNCHES_PER_CALL),
+                            * (LAUNCHES_PER_SMALL_CALL if count <= 12288 else LAUNCHES_PER_CALL),
             "roofline": roof, "cpu_baseline": cpu, "wall_s_timed_region": t_wall,
         }
         line.update(side)

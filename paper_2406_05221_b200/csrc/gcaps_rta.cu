@@ -305,7 +305,8 @@ void fill_params(KParams *p, const gcaps_tasksets_t *ts, int64_t n_tasksets, int
   p->out_sched = out_sched;
 }
 
-int enqueue_plan(KParams &p, void *workspace, size_t workspace_bytes, cudaStream_t st) {
+// Points p at the plan areas of `workspace`.
+static int place_plan(KParams &p, void *workspace, size_t workspace_bytes) {
   const size_t need = gcaps_rta_workspace_bytes(p.n_tasksets);
   if (!workspace || workspace_bytes < need || ((uintptr_t)workspace & 255u))
     return GCAPS_ERR_WORKSPACE;
@@ -314,14 +315,24 @@ int enqueue_plan(KParams &p, void *workspace, size_t workspace_bytes, cudaStream
   p.hdr = (PlanHeader *)w;
   p.block_cnt = (unsigned int *)(w + 256);
   p.perm = (unsigned int *)(w + 256 + align_up(nb * kBinStride * sizeof(unsigned int), 256));
+  return GCAPS_OK;
+}
+
+static void enqueue_plan_kernels(const KParams &p, cudaStream_t st) {
+  const size_t nb = plan_blocks(p.n_tasksets);
   if (p.n_tasksets <= kPlanSmall) {
     plan_small_kernel<<<1, 1024, 0, st>>>(p);
-    return GCAPS_OK;
+    return;
   }
   plan_count_kernel<<<(unsigned int)nb, 256, 0, st>>>(p);
   plan_scan_kernel<<<1, 32 * kNumBins, 0, st>>>(p, (unsigned int)nb);
   plan_scatter_kernel<<<(unsigned int)nb, 256, 0, st>>>(p);
-  return GCAPS_OK;
+}
+
+int enqueue_plan(KParams &p, void *workspace, size_t workspace_bytes, cudaStream_t st) {
+  const int rc = place_plan(p, workspace, workspace_bytes);
+  if (rc == GCAPS_OK) enqueue_plan_kernels(p, st);
+  return rc;
 }
 
 }  // namespace gcaps_detail
@@ -371,7 +382,6 @@ cudaError_t launch_deferred(const KParams &p, int sm_count, cudaStream_t st) {
 template <int MODE>
 cudaError_t launch_all_bins(const KParams &p, int sm_count, cudaStream_t st) {
   constexpr int kWarps = kBlockThreads / 32;
-  if (p.n_tasksets <= kPlanSmall) return launch_any_bins(MODE, p, sm_count, st);  // one launch for every bin
   static int blocks_per_sm[64] = {0};
   const size_t smem = sizeof(u32) * kSmallWarpWords * kWarps;
   cudaError_t e = launch_persistent(rta_small_kernel<MODE>, blocks_per_sm, smem,
@@ -393,8 +403,12 @@ cudaError_t launch_all_bins(const KParams &p, int sm_count, cudaStream_t st) {
 int enqueue_batch(KParams p, void *workspace, size_t workspace_bytes, int sm_count, cudaStream_t st,
                   const SweepArgs *sw = nullptr, int analyses = 0) {
   if (p.n_tasksets == 0) return GCAPS_OK;
-  const int rc = enqueue_plan(p, workspace, workspace_bytes, st);
+  const bool rr = (p.policy & 0xff) == GCAPS_POLICY_RR, busy = (p.policy & GCAPS_RTA_BUSY) != 0;
+  const int mode = (rr ? 2 : 0) + (busy ? 1 : 0);
+  const bool direct = !sw && p.n_tasksets <= kDirectMost;
+  const int rc = place_plan(p, workspace, workspace_bytes);
   if (rc != GCAPS_OK) return rc;
+  if (!direct) enqueue_plan_kernels(p, st);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess && sw) {
     SweepArgs set = *sw;
@@ -412,10 +426,10 @@ int enqueue_batch(KParams p, void *workspace, size_t workspace_bytes, int sm_cou
       if (e == cudaSuccess) e = launch_sweep_set(p, set, sm_count, st);
     }
   } else if (e == cudaSuccess) {
-    const bool rr = (p.policy & 0xff) == GCAPS_POLICY_RR, busy = (p.policy & GCAPS_RTA_BUSY) != 0;
-    if (!rr && !busy) e = launch_all_bins<0>(p, sm_count, st);
-    else if (!rr) e = launch_all_bins<1>(p, sm_count, st);
-    else if (!busy) e = launch_all_bins<2>(p, sm_count, st);
+    if (direct) e = launch_one_warp_each(mode, p, st);
+    else if (mode == 0) e = launch_all_bins<0>(p, sm_count, st);
+    else if (mode == 1) e = launch_all_bins<1>(p, sm_count, st);
+    else if (mode == 2) e = launch_all_bins<2>(p, sm_count, st);
     else e = launch_all_bins<3>(p, sm_count, st);
   }
   if (e != cudaSuccess) {

@@ -26,6 +26,7 @@ constexpr int kBlockThreads = 128;
 constexpr int kStagedBlockThreads = 64;  // kernels that stage tasksets by bulk copies
 constexpr int kPlanItems = 1024;  // tasksets per plan block
 constexpr int kPlanSmall = 8192;  // batches up to this size are planned by one block in one launch
+constexpr int kDirectMost = 12288;  // batches up to this size run without a plan (see gcaps_rta_direct.cu)
 constexpr u64 kClamp = 1ull << 50;  // any quantity >= 2^50 exceeds every deadline (<= 2^40)
 
 struct PlanHeader {
@@ -273,9 +274,10 @@ void fill_params(KParams *p, const gcaps_tasksets_t *ts, int64_t n_tasksets, int
 // Points p at the plan areas of `workspace` and enqueues the three plan kernels (size bins, a
 // permutation of the taskset indices, zeroed work counters).  GCAPS_OK or GCAPS_ERR_WORKSPACE.
 int enqueue_plan(KParams &p, void *workspace, size_t workspace_bytes, cudaStream_t st);
-// One launch over all size bins for analysis `mode` (0 GCAPS self-suspension, 1 GCAPS
-// busy-waiting, 2 RR self-suspension, 3 RR busy-waiting); defined in gcaps_rta_any.cu.
-cudaError_t launch_any_bins(int mode, const KParams &p, int sm_count, cudaStream_t st);
+// One launch for analysis `mode` (0 GCAPS self-suspension, 1 GCAPS busy-waiting, 2 RR self-suspension, 3 RR
+// busy-waiting) without a plan, a block of one warp per taskset, for batches of at most kDirectMost
+// tasksets; defined in gcaps_rta_direct.cu.
+cudaError_t launch_one_warp_each(int mode, const KParams &p, cudaStream_t st);
 // Launches over all size bins for the analyses sw.enabled names (bit m = mode m; one of 1, 2, 4, 8,
 // 5, 10) under every pair of `sw`; defined in gcaps_rta_sweep.cu.
 cudaError_t launch_sweep_set(const KParams &p, const SweepArgs &sw, int sm_count, cudaStream_t st);

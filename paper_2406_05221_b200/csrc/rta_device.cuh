@@ -1,6 +1,6 @@
 // rta_device.cuh -- device code of the analysis kernels, shared by the translation units that
-// instantiate them: gcaps_rta.cu (one analysis per launch), gcaps_rta_any.cu (all size bins in one
-// launch), gcaps_rta_sweep.cu (several analyses per launch).  Internal.
+// instantiate them: gcaps_rta.cu (one analysis per launch), gcaps_rta_direct.cu (small batches, a
+// warp per taskset), gcaps_rta_sweep.cu (several analyses per launch).  Internal.
 //
 // One warp analyses one taskset at a time:
 //   stage      coalesced loads of the taskset's per-task slices into registers (lane = task)
@@ -375,6 +375,10 @@ struct ModeTag {
   __host__ __device__ constexpr operator int() const { return V; }
 };
 
+__device__ __forceinline__ void prefetch_l2(const void *ptr) {
+  asm volatile("prefetch.global.L2 [%0];" ::"l"(ptr));
+}
+
 // What a taskset's staging, ordering and aggregation leave in a lane (slot s: position lane + LPT * s);
 // info rows (deadline, core) by rank are in shared memory.
 template <int SLOTS>
@@ -392,7 +396,9 @@ struct TaskValues {
 // so that each shuffle, vote and reduction is one instruction for all of them.  False if no group of
 // the warp has a taskset that fits the 32-bit path; else o.live says which do.  BC: prefix blocks of
 // the CPU segments whose loads are issued together.  ovh_max: the largest epsilon of a GCAPS analysis.
-template <int LPT, int SLOTS, int BC, bool kAnyGcaps, class RowsT>
+// PREFETCH: the caller has not prefetched the segments; the G^m and G^e slices start their way into L2 as
+// soon as their place is known, so that they do not wait for the CPU segments' sums.
+template <int LPT, int SLOTS, int BC, bool kAnyGcaps, bool PREFETCH = false, class RowsT>
 __device__ __forceinline__ bool stage_fast(const KParams &p, bool live, i64 a, int n, u32 *buf, const RowsT rows, int lane,
                                            unsigned int gmask, bool best_effort, u32 ovh_max, TaskValues<SLOTS> &o) {
   typedef FastLayout<LPT, SLOTS> Lay;
@@ -436,6 +442,10 @@ __device__ __forceinline__ bool stage_fast(const KParams &p, bool live, i64 a, i
       live = false;
     Nc = (int)Nc64, Ng = (int)Ng64;
     GCAPS_LEAVE_IF_NONE_LIVE();
+    if constexpr (PREFETCH) {
+      for (int e = 16 * lane; e < Ng; e += 16 * LPT)
+        prefetch_l2(p.gseg_misc + gfirst + e), prefetch_l2(p.gseg_exec + gfirst + e);
+    }
     u32 high = 0;  // any set bit: some value does not fit the 32-bit path
     bool ok = true, any_wide = false;
     u32 D[SLOTS], core[SLOTS];
@@ -632,7 +642,7 @@ __device__ __forceinline__ bool stage_fast(const KParams &p, bool live, i64 a, i
 // Returns, per group, kFastDone (outputs written) or kFastDeclined (some value does not fit the
 // 32-bit path or the taskset is invalid; nothing written: the caller runs the exact path).
 constexpr int kFastDeclined = 0, kFastDone = 1;
-template <int LPT, int SLOTS, int MASK, bool SWEEP = false>
+template <int LPT, int SLOTS, int MASK, bool SWEEP = false, bool PREFETCH = false>
 __device__ __forceinline__ int analyse_fast(const KParams &p, bool live, i64 t, i64 a, int n, u32 *buf, int lane,
                                             unsigned int gmask, const SweepArgs *sw = nullptr) {
   typedef FastLayout<LPT, SLOTS> Lay;
@@ -651,7 +661,7 @@ __device__ __forceinline__ int analyse_fast(const KParams &p, bool live, i64 t, 
   const Rows<LPT, SLOTS, SWEEP> rows{buf};
   u32 *Q0 = buf + Lay::kQ0, *Q1 = buf + Lay::kQ1;
   TaskValues<SLOTS> o;
-  if (!stage_fast<LPT, SLOTS, BC, kAnyGcaps>(p, live, a, n, buf, rows, lane, gmask, best_effort,
+  if (!stage_fast<LPT, SLOTS, BC, kAnyGcaps, PREFETCH>(p, live, a, n, buf, rows, lane, gmask, best_effort,
                                              SWEEP ? (u32)sw->max_ovh : (u32)p.ovh, o))
     return kFastDeclined;
   live = o.live, n = o.n;
@@ -818,10 +828,6 @@ __device__ __forceinline__ int analyse_fast(const KParams &p, bool live, i64 t, 
     }
   }
   return live ? kFastDone : kFastDeclined;
-}
-
-__device__ __forceinline__ void prefetch_l2(const void *ptr) {
-  asm volatile("prefetch.global.L2 [%0];" ::"l"(ptr));
 }
 
 // What a warp knows in advance about one taskset of a chunk (kept in shared memory).

@@ -80,7 +80,7 @@ def test_tasks_without_demand(n):
         check(tasksets, ALL_MODES, ovh=ovh)
 
 
-@pytest.mark.parametrize("count", [1, 2, 3, 4, 5, 8191, 8193])
+@pytest.mark.parametrize("count", [1, 2, 3, 4, 5, 8193, 12288, 12289])
 def test_groups_of_a_warp(count):
     """Tasksets that share a warp end at different ranks and sweeps (one that declines the 32-bit
     path among them)."""

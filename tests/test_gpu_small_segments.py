@@ -11,7 +11,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("n", [1, 7, 8, 15, 16, 24, 32])
-@pytest.mark.parametrize("count", [40, 8300])
+@pytest.mark.parametrize("count", [40, 12300])
 def test_segment_counts_around_the_capacity(n, count):
     torch = pytest.importorskip("torch")
     rng = np.random.default_rng(n)

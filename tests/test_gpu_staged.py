@@ -12,7 +12,7 @@ from tests.helpers import ALL_MODES, BEST_EFFORT, batch_of
 
 pytestmark = pytest.mark.gpu
 
-FILLERS = 8192   # more tasksets than the one-launch path takes (kPlanSmall of csrc/rta_common.cuh)
+FILLERS = 12288   # more tasksets than the path without a plan takes (kDirectMost of csrc/rta_common.cuh)
 
 
 def taskset(rng, n, load, segs, gaps=False):
@@ -95,4 +95,4 @@ def test_deferred_tasksets(every):
     rng = np.random.default_rng(every)
     kinds = [taskset(rng, n, load, 2) for n in (40, 80, 130, 200, 250) for load in (0.02, 6.0)]
     tasksets = [kinds[2 * (k % 5) + (0 if k % every == 0 else 1)] for k in range(4200)]
-    check(tasksets, [0, 1], fillers=4200)
+    check(tasksets, [0, 1], fillers=8400)
