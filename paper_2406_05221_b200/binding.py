@@ -340,7 +340,7 @@ def generate_device(params: GenParams, first: int, count: int, device="cuda:0", 
     with _device_and_stream(dev, stream) as st:
         ws = torch.empty(max(int(lib.gcaps_gen_workspace_bytes(ctypes.byref(cp), count)), 256), dtype=torch.uint8,
                          device=dev)
-        totals = torch.zeros(3, dtype=torch.int64, device=dev)
+        totals = torch.empty(3, dtype=torch.int64, device=dev)  # (gcaps_gen_count writes all three)
         ev = [torch.cuda.Event(enable_timing=True) for _ in range(4)] if timing is not None else None
         if ev:
             ev[0].record()
@@ -352,7 +352,9 @@ def generate_device(params: GenParams, first: int, count: int, device="cuda:0", 
         sizes = {"task_off": max(count, 0) + 1, "period": n_tasks, "deadline": n_tasks,
                  "priority": n_tasks, "core": n_tasks, "cseg_off": n_tasks + 1, "cseg_wcet": n_c,
                  "gseg_off": n_tasks + 1, "gseg_misc": n_g, "gseg_exec": n_g}
-        t = {f: torch.zeros(sizes[f], dtype=torch.int64, device=dev) for f in ARRAY_FIELDS}
+        # gcaps_gen_fill writes every element of arrays of exactly these sizes (nothing for an empty batch)
+        make = torch.empty if count > 0 else torch.zeros
+        t = {f: make(sizes[f], dtype=torch.int64, device=dev) for f in ARRAY_FIELDS}
         ts = DeviceTasksets(t)
         if ev:
             ev[2].record()
