@@ -8,8 +8,9 @@
 // random stream in the workspace; three exclusive scans turn the sizes into offsets (block sums,
 // one block over the block sums, block-local scan).  gcaps_gen_fill: one warp per taskset, lane =
 // task; the random draws of a task start at a position that is a prefix sum over the tasks
-// before it (the random source is counter-based), so every lane splits its own task's demand
-// into segments (igen_task_segments) and writes them at offsets that are prefix sums again.
+// before it (the random source is counter-based).  The segments of 32 tasks at a time are split with
+// lane = segment: random weights, quotients and stores all run over the segments side by side, and
+// only the two sums of a task (its weights, its shares) are added up by the task's lane.
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <string.h>
@@ -158,8 +159,85 @@ __device__ __forceinline__ u32 warp_exclusive(u32 v, int lane, u32 *total) {
   return x - v;
 }
 
+constexpr int kFillParts = 32 * (IGEN_MAX_SEGS + 1);  // segments of a kind of 32 tasks, at most
+
+// Shared memory of one warp of the fill kernel, for 32 tasks.
+struct FillWarp {
+  uint64_t weights[32];  // by task: sum of its weights (Q32)
+  double inverse[32];    // ... and its reciprocal
+  u32 spare[32];         // what is shared out beyond 1 us per segment
+  u32 draw[32];          // position of the first weight's draw within the taskset's stream
+  u32 share[kFillParts];  // by segment: the random fraction of its weight, then its share of `spare`
+  unsigned short first[32];         // first segment of the task
+  unsigned char owner[kFillParts];  // by segment: the task's lane
+};
+
+// Splits `total` us of this lane's task into `parts` segments (0: none) like igen_split does, the tasks
+// of all lanes at once.  `draw`: position of the task's first weight.  The segments of the lanes lie one
+// behind the other from out[0] on; FIFTH: a fifth of each goes to `fifth`.
+//
+// igen_split's quotient floor(spare * w / sum of weights) is taken in double precision with the task's
+// reciprocal (wrong by at most 1, as all values stay below 2^31) and settled by its remainder.
+template <bool FIFTH>
+__device__ __forceinline__ void split_tasks(FillWarp &w, uint64_t key, uint64_t ctr, u32 draw, u32 total, u32 parts,
+                                            i64 *out, i64 *fifth, int lane) {
+  u32 n_parts;
+  const u32 first = warp_exclusive(parts, lane, &n_parts);
+  w.spare[lane] = total - parts;
+  w.draw[lane] = draw;
+  w.first[lane] = (unsigned short)first;
+#pragma unroll 1
+  for (u32 j = 0; j < parts; ++j) w.owner[first + j] = (unsigned char)lane;
+  __syncwarp();
+#pragma unroll 1
+  for (u32 q = lane; q < n_parts; q += 32) {
+    const int i = w.owner[q];
+    igen_rng_t rng;
+    rng.key = key, rng.ctr = ctr + w.draw[i] + (q - w.first[i]);
+    w.share[q] = (u32)igen_unit(&rng);
+  }
+  __syncwarp();
+  uint64_t sum = (uint64_t)parts << 32;
+#pragma unroll 1
+  for (u32 j = 0; j < parts; ++j) sum += w.share[first + j];
+  w.weights[lane] = sum;
+  w.inverse[lane] = 1.0 / (double)(sum + (parts == 0 ? 1 : 0));
+  __syncwarp();
+#pragma unroll 1
+  for (u32 q = lane; q < n_parts; q += 32) {
+    const int i = w.owner[q];
+    const u32 spare = w.spare[i], u = w.share[q];
+    const uint64_t of = w.weights[i];
+    u32 x = (u32)((double)spare * ((double)u + 4294967296.0) * w.inverse[i]);
+    const i64 rem = (i64)(((uint64_t)spare << 32) + (uint64_t)spare * u - (uint64_t)x * of);
+    if (rem < 0) x -= 1;
+    else if ((uint64_t)rem >= of) x += 1;
+    w.share[q] = x;
+  }
+  __syncwarp();
+  if (parts > 0) {  // the last segment takes what is left
+    u32 left = w.spare[lane];
+#pragma unroll 1
+    for (u32 j = 0; j + 1 < parts; ++j) left -= w.share[first + j];
+    w.share[first + parts - 1] = left;
+  }
+  __syncwarp();
+#pragma unroll 1
+  for (u32 q = lane; q < n_parts; q += 32) {
+    const u32 part = 1 + w.share[q], small = FIFTH ? part / 5u : 0u;
+    out[q] = (i64)(part - small);
+    if (FIFTH) fifth[q] = (i64)small;
+  }
+  __syncwarp();
+}
+
+// Bound by instruction issue and by the stores: 250,000 `large` tasksets (2.3 GB) 0.97 ms; a lane per
+// task for everything took 1.43 ms (lanes wait for the task with the most segments, weights drawn
+// twice, 8-byte stores far apart).
 __global__ void __launch_bounds__(kGenThreads) gen_fill_kernel(igen_params_t p, i64 first, i64 count,
                                                                 GenSpace w, GenOut o) {
+  __shared__ FillWarp warps[kGenThreads / 32];
+  FillWarp &mine_w = warps[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31;
   const i64 t = (i64)blockIdx.x * (kGenThreads / 32) + (threadIdx.x >> 5);
   if (t >= count) return;
@@ -172,30 +250,33 @@ __global__ void __launch_bounds__(kGenThreads) gen_fill_kernel(igen_params_t p, 
     const uint64_t key = (uint64_t)st[0] | ((uint64_t)st[1] << 32);
     uint64_t ctr = (uint64_t)st[2] | ((uint64_t)st[3] << 32);
     u32 c_run = 0, g_run = 0;  // segments of the tasks before this round of 32
+#pragma unroll 1
     for (i64 i0 = 0; i0 < n; i0 += 32) {
       const i64 i = i0 + lane;
       const bool mine = i < n;
       u32 T = 0, E = 0, pk = 0;
       if (mine) T = st[4 + 3 * i], E = st[5 + 3 * i], pk = st[6 + 3 * i];
-      const int eta = (int)(pk >> 24);
+      const u32 eta = pk >> 24, c_parts = mine ? eta + 1 : 0;
       u32 draws_total, c_total, g_total;
-      const u32 draws_before = warp_exclusive(mine ? igen_task_draws(eta) : 0u, lane, &draws_total);
-      const u32 c_before = warp_exclusive(mine ? (u32)eta + 1u : 0u, lane, &c_total);
-      const u32 g_before = warp_exclusive(mine ? (u32)eta : 0u, lane, &g_total);
+      const u32 draws_before = warp_exclusive(mine ? igen_task_draws((int)eta) : 0u, lane, &draws_total);
+      const u32 c_before = warp_exclusive(c_parts, lane, &c_total);
+      const u32 g_before = warp_exclusive(eta, lane, &g_total);
+      // the draws of a task: the ratio, one weight per GPU segment, one per CPU segment
+      igen_rng_t rng;
+      rng.key = key, rng.ctr = ctr + draws_before;
+      const u32 G = mine ? (u32)igen_task_gpu(&rng, (int64_t)E, (int)eta, p.ratio_lo, p.ratio_hi) : 0u;
       if (mine) {
-        igen_rng_t rng;
-        rng.key = key, rng.ctr = ctr + draws_before;
-        const i64 c0 = c_start + c_run + c_before, g0 = g_start + g_run + g_before;
-        // the segment values go straight to their places in the output arrays
-        igen_task_segments(&rng, (int64_t)E, eta, p.ratio_lo, p.ratio_hi, (int64_t *)(o.cseg_wcet + c0),
-                           (int64_t *)(o.gseg_misc + g0), (int64_t *)(o.gseg_exec + g0));
         o.period[k0 + i] = T;
         o.deadline[k0 + i] = T;
         o.priority[k0 + i] = pk & 0xffffu;
         o.core[k0 + i] = (pk >> 16) & 0xffu;
-        o.cseg_off[k0 + i] = c0;
-        o.gseg_off[k0 + i] = g0;
+        o.cseg_off[k0 + i] = c_start + c_run + c_before;
+        o.gseg_off[k0 + i] = g_start + g_run + g_before;
       }
+      split_tasks<true>(mine_w, key, ctr, draws_before + 1, G, eta, o.gseg_exec + g_start + g_run,
+                        o.gseg_misc + g_start + g_run, lane);
+      split_tasks<false>(mine_w, key, ctr, draws_before + 1 + eta, E - G, c_parts, o.cseg_wcet + c_start + c_run, nullptr,
+                         lane);
       ctr += draws_total, c_run += c_total, g_run += g_total;
     }
   }

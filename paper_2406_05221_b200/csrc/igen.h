@@ -158,32 +158,6 @@ IGEN_FN uint64_t igen_exp2(uint64_t y) {
   return ((r >> (61 - k)) + 1) >> 1;
 }
 
-/* floor(a / d) for 0 < d < 2^40 and a < 2^63 */
-IGEN_FN uint64_t igen_div(uint64_t a, uint64_t d) {
-#ifdef __CUDA_ARCH__
-  /* no 64-bit division: two single-precision estimates, the second of what the first left over,
-   * then the remainder settles the quotient exactly (differences are taken modulo 2^64 and read
-   * as signed: the true ones are far below 2^63) */
-  const float inv = 1.0f / (float)d;
-  uint64_t q = (uint64_t)((float)a * inv);
-  int64_t rem = (int64_t)(a - q * d);
-  const int64_t q2 = (int64_t)((float)rem * inv);
-  q += (uint64_t)q2;
-  rem -= q2 * (int64_t)d;
-  while (rem < 0) {
-    rem += (int64_t)d;
-    q -= 1;
-  }
-  while (rem >= (int64_t)d) {
-    rem -= (int64_t)d;
-    q += 1;
-  }
-  return q;
-#else
-  return a / d;
-#endif
-}
-
 /* Splits `total` into `parts` integers >= 1 (needs total >= parts) in proportion to random
  * weights in [1,2); the last part takes the rounding remainder.  With `fifth` given, a fifth of
  * every part (rounded down) goes there and the rest to `out`.  The weights are drawn twice (once
@@ -201,7 +175,7 @@ IGEN_FN void igen_split(igen_rng_t *r, int64_t total, int parts, int64_t *out, i
     if (j == parts - 1) {
       x = spare - used;
     } else {
-      x = igen_div(spare * w, ws);
+      x = spare * w / ws;
       if (x > spare - used) x = spare - used;
     }
     used += x;
@@ -334,19 +308,22 @@ IGEN_FN void igen_begin(const igen_params_t *p, uint64_t index, igen_state_t *s)
  * weights of the GPU split (none for a CPU-only task), eta + 1 weights of the CPU split. */
 IGEN_FN uint32_t igen_task_draws(int eta) { return 2u * (uint32_t)eta + 2u; }
 
+/* The GPU part G_i of a task with execution demand E and eta GPU segments (one draw: the ratio). */
+IGEN_FN int64_t igen_task_gpu(igen_rng_t *rng, int64_t E, int eta, uint64_t ratio_lo, uint64_t ratio_hi) {
+  const uint64_t rho = igen_range(rng, ratio_lo, ratio_hi);
+  int64_t G = (int64_t)((rho * (uint64_t)E + (1ULL << 31)) >> 32); /* rho < 2^32, E < 2^31 */
+  if (eta == 0) return 0;
+  if (G < eta) G = eta;
+  if (G > E - eta - 1) G = E - eta - 1;
+  return G;
+}
+
 /* The segments of a task with execution demand E and eta GPU segments, drawn from `rng`:
  * cseg[0 .. eta], gm / ge[0 .. eta-1]. */
 IGEN_FN void igen_task_segments(igen_rng_t *rng, int64_t E, int eta, uint64_t ratio_lo,
                                 uint64_t ratio_hi, int64_t *cseg, int64_t *gm, int64_t *ge) {
-  const uint64_t rho = igen_range(rng, ratio_lo, ratio_hi);
-  int64_t G = (int64_t)((rho * (uint64_t)E + (1ULL << 31)) >> 32); /* rho < 2^32, E < 2^31 */
-  if (eta == 0) {
-    G = 0;
-  } else {
-    if (G < eta) G = eta;
-    if (G > E - eta - 1) G = E - eta - 1;
-    igen_split(rng, G, eta, ge, gm); /* 20 % miscellaneous CPU work, 80 % pure GPU work */
-  }
+  const int64_t G = igen_task_gpu(rng, E, eta, ratio_lo, ratio_hi);
+  if (eta > 0) igen_split(rng, G, eta, ge, gm); /* 20 % miscellaneous CPU work, 80 % pure GPU work */
   igen_split(rng, E - G, eta + 1, cseg, 0);
 }
 
