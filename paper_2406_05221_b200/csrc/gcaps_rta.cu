@@ -759,12 +759,13 @@ int gcaps_rta_batch_host_multi(const gcaps_tasksets_t *ts, int64_t n_tasksets, c
     g_stage.streams_ok = true;
   }
   const int64_t kChunkTasksets = 1 << 16;
-  // About 30 MB per chunk (0.6 ms of the host link): what the first chunk's checks, the last
-  // chunk's analysis and its way back take is not hidden behind a transfer, so chunks are small,
-  // but still long against the launches and copies of one (60,000 80-task tasksets, two policies,
-  // page-locked arrays: 15.4 -> 11.9 ms against chunks of up to 3 M tasks in two slots; 10 ms of it is
-  // the inputs on the link).
-  const int64_t kChunkTasks = 1 << 18;
+  // What the first chunk's checks, the last chunk's analysis and its way back take is not hidden behind a
+  // transfer, so the chunks of a short batch are small (256 k tasks, 30 MB, 0.6 ms of the host link:
+  // 60,000 80-task tasksets, two policies, page-locked arrays: 15.4 -> 12.0 ms against chunks of up to
+  // 3 M tasks); every chunk costs its ten copies and its launches, so those of a long one are larger
+  // (300,000 such tasksets: 54.8 ms; 58.5 in chunks of 256 k, 56.1 in chunks of 3 M tasks).
+  int64_t chunk_tasks = ts->n_tasks / 24;
+  chunk_tasks = chunk_tasks < (1 << 18) ? (1 << 18) : chunk_tasks > (1 << 21) ? (1 << 21) : chunk_tasks;
   int64_t t = 0;
   int slot = 0;
   while (t < n_tasksets) {
@@ -774,7 +775,7 @@ int gcaps_rta_batch_host_multi(const gcaps_tasksets_t *ts, int64_t n_tasksets, c
     int64_t k1 = k0;
     while (t1 < n_tasksets && t1 - t < kChunkTasksets) {
       const int64_t kn = ts->task_off[t1 + 1];
-      if (kn < k1 || (t1 > t && kn - k0 > kChunkTasks)) break;
+      if (kn < k1 || (t1 > t && kn - k0 > chunk_tasks)) break;
       k1 = kn;
       t1 += 1;
     }
