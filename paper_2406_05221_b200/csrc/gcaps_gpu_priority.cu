@@ -414,7 +414,7 @@ __device__ __noinline__ void analyse_gpu_priority(const GpParams &g, i64 t, GpSm
 // slots; about 15 bounds and 43 sweeps each).  100,000 of them 1.19 -> 0.77 ms: what went are per-lane
 // loops over global memory for the sums, a quadratic loop for every core's lowest task, 64-bit state
 // and the integer form of the terms (7,230 instructions).
-template <int LPT, int S, bool BUSY>
+template <int LPT, int S, bool BUSY, bool PREFETCH = false>
 __device__ __forceinline__ bool search_narrow(const GpParams &g, bool live, i64 t, i64 a, int n, u32 *buf, int lane,
                                               unsigned int gmask) {
   const KParams &p = g.k;
@@ -422,7 +422,7 @@ __device__ __forceinline__ bool search_narrow(const GpParams &g, bool live, i64 
   const u32 eps = (u32)p.ovh;
   const Rows<LPT, S, false> rows{buf};
   TaskValues<S> o;
-  if (!stage_fast<LPT, S, (S <= 3 ? S : 2), true>(p, live, a, n, buf, rows, lane, gmask, false, eps, o)) return false;
+  if (!stage_fast<LPT, S, (S <= 3 ? S : 2), true, PREFETCH>(p, live, a, n, buf, rows, lane, gmask, false, eps, o)) return false;
   live = o.live && o.n_narrow == o.n;
   if (LPT == 32 ? !live : !__any_sync(kFull, live)) return false;
   n = live ? o.n : 0;
@@ -689,6 +689,31 @@ __global__ void __launch_bounds__(kBlockThreads, gp_min_blocks(S)) gpu_priority_
   wait_for_previous_grid();
 }
 
+// A batch of at most kDirectSweepMost tasksets in one launch: a block of one warp per taskset, no plan
+// (1,000 tasksets of 8 / 20 / 80 tasks: 25 / 26 / 45 us, with plan and binned kernels 39 / 59 / 66 us; 8,192
+// of 80 tasks: 147 against 132 us).
+template <bool BUSY>
+__global__ void __launch_bounds__(32) gpu_priority_direct_kernel(GpParams g) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  u32 *const buf = reinterpret_cast<u32 *>(smem_raw);
+  const KParams &p = g.k;
+  const int lane = threadIdx.x;
+  const i64 t = blockIdx.x;
+  const i64 a = p.task_off[t], b = p.task_off[t + 1];
+  bool done = false;
+  if (g.assign && a >= 0 && b > a && b <= p.n_tasks && b - a <= GCAPS_RTA_MAX_TASKS && p.ovh < (1 << 20)) {
+    const int n = (int)(b - a);
+    if (n <= 32) done = search_narrow<32, 1, BUSY, true>(g, true, t, a, n, buf, lane, kFull);
+    else if (n <= 64) done = search_narrow<32, 2, BUSY, true>(g, true, t, a, n, buf, lane, kFull);
+    else if (n <= 96) done = search_narrow<32, 3, BUSY, true>(g, true, t, a, n, buf, lane, kFull);
+    else if (n <= 128) done = search_narrow<32, 4, BUSY, true>(g, true, t, a, n, buf, lane, kFull);
+    else if (n <= 192) done = search_narrow<32, 6, BUSY, true>(g, true, t, a, n, buf, lane, kFull);
+    else done = search_narrow<32, 8, BUSY, true>(g, true, t, a, n, buf, lane, kFull);
+  }
+  __syncwarp();
+  if (!done) analyse_gpu_priority<32, 8>(g, t, *reinterpret_cast<GpSmem<256> *>(buf), lane, kFull);
+}
+
 template <int S, bool BUSY>
 cudaError_t launch_big(const GpParams &g, int bin, int sm_count, cudaStream_t st) {
   constexpr int kWarps = kBlockThreads / 32;
@@ -736,11 +761,19 @@ extern "C" int gcaps_rta_gpu_priority_batch(const gcaps_tasksets_t *ts, int64_t 
   g.gpu_prio_out = (i64 *)out_gpu_priority;
   g.assign = assign ? 1 : 0;
   cudaStream_t st = (cudaStream_t)stream;
-  rc = enqueue_plan(g.k, workspace, workspace_bytes, st);
+  const bool direct = n_tasksets <= kDirectSweepMost, busy = (flags & GCAPS_RTA_BUSY) != 0;
+  rc = direct ? place_plan(g.k, workspace, workspace_bytes) : enqueue_plan(g.k, workspace, workspace_bytes, st);
   if (rc != GCAPS_OK) return rc;
   cudaError_t e = cudaGetLastError();
-  if (e == cudaSuccess)
-    e = (flags & GCAPS_RTA_BUSY) ? launch_gp_bins<true>(g, di.sm_count, st) : launch_gp_bins<false>(g, di.sm_count, st);
+  if (e == cudaSuccess && direct) {
+    constexpr int smem = (int)sizeof(u32) * bin_warp_words<32, 8>();
+    static_assert(sizeof(GpSmem<256>) <= (size_t)smem && smem <= 48 * 1024, "no attribute to set");
+    if (busy) gpu_priority_direct_kernel<true><<<(unsigned int)n_tasksets, 32, smem, st>>>(g);
+    else gpu_priority_direct_kernel<false><<<(unsigned int)n_tasksets, 32, smem, st>>>(g);
+    e = cudaGetLastError();
+  } else if (e == cudaSuccess) {
+    e = busy ? launch_gp_bins<true>(g, di.sm_count, st) : launch_gp_bins<false>(g, di.sm_count, st);
+  }
   if (e != cudaSuccess) {
     g_last_cuda_error = (int)e;
     return GCAPS_ERR_CUDA;

@@ -305,8 +305,7 @@ void fill_params(KParams *p, const gcaps_tasksets_t *ts, int64_t n_tasksets, int
   p->out_sched = out_sched;
 }
 
-// Points p at the plan areas of `workspace`.
-static int place_plan(KParams &p, void *workspace, size_t workspace_bytes) {
+int place_plan(KParams &p, void *workspace, size_t workspace_bytes) {
   const size_t need = gcaps_rta_workspace_bytes(p.n_tasksets);
   if (!workspace || workspace_bytes < need || ((uintptr_t)workspace & 255u))
     return GCAPS_ERR_WORKSPACE;
@@ -405,7 +404,7 @@ int enqueue_batch(KParams p, void *workspace, size_t workspace_bytes, int sm_cou
   if (p.n_tasksets == 0) return GCAPS_OK;
   const bool rr = (p.policy & 0xff) == GCAPS_POLICY_RR, busy = (p.policy & GCAPS_RTA_BUSY) != 0;
   const int mode = (rr ? 2 : 0) + (busy ? 1 : 0);
-  const bool direct = !sw && p.n_tasksets <= kDirectMost;
+  const bool direct = p.n_tasksets <= (sw ? kDirectSweepMost : kDirectMost);
   const int rc = place_plan(p, workspace, workspace_bytes);
   if (rc != GCAPS_OK) return rc;
   if (!direct) enqueue_plan_kernels(p, st);
@@ -421,9 +420,10 @@ int enqueue_batch(KParams p, void *workspace, size_t workspace_bytes, int sm_cou
     for (int half = 0; half < 2 && e == cudaSuccess; ++half) {
       set.enabled = analyses & (half == 0 ? 5 : 10);
       if (set.enabled == 0) continue;
-      if (!first) e = cudaMemsetAsync(p.hdr->next, 0, sizeof(p.hdr->next), st);
+      if (!first && !direct) e = cudaMemsetAsync(p.hdr->next, 0, sizeof(p.hdr->next), st);
       first = false;
-      if (e == cudaSuccess) e = launch_sweep_set(p, set, sm_count, st);
+      if (e == cudaSuccess)
+        e = direct ? launch_sweep_one_warp_each(p, set, sm_count, st) : launch_sweep_set(p, set, sm_count, st);
     }
   } else if (e == cudaSuccess) {
     if (direct) e = launch_one_warp_each(mode, p, st);

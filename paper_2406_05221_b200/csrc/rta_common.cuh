@@ -27,6 +27,8 @@ constexpr int kStagedBlockThreads = 64;  // kernels that stage tasksets by bulk 
 constexpr int kPlanItems = 1024;  // tasksets per plan block
 constexpr int kPlanSmall = 8192;  // batches up to this size are planned by one block in one launch
 constexpr int kDirectMost = 12288;  // batches up to this size run without a plan (see gcaps_rta_direct.cu)
+constexpr int kDirectSweepMost = 4096;  // the same for several analyses per taskset, and for the search of GPU
+                                        // priorities
 constexpr u64 kClamp = 1ull << 50;  // any quantity >= 2^50 exceeds every deadline (<= 2^40)
 
 struct PlanHeader {
@@ -273,6 +275,7 @@ void fill_params(KParams *p, const gcaps_tasksets_t *ts, int64_t n_tasksets, int
                  int64_t ovh, int64_t *out_wcrt, uint8_t *out_sched);
 // Points p at the plan areas of `workspace` and enqueues the three plan kernels (size bins, a
 // permutation of the taskset indices, zeroed work counters).  GCAPS_OK or GCAPS_ERR_WORKSPACE.
+int place_plan(KParams &p, void *workspace, size_t workspace_bytes);  // only the first part
 int enqueue_plan(KParams &p, void *workspace, size_t workspace_bytes, cudaStream_t st);
 // One launch for analysis `mode` (0 GCAPS self-suspension, 1 GCAPS busy-waiting, 2 RR self-suspension, 3 RR
 // busy-waiting) without a plan, a block of one warp per taskset, for batches of at most kDirectMost
@@ -281,6 +284,9 @@ cudaError_t launch_one_warp_each(int mode, const KParams &p, cudaStream_t st);
 // Launches over all size bins for the analyses sw.enabled names (bit m = mode m; one of 1, 2, 4, 8,
 // 5, 10) under every pair of `sw`; defined in gcaps_rta_sweep.cu.
 cudaError_t launch_sweep_set(const KParams &p, const SweepArgs &sw, int sm_count, cudaStream_t st);
+// The same for at most kDirectSweepMost tasksets in one launch without a plan; defined in
+// gcaps_rta_direct_sweep.cu.
+cudaError_t launch_sweep_one_warp_each(const KParams &p, const SweepArgs &sw, int sm_count, cudaStream_t st);
 
 }  // namespace gcaps_detail
 #endif  // GCAPS_RTA_COMMON_CUH_

@@ -644,7 +644,8 @@ __device__ __forceinline__ bool stage_fast(const KParams &p, bool live, i64 a, i
 constexpr int kFastDeclined = 0, kFastDone = 1;
 template <int LPT, int SLOTS, int MASK, bool SWEEP = false, bool PREFETCH = false>
 __device__ __forceinline__ int analyse_fast(const KParams &p, bool live, i64 t, i64 a, int n, u32 *buf, int lane,
-                                            unsigned int gmask, const SweepArgs *sw = nullptr) {
+                                            unsigned int gmask, const SweepArgs *sw = nullptr, int q_first = 0,
+                                            int q_end = GCAPS_RTA_MAX_SWEEP) {
   typedef FastLayout<LPT, SLOTS> Lay;
   constexpr int MAXN = Lay::MAXN, CAP = Lay::CAP;
   // prefix blocks of the CPU segments whose loads are issued together.  Tasksets of 65..96 tasks
@@ -795,7 +796,7 @@ __device__ __forceinline__ int analyse_fast(const KParams &p, bool live, i64 t, 
     i64 sl_L = -1;
     const int enabled = kMulti ? sw->enabled : MASK;
 #pragma unroll 1
-    for (int q = 0; q < sw->n; ++q) {
+    for (int q = q_first; q < (q_end < sw->n ? q_end : sw->n); ++q) {
       const i64 L64 = sw->q[q].L;
       PairConsts pc;
       pc.ovh = (u32)sw->q[q].ovh;  // the fast path needs eps, theta < 2^20
@@ -882,6 +883,30 @@ __host__ __device__ constexpr int min_blocks(int slots) {
   return slots <= 3 ? 6 : slots == 4 ? 4 : slots == 6 ? 3 : 2;
 }
 
+// The exact path once per (timeslice, overhead) pair q_first .. q_end-1 and analysis of a sweep.
+template <int LPT, int MAXN, int MASK>
+__device__ __forceinline__ void exact_by_pair(const KParams &p, const SweepArgs &sw, i64 t, GroupSmem<MAXN> &s, int lane,
+                                              unsigned int gmask, int q_first, int q_end) {
+  constexpr bool kMulti = (MASK & (MASK - 1)) != 0;
+  const int enabled = kMulti ? sw.enabled : MASK;
+#pragma unroll 1
+  for (int q = q_first; q < q_end; ++q) {
+#pragma unroll 1
+    for (int m = 0; m < 4; ++m) {
+      if (!((MASK & enabled) >> m & 1)) continue;
+      const int block = q * sw.block_stride + sw.block_of_mode[m];
+      KParams pq = p;
+      pq.policy = (p.policy & ~(0xff | GCAPS_RTA_BUSY)) | (m >= 2 ? GCAPS_POLICY_RR : GCAPS_POLICY_GCAPS) |
+                  ((m & 1) ? GCAPS_RTA_BUSY : 0);
+      pq.L = sw.q[q].L, pq.ovh = sw.q[q].ovh;
+      pq.out_wcrt = p.out_wcrt ? p.out_wcrt + (i64)block * p.n_tasks : nullptr;
+      pq.out_sched = p.out_sched + (i64)block * p.n_tasksets;
+      analyse_taskset<LPT, MAXN>(pq, t, s, lane, gmask);
+      __syncwarp(gmask);
+    }
+  }
+}
+
 // One size bin, worked through by all warps of a persistent launch.  A warp is 32/LPT groups of
 // LPT lanes; every group analyses one taskset at a time.  Warps pull chunks of taskset indices
 // from the bin's counter; the index, task range and first segment offsets of the next chunk are
@@ -950,23 +975,8 @@ __device__ __forceinline__ void run_bin(const KParams &p, int bin, u32 *warp_buf
         if (!SWEEP) {
           // the exact path reads task_off again and validates everything itself
           analyse_taskset<LPT, MAXN>(p, t, *reinterpret_cast<GroupSmem<MAXN> *>(buf), lane, gmask);
-        } else {  // the exact path once per (timeslice, overhead) pair
-          constexpr bool kMulti = (MASK & (MASK - 1)) != 0;
-          const int enabled = kMulti ? sw->enabled : MASK;
-          for (int q = 0; q < sw->n; ++q) {
-            for (int m = 0; m < 4; ++m) {
-              if (!((MASK & enabled) >> m & 1)) continue;
-              const int block = q * sw->block_stride + sw->block_of_mode[m];
-              KParams pq = p;
-              pq.policy = (p.policy & ~(0xff | GCAPS_RTA_BUSY)) | (m >= 2 ? GCAPS_POLICY_RR : GCAPS_POLICY_GCAPS) |
-                          ((m & 1) ? GCAPS_RTA_BUSY : 0);
-              pq.L = sw->q[q].L, pq.ovh = sw->q[q].ovh;
-              pq.out_wcrt = p.out_wcrt ? p.out_wcrt + (i64)block * p.n_tasks : nullptr;
-              pq.out_sched = p.out_sched + (i64)block * p.n_tasksets;
-              analyse_taskset<LPT, MAXN>(pq, t, *reinterpret_cast<GroupSmem<MAXN> *>(buf), lane, gmask);
-              __syncwarp(gmask);
-            }
-          }
+        } else {
+          exact_by_pair<LPT, MAXN, MASK>(p, *sw, t, *reinterpret_cast<GroupSmem<MAXN> *>(buf), lane, gmask, 0, sw->n);
         }
       }
       __syncwarp();
