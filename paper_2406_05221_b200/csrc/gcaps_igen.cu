@@ -2,9 +2,10 @@
 // GCAPS, ECRTS 2024, arXiv 2406.05221, Sec. 7.1 / Table 3) for NVIDIA B200 (sm_100a).
 //
 // The generator itself is igen.h (integer-only; the host generator compiles the same
-// definition).  gcaps_gen_count: one thread per taskset runs the per-task part of the generator
-// (igen_begin), writes the three sizes of the taskset and leaves what it drew per task (period,
-// execution demand, priority, core, GPU segments: 12 bytes per task) and the position of the
+// definition).  gcaps_gen_count: one warp per taskset does what igen_begin defines (lane = task; the
+// random source is counter-based, so every draw's position is known without the ones before it),
+// writes the three sizes of the taskset and leaves what it drew per task (period, execution demand,
+// priority, core, GPU segments: 12 bytes per task) and the position of the
 // random stream in the workspace; three exclusive scans turn the sizes into offsets (block sums,
 // one block over the block sums, block-local scan).  gcaps_gen_fill: one warp per taskset, lane =
 // task; the random draws of a task start at a position that is a prefix sum over the tasks
@@ -46,20 +47,300 @@ __host__ __device__ inline i64 max_tasks_of(const igen_params_t &p) {
 
 __host__ __device__ inline i64 scan_blocks(i64 count) { return (count + kScanItems - 1) / kScanItems; }
 
+// ---- the per-task part of the generator, a warp per taskset -----------------------------------------
+constexpr int kExpBits = 10;  // leading bits of the fraction that 2^y looks up
+
+// Shared memory of one warp of the count kernel.
+struct CountWarp {
+  union {
+    struct {
+      u32 cut[IGEN_MAX_TASKS];  // by task: cut points of its core's utilisation as drawn, then its utilisation
+      union {
+        u32 sorted[IGEN_MAX_TASKS];  // the cut points in ascending order
+        int writer[IGEN_MAX_TASKS];  // the draw of GPU-using tasks, see below
+        __align__(16) u32 key[IGEN_MAX_TASKS];  // (T << 8 | position), for the ranks
+      };
+    };
+    uint64_t load[IGEN_MAX_TASKS];  // worst fit: E / T in Q32
+  };
+  u32 T[IGEN_MAX_TASKS];
+  short last[IGEN_MAX_TASKS], from[IGEN_MAX_TASKS];
+  unsigned char core[IGEN_MAX_TASKS], eta[IGEN_MAX_TASKS];
+  u32 start[IGEN_MAX_CORES + 1];  // first task of a core
+  u32 ctr[IGEN_MAX_CORES];        // draws in front of a core's
+  u32 util[IGEN_MAX_CORES];       // utilisation of a core, Q32
+  u32 pad_[3];
+};
+static_assert(sizeof(CountWarp) % 16 == 0, "16-byte rows");
+
+__device__ __forceinline__ uint64_t draw_at(uint64_t key, u32 position) {  // the position-th draw, from 1 on
+  igen_rng_t r;
+  r.key = key, r.ctr = position - 1;
+  return igen_u64(&r);
+}
+
+// x mod d for 0 < d < 2^16, in 32-bit steps
+__device__ __forceinline__ u32 mod_small(uint64_t x, u32 d) {
+  u32 r = (u32)(x >> 32) % d;
+  r = ((r << 16) | (u32)(x >> 16 & 0xffffu)) % d;
+  return ((r << 16) | (u32)(x & 0xffffu)) % d;
+}
+__device__ __forceinline__ int int_from(uint64_t x, int lo, int hi) {  // igen_int of the draw x
+  return hi <= lo ? lo : lo + (int)mod_small(x, (u32)(hi - lo) + 1u);
+}
+__device__ __forceinline__ uint64_t range_from(uint64_t x, uint64_t lo, uint64_t hi) {  // igen_range of the draw x
+  return hi <= lo ? lo : lo + igen_mul_shr32(hi - lo, x >> 32);
+}
+
+// 2^(2^-i) = 1 + e_i as 4 * e_i in Q62: r * (1 + e_i) in Q62, rounded down, is r + umulhi(r, 4 e_i), the same
+// integer as igen_mul_q62(r, igen_root(i)).
+__device__ __forceinline__ uint64_t times_root(uint64_t r, int i) {
+  return r + __umul64hi(r, (igen_root(i) - (1ULL << 62)) << 2);
+}
+// igen_exp2 with the product of the first kExpBits roots looked up
+__device__ __forceinline__ uint64_t exp2_from(const uint64_t *table, uint64_t y) {
+  const int k = (int)(y >> 32);
+  const u32 f = (u32)y >> (32 - IGEN_FRAC_BITS);
+  uint64_t r = table[f >> (IGEN_FRAC_BITS - kExpBits)];
+#pragma unroll
+  for (int i = kExpBits + 1; i <= IGEN_FRAC_BITS; ++i)
+    if ((f >> (IGEN_FRAC_BITS - i)) & 1u) r = times_root(r, i);
+  return ((r >> (61 - k)) + 1) >> 1;
+}
+
+// Bound by instruction issue (3,790 warp instructions per `large` taskset, 70 % of the slots; the ranks are
+// 16 % of the time, 2^y 12 %): 250,000 of them 1.20 ms.  A thread per taskset took 1.40 ms (2.3 KB of state
+// per thread in local memory).
 __global__ void __launch_bounds__(kGenThreads) gen_count_kernel(igen_params_t p, i64 first, i64 count,
                                                                  GenSpace w) {
-  const i64 t = (i64)blockIdx.x * kGenThreads + threadIdx.x;
-  if (t >= count) return;
-  igen_state_t s;
-  igen_begin(&p, (uint64_t)(first + t), &s);
-  w.off[0][t] = s.n, w.off[1][t] = s.n_csegs, w.off[2][t] = s.n_gsegs;
-  u32 *st = w.state + t * w.state_stride;
-  st[0] = (u32)s.rng.key, st[1] = (u32)(s.rng.key >> 32);
-  st[2] = (u32)s.rng.ctr, st[3] = (u32)(s.rng.ctr >> 32);
-  for (int i = 0; i < s.n; ++i) {
-    st[4 + 3 * i] = s.T[i];
-    st[5 + 3 * i] = s.E[i];
-    st[6 + 3 * i] = (u32)s.prio[i] | ((u32)s.core[i] << 16) | ((u32)s.eta[i] << 24);
+  __shared__ CountWarp warps[kGenThreads / 32];
+  __shared__ uint64_t table[1 << kExpBits];
+  CountWarp &s = warps[threadIdx.x >> 5];
+  const int lane = threadIdx.x & 31;
+#pragma unroll 1
+  for (int f = threadIdx.x; f < (1 << kExpBits); f += kGenThreads) {
+    uint64_t r = 1ULL << 62;
+#pragma unroll
+    for (int i = 1; i <= kExpBits; ++i)
+      if ((f >> (kExpBits - i)) & 1) r = times_root(r, i);
+    table[f] = r;
+  }
+  __syncthreads();
+#pragma unroll 1
+  for (i64 t = (i64)blockIdx.x * (kGenThreads / 32) + (threadIdx.x >> 5); t < count; t += (i64)gridDim.x * (kGenThreads / 32)) {
+    igen_rng_t rng;
+    igen_rng_init(&rng, p.seed, p.stream, (uint64_t)(first + t));
+    const uint64_t key = rng.key;
+    int cores = int_from(draw_at(key, 1), p.cores_lo, p.cores_hi);
+    if (cores > IGEN_MAX_CORES) cores = IGEN_MAX_CORES;
+    const bool harmonic = (draw_at(key, 2) >> 32) < p.harmonic;
+    u32 ctr = 2;  // draws so far
+    int n = 0;
+    // tasks per core: a core takes a draw for its tasks, one for its utilisation, one per cut point
+#pragma unroll 1
+    for (int c = 0; c < cores; ++c) {
+      int m = p.tpc_hi <= p.tpc_lo ? p.tpc_lo : int_from(draw_at(key, ctr + 1), p.tpc_lo, p.tpc_hi);
+      if (n + m > IGEN_MAX_TASKS) m = IGEN_MAX_TASKS - n;
+      if (lane == 0) s.start[c] = (u32)n, s.ctr[c] = ctr;
+      for (int k = lane; k < m; k += 32) s.core[n + k] = (unsigned char)c;
+      ctr += 2 + (m > 1 ? m - 1 : 0);
+      n += m;
+    }
+    if (lane == 0) s.start[cores] = (u32)n;
+    __syncwarp();
+    for (int c = lane; c < cores; c += 32) s.util[c] = (u32)range_from(draw_at(key, s.ctr[c] + 2), p.util_lo, p.util_hi);
+#pragma unroll 1
+    for (int i = lane; i < n; i += 32) {
+      const int c = s.core[i], k = i - (int)s.start[c];
+      if (i + 1 < (int)s.start[c + 1]) s.cut[i] = (u32)(draw_at(key, s.ctr[c] + 3 + k) >> 32);
+      s.eta[i] = 0, s.last[i] = -1;
+    }
+    __syncwarp();
+#pragma unroll 1
+    for (int i = lane; i < n; i += 32) {  // the cut points of a core in ascending order
+      const int c = s.core[i], from = (int)s.start[c], last = (int)s.start[c + 1] - 1;
+      if (i < last) {
+        const u32 x = s.cut[i];
+        int r = from;
+#pragma unroll 1
+        for (int q = from; q < last; ++q) {
+          const u32 y = s.cut[q];
+          r += (y < x || (y == x && q < i)) ? 1 : 0;
+        }
+        s.sorted[r] = x;
+      }
+    }
+    __syncwarp();
+#pragma unroll 1
+    for (int i = lane; i < n; i += 32) {  // a task's share of its core (the last one takes what is left)
+      const int c = s.core[i], from = (int)s.start[c], last = (int)s.start[c + 1] - 1;
+      if (i < last) s.cut[i] = (u32)(((uint64_t)s.util[c] * (s.sorted[i] - (i > from ? s.sorted[i - 1] : 0u))) >> 32);
+    }
+    __syncwarp();
+#pragma unroll 1
+    for (int i = lane; i < n; i += 32) {
+      const int c = s.core[i], from = (int)s.start[c], last = (int)s.start[c + 1] - 1;
+      if (i == last) {
+        u32 left = s.util[c];
+#pragma unroll 1
+        for (int q = from; q < last; ++q) left -= s.cut[q];
+        s.cut[i] = left;
+      }
+    }
+    // periods
+#pragma unroll 1
+    for (int i = lane; i < n; i += 32) {
+      i64 T;
+      if (harmonic) {
+        const i64 T0 = (i64)exp2_from(table, range_from(draw_at(key, ctr + 1 + 2 * i), p.log2_lo, p.log2_hi0));
+        T = T0 << int_from(draw_at(key, ctr + 2 + 2 * i), 0, 10);
+      } else {
+        T = (i64)exp2_from(table, range_from(draw_at(key, ctr + 1 + i), p.log2_lo, p.log2_hi));
+      }
+      if (T < p.period_lo) T = p.period_lo;
+      if (T > p.period_hi) T = p.period_hi;
+      s.T[i] = (u32)T;
+    }
+    ctr += harmonic ? 2 * n : n;
+    // which tasks use the GPU, and how many segments they ask for
+    if (p.gpu_mode == 0) {
+      // A partial Fisher-Yates shuffle of 0 .. n-1: step k swaps positions k and j_k >= k, and the task
+      // then at position k is drawn.  Position k is last written, before step k, by the largest k' < k
+      // with j_k' = k (`writer`), and then holds what was at position k' before step k': following the
+      // writers to the end gives the task (v).  What step k draws was at position j_k: v of the last
+      // k' < k with the same j, or j_k itself.
+      int ng = (int)((p.gpu_frac * (uint64_t)n + (1ULL << 31)) >> 32);
+      if (ng > n) ng = n;
+      for (int i = lane; i < n; i += 32) s.writer[i] = -1;
+      __syncwarp();
+#pragma unroll 1
+      for (int k0 = 0; k0 < ng; k0 += 32) {
+        const int k = k0 + lane;
+        const int j = k < ng ? k + (int)mod_small(draw_at(key, ctr + 1 + 2 * k), (u32)(n - k)) : -1 - lane;
+        const u32 same = __match_any_sync(kFull, j);
+        const u32 below = same & ((1u << lane) - 1u);
+        int before = -1;
+        if (k < ng) {
+          before = below ? k0 + 31 - __clz((int)below) : (int)s.last[j];
+          if (j != k) atomicMax(&s.writer[j], k);
+        }
+        __syncwarp();
+        if (k < ng) {
+          if ((same >> lane) == 1u) s.last[j] = (short)k;  // the last of its kind in this round
+          s.from[k] = (short)(before >= 0 ? before : ~j);   // a step to follow, or ~task
+        }
+        __syncwarp();
+      }
+#pragma unroll 1
+      for (int k = lane; k < ng; k += 32) {
+        int task = s.from[k];
+        if (task >= 0) {
+          while (s.writer[task] >= 0) task = s.writer[task];
+        } else {
+          task = ~task;
+        }
+        s.eta[task] = (unsigned char)int_from(draw_at(key, ctr + 2 + 2 * k), p.seg_lo < 1 ? 1 : p.seg_lo, p.seg_hi);
+      }
+      ctr += 2 * ng;
+    } else {
+#pragma unroll 1
+      for (int i = lane; i < n; i += 32) s.eta[i] = (unsigned char)int_from(draw_at(key, ctr + 1 + i), p.seg_lo, p.seg_hi);
+      ctr += n;
+    }
+    __syncwarp();
+    // execution demand; a task drops segments until every one gets at least 1 us
+    u32 *st = w.state + t * w.state_stride;
+    u32 nc = 0, ngs = 0;
+#pragma unroll 1
+    for (int i = lane; i < n; i += 32) {
+      const u32 T = s.T[i];
+      uint64_t E = ((uint64_t)s.cut[i] * T + (1ULL << 31)) >> 32;
+      if (E < 1) E = 1;
+      if (E > T) E = T;
+      u32 eta = s.eta[i] > IGEN_MAX_SEGS ? IGEN_MAX_SEGS : s.eta[i];
+      if (eta > ((u32)E - 1) / 2) eta = ((u32)E - 1) / 2;
+      s.eta[i] = (unsigned char)eta;
+      nc += eta + 1, ngs += eta;
+      st[4 + 3 * i] = T, st[5 + 3 * i] = (u32)E;
+    }
+    __syncwarp();
+    if (p.wfd) {
+      // worst fit, decreasing by utilisation (ties: lower index first): the order by counting, then one
+      // task after the other to the core with the least load (lane: cores lane and lane + 32)
+#pragma unroll 1
+      for (int i = lane; i < n; i += 32) s.load[i] = ((uint64_t)st[5 + 3 * i] << 32) / s.T[i];
+      __syncwarp();
+#pragma unroll 1
+      for (int i = lane; i < n; i += 32) {
+        const uint64_t u = s.load[i];
+        int r = 0;
+#pragma unroll 1
+        for (int q = 0; q < n; ++q) {
+          const uint64_t y = s.load[q];
+          r += (y > u || (y == u && q < i)) ? 1 : 0;
+        }
+        s.from[r] = (short)i;
+      }
+      __syncwarp();
+      uint64_t load0 = lane < cores ? 0 : ~0ULL >> 8, load1 = lane + 32 < cores ? 0 : ~0ULL >> 8;
+#pragma unroll 1
+      for (int k = 0; k < n; ++k) {
+        const int i = s.from[k];
+        // least (load, core): loads stay below 2^41, in two halves with the core behind the lower one
+        const bool second = load1 < load0;
+        const uint64_t mine = second ? load1 : load0;
+        const u32 hi = mine >= (1ULL << 48) ? 0xffffffffu : (u32)(mine >> 20);
+        const u32 least = __reduce_min_sync(kFull, hi);
+        const u32 lo = hi == least ? (((u32)mine & 0xfffffu) << 6) | (u32)(second ? lane + 32 : lane) : 0xffffffffu;
+        const u32 best = __reduce_min_sync(kFull, lo) & 63u;
+        if ((best & 31u) == (u32)lane) {
+          if (best >= 32) load1 += s.load[i];
+          else load0 += s.load[i];
+        }
+        if (lane == 0) s.core[i] = (unsigned char)best;
+      }
+      __syncwarp();
+    }
+    // rate-monotonic priorities: shorter period = higher, ties by position.  Periods below 2^24 with the
+    // position behind them are distinct 32-bit keys; 96 tasks are compared with four at a time.
+    if (p.period_hi < (1LL << 24)) {
+      for (int i = lane; i < ((n + 3) & ~3); i += 32) s.key[i] = i < n ? (s.T[i] << 8) | (u32)i : 0xffffffffu;
+      __syncwarp();
+#pragma unroll 1
+      for (int i0 = lane; i0 - lane < n; i0 += 96) {
+        u32 mine[3];
+        int higher[3] = {0, 0, 0};
+#pragma unroll
+        for (int e = 0; e < 3; ++e) mine[e] = i0 + 32 * e < n ? s.key[i0 + 32 * e] : 0u;
+#pragma unroll 1
+        for (int q = 0; q < n; q += 4) {
+          const uint4 y = *reinterpret_cast<const uint4 *>(&s.key[q]);
+#pragma unroll
+          for (int e = 0; e < 3; ++e)
+            higher[e] += (y.x < mine[e] ? 1 : 0) + (y.y < mine[e] ? 1 : 0) + (y.z < mine[e] ? 1 : 0) + (y.w < mine[e] ? 1 : 0);
+        }
+#pragma unroll
+        for (int e = 0; e < 3; ++e) {
+          const int i = i0 + 32 * e;
+          if (i < n) st[6 + 3 * i] = (u32)(n - higher[e]) | ((u32)s.core[i] << 16) | ((u32)s.eta[i] << 24);
+        }
+      }
+    } else {
+#pragma unroll 1
+      for (int i = lane; i < n; i += 32) {
+        int higher = 0;
+        const u32 T = s.T[i];
+#pragma unroll 1
+        for (int q = 0; q < n; ++q) higher += s.T[q] < T + (q < i ? 1u : 0u) ? 1 : 0;
+        st[6 + 3 * i] = (u32)(n - higher) | ((u32)s.core[i] << 16) | ((u32)s.eta[i] << 24);
+      }
+    }
+    nc = __reduce_add_sync(kFull, nc), ngs = __reduce_add_sync(kFull, ngs);
+    if (lane == 0) {
+      w.off[0][t] = n, w.off[1][t] = nc, w.off[2][t] = ngs;
+      st[0] = (u32)key, st[1] = (u32)(key >> 32), st[2] = ctr, st[3] = 0;
+    }
+    __syncwarp();
   }
 }
 
@@ -289,6 +570,8 @@ __global__ void __launch_bounds__(kGenThreads) gen_fill_kernel(igen_params_t p, 
   }
 }
 
+int g_count_blocks[64] = {0};
+
 size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 
 bool params_ok(const gcaps_gen_params_t *p) {
@@ -355,11 +638,17 @@ int gcaps_gen_count(const gcaps_gen_params_t *params, int64_t first, int64_t cou
   if (rc != GCAPS_OK) return rc;
   igen_params_t p;
   memcpy(&p, params, sizeof(p));
-  gen_count_kernel<<<(unsigned int)((count + kGenThreads - 1) / kGenThreads), kGenThreads, 0, st>>>(p, first, count, w);
+  constexpr int kWarps = kGenThreads / 32;
+  cudaError_t e = launch_persistent(gen_count_kernel, g_count_blocks, 0, (long long)((count + kWarps - 1) / kWarps), di.sm_count, st, p,
+                                    (i64)first, (i64)count, w);
+  if (e != cudaSuccess) {
+    g_last_cuda_error = (int)e;
+    return GCAPS_ERR_CUDA;
+  }
   scan_sums_kernel<<<dim3((unsigned int)w.n_blocks, 3), kScanThreads, 0, st>>>(w, count);
   scan_blocks_kernel<<<3, kScanThreads, 0, st>>>(w, count, (i64 *)out_totals);
   scan_apply_kernel<<<dim3((unsigned int)w.n_blocks, 3), kScanThreads, 0, st>>>(w, count);
-  cudaError_t e = cudaGetLastError();
+  e = cudaGetLastError();
   if (e != cudaSuccess) {
     g_last_cuda_error = (int)e;
     return GCAPS_ERR_CUDA;

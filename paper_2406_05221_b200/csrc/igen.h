@@ -1,6 +1,7 @@
 /*
- * igen.h -- the integer-only taskset generator, as one definition that compiles both as C (the
- * host generator, gcc) and as CUDA device code (the on-device generator, nvcc).
+ * igen.h -- the integer-only taskset generator: the definition, as the host generator runs it
+ * (gcc), and the draws and arithmetic that the on-device generator (nvcc) shares with it.  The
+ * device takes the same steps with a warp per taskset (gcaps_igen.cu).
  *
  * It follows the generation procedure of the paper's Sec. 7.1 / Table 3 like the floating-point
  * host generator (taskgen.c) does -- tasks per CPU, utilisation per CPU split over its tasks,

@@ -1,0 +1,28 @@
+"""The per-task part of the on-device generator against its oracle where the warp's way differs from the
+step-by-step definition: few and many cores, cores without tasks, the limit of 256 tasks, every share
+of GPU-using tasks, harmonic periods, periods beyond 2^24, worst fit on up to 64 cores."""
+import numpy as np
+import pytest
+
+from oracle.igen_oracle import reference_taskset
+from paper_2406_05221_b200 import binding, taskgen
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("wfd", [False, True])
+@pytest.mark.parametrize("cores,per_core,gpu_frac,harmonic,period", [
+    ((1, 1), (0, 1), 1.0, 0.0, (1000, 1e6)), ((1, 2), (1, 33), 0.5, 0.5, (100, 1e7)),
+    ((33, 64), (0, 3), 0.9, 0.0, (1e4, 1e6)), ((20, 40), (7, 9), 0.0, 1.0, (50, 1e5)),
+    ((64, 64), (4, 5), 1.0, 0.3, (1e3, 1.07e9)), ((2, 3), (100, 120), 0.77, 0.5, (2, 40))])
+def test_tasks_match_the_oracle(cores, per_core, gpu_frac, harmonic, period, wfd):
+    torch = pytest.importorskip("torch")
+    for count in (1, 37):
+        params = taskgen.GenParams(seed=9, stream=2, cores=cores, tasks_per_core=per_core, util_per_core=(0.05, 0.9),
+                                   period_us=period, gpu_frac=gpu_frac, harmonic_frac=harmonic, wfd=wfd)
+        ts = binding.generate_device(params, 100, count)
+        torch.cuda.synchronize()
+        p = params.int_params()
+        want = taskgen.TasksetBatch.from_tasksets([reference_taskset(p, 100 + t) for t in range(count)])
+        for f in taskgen.ARRAY_FIELDS:
+            assert np.array_equal(ts.t[f].cpu().numpy(), getattr(want, f)), f
