@@ -639,8 +639,15 @@ int gcaps_gen_count(const gcaps_gen_params_t *params, int64_t first, int64_t cou
   igen_params_t p;
   memcpy(&p, params, sizeof(p));
   constexpr int kWarps = kGenThreads / 32;
-  cudaError_t e = launch_persistent(gen_count_kernel, g_count_blocks, 0, (long long)((count + kWarps - 1) / kWarps), di.sm_count, st, p,
-                                    (i64)first, (i64)count, w);
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  // (once per device, before the number of resident blocks is looked up: as much shared memory as there is,
+  // 24 instead of 16 warps per SM)
+  if (e == cudaSuccess && __atomic_load_n(&g_count_blocks[dev & 63], __ATOMIC_ACQUIRE) == 0)
+    e = cudaFuncSetAttribute(gen_count_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+  if (e == cudaSuccess)
+    e = launch_persistent(gen_count_kernel, g_count_blocks, 0, (long long)((count + kWarps - 1) / kWarps), di.sm_count, st,
+                          p, (i64)first, (i64)count, w);
   if (e != cudaSuccess) {
     g_last_cuda_error = (int)e;
     return GCAPS_ERR_CUDA;

@@ -196,8 +196,6 @@ cudaError_t launch_persistent_ex(bool overlap_previous, void (*kernel)(Args...),
     std::lock_guard<std::mutex> lock(g_init_mutex);
     e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-    if (e != cudaSuccess) return e;
     int per_sm = 1;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kBlockThreads, smem);
     if (e != cudaSuccess) return e;
