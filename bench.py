@@ -45,10 +45,10 @@ LAUNCHES_PER_SMALL_CALL = 1  # batches of up to 12,288 tasksets: a warp per task
 # ncu capture of a 131,072-taskset launch (traffic grows in proportion to the tasksets of a
 # launch).  Only reported while the kernel source is the one the counters were taken from.
 CAPTURED_TRAFFIC = {
-    "source_sha256": "9fc3a243eb31c6fb7c4e05766b9dc8d537e4e9f0aa84ad3911c2ef4eedab4396",
+    "source_sha256": "68df5a3333bb4154f1141fb0bd779590e78a1e72fe799874d64ebe93c2b9038c",
     "workload": "large",
-    "bytes_per_taskset": {"gcaps": (1248476000 + 84340736) / 131072.0,
-                          "rr": (1258324000 + 95665152) / 131072.0},
+    "bytes_per_taskset": {"gcaps": (1236099000 + 80368384) / 131072.0,
+                          "rr": (1236100000 + 80585984) / 131072.0},
 }
 
 
