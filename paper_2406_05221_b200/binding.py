@@ -145,7 +145,8 @@ class _device_and_stream:
 
     With ``dev`` current already and no stream given there is nothing to switch: only the handle is
     looked up (entering torch's two context managers took 13 us, half of a call of 1,000 small
-    tasksets)."""
+    tasksets).  Both ways refuse a device that is not a CUDA one, as the kernels would follow host
+    pointers."""
     __slots__ = ("dev", "stream", "inside")
 
     def __init__(self, dev, stream):
@@ -153,6 +154,8 @@ class _device_and_stream:
 
     def __enter__(self) -> int:
         import torch
+        if self.dev.type != "cuda":
+            raise ValueError("Expected a cuda device, but got: %s" % self.dev)
         index = self.dev.index
         here = torch.cuda.current_device()
         if self.stream is None and (index is None or index == here):
