@@ -1,6 +1,7 @@
 """In-tree build of the native sources: the CUDA library (nvcc, sm_100a) and the generator."""
 from __future__ import annotations
 
+import glob
 import os
 import subprocess
 import sys
@@ -12,7 +13,7 @@ CUDA_SRCS = [CUDA_SRC, os.path.join(_HERE, "csrc", "gcaps_rta_direct.cu"),
              os.path.join(_HERE, "csrc", "gcaps_rta_direct_sweep.cu"),
              os.path.join(_HERE, "csrc", "gcaps_gpu_priority.cu"),
              os.path.join(_HERE, "csrc", "gcaps_igen.cu"), os.path.join(_HERE, "csrc", "gcaps_diag.cu")]
-CUDA_DEPS = CUDA_SRCS + [os.path.join(_HERE, "csrc", f) for f in ("rta_common.cuh", "rta_device.cuh", "igen.h")]
+CUDA_DEPS = CUDA_SRCS + sorted(glob.glob(os.path.join(_HERE, "csrc", "*.cuh")) + glob.glob(os.path.join(_HERE, "csrc", "*.h")))
 CUDA_LIB = os.path.join(_HERE, "libgcaps_rta.so")
 HEADER = os.path.join(os.path.dirname(_HERE), "include", "gcaps_rta.h")
 
