@@ -17,6 +17,7 @@ from __future__ import annotations
 import argparse
 import json
 import os
+import re
 import statistics
 import subprocess
 import sys
@@ -25,6 +26,8 @@ import time
 ROOT = os.path.dirname(os.path.abspath(__file__))
 if ROOT not in sys.path:
     sys.path.insert(0, ROOT)
+
+from paper_2406_05221_b200 import build  # noqa: E402
 
 METRIC = "tasksets analysed/sec (GCAPS & RR RTA)"
 UNIT = "tasksets/s"
@@ -45,20 +48,32 @@ LAUNCHES_PER_SMALL_CALL = 1  # batches of up to 12,288 tasksets: a warp per task
 # ncu capture of a 131,072-taskset launch (traffic grows in proportion to the tasksets of a
 # launch).  Only reported while the kernel source is the one the counters were taken from.
 CAPTURED_TRAFFIC = {
-    "source_sha256": "68df5a3333bb4154f1141fb0bd779590e78a1e72fe799874d64ebe93c2b9038c",
+    "source_sha256": "d72161a2f977194ed98022d5ce4278143fd1418fff695841a09c0b0cc3b32e18",
     "workload": "large",
     "bytes_per_taskset": {"gcaps": (1236099000 + 80368384) / 131072.0,
                           "rr": (1236100000 + 80585984) / 131072.0},
 }
 
 
+def kernel_sources():
+    """The source of the kernels that CAPTURED_TRAFFIC was taken from and all it includes from csrc."""
+    found, todo = [], [build.CUDA_SRC]
+    while todo:
+        path = todo.pop()
+        found.append(path)
+        with open(path) as fh:
+            names = re.findall(r'^\s*#\s*include\s+"([^"/]+)"', fh.read(), flags=re.M)
+        todo += [p for p in (os.path.join(os.path.dirname(path), n) for n in names) if p not in found + todo]
+    return sorted(found)
+
+
 def kernel_source_digest():
-    """sha256 over the sources of the analysis kernel (gcaps_rta.cu and the headers it shares)."""
+    """sha256 over kernel_sources()."""
     import hashlib
     h = hashlib.sha256()
     try:
-        for name in ("gcaps_rta.cu", "rta_device.cuh", "rta_common.cuh"):
-            with open(os.path.join(ROOT, "paper_2406_05221_b200", "csrc", name), "rb") as fh:
+        for path in kernel_sources():
+            with open(path, "rb") as fh:
                 h.update(fh.read())
     except OSError:
         return None
