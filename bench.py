@@ -39,11 +39,18 @@ ALU_PEAK_DERIVED = 148 * 128 * 1.965e9
 # workload is generated, analysed and verified in chunks of 1,000,000)
 MAX_TASKSETS_PER_GPU = 1_000_000
 K_TERM, K_SETUP = 6, 16   # algorithmic integer lane-operations per interference term / per task
-# kernels launched by one gcaps_rta_batch call: 3 plan kernels, one analysis kernel for the bins
-# of up to 32 tasks, one each for the 64-, 96-, 128-, 192- and 256-task bins and two for the larger
-# tasksets that those left over
-LAUNCHES_PER_CALL = 11       # three plan kernels + one kernel per group of size bins + two
-LAUNCHES_PER_SMALL_CALL = 1  # batches of up to 12,288 tasksets: a warp per taskset, no plan
+
+def kernel_launches(tasksets, several=False):
+    """Kernels of one call on a batch: gcaps_rta_batch, or with `several` a sweep, a call for several
+    analyses of one waiting mode or a search of GPU priorities.  Small batches are one launch without a
+    plan.  Otherwise the plan takes one kernel or three; then one kernel serves the bins of up to 32
+    tasks, one each those of up to 64, 96, 128, 192 and 256, and for a single analysis two more what
+    the larger bins left over."""
+    if tasksets <= build.source_constant("kDirectSweepMost" if several else "kDirectMost"):
+        return 1
+    return (1 if tasksets <= build.source_constant("kPlanSmall") else 3) + (6 if several else 8)
+
+
 # DRAM bytes (read + write) per taskset of the analysis kernel on the 'large' workload, from an
 # ncu capture of a 131,072-taskset launch (traffic grows in proportion to the tasksets of a
 # launch).  Only reported while the kernel source is the one the counters were taken from.
@@ -608,9 +615,10 @@ def main():
                        "schedulable_fraction_last_policy": sched_frac,
                        "input_checksum": batch.checksum() if count <= 200_000 else None},
             "clocks": clocks, "e2e": e2e,
-            "gpu_launches": args.steps * (len(policies) if args.mode == "policies"
-                                          else (1 + len(pairs)) if args.mode == "sweep" else 2)
-                            * (LAUNCHES_PER_SMALL_CALL if count <= 12288 else LAUNCHES_PER_CALL),
+            "gpu_launches": args.steps * sum(
+                len(pairs) * kernel_launches(count) if name == "one_call_per_pair" else
+                kernel_launches(count, several=name in ("gcaps+rr", "fused_sweep", "gpu_priority_search"))
+                for name in names),
             "roofline": roof, "cpu_baseline": cpu, "wall_s_timed_region": t_wall,
         }
         line.update(side)

@@ -3,6 +3,7 @@ from __future__ import annotations
 
 import glob
 import os
+import re
 import subprocess
 import sys
 
@@ -19,6 +20,12 @@ HEADER = os.path.join(os.path.dirname(_HERE), "include", "gcaps_rta.h")
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-shared", "-Xcompiler", "-fPIC", "--threads", "7"]
+
+
+def source_constant(name: str) -> int:
+    """The value of a `constexpr int` of csrc/rta_common.cuh (sizes at which the launches of a call change)."""
+    with open(os.path.join(_HERE, "csrc", "rta_common.cuh")) as fh:
+        return int(re.search(r"constexpr int %s = (\d+);" % name, fh.read()).group(1))
 
 
 def _nvcc() -> str:
