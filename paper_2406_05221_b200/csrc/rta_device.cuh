@@ -836,7 +836,7 @@ struct Ahead {
   i64 a;           // first task
   i64 c_lo, g_lo;  // first CPU segment, first GPU segment
   u32 t;           // taskset index
-  u32 packed;      // tasks (bits 0-8) | CPU segments (9-19) | GPU segments (20-30) | fast (31)
+  u32 packed;      // tasks (bits 0-8) | CPU segments (9-19) | GPU segments (20-30) | offsets in range (31)
 };
 static_assert(sizeof(Ahead) == 32, "two 16-byte rows");
 constexpr int kMaxAhead = 16;  // tasksets of one pull
@@ -844,7 +844,9 @@ constexpr int kAheadWords = 2 * kMaxAhead * (int)(sizeof(Ahead) / sizeof(u32)); 
 
 constexpr u32 kNoTaskset = 0xffffffffu;
 
-// Looks up one taskset (or none) of a bin for at most MAXN tasks and CAP-1 segments of a kind.
+// Looks up one taskset (or none) of a bin for at most MAXN tasks and CAP-1 segments of a kind.  One whose
+// first or last offset lies outside its array has bit 31 of `packed` clear, and the exact path says what it
+// is: the stages see differences of offsets only, and without a segment all of those are 0.
 template <int MAXN, int CAP>
 __device__ __forceinline__ Ahead look_up_taskset(const KParams &p, u32 t) {
   static_assert(MAXN <= 256 && CAP <= 2048, "fields of Ahead::packed");
@@ -854,12 +856,14 @@ __device__ __forceinline__ Ahead look_up_taskset(const KParams &p, u32 t) {
     me.a = p.task_off[t] - p.task_base;
     const i64 b = p.task_off[(i64)t + 1] - p.task_base;
     if (me.a >= 0 && b > me.a && b <= p.n_tasks && b - me.a <= MAXN) {
-      u32 nc = 0, ng = 0;
       me.c_lo = p.cseg_off[me.a] - p.cseg_base, me.g_lo = p.gseg_off[me.a] - p.gseg_base;
       const i64 c_hi = p.cseg_off[b] - p.cseg_base, g_hi = p.gseg_off[b] - p.gseg_base;
-      if (me.c_lo >= 0 && c_hi <= p.n_csegs && c_hi - me.c_lo < CAP && c_hi > me.c_lo) nc = (u32)(c_hi - me.c_lo);
-      if (me.g_lo >= 0 && g_hi <= p.n_gsegs && g_hi - me.g_lo < CAP && g_hi > me.g_lo) ng = (u32)(g_hi - me.g_lo);
-      me.packed = (u32)(b - me.a) | (nc << 9) | (ng << 20) | 0x80000000u;
+      const bool in_range = me.c_lo >= 0 && c_hi >= me.c_lo && c_hi <= p.n_csegs && me.g_lo >= 0 && g_hi >= me.g_lo &&
+                            g_hi <= p.n_gsegs;
+      // (too many segments for the 32-bit path: none are fetched in advance)
+      const u32 nc = in_range && c_hi - me.c_lo < CAP ? (u32)(c_hi - me.c_lo) : 0u;
+      const u32 ng = in_range && g_hi - me.g_lo < CAP ? (u32)(g_hi - me.g_lo) : 0u;
+      me.packed = (u32)(b - me.a) | (nc << 9) | (ng << 20) | (in_range ? 0x80000000u : 0u);
     }
   }
   return me;

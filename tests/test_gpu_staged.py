@@ -1,7 +1,8 @@
 """Analysis of larger tasksets out of stages in shared memory against the oracle, where it can go
 wrong: sizes at the edges of the bins, arrays that start on odd elements, slices at the very ends of
-their arrays, tasksets too large for a stage, values beyond the 32-bit path, undecided tasksets that
-are kept or left to the second launch, priorities with gaps and best-effort tasks."""
+their arrays, tasksets too large for a stage, values beyond the 32-bit path, offsets out of range,
+undecided tasksets that are kept or left to the second launch, priorities with gaps and best-effort
+tasks."""
 import numpy as np
 import pytest
 
@@ -30,13 +31,16 @@ def taskset(rng, n, load, segs, gaps=False):
     return ts
 
 
-def check(tasksets, policies, shift=0, L=1024, ovh=20, fillers=FILLERS):
-    """Parity on `tasksets` at the two ends of a batch whose middle is one-task tasksets."""
+def check(tasksets, policies, shift=0, L=1024, ovh=20, fillers=FILLERS, spoil=None):
+    """Parity on `tasksets` at the two ends of a batch whose middle is one-task tasksets, after
+    `spoil(batch)` has changed it."""
     torch = pytest.importorskip("torch")
     half = len(tasksets) // 2
     few = batch_of([[dict(T=50, prio=1, core=0, cseg=[7])]] * 64)
     middle = TasksetBatch.concat([few] * (fillers // 64 + 1))
     batch = TasksetBatch.concat([batch_of(tasksets[:half]), middle, batch_of(tasksets[half:])])
+    if spoil:
+        spoil(batch)
     t = {}
     for f in ARRAY_FIELDS:   # the arrays start `shift` elements into an allocation of exactly their size
         room = torch.empty(getattr(batch, f).shape[0] + shift, dtype=torch.int64, device="cuda")
@@ -96,3 +100,29 @@ def test_deferred_tasksets(every):
     kinds = [taskset(rng, n, load, 2) for n in (40, 80, 130, 200, 250) for load in (0.02, 6.0)]
     tasksets = [kinds[2 * (k % 5) + (0 if k % every == 0 else 1)] for k in range(4200)]
     check(tasksets, [0, 1], fillers=8400)
+
+
+@pytest.mark.parametrize("kind", ["cseg", "gseg"])
+@pytest.mark.parametrize("where", ["below", "beyond"])
+def test_constant_offsets_out_of_range(kind, where):
+    """Tasksets without segments of one kind whose offsets of that kind are all the same value outside
+    the array: no segment is read for them, every step between two offsets is 0, and they are
+    INVALID all the same.  The segments of the other kind make them miss within the first ranks."""
+    rng = np.random.default_rng(3)
+    tasksets = []
+    for n in (33, 64, 80, 96, 120, 128, 180, 192, 200, 256) * 2:
+        ts = taskset(rng, n, 60.0, 2)
+        for tk in ts:
+            if kind == "gseg":
+                tk["gseg"] = []
+            else:
+                tk["cseg"], tk["gseg"] = [], tk["gseg"] or [(1, 5)]
+        tasksets += [ts, taskset(rng, n, 60.0, 2)]   # (the second: its own first offset is in front of it)
+
+    def spoil(batch):
+        off, total = getattr(batch, kind + "_off"), getattr(batch, kind + "_off")[-1]
+        large = np.nonzero(np.diff(batch.task_off) > 32)[0]
+        for t in large[::2]:
+            a, b = batch.task_off[t], batch.task_off[t + 1]
+            off[a:b + 1] = -3 if where == "below" else total + 5
+    check(tasksets, [0, binding.BUSY, 1, 1 | binding.BUSY], spoil=spoil)
