@@ -10,9 +10,10 @@
 // far from schedulable (the first deadline miss comes within 16 ranks for all but 0.02 % of the `large`
 // and `divergence` tasksets) that is all there is to do.  Every value of the taskset is still read and
 // range-checked.  A taskset that none of these ranks decides, or that this kernel cannot take (too
-// many segments for a stage, values beyond the 32-bit path, at the very end of an array), is marked
-// in the permutation and left to a second launch (run_deferred_bin), which needs no stages and so has
-// more warps for the recurrence.
+// many segments for a stage, values beyond the 32-bit path, at the very end of an array), takes the full
+// pass: at the end of the warp's own work while there are few, else it is marked in the permutation and
+// left to a second launch (run_deferred_bin), which needs no stages and so has more warps for the
+// recurrence.  Which of the two is staged_walk.h.
 //
 // 1,000,000 `large` tasksets (9.75 GB in and out): GCAPS 2.39 -> 1.58 ms, round robin 2.18 -> 1.52 ms
 // (6.2 and 6.4 TB/s): bound by HBM.  Before, 1,775 warp instructions per taskset and the latency of
@@ -26,12 +27,12 @@
 #include <stdint.h>
 
 #include "rta_device.cuh"
+#include "staged_walk.h"
 
 namespace {
 
 constexpr int kStagedThreads = kStagedBlockThreads;  // two warps: the number of stages per SM adapts finely
 constexpr int kHeadRanks = 16;  // two lanes per rank
-constexpr int kLeftMost = 8;    // undecided tasksets a warp keeps for its own end
 constexpr int kStagedChunk = 8;  // tasksets of one pull
 constexpr int kArrays = 9;       // period, deadline, priority, core, cseg_off, gseg_off, cseg, gm, ge
 constexpr int kHeadUndecided = 2;
@@ -51,7 +52,7 @@ template <int SLOTS>
 struct __align__(16) StagedWarp {
   Ahead ahead[2 * kStagedChunk];
   __align__(16) unsigned char rows[40 * kHeadRanks];
-  u32 left[kLeftMost];
+  u32 left[kLeftMost];  // entries of the bin
   __align__(16) u32 offset[12];  // where in the stage each array's slice starts; [9]: where all end
   __align__(16) unsigned char pos_of_rank[32 * SLOTS];
   __align__(16) unsigned long long barrier;
@@ -317,137 +318,98 @@ __device__ __forceinline__ void full_pass(const KParams &p, const Ahead me, bool
   __syncwarp();
 }
 
+// The steps of walk_staged_bin on the device.
+template <int SLOTS, int MODE>
+struct StagedSteps {
+  typedef FastLayout<32, SLOTS> Lay;
+  static constexpr int MAXN = 32 * SLOTS;
+  const KParams &p;
+  const SliceTable &tab;
+  StagedWarp<SLOTS> &w;
+  unsigned char *stage;
+  u32 stage_bytes;
+  int bin, lane;
+  unsigned int start, count, chunk;
+  bool fast_call;
+  u32 phase;
+  unsigned int asked;
+  Ahead me;
+
+  __device__ __forceinline__ unsigned int pull(unsigned int n) {
+    ask(n);
+    return answer();
+  }
+  __device__ __forceinline__ void ask(unsigned int n) {
+    asked = 0;
+    if (lane == 0) asked = atomicAdd(&p.hdr->next[bin], n);
+  }
+  __device__ __forceinline__ unsigned int answer() { return __shfl_sync(kFull, asked, 0); }
+  // lanes 0..chunk-1 each look up one taskset
+  __device__ __forceinline__ void look_up(unsigned int first, int half) {
+    if ((unsigned int)lane < chunk)
+      w.ahead[half * kStagedChunk + lane] =
+          look_up_taskset<MAXN, Lay::CAP>(p, first + lane < count ? p.perm[start + first + lane] : kNoTaskset);
+    __syncwarp();
+  }
+  __device__ __forceinline__ void take(int half, int place) { me = w.ahead[half * kStagedChunk + place]; }
+  __device__ __forceinline__ bool start_copies(int half, int place) {
+    const Ahead &coming = w.ahead[half * kStagedChunk + place];
+    return (coming.packed >> 31) != 0 && stage_taskset<SLOTS>(tab, coming, w, stage, stage_bytes, lane);
+  }
+  __device__ __forceinline__ bool wait() {
+    const bool arrived = __all_sync(kFull, barrier_wait(&w.barrier, phase));
+    if (arrived) phase ^= 1u;
+    return arrived;
+  }
+  template <class Next>
+  __device__ __forceinline__ bool head(Next next) {
+    const int how = staged_head<SLOTS, MODE>(p, me, w, stage, lane, next);
+    __syncwarp();
+    return how == kFastDone;
+  }
+  __device__ __forceinline__ void first_try(bool decided) {
+    if (lane == 0) atomicAdd(&p.hdr->first_tries[bin], decided ? 1u : 0x10001u);  // undecided | all
+  }
+  __device__ __forceinline__ bool most_undecided() const {
+    const unsigned int tries = __ldcg(&p.hdr->first_tries[bin]);
+    return (tries & 0xffffu) >= 32 && 4 * (tries >> 16) >= 3 * (tries & 0xffffu);
+  }
+  __device__ __forceinline__ void keep(int k, unsigned int entry) {
+    if (lane == 0) w.left[k] = entry;
+  }
+  // (this warp pulled the entries: no one else looks at them in this launch)
+  __device__ __forceinline__ void mark(unsigned int first, unsigned int n) {
+    if ((unsigned int)lane < n) p.perm[start + first + lane] |= kDeferred;
+  }
+  __device__ __forceinline__ void mark_kept(int k) {
+    __syncwarp();
+    mark(w.left[k], 1);
+  }
+  __device__ __forceinline__ void full_pass(int k) {
+    __syncwarp();
+    ::full_pass<SLOTS, MODE>(p, look_up_taskset<MAXN, Lay::CAP>(p, p.perm[start + w.left[k]]), fast_call,
+                             reinterpret_cast<u32 *>(stage), lane);
+  }
+  __device__ __forceinline__ void marked(unsigned int n) {
+    if (lane == 0) atomicAdd(&p.hdr->deferred[bin], n);
+  }
+};
+
 // One size bin, worked through by all warps of a persistent launch, a warp per taskset.
-//
-// Far from schedulable, a taskset ends with a miss among its first ranks, and this is the way to find
-// it; where more ranks converge, looking at the first ones alone is wasted.  Tasksets of a batch tend
-// to be alike: a warp that meets eight undecided ones in a row, or one when most warps' first taskset
-// was undecided too, marks what it pulls for the second launch (run_deferred_bin) and only tries one
-// in 256.  A few undecided ones it keeps and takes through the full pass itself when there is nothing
-// left to pull.
 template <int SLOTS, int MODE>
 __device__ __forceinline__ void run_staged_bin(const KParams &p, int bin, u32 stage_bytes, StagedWarp<SLOTS> &w,
                                                unsigned char *stage, const SliceTable &tab) {
-  typedef FastLayout<32, SLOTS> Lay;
-  constexpr int MAXN = 32 * SLOTS;
-  const int lane = threadIdx.x & 31;
-  const unsigned int start = p.hdr->bin_start[bin], count = p.hdr->bin_count[bin];
+  const unsigned int count = p.hdr->bin_count[bin];
   if (count == 0) return;
-  const bool fast_call = p.ovh < (1 << 20);
+  const int lane = threadIdx.x & 31;
   const unsigned int n_warps = gridDim.x * (kStagedThreads / 32);
-  const int chunk = count >= 32 * n_warps ? kStagedChunk : (count >= 8 * n_warps ? 4 : 1);
+  const unsigned int chunk = count >= 32 * n_warps ? kStagedChunk : (count >= 8 * n_warps ? 4 : 1);
+  const bool fast_call = p.ovh < (1 << 20);
   if (lane == 0) barrier_init(&w.barrier);
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   __syncwarp();
-
-  // lanes 0..chunk-1 each look up one taskset of a chunk and leave what they found in `slot`
-  auto look_up = [&](unsigned int first, Ahead *slot) {
-    if (lane < chunk)
-      slot[lane] = look_up_taskset<MAXN, Lay::CAP>(p, first + lane < count ? p.perm[start + first + lane] : kNoTaskset);
-    __syncwarp();
-  };
-  auto pull = [&](unsigned int n) {
-    unsigned int first = 0;
-    if (lane == 0) first = atomicAdd(&p.hdr->next[bin], n);
-    return __shfl_sync(kFull, first, 0);
-  };
-  // leaves entries [first, first + n) to the second launch (this warp pulled them: no one else looks
-  // at them in this launch)
-  unsigned int deferred = 0;
-  auto defer = [&](unsigned int first, unsigned int n) {
-    if ((unsigned int)lane < n) p.perm[start + first + lane] |= kDeferred;
-    deferred += n;
-  };
-
-  bool defer_all = !fast_call, first_one = true;
-  int undecided_run = 0, n_left = 0;
-  bool staged = false;  // the copies of the coming taskset have been started
-  u32 phase = 0;
-  auto start_copies = [&](const Ahead &me) {
-    staged = !defer_all && (me.packed >> 31) != 0 && stage_taskset<SLOTS>(tab, me, w, stage, stage_bytes, lane);
-  };
-  unsigned int first = pull(chunk);
-  if (first >= count) return;
-  int which = 0;
-  look_up(first, w.ahead);
-  start_copies(w.ahead[0]);
-  while (first < count) {
-    unsigned int nfirst = 0;
-    if (lane == 0) nfirst = atomicAdd(&p.hdr->next[bin], (unsigned int)chunk);
-    const Ahead *cur = w.ahead + which * kStagedChunk;
-    Ahead *nxt = w.ahead + (which ^ 1) * kStagedChunk;
-    const int in_chunk = count - first < (unsigned int)chunk ? (int)(count - first) : chunk;
-#pragma unroll 1
-    for (int c = 0; c < in_chunk; ++c) {
-      if (c == 1 || in_chunk == 1) {  // the next chunk's index has arrived by now
-        nfirst = __shfl_sync(kFull, nfirst, 0);
-        look_up(nfirst, nxt);
-      }
-      const Ahead me = cur[c];
-      const bool more = c + 1 < in_chunk || nfirst < count;
-      const Ahead &coming = c + 1 < in_chunk ? cur[c + 1] : nxt[0];
-      int how = kHeadUndecided;
-      if (staged) {
-        if (!barrier_wait(&w.barrier, phase)) {  // (does not happen: the copies were in bounds)
-          if (lane == 0) p.out_sched[me.t] = GCAPS_SCHED_INVALID;
-          return;
-        }
-        phase ^= 1u;
-        staged = false;
-        if (!defer_all) {
-          how = staged_head<SLOTS, MODE>(p, me, w, stage, lane, [&] {
-            if (more) start_copies(coming);
-          });
-          undecided_run = how == kFastDone ? 0 : undecided_run + 1;
-          if (first_one && lane == 0)
-            atomicAdd(&p.hdr->first_tries[bin], how == kFastDone ? 1u : 0x10001u);  // undecided | all
-          first_one = false;
-          if (undecided_run > 0) {
-            const unsigned int tries = __ldcg(&p.hdr->first_tries[bin]);
-            defer_all = undecided_run >= 8 || ((tries & 0xffffu) >= 32 && 4 * (tries >> 16) >= 3 * (tries & 0xffffu));
-          }
-        }
-      } else if (more) {
-        start_copies(coming);
-      }
-      if (how == kHeadUndecided) {
-        if (defer_all || n_left == kLeftMost) {
-          defer(first + c, 1);
-        } else {
-          if (lane == 0) w.left[n_left] = me.t;
-          n_left += 1;
-        }
-      }
-      __syncwarp();
-    }
-    first = nfirst;
-    which ^= 1;
-    if (defer_all && first < count) {
-      if (staged) {  // (what has been copied for the coming taskset is not looked at)
-        if (!barrier_wait(&w.barrier, phase)) return;
-        phase ^= 1u;
-        staged = false;
-      }
-      defer(first, count - first < (unsigned int)chunk ? count - first : chunk);
-      int k = 0;
-      do {
-        first = pull(32);
-        if (first < count) defer(first, count - first < 32u ? count - first : 32u);
-      } while (first < count && (++k < 8 || !fast_call));
-      if (first < count) first = pull(chunk);
-      if (first < count) {  // one try: if it is undecided too, the rest of its chunk is deferred again
-        look_up(first, w.ahead + which * kStagedChunk);
-        defer_all = false;
-        undecided_run = 7;
-        start_copies(w.ahead[which * kStagedChunk]);
-      }
-    }
-  }
-  if (deferred > 0 && lane == 0) atomicAdd(&p.hdr->deferred[bin], deferred);
-  u32 *const buf = reinterpret_cast<u32 *>(stage);
-#pragma unroll 1
-  for (int k = 0; k < n_left; ++k)
-    full_pass<SLOTS, MODE>(p, look_up_taskset<MAXN, Lay::CAP>(p, w.left[k]), fast_call, buf, lane);
+  StagedSteps<SLOTS, MODE> steps = {p, tab, w, stage, stage_bytes, bin, lane, p.hdr->bin_start[bin], count, chunk, fast_call, 0u, 0u, {}};
+  walk_staged_bin(steps, count, chunk, fast_call);
 }
 
 // The tasksets of a bin that its first launch marked, a warp per taskset, without stages.  Where most
