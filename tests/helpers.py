@@ -5,6 +5,7 @@ import os
 
 import numpy as np
 
+from paper_2406_05221_b200 import build
 from paper_2406_05221_b200.taskgen import TasksetBatch
 
 GOLDEN = os.path.join(os.path.dirname(os.path.abspath(__file__)), "golden")
@@ -77,3 +78,23 @@ def random_tasksets(rng, count, max_tasks=6, max_cores=3, periods=(20, 30, 40, 6
 
 def batch_of(tasksets):
     return TasksetBatch.from_tasksets(tasksets)
+
+
+def direct_most(several=False):
+    """Batches of up to this many tasksets run without a plan; `several`: sweeps, several analyses and
+    searches of GPU priorities."""
+    return build.source_constant("kDirectSweepMost" if several else "kDirectMost")
+
+
+def with_fillers(batch, several=False, middle=False):
+    """`batch` and so many one-task tasksets behind it (or in its middle) that it runs with a plan and the
+    kernels of the size bins."""
+    few = batch_of([[dict(T=50, prio=1, core=0, cseg=[7])]] * 64)
+    fillers = [few] * (max(0, direct_most(several) - batch.n_tasksets) // 64 + 1)
+    half = batch.n_tasksets // 2 if middle else batch.n_tasksets
+    return TasksetBatch.concat([batch.slice(0, half)] + fillers + [batch.slice(half, batch.n_tasksets)])
+
+
+def both_ways(batch, several=False):
+    """The batch as it is and, where that runs without a plan, with fillers behind it."""
+    return [batch] if batch.n_tasksets > direct_most(several) else [batch, with_fillers(batch, several)]

@@ -5,7 +5,7 @@ import pytest
 
 from oracle import rta
 from paper_2406_05221_b200 import binding, taskgen
-from tests.helpers import ALL_MODES, BEST_EFFORT, batch_of, parse_vectors, random_tasksets
+from tests.helpers import ALL_MODES, BEST_EFFORT, batch_of, both_ways, parse_vectors, random_tasksets
 from tests.test_oracle_best_effort import _demote
 
 torch = pytest.importorskip("torch")
@@ -20,17 +20,18 @@ def _need_gpu():
 
 
 def parity(batch, policy, L, ovh, what=""):
-    ts = binding.DeviceTasksets.from_host(batch)
-    wc = torch.full((ts.n_tasks,), binding.WCRT_INVALID, dtype=torch.int64, device="cuda")
-    sc = torch.full((max(ts.n_tasksets, 0),), binding.SCHED_INVALID, dtype=torch.uint8, device="cuda")
-    binding.rta_batch(ts, policy, L, ovh, out_wcrt=wc, out_sched=sc)
-    torch.cuda.synchronize()
     w_ref, s_ref, _ = rta.analyse(batch, policy, L, ovh)
-    wc, sc = wc.cpu().numpy(), sc.cpu().numpy()
-    bad = np.nonzero(sc != s_ref)[0]
-    assert bad.size == 0, "%s: out_sched differs at tasksets %s" % (what, bad[:5])
-    bad = np.nonzero(wc != w_ref)[0]
-    assert bad.size == 0, "%s: out_wcrt differs at %s: %s vs oracle %s" % (what, bad[:5], wc[bad[:5]], w_ref[bad[:5]])
+    for b in both_ways(batch):
+        ts = binding.DeviceTasksets.from_host(b)
+        wc = torch.full((ts.n_tasks,), binding.WCRT_INVALID, dtype=torch.int64, device="cuda")
+        sc = torch.full((max(ts.n_tasksets, 0),), binding.SCHED_INVALID, dtype=torch.uint8, device="cuda")
+        binding.rta_batch(ts, policy, L, ovh, out_wcrt=wc, out_sched=sc)
+        torch.cuda.synchronize()
+        wc, sc = wc.cpu().numpy()[:w_ref.size], sc.cpu().numpy()[:s_ref.size]
+        bad = np.nonzero(sc != s_ref)[0]
+        assert bad.size == 0, "%s: out_sched differs at tasksets %s" % (what, bad[:5])
+        bad = np.nonzero(wc != w_ref)[0]
+        assert bad.size == 0, "%s: out_wcrt differs at %s: %s vs oracle %s" % (what, bad[:5], wc[bad[:5]], w_ref[bad[:5]])
     return wc, sc
 
 
@@ -85,13 +86,14 @@ def test_sweep_entry_point_with_the_flag():
     rng = np.random.default_rng(8)
     sets, _ = _demote(random_tasksets(rng, 1500, max_tasks=12, max_cores=4, wcet_hi=8), rng)
     b = batch_of(sets)
-    ts = binding.DeviceTasksets.from_host(b)
     for policy in (0, 1, 0x101):
         Ls, ov = [2, 2, 5, 1 << 30], [0, 3, 1, 1 << 21]
-        wc, sc = binding.rta_sweep(ts, policy | BEST_EFFORT, Ls, ov)
-        torch.cuda.synchronize()
         w_ref, s_ref = rta.analyse_sweep(b, policy | BEST_EFFORT, Ls, ov)
-        assert (wc.cpu().numpy() == w_ref).all() and (sc.cpu().numpy() == s_ref).all()
+        for way in both_ways(b, several=True):
+            wc, sc = binding.rta_sweep(binding.DeviceTasksets.from_host(way), policy | BEST_EFFORT, Ls, ov)
+            torch.cuda.synchronize()
+            wc, sc = wc.cpu().numpy()[:, :w_ref.shape[1]], sc.cpu().numpy()[:, :s_ref.shape[1]]
+            assert (wc == w_ref).all() and (sc == s_ref).all()
 
 
 def test_flag_is_refused_by_the_gpu_priority_entry_point():

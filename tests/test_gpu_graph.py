@@ -29,7 +29,9 @@ def capture(fn):
     return g
 
 
-@pytest.mark.parametrize("name,count", [("pr1", 1000), ("divergence", 1500), ("large", 300)])
+# (one launch without a plan; the plan, the kernels of the size bins and what they leave over)
+@pytest.mark.parametrize("name,count", [("pr1", 1000), ("divergence", 1500), ("large", 300), ("pr1", 13000),
+                                        ("divergence", 14000), ("large_light", 13000)])
 def test_replayed_batch_call_follows_the_buffers(name, count):
     w = taskgen.WORKLOADS[name]
     b = w.generate(17, count)
@@ -57,9 +59,10 @@ def test_replayed_batch_call_follows_the_buffers(name, count):
         torch.cuda.synchronize()
 
 
-def test_replayed_sweep_and_gpu_priority_calls():
+@pytest.mark.parametrize("count", [1200, 4500])
+def test_replayed_sweep_and_gpu_priority_calls(count):
     w = taskgen.WORKLOADS["rr_model"]
-    b = w.generate(5, 1200)
+    b = w.generate(5, count)
     ts = binding.DeviceTasksets.from_host(b)
     Ls = [L for L in w.timeslices for _ in w.overheads]
     th = [t for _ in w.timeslices for t in w.overheads]

@@ -11,7 +11,8 @@ import pytest
 
 from oracle import rta
 from paper_2406_05221_b200 import binding, taskgen
-from tests.helpers import ALL_MODES, BUSY, LITERAL, batch_of, parse_vector_sets, random_tasksets
+from tests.helpers import (ALL_MODES, BUSY, LITERAL, batch_of, both_ways, parse_vector_sets, random_tasksets,
+                           with_fillers)
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -37,12 +38,14 @@ def gpu_run(batch, policy, L=1024, ovh=0):
 
 def assert_parity(batch, policy, L=1024, ovh=0, what=""):
     w_ref, s_ref, _ = rta.analyse(batch, policy, L, ovh)
-    w, s = gpu_run(batch, policy, L, ovh)
-    bad_s = np.nonzero(s != s_ref)[0]
-    assert bad_s.size == 0, "%s: out_sched differs at tasksets %s" % (what, bad_s[:5])
-    bad_w = np.nonzero(w != w_ref)[0]
-    assert bad_w.size == 0, "%s: out_wcrt differs at tasks %s: %s vs oracle %s" % (
-        what, bad_w[:5], w[bad_w[:5]], w_ref[bad_w[:5]])
+    for b in both_ways(batch):
+        w, s = gpu_run(b, policy, L, ovh)
+        w, s = w[:w_ref.size], s[:s_ref.size]
+        bad_s = np.nonzero(s != s_ref)[0]
+        assert bad_s.size == 0, "%s: out_sched differs at tasksets %s" % (what, bad_s[:5])
+        bad_w = np.nonzero(w != w_ref)[0]
+        assert bad_w.size == 0, "%s: out_wcrt differs at tasks %s: %s vs oracle %s" % (
+            what, bad_w[:5], w[bad_w[:5]], w_ref[bad_w[:5]])
     return w, s
 
 
@@ -52,8 +55,9 @@ def test_hand_derived_vectors(fixture):
     for set_name, tasks, cases in parse_vector_sets(fixture):
         b = batch_of([tasks])
         for c in cases:
-            w, s = gpu_run(b, c["policy"], c["L"], c["ovh"])
-            assert w.tolist() == c["expect"], (set_name, c["name"])
+            for way in both_ways(b):
+                w, s = gpu_run(way, c["policy"], c["L"], c["ovh"])
+                assert w[:len(tasks)].tolist() == c["expect"], (set_name, c["name"])
             assert s[0] == (1 if min(c["expect"]) >= 0 else 0), (set_name, c["name"])
 
 
@@ -178,9 +182,9 @@ def test_invalid_tasksets_are_flagged_not_trapped():
     err = binding.rta_validate(binding.DeviceTasksets.from_host(b)).cpu().numpy()
     assert err.tolist() == rta.validate(b).tolist()
     # broken offsets: the oracle and the library agree and nothing faults
-    for field, idx, val in (("task_off", 2, 9999), ("task_off", 3, -4), ("cseg_off", 2, -1),
-                            ("gseg_off", 1, 1 << 50), ("cseg_off", 5, 0)):
-        bb = copy.deepcopy(b)
+    for field, idx, val, way in [broken + (way,) for way in both_ways(b) for broken in (
+            ("task_off", 2, 9999), ("task_off", 3, -4), ("cseg_off", 2, -1), ("gseg_off", 1, 1 << 50), ("cseg_off", 5, 0))]:
+        bb = copy.deepcopy(way)
         getattr(bb, field)[idx] = val
         w_ref, s_ref, _ = rta.analyse(bb, 0, 4, 0)
         w, s = gpu_run(bb, 0, 4, 0)
@@ -274,23 +278,24 @@ def test_arrays_that_start_on_odd_8_byte_boundaries():
     start at their first element), for batches whose slices touch both ends of the arrays."""
     for name, count in (("large", 40), ("sweep", 70), ("divergence", 300), ("pr1", 1)):
         w = taskgen.WORKLOADS[name]
-        b = w.generate(11, count)
-        tens = {}
-        for f, arr in b.arrays().items():
-            for shift in (1,):
-                pad = torch.full((arr.shape[0] + 3,), (1 << 62) + 12345, dtype=torch.int64, device="cuda")
-                pad[shift:shift + arr.shape[0]] = torch.from_numpy(arr).cuda()
-                tens[f] = pad[shift:shift + arr.shape[0]]
-        ts = binding.DeviceTasksets(tens)
-        for policy in MODES4:
-            w_ref, s_ref, _ = rta.analyse(b, policy, w.timeslice_us, w.overhead_us)
-            wc, sc = binding.rta_batch(ts, policy, w.timeslice_us, w.overhead_us)
-            torch.cuda.synchronize()
-            assert (sc.cpu().numpy() == s_ref).all() and (wc.cpu().numpy() == w_ref).all(), (name, policy)
+        for b in (w.generate(11, count), with_fillers(w.generate(11, count), middle=True)):
+            tens = {}
+            for f, arr in b.arrays().items():
+                for shift in (1,):
+                    pad = torch.full((arr.shape[0] + 3,), (1 << 62) + 12345, dtype=torch.int64, device="cuda")
+                    pad[shift:shift + arr.shape[0]] = torch.from_numpy(arr).cuda()
+                    tens[f] = pad[shift:shift + arr.shape[0]]
+            ts = binding.DeviceTasksets(tens)
+            for policy in MODES4:
+                w_ref, s_ref, _ = rta.analyse(b, policy, w.timeslice_us, w.overhead_us)
+                wc, sc = binding.rta_batch(ts, policy, w.timeslice_us, w.overhead_us)
+                torch.cuda.synchronize()
+                assert (sc.cpu().numpy() == s_ref).all() and (wc.cpu().numpy() == w_ref).all(), (name, policy)
 
 
-def test_determinism_and_output_reuse():
-    b = taskgen.WORKLOADS["divergence"].generate(1000, 4000)
+@pytest.mark.parametrize("count", [4000, 14000])
+def test_determinism_and_output_reuse(count):
+    b = taskgen.WORKLOADS["divergence"].generate(1000, count)
     ts = binding.DeviceTasksets.from_host(b)
     outs = []
     for _ in range(3):

@@ -6,7 +6,7 @@ import pytest
 
 from oracle import rta
 from paper_2406_05221_b200 import binding
-from tests.helpers import BUSY, LITERAL, batch_of
+from tests.helpers import BUSY, LITERAL, batch_of, both_ways
 
 pytestmark = pytest.mark.gpu
 
@@ -35,12 +35,14 @@ def test_search_matches_oracle(n, cores):
             ts[i]["prio"] = n - r if k % 3 else 2 * (n - r)
         tasksets.append(ts)
     batch = batch_of(tasksets)
-    dev = binding.DeviceTasksets.from_host(batch)
+    nt, ns = batch.n_tasks, batch.n_tasksets
+    devs = [binding.DeviceTasksets.from_host(b) for b in both_ways(batch, several=True)]
     for flags in (0, BUSY, LITERAL, BUSY | LITERAL):
         for eps in (0, 5):
-            w, s, g = binding.rta_gpu_priority(dev, flags | binding.ASSIGN, eps)
-            torch.cuda.synchronize()
             wr, sr, gr = rta.analyse_gpu_priority(batch, flags | binding.ASSIGN, eps)
-            assert np.array_equal(w.cpu().numpy(), wr), (flags, eps)
-            assert np.array_equal(g.cpu().numpy(), gr), (flags, eps)
-            assert np.array_equal(s.cpu().numpy(), sr), (flags, eps)
+            for dev in devs:   # a warp each, then the lane groups of the size bins
+                w, s, g = binding.rta_gpu_priority(dev, flags | binding.ASSIGN, eps)
+                torch.cuda.synchronize()
+                assert np.array_equal(w.cpu().numpy()[:nt], wr), (flags, eps)
+                assert np.array_equal(g.cpu().numpy()[:nt], gr), (flags, eps)
+                assert np.array_equal(s.cpu().numpy()[:ns], sr), (flags, eps)

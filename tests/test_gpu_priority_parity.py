@@ -5,7 +5,7 @@ import pytest
 
 from oracle import rta
 from paper_2406_05221_b200 import binding, taskgen
-from tests.helpers import BUSY, LITERAL, batch_of, parse_vectors, random_tasksets
+from tests.helpers import BUSY, LITERAL, batch_of, both_ways, parse_vectors, random_tasksets
 from tests.test_oracle_gpu_priority import gp_cases
 
 torch = pytest.importorskip("torch")
@@ -30,11 +30,16 @@ def gpu_gp(batch, flags, eps, gpu_priority=None):
 
 def assert_gp_parity(batch, flags, eps, gpu_priority=None, what=""):
     w_ref, s_ref, g_ref = rta.analyse_gpu_priority(batch, flags, eps, gpu_priority=gpu_priority)
-    w, s, g = gpu_gp(batch, flags, eps, gpu_priority)
-    assert (s == s_ref).all(), what
-    assert (w == w_ref).all(), what
-    if flags & ASSIGN:
-        assert (g == g_ref).all(), what
+    for way in both_ways(batch, several=True):
+        given = gpu_priority
+        if given is not None:   # (one-task tasksets: any value)
+            given = np.concatenate([given, np.ones(way.n_tasks - batch.n_tasks, np.int64)])
+        w, s, g = gpu_gp(way, flags, eps, given)
+        w, s, g = w[:batch.n_tasks], s[:batch.n_tasksets], g[:batch.n_tasks]
+        assert (s == s_ref).all(), what
+        assert (w == w_ref).all(), what
+        if flags & ASSIGN:
+            assert (g == g_ref).all(), what
     return w, s, g
 
 

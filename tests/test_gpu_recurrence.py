@@ -7,7 +7,7 @@ import pytest
 
 from oracle import rta
 from paper_2406_05221_b200 import binding, taskgen
-from tests.helpers import ALL_MODES, batch_of
+from tests.helpers import ALL_MODES, batch_of, both_ways
 
 pytestmark = pytest.mark.gpu
 
@@ -17,19 +17,25 @@ NARROW_LIMIT = 2_796_200   # kNarrowLimit of csrc/rta_recurrence.cuh
 def check(tasksets, policies, L=1024, ovh=3):
     torch = pytest.importorskip("torch")
     batch = batch_of(tasksets)
-    ts = binding.DeviceTasksets.from_host(batch)
+    n, k = batch.n_tasks, batch.n_tasksets
+    # (with fillers: the groups of 8 and 16 lanes, the stages and the second launch; without: a warp each)
+    one = [binding.DeviceTasksets.from_host(b) for b in both_ways(batch)]
+    several = [binding.DeviceTasksets.from_host(b) for b in both_ways(batch, several=True)]
     for policy in policies:
-        wcrt, sched = binding.rta_batch(ts, policy, L, ovh)
         analysis = {0: 1, binding.BUSY: 2, 1: 4, 1 | binding.BUSY: 8}[policy & 0x101]
-        many, many_s = binding.rta_multi(ts, analysis, [L, L + 1], [ovh, 0], flags=policy & binding.LITERAL)
-        torch.cuda.synchronize()
         ref, ref_s, _ = rta.analyse(batch, policy, L, ovh)
-        assert np.array_equal(wcrt.cpu().numpy(), ref), hex(policy)
-        assert np.array_equal(sched.cpu().numpy(), ref_s), hex(policy)
-        assert np.array_equal(many[0, 0].cpu().numpy(), ref), hex(policy)
-        ref, ref_s, _ = rta.analyse(batch, policy, L + 1, 0)
-        assert np.array_equal(many[1, 0].cpu().numpy(), ref), hex(policy)
-        assert np.array_equal(many_s[1, 0].cpu().numpy(), ref_s), hex(policy)
+        for ts in one:
+            wcrt, sched = binding.rta_batch(ts, policy, L, ovh)
+            torch.cuda.synchronize()
+            assert np.array_equal(wcrt.cpu().numpy()[:n], ref), hex(policy)
+            assert np.array_equal(sched.cpu().numpy()[:k], ref_s), hex(policy)
+        ref2, ref2_s, _ = rta.analyse(batch, policy, L + 1, 0)
+        for ts in several:
+            many, many_s = binding.rta_multi(ts, analysis, [L, L + 1], [ovh, 0], flags=policy & binding.LITERAL)
+            torch.cuda.synchronize()
+            assert np.array_equal(many[0, 0].cpu().numpy()[:n], ref), hex(policy)
+            assert np.array_equal(many[1, 0].cpu().numpy()[:n], ref2), hex(policy)
+            assert np.array_equal(many_s[1, 0].cpu().numpy()[:k], ref2_s), hex(policy)
 
 
 @pytest.mark.parametrize("n", [1, 7, 8, 9, 16, 24, 25, 31, 32, 33, 64, 65, 80, 96, 97, 128, 129, 192, 255, 256])

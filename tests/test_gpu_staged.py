@@ -9,11 +9,11 @@ import pytest
 from oracle import rta
 from paper_2406_05221_b200 import binding
 from paper_2406_05221_b200.taskgen import ARRAY_FIELDS, TasksetBatch
-from tests.helpers import ALL_MODES, BEST_EFFORT, batch_of
+from tests.helpers import ALL_MODES, BEST_EFFORT, batch_of, direct_most
 
 pytestmark = pytest.mark.gpu
 
-FILLERS = 12288   # more tasksets than the path without a plan takes (kDirectMost of csrc/rta_common.cuh)
+FILLERS = direct_most()   # with these a batch is more than the path without a plan takes
 
 
 def taskset(rng, n, load, segs, gaps=False):
