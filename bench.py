@@ -40,15 +40,15 @@ ALU_PEAK_DERIVED = 148 * 128 * 1.965e9
 MAX_TASKSETS_PER_GPU = 1_000_000
 K_TERM, K_SETUP = 6, 16   # algorithmic integer lane-operations per interference term / per task
 
-def kernel_launches(tasksets, several=False):
-    """Kernels of one call on a batch: gcaps_rta_batch, or with `several` a sweep, a call for several
-    analyses of one waiting mode or a search of GPU priorities.  Small batches are one launch without a
-    plan.  Otherwise the plan takes one kernel or three; then one kernel serves the bins of up to 32
-    tasks, one each those of up to 64, 96, 128, 192 and 256, and for a single analysis two more what
-    the larger bins left over."""
-    if tasksets <= build.source_constant("kDirectSweepMost" if several else "kDirectMost"):
+def kernel_launches(tasksets, kind="one"):
+    """Kernels of one call on a batch: "one" analysis, "several" (a sweep, or analyses of one waiting
+    mode) or a "search" of GPU priorities.  Small batches are one launch without a plan.  Otherwise the
+    plan takes one kernel or three; then one kernel serves the bins of up to 32 tasks, one each those of
+    up to 64, 96, 128, 192 and 256, and for a single analysis two more, for a search one more, what
+    these left over."""
+    if tasksets <= build.source_constant("kDirectMost" if kind == "one" else "kDirectSweepMost"):
         return 1
-    return (1 if tasksets <= build.source_constant("kPlanSmall") else 3) + (6 if several else 8)
+    return (1 if tasksets <= build.source_constant("kPlanSmall") else 3) + {"one": 8, "several": 6, "search": 7}[kind]
 
 
 # DRAM bytes (read + write) per taskset of the analysis kernel on the 'large' workload, from an
@@ -617,7 +617,8 @@ def main():
             "clocks": clocks, "e2e": e2e,
             "gpu_launches": args.steps * sum(
                 len(pairs) * kernel_launches(count) if name == "one_call_per_pair" else
-                kernel_launches(count, several=name in ("gcaps+rr", "fused_sweep", "gpu_priority_search"))
+                kernel_launches(count, {"gcaps+rr": "several", "fused_sweep": "several",
+                                        "gpu_priority_search": "search"}.get(name, "one"))
                 for name in names),
             "roofline": roof, "cpu_baseline": cpu, "wall_s_timed_region": t_wall,
         }

@@ -13,9 +13,10 @@
 //
 // search_narrow does the search for tasksets whose periods all lie below kNarrowLimit: staged and
 // aggregated like the default analysis (stage_fast), bounded in packed single precision with exact
-// integer results (see rta_recurrence.cuh).  analyse_gpu_priority takes all others, and given
-// priorities: 32-bit integers while all values of a taskset are below 2^26 us, else the same loop in
-// saturating 64-bit.
+// integer results (see rta_recurrence.cuh).  All others, and given priorities, go through integers
+// (analyse_gpu_priority): 32-bit while all values of a taskset are below 2^26 us, else the same loop in
+// saturating 64-bit.  The kernels of the size bins hold only the one or the other: out of line in the
+// search's kernels, with their registers and shared memory, the integer code took up to 2.7 times as long.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -29,7 +30,6 @@ struct GpParams {
   KParams k;
   const i64 *gpu_prio_in;
   i64 *gpu_prio_out;
-  int assign;
 };
 
 // Per-taskset shared memory of a group, by position.
@@ -139,9 +139,125 @@ __device__ __forceinline__ i64 bound_of(const GpLane<S> &me, int lane, unsigned 
   }
 }
 
+// What the lane's tasks contribute, and what the group looks up by position, from the tasks' values.
 template <int LPT, int S>
-__device__ __noinline__ void analyse_gpu_priority(const GpParams &g, i64 t, GpSmem<LPT * S> &sm, int lane,
-                                     unsigned int gmask) {
+__device__ __forceinline__ void lane_values(u64 eps, bool busy, bool fits32, const u64 (&T)[S], const u64 (&D)[S],
+                                            const u64 (&A)[S], const u64 (&Ge)[S], const u64 (&Star)[S], const int (&eta)[S],
+                                            const int (&core)[S], const bool (&valid)[S], GpLane<S> &me,
+                                            GpSmem<LPT * S> &sm, int lane) {
+#pragma unroll
+  for (int s = 0; s < S; ++s) {
+    const int i = lane + LPT * s;
+    const bool gh = eta[s] > 0;
+    // Sec. 6.4: J^c_h = D_h - (C_h + G^m_h), J^g_h = D_h - G^e_h (a task whose own execution
+    // exceeds its deadline has no such slack: 0); a CPU-only tau_h has no J^c (Lemma 15)
+    const u64 Jc = (gh && D[s] > A[s]) ? D[s] - A[s] : 0, Jg = D[s] > Ge[s] ? D[s] - Ge[s] : 0;
+    me.T[s] = T[s], me.Kc[s] = Jc + T[s] - 1, me.Kg[s] = Jg + T[s] - 1;
+    me.Wc[s] = A[s] + ((gh && !busy) ? Star[s] : 0);  // Lemma 15: C_h + G^{m*}_h; Lemma 12: C_h + G^m_h
+    me.We[s] = Ge[s], me.Wes[s] = Ge[s] + Star[s];
+    me.core[s] = core[s], me.gpu[s] = gh, me.valid[s] = valid[s];
+    me.magic[s] = 0, me.shift[s] = 0;
+    if (fits32) make_reciprocal((u32)T[s], me.magic[s], me.shift[s]);
+    if (valid[s]) {
+      sm.cpu_rank[i] = (short)me.cpu_rank[s];
+      sm.by_cpu_rank[me.cpu_rank[s]] = (short)i;
+      sm.uses_gpu[i] = gh ? 1 : 0;
+      sm.base[i] = (i64)(A[s] + Ge[s] + Star[s] + ((u64)eta[s] + 1) * eps);  // C_i + G*_i + B^C_i
+      sm.D[i] = (i64)D[s];
+    }
+  }
+}
+
+// The bound of the task at position i by bound_of, in 32 bits where its values fit.
+template <int LPT, int S>
+__device__ __forceinline__ i64 bound_at(const GpLane<S> &me, const GpSmem<LPT * S> &sm, int i, const bool (&above)[S],
+                                        bool fits32, bool busy, bool literal, int lane, unsigned int gmask) {
+  const int core_i = sm.core[i], rank_i = sm.cpu_rank[i];
+  const bool gi = sm.uses_gpu[i] != 0;
+  const u64 bi = (u64)sm.base[i], Di = (u64)sm.D[i];
+  if (fits32 && bi < kFastClamp)
+    return bound_of<LPT, S, true>(me, lane, gmask, i, core_i, rank_i, gi, bi, Di, above, busy, literal);
+  return bound_of<LPT, S, false>(me, lane, gmask, i, core_i, rank_i, gi, bi, Di, above, busy, literal);
+}
+
+// The search of Sec. 5.3 in integers: levels from the lowest.  Returns GCAPS_SCHED_YES or _NO.
+template <int LPT, int S>
+__device__ __forceinline__ int search_levels(const GpParams &g, i64 a, int n, const GpLane<S> &me, const int (&core)[S],
+                                             const bool (&valid)[S], GpSmem<LPT * S> &sm, bool fits32, bool busy, bool literal,
+                                             int lane, unsigned int gmask) {
+  const KParams &p = g.k;
+  int sched = GCAPS_SCHED_YES;
+  bool unplaced[S];
+  if (lane < 8) sm.cand[lane] = 0;
+#pragma unroll
+  for (int s = 0; s < S; ++s) {
+    unplaced[s] = valid[s];
+    if (valid[s]) {
+      p.out_wcrt[a + lane + LPT * s] = GCAPS_WCRT_MISS;
+      g.gpu_prio_out[a + lane + LPT * s] = 0;
+    }
+  }
+  __syncwarp(gmask);
+  {  // the lowest CPU priority of every core starts as a candidate
+    bool lowest[S];
+#pragma unroll
+    for (int s = 0; s < S; ++s) lowest[s] = valid[s];
+    for (int q = 0; q < n; ++q) {
+      const int core_q = sm.core[q], rank_q = sm.cpu_rank[q];
+#pragma unroll
+      for (int s = 0; s < S; ++s) lowest[s] &= !(core_q == core[s] && rank_q > me.cpu_rank[s]);
+    }
+#pragma unroll
+    for (int s = 0; s < S; ++s)
+      if (lowest[s]) atomicOr(&sm.cand[me.cpu_rank[s] >> 5], 1u << (me.cpu_rank[s] & 31));
+  }
+  __syncwarp(gmask);
+  for (int level = 1; level <= n && sched == GCAPS_SCHED_YES; ++level) {
+    bool placed = false;
+    int want = n;
+    while (!placed) {  // candidates from the lowest CPU priority upwards
+      want = highest_below(sm.cand, want);
+      if (want < 0) break;
+      const int c = sm.by_cpu_rank[want];
+      // every other unplaced task above c (c itself is skipped)
+      const i64 r = bound_at<LPT, S>(me, sm, c, unplaced, fits32, busy, literal, lane, gmask);
+      if (r >= 0) {
+        placed = true;
+        const int core_c = sm.core[c];
+        int next = -1;  // the task of c's core that becomes a candidate now
+#pragma unroll
+        for (int s = 0; s < S; ++s) {
+          if (lane + LPT * s == c) {
+            unplaced[s] = false;
+            p.out_wcrt[a + c] = r;
+            g.gpu_prio_out[a + c] = (i64)level;
+          }
+          if (unplaced[s] && core[s] == core_c && me.cpu_rank[s] < want && me.cpu_rank[s] > next)
+            next = me.cpu_rank[s];
+        }
+#pragma unroll
+        for (int d = LPT / 2; d >= 1; d >>= 1) {
+          const int other = __shfl_xor_sync(gmask, next, d, LPT);
+          next = other > next ? other : next;
+        }
+        __syncwarp(gmask);
+        if (lane == 0) {
+          sm.cand[want >> 5] &= ~(1u << (want & 31));
+          if (next >= 0) sm.cand[next >> 5] |= 1u << (next & 31);
+        }
+        __syncwarp(gmask);
+      }
+    }
+    if (!placed) sched = GCAPS_SCHED_NO;
+  }
+  return sched;
+}
+
+// One taskset in integers from global memory, by a group of LPT lanes.  ASSIGN: the search, else the given
+// GPU priorities.
+template <int LPT, int S, bool ASSIGN>
+__device__ __forceinline__ void analyse_gpu_priority(const GpParams &g, i64 t, GpSmem<LPT * S> &sm, int lane,
+                                                     unsigned int gmask) {
   constexpr int MAXN = LPT * S;
   const KParams &p = g.k;
   const bool busy = (p.policy & GCAPS_RTA_BUSY) != 0, literal = (p.policy & GCAPS_RTA_LITERAL) != 0;
@@ -257,39 +373,10 @@ __device__ __noinline__ void analyse_gpu_priority(const GpParams &g, i64 t, GpSm
     }
   }
   __syncwarp(gmask);
-#pragma unroll
-  for (int s = 0; s < S; ++s) {
-    const int i = lane + LPT * s;
-    const bool gh = eta[s] > 0;
-    // Sec. 6.4: J^c_h = D_h - (C_h + G^m_h), J^g_h = D_h - G^e_h (a task whose own execution
-    // exceeds its deadline has no such slack: 0); a CPU-only tau_h has no J^c (Lemma 15)
-    const u64 Jc = (gh && D[s] > A[s]) ? D[s] - A[s] : 0, Jg = D[s] > Ge[s] ? D[s] - Ge[s] : 0;
-    me.T[s] = T[s], me.Kc[s] = Jc + T[s] - 1, me.Kg[s] = Jg + T[s] - 1;
-    me.Wc[s] = A[s] + ((gh && !busy) ? Star[s] : 0);  // Lemma 15: C_h + G^{m*}_h; Lemma 12: C_h + G^m_h
-    me.We[s] = Ge[s], me.Wes[s] = Ge[s] + Star[s];
-    me.core[s] = core[s], me.gpu[s] = gh, me.valid[s] = valid[s];
-    me.magic[s] = 0, me.shift[s] = 0;
-    if (fits32) make_reciprocal((u32)T[s], me.magic[s], me.shift[s]);
-    if (valid[s]) {
-      sm.cpu_rank[i] = (short)me.cpu_rank[s];
-      sm.by_cpu_rank[me.cpu_rank[s]] = (short)i;
-      sm.uses_gpu[i] = gh ? 1 : 0;
-      sm.base[i] = (i64)(A[s] + Ge[s] + Star[s] + ((u64)eta[s] + 1) * eps);  // C_i + G*_i + B^C_i
-      sm.D[i] = (i64)D[s];
-    }
-  }
+  lane_values<LPT, S>(eps, busy, fits32, T, D, A, Ge, Star, eta, core, valid, me, sm, lane);
   __syncwarp(gmask);
-  auto bound = [&](int i, const bool(&above)[S]) -> i64 {
-    const int core_i = sm.core[i], rank_i = sm.cpu_rank[i];
-    const bool gi = sm.uses_gpu[i] != 0;
-    const u64 bi = (u64)sm.base[i], Di = (u64)sm.D[i];
-    if (fits32 && bi < kFastClamp)
-      return bound_of<LPT, S, true>(me, lane, gmask, i, core_i, rank_i, gi, bi, Di, above, busy, literal);
-    return bound_of<LPT, S, false>(me, lane, gmask, i, core_i, rank_i, gi, bi, Di, above, busy, literal);
-  };
-
   int sched = GCAPS_SCHED_YES;
-  if (!g.assign) {
+  if constexpr (!ASSIGN) {
     // ---- the given GPU priorities ---------------------------------------------------------------
 #pragma unroll
     for (int s = 0; s < S; ++s)
@@ -330,7 +417,7 @@ __device__ __noinline__ void analyse_gpu_priority(const GpParams &g, i64 t, GpSm
       bool above[S];
 #pragma unroll
       for (int s = 0; s < S; ++s) above[s] = gpu_rank[s] < rank_i;
-      const i64 r = bound(i, above);
+      const i64 r = bound_at<LPT, S>(me, sm, i, above, fits32, busy, literal, lane, gmask);
       if (lane == 0) {
         p.out_wcrt[a + i] = r;
         if (g.gpu_prio_out) g.gpu_prio_out[a + i] = g.gpu_prio_in[a + i];
@@ -338,83 +425,62 @@ __device__ __noinline__ void analyse_gpu_priority(const GpParams &g, i64 t, GpSm
       if (r < 0) sched = GCAPS_SCHED_NO;
     }
   } else {
-    // ---- the search of Sec. 5.3: levels from the lowest ----------------------------------------
-    bool unplaced[S];
-    if (lane < 8) sm.cand[lane] = 0;
+    sched = search_levels<LPT, S>(g, a, n, me, core, valid, sm, fits32, busy, literal, lane, gmask);
+  }
+  if (lane == 0) p.out_sched[t] = (uint8_t)sched;
+  __syncwarp(gmask);
+}
+
+// The search in integers for the kernel that holds search_narrow too: from global memory (a taskset that
+// stage_fast declines), and from what stage_fast has left (one with a period of kNarrowLimit or more).
+template <int LPT, int S>
+__device__ __noinline__ void search_exact(const GpParams &g, i64 t, GpSmem<LPT * S> &sm, int lane, unsigned int gmask) {
+  analyse_gpu_priority<LPT, S, true>(g, t, sm, lane, gmask);
+}
+template <int LPT, int S>
+__device__ __noinline__ void search_wide(const GpParams &g, i64 t, i64 a, const TaskValues<S> &o, u32 *buf, int lane,
+                                         unsigned int gmask) {
+  const KParams &p = g.k;
+  const bool busy = (p.policy & GCAPS_RTA_BUSY) != 0, literal = (p.policy & GCAPS_RTA_LITERAL) != 0;
+  const Rows<LPT, S, false> rows{buf};
+  GpSmem<LPT * S> &sm = *reinterpret_cast<GpSmem<LPT * S> *>(buf);
+  u64 T[S], D[S], A[S], Ge[S], Star[S];
+  int eta[S], core[S];
+  bool valid[S];
+  GpLane<S> me;
 #pragma unroll
-    for (int s = 0; s < S; ++s) {
-      unplaced[s] = valid[s];
-      if (valid[s]) {
-        p.out_wcrt[a + lane + LPT * s] = GCAPS_WCRT_MISS;
-        g.gpu_prio_out[a + lane + LPT * s] = 0;
-      }
-    }
-    __syncwarp(gmask);
-    {  // the lowest CPU priority of every core starts as a candidate
-      bool lowest[S];
-#pragma unroll
-      for (int s = 0; s < S; ++s) lowest[s] = valid[s];
-      for (int q = 0; q < n; ++q) {
-        const int core_q = sm.core[q], rank_q = sm.cpu_rank[q];
-#pragma unroll
-        for (int s = 0; s < S; ++s) lowest[s] &= !(core_q == core[s] && rank_q > me.cpu_rank[s]);
-      }
-#pragma unroll
-      for (int s = 0; s < S; ++s)
-        if (lowest[s]) atomicOr(&sm.cand[me.cpu_rank[s] >> 5], 1u << (me.cpu_rank[s] & 31));
-    }
-    __syncwarp(gmask);
-    for (int level = 1; level <= n && sched == GCAPS_SCHED_YES; ++level) {
-      bool placed = false;
-      int want = n;
-      while (!placed) {  // candidates from the lowest CPU priority upwards
-        want = highest_below(sm.cand, want);
-        if (want < 0) break;
-        const int c = sm.by_cpu_rank[want];
-        const i64 r = bound(c, unplaced);  // every other unplaced task above c (c itself is skipped)
-        if (r >= 0) {
-          placed = true;
-          const int core_c = sm.core[c];
-          int next = -1;  // the task of c's core that becomes a candidate now
-#pragma unroll
-          for (int s = 0; s < S; ++s) {
-            if (lane + LPT * s == c) {
-              unplaced[s] = false;
-              p.out_wcrt[a + c] = r;
-              g.gpu_prio_out[a + c] = (i64)level;
-            }
-            if (unplaced[s] && core[s] == core_c && me.cpu_rank[s] < want && me.cpu_rank[s] > next)
-              next = me.cpu_rank[s];
-          }
-#pragma unroll
-          for (int d = LPT / 2; d >= 1; d >>= 1) {
-            const int other = __shfl_xor_sync(gmask, next, d, LPT);
-            next = other > next ? other : next;
-          }
-          __syncwarp(gmask);
-          if (lane == 0) {
-            sm.cand[want >> 5] &= ~(1u << (want & 31));
-            if (next >= 0) sm.cand[next >> 5] |= 1u << (next & 31);
-          }
-          __syncwarp(gmask);
-        }
-      }
-      if (!placed) sched = GCAPS_SCHED_NO;
+  for (int s = 0; s < S; ++s) {
+    valid[s] = lane + LPT * s < o.n;
+    T[s] = 2, D[s] = 1, A[s] = 0, Ge[s] = 0, Star[s] = 0, eta[s] = 0, core[s] = -1, me.cpu_rank[s] = 0;
+    if (valid[s]) {
+      const uint4 row = rows.a(o.rank[s]);
+      T[s] = o.T[s], D[s] = row.x, A[s] = o.A[s], Ge[s] = o.Ge[s], eta[s] = (int)o.eta[s], core[s] = (int)row.y;
+      Star[s] = 2 * (u64)p.ovh * (u64)o.eta[s], me.cpu_rank[s] = o.rank[s];
     }
   }
+  __syncwarp(gmask);  // (the rows are read: their place holds `sm` from here on)
+#pragma unroll
+  for (int s = 0; s < S; ++s)
+    if (valid[s]) sm.core[lane + LPT * s] = core[s];
+  lane_values<LPT, S>((u64)p.ovh, busy, true, T, D, A, Ge, Star, eta, core, valid, me, sm, lane);
+  __syncwarp(gmask);
+  const int sched = search_levels<LPT, S>(g, a, o.n, me, core, valid, sm, true, busy, literal, lane, gmask);
   if (lane == 0) p.out_sched[t] = (uint8_t)sched;
   __syncwarp(gmask);
 }
 
 // The search of Sec. 5.3 in single precision.  Called by the whole warp; its groups step from bound to
 // bound side by side and sweep until the last of them has settled.  Returns, per group, whether its
-// taskset is done (outputs written); the others are analyse_gpu_priority's.
+// taskset is done (outputs written).
 //
 // Bound by instruction issue (4,420 warp instructions per 80-task taskset of `large`, 60 % of the issue
 // slots; about 15 bounds and 43 sweeps each).  100,000 of them 1.19 -> 0.77 ms: what went are per-lane
 // loops over global memory for the sums, a quadratic loop for every core's lowest task, 64-bit state
 // and the integer form of the terms (7,230 instructions).
-template <int LPT, int S, bool BUSY, bool PREFETCH = false>
+//
+// DIRECT (a block of its own per taskset): prefetches, and searches a taskset with a longer period in
+// integers; otherwise such a taskset is declined before its segments are read.
+template <int LPT, int S, bool BUSY, bool DIRECT = false>
 __device__ __forceinline__ bool search_narrow(const GpParams &g, bool live, i64 t, i64 a, int n, u32 *buf, int lane,
                                               unsigned int gmask) {
   const KParams &p = g.k;
@@ -422,10 +488,16 @@ __device__ __forceinline__ bool search_narrow(const GpParams &g, bool live, i64 
   const u32 eps = (u32)p.ovh;
   const Rows<LPT, S, false> rows{buf};
   TaskValues<S> o;
-  if (!stage_fast<LPT, S, (S <= 3 ? S : 2), true, PREFETCH>(p, live, a, n, buf, rows, lane, gmask, false, eps, o)) return false;
-  live = o.live && o.n_narrow == o.n;
-  if (LPT == 32 ? !live : !__any_sync(kFull, live)) return false;
-  n = live ? o.n : 0;
+  if (!stage_fast<LPT, S, (S <= 3 ? S : 2), true, DIRECT, !DIRECT>(p, live, a, n, buf, rows, lane, gmask, false, eps, o)) return false;
+  live = o.live;
+  if constexpr (DIRECT) {
+    if (__any_sync(kFull, live && o.n_narrow != o.n)) {
+      const TaskValues<S> there = o;  // (in memory for the call; `o` itself stays in registers)
+      if (live) search_wide<LPT, S>(g, t, a, there, buf, lane, gmask);
+      return live;
+    }
+  }
+  n = o.n;
   // what this lane's tasks contribute as interferers; inv = 0 where there is no task
   float inv[S], Kc[S], Kg[S], Wc[S], We[S], Wes[S];
   u32 core[S], found[S];  // found: level << 23 | bound, 0 without a level
@@ -615,15 +687,14 @@ template <int LPT, int S, bool BUSY>
 __device__ __forceinline__ void run_gp_bin(const GpParams &g, int bin, u32 *warp_buf, Ahead *ahead) {
   constexpr int G = 32 / LPT, MAXN = LPT * S;  // tasksets per warp
   typedef FastLayout<LPT, S> Lay;
-  typedef GpSmem<MAXN> Sm;
-  static_assert(sizeof(Sm) <= sizeof(u32) * Lay::kWords && sizeof(u32) * Lay::kWords % 16 == 0, "the other path fits");
   const KParams &p = g.k;
   const int lane32 = threadIdx.x & 31, group = lane32 / LPT, lane = lane32 % LPT;
   const unsigned int gmask = LPT == 32 ? kFull : (((1u << LPT) - 1u) << (group * LPT));
   u32 *const buf = warp_buf + group * Lay::kWords;
   const unsigned int start = p.hdr->bin_start[bin], count = p.hdr->bin_count[bin];
   if (count == 0) return;
-  const bool fast_call = g.assign && p.ovh < (1 << 20);
+  const bool fast_call = p.ovh < (1 << 20);
+  unsigned int marked = 0;  // tasksets of this lane's group left to gpu_priority_rest_kernel
   const unsigned int n_groups = gridDim.x * (kBlockThreads / 32) * G;
   const int chunk = G * (count >= 32 * n_groups ? (G == 1 ? 8 : kMaxAhead / G) : (count >= 8 * n_groups ? 2 : 1));
   auto look_up = [&](unsigned int first, Ahead *slot) {
@@ -655,11 +726,52 @@ __device__ __forceinline__ void run_gp_bin(const GpParams &g, int bin, u32 *warp
         done = search_narrow<LPT, S, BUSY>(g, fast, (i64)me.t, me.a, (int)(me.packed & 0x1ffu), buf, lane, gmask);
       }
       __syncwarp();
-      if (have && !done) analyse_gpu_priority<LPT, S>(g, (i64)me.t, *reinterpret_cast<Sm *>(buf), lane, gmask);
+      if (have && !done && lane == 0) p.perm[start + first + c + group] |= kDeferred, marked += 1;
       __syncwarp();
     }
     first = nfirst;
     which ^= 1;
+  }
+  if (marked > 0) atomicAdd(&p.hdr->deferred[bin], marked);
+}
+
+// What run_gp_bin has marked in a bin: tasksets with a period of kNarrowLimit or more, values beyond the 32-bit
+// path, malformed ones.  Where most of the bin is marked its entries are pulled from a counter, as many as
+// the warp has groups; where few are, every warp looks through its share, 32 entries at a time.
+template <int LPT, int S>
+__device__ __forceinline__ void run_rest_bin(const GpParams &g, int bin, unsigned char *warp_smem) {
+  constexpr unsigned int G = 32 / LPT;
+  typedef GpSmem<LPT * S> Sm;
+  const KParams &p = g.k;
+  const unsigned int lane32 = threadIdx.x & 31, group = lane32 / LPT;
+  const int lane = (int)(lane32 % LPT);
+  const unsigned int gmask = LPT == 32 ? kFull : (((1u << LPT) - 1u) << (group * LPT));
+  const unsigned int start = p.hdr->bin_start[bin], count = p.hdr->bin_count[bin];
+  const unsigned int marked = count > 0 ? __ldcg(&p.hdr->deferred[bin]) : 0;
+  if (marked == 0) return;
+  const bool dense = marked >= count / 4;
+  const unsigned int n_warps = gridDim.x * (kBlockThreads / 32), step = dense ? G : 32;
+  unsigned int window = (blockIdx.x * (kBlockThreads / 32) + (threadIdx.x >> 5)) * 32;  // (!dense)
+  for (;;) {
+    unsigned int first = window;
+    if (dense) {
+      if (lane32 == 0) first = atomicAdd(&p.hdr->next2[bin], step);
+      first = __shfl_sync(kFull, first, 0);
+    }
+    window += n_warps * 32;
+    if (first >= count) break;
+    u32 t = 0;
+    if (lane32 < step && first + lane32 < count) t = __ldcg(&p.perm[start + first + lane32]);
+    unsigned int found = __ballot_sync(kFull, (t & kDeferred) != 0);
+    while (found) {  // the next G of them, one per group
+      unsigned int rest = found;
+      for (unsigned int k = 0; k < group; ++k) rest &= rest - 1;
+      const bool have = rest != 0;
+      const u32 mine = __shfl_sync(kFull, t, have ? __ffs((int)rest) - 1 : 0) & ~kDeferred;
+      if (have) analyse_gpu_priority<LPT, S, true>(g, (i64)mine, reinterpret_cast<Sm *>(warp_smem)[group], lane, gmask);
+      __syncwarp();
+      for (unsigned int k = 0; k < G; ++k) found &= found - 1;
+    }
   }
 }
 
@@ -690,8 +802,14 @@ __global__ void __launch_bounds__(kBlockThreads, gp_min_blocks(S)) gpu_priority_
 }
 
 // A batch of at most kDirectSweepMost tasksets in one launch: a block of one warp per taskset, no plan
-// (1,000 tasksets of 8 / 20 / 80 tasks: 25 / 26 / 45 us, with plan and binned kernels 39 / 59 / 66 us; 8,192
-// of 80 tasks: 147 against 132 us).
+// (1,000 tasksets of 8 / 20 / 80 tasks: 25 / 26 / 45 us, with plan and binned kernels 39 / 59 / 66 us; 4,096
+// of them: 36 / 60 / 87 against 40 / 65 / 88 us, and 313 against 250 us where all 80 tasks find a level).
+template <int S, bool BUSY>
+__device__ __forceinline__ void search_direct(const GpParams &g, bool fast, i64 t, i64 a, int n, u32 *buf, int lane) {
+  const bool done = fast && search_narrow<32, S, BUSY, true>(g, true, t, a, n, buf, lane, kFull);
+  __syncwarp();
+  if (!done) search_exact<32, S>(g, t, *reinterpret_cast<GpSmem<32 * S> *>(buf), lane, kFull);
+}
 template <bool BUSY>
 __global__ void __launch_bounds__(32) gpu_priority_direct_kernel(GpParams g) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -700,18 +818,96 @@ __global__ void __launch_bounds__(32) gpu_priority_direct_kernel(GpParams g) {
   const int lane = threadIdx.x;
   const i64 t = blockIdx.x;
   const i64 a = p.task_off[t], b = p.task_off[t + 1];
-  bool done = false;
-  if (g.assign && a >= 0 && b > a && b <= p.n_tasks && b - a <= GCAPS_RTA_MAX_TASKS && p.ovh < (1 << 20)) {
-    const int n = (int)(b - a);
-    if (n <= 32) done = search_narrow<32, 1, BUSY, true>(g, true, t, a, n, buf, lane, kFull);
-    else if (n <= 64) done = search_narrow<32, 2, BUSY, true>(g, true, t, a, n, buf, lane, kFull);
-    else if (n <= 96) done = search_narrow<32, 3, BUSY, true>(g, true, t, a, n, buf, lane, kFull);
-    else if (n <= 128) done = search_narrow<32, 4, BUSY, true>(g, true, t, a, n, buf, lane, kFull);
-    else if (n <= 192) done = search_narrow<32, 6, BUSY, true>(g, true, t, a, n, buf, lane, kFull);
-    else done = search_narrow<32, 8, BUSY, true>(g, true, t, a, n, buf, lane, kFull);
+  // (a broken range goes to the exact search of the smallest size, which finds it INVALID)
+  const bool in_range = a >= 0 && b > a && b <= p.n_tasks && b - a <= GCAPS_RTA_MAX_TASKS;
+  const bool fast = in_range && p.ovh < (1 << 20);
+  const int n = in_range ? (int)(b - a) : 0;
+  if (n <= 32) search_direct<1, BUSY>(g, fast, t, a, n, buf, lane);
+  else if (n <= 64) search_direct<2, BUSY>(g, fast, t, a, n, buf, lane);
+  else if (n <= 96) search_direct<3, BUSY>(g, fast, t, a, n, buf, lane);
+  else if (n <= 128) search_direct<4, BUSY>(g, fast, t, a, n, buf, lane);
+  else if (n <= 192) search_direct<6, BUSY>(g, fast, t, a, n, buf, lane);
+  else search_direct<8, BUSY>(g, fast, t, a, n, buf, lane);
+}
+
+// Given GPU priorities: every task is bounded once, in integers.
+template <int LPT, int S>
+__device__ __forceinline__ void run_given_bin(const GpParams &g, int bin, unsigned char *warp_smem) {
+  constexpr int G = 32 / LPT;  // tasksets per warp
+  typedef GpSmem<LPT * S> Sm;
+  const KParams &p = g.k;
+  const int lane32 = threadIdx.x & 31, group = lane32 / LPT, lane = lane32 % LPT;
+  const unsigned int gmask = LPT == 32 ? kFull : (((1u << LPT) - 1u) << (group * LPT));
+  const unsigned int start = p.hdr->bin_start[bin], count = p.hdr->bin_count[bin];
+  for (;;) {
+    unsigned int first = 0;
+    if (lane32 == 0) first = atomicAdd(&p.hdr->next[bin], (unsigned int)G);
+    first = __shfl_sync(kFull, first, 0);
+    if (first >= count) break;
+    if (first + group < count)
+      analyse_gpu_priority<LPT, S, false>(g, (i64)p.perm[start + first + group], reinterpret_cast<Sm *>(warp_smem)[group],
+                                          lane, gmask);
+    __syncwarp();
   }
-  __syncwarp();
-  if (!done) analyse_gpu_priority<32, 8>(g, t, *reinterpret_cast<GpSmem<256> *>(buf), lane, kFull);
+}
+template <int LPT, int S>
+__host__ __device__ constexpr int given_warp_bytes() {
+  return (32 / LPT) * (int)sizeof(GpSmem<LPT * S>);
+}
+constexpr int kGivenSmallWarpBytes = cmax(cmax(given_warp_bytes<16, 2>(), given_warp_bytes<8, 3>()),
+                                          cmax(given_warp_bytes<8, 2>(), given_warp_bytes<8, 1>()));
+static_assert(kGivenSmallWarpBytes % 16 == 0, "every warp's area starts 16-byte aligned");
+__global__ void __launch_bounds__(kBlockThreads) gpu_priority_given_small_kernel(GpParams g) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  let_dependents_start();
+  unsigned char *mine = smem_raw + (threadIdx.x >> 5) * kGivenSmallWarpBytes;
+  run_given_bin<16, 2>(g, 3, mine);
+  run_given_bin<8, 3>(g, 2, mine);
+  run_given_bin<8, 2>(g, 1, mine);
+  run_given_bin<8, 1>(g, 0, mine);
+  wait_for_previous_grid();
+}
+template <int S>
+__global__ void __launch_bounds__(kBlockThreads, S <= 4 ? 5 : 2) gpu_priority_given_big_kernel(GpParams g, int bin) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  let_dependents_start();
+  run_given_bin<32, S>(g, bin, smem_raw + (threadIdx.x >> 5) * given_warp_bytes<32, S>());
+  wait_for_previous_grid();
+}
+// ... of a batch of at most kDirectGivenMost tasksets, a block of one warp per taskset, without a plan: 1,000
+// tasksets of 8 / 20 / 80 / 128 tasks 24 / 27 / 113 / 196 us, with plan and binned kernels 40 / 63 / 155 / 280
+// us; 4,096 of them 36 / 72 / 359 / 615 against 53 / 86 / 274 / 508 us.
+__global__ void __launch_bounds__(32) gpu_priority_given_direct_kernel(GpParams g) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const KParams &p = g.k;
+  const int lane = threadIdx.x;
+  const i64 t = blockIdx.x, n = p.task_off[t + 1] - p.task_off[t];
+  // (a broken range is found INVALID whatever its size)
+  if (n <= 32) analyse_gpu_priority<32, 1, false>(g, t, *reinterpret_cast<GpSmem<32> *>(smem_raw), lane, kFull);
+  else if (n <= 64) analyse_gpu_priority<32, 2, false>(g, t, *reinterpret_cast<GpSmem<64> *>(smem_raw), lane, kFull);
+  else if (n <= 96) analyse_gpu_priority<32, 3, false>(g, t, *reinterpret_cast<GpSmem<96> *>(smem_raw), lane, kFull);
+  else if (n <= 128) analyse_gpu_priority<32, 4, false>(g, t, *reinterpret_cast<GpSmem<128> *>(smem_raw), lane, kFull);
+  else if (n <= 192) analyse_gpu_priority<32, 6, false>(g, t, *reinterpret_cast<GpSmem<192> *>(smem_raw), lane, kFull);
+  else analyse_gpu_priority<32, 8, false>(g, t, *reinterpret_cast<GpSmem<256> *>(smem_raw), lane, kFull);
+}
+
+// What the search's kernels have left over, largest tasksets first (100,000 tasksets of 20 tasks with periods
+// to 60 s: 572 us; out of line in those kernels 762, without the look at them first 520).
+constexpr int kRestWarpBytes = cmax(given_warp_bytes<32, 8>(), kGivenSmallWarpBytes);
+static_assert(kRestWarpBytes % 16 == 0, "every warp's area starts 16-byte aligned");
+__global__ void __launch_bounds__(kBlockThreads, 4) gpu_priority_rest_kernel(GpParams g) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  wait_for_previous_grid();  // the marks in the permutation are complete from here on
+  unsigned char *mine = smem_raw + (threadIdx.x >> 5) * kRestWarpBytes;
+  run_rest_bin<32, 8>(g, 8, mine);
+  run_rest_bin<32, 6>(g, 7, mine);
+  run_rest_bin<32, 4>(g, 6, mine);
+  run_rest_bin<32, 3>(g, 5, mine);
+  run_rest_bin<32, 2>(g, 4, mine);
+  run_rest_bin<16, 2>(g, 3, mine);
+  run_rest_bin<8, 3>(g, 2, mine);
+  run_rest_bin<8, 2>(g, 1, mine);
+  run_rest_bin<8, 1>(g, 0, mine);
 }
 
 template <int S, bool BUSY>
@@ -734,6 +930,31 @@ cudaError_t launch_gp_bins(const GpParams &g, int sm_count, cudaStream_t st) {
   if (e == cudaSuccess) e = launch_big<4, BUSY>(g, 6, sm_count, st);
   if (e == cudaSuccess) e = launch_big<6, BUSY>(g, 7, sm_count, st);
   if (e == cudaSuccess) e = launch_big<8, BUSY>(g, 8, sm_count, st);
+  static int rest_blocks_per_sm[64] = {0};
+  if (e == cudaSuccess)
+    e = launch_persistent_ex(true, gpu_priority_rest_kernel, rest_blocks_per_sm, (size_t)kRestWarpBytes * kWarps,
+                             (g.k.n_tasksets + kWarps - 1) / kWarps, sm_count, st, g);
+  return e;
+}
+
+template <int S>
+cudaError_t launch_given_big(const GpParams &g, int bin, int sm_count, cudaStream_t st) {
+  constexpr int kWarps = kBlockThreads / 32;
+  static int blocks_per_sm[64] = {0};
+  return launch_persistent_ex(true, gpu_priority_given_big_kernel<S>, blocks_per_sm, (size_t)given_warp_bytes<32, S>() * kWarps,
+                              (g.k.n_tasksets + kWarps - 1) / kWarps, sm_count, st, g, bin);
+}
+
+cudaError_t launch_given_bins(const GpParams &g, int sm_count, cudaStream_t st) {
+  constexpr int kWarps = kBlockThreads / 32;
+  static int blocks_per_sm[64] = {0};
+  cudaError_t e = launch_persistent(gpu_priority_given_small_kernel, blocks_per_sm, (size_t)kGivenSmallWarpBytes * kWarps,
+                                    (g.k.n_tasksets + kWarps - 1) / kWarps, sm_count, st, g);
+  if (e == cudaSuccess) e = launch_given_big<2>(g, 4, sm_count, st);
+  if (e == cudaSuccess) e = launch_given_big<3>(g, 5, sm_count, st);
+  if (e == cudaSuccess) e = launch_given_big<4>(g, 6, sm_count, st);
+  if (e == cudaSuccess) e = launch_given_big<6>(g, 7, sm_count, st);
+  if (e == cudaSuccess) e = launch_given_big<8>(g, 8, sm_count, st);
   return e;
 }
 
@@ -759,18 +980,20 @@ extern "C" int gcaps_rta_gpu_priority_batch(const gcaps_tasksets_t *ts, int64_t 
   fill_params(&g.k, ts, n_tasksets, policy, 1, runlist_update_us, out_wcrt, out_sched);
   g.gpu_prio_in = (const i64 *)gpu_priority;
   g.gpu_prio_out = (i64 *)out_gpu_priority;
-  g.assign = assign ? 1 : 0;
   cudaStream_t st = (cudaStream_t)stream;
-  const bool direct = n_tasksets <= kDirectSweepMost, busy = (flags & GCAPS_RTA_BUSY) != 0;
+  const bool direct = n_tasksets <= (assign ? kDirectSweepMost : kDirectGivenMost), busy = (flags & GCAPS_RTA_BUSY) != 0;
   rc = direct ? place_plan(g.k, workspace, workspace_bytes) : enqueue_plan(g.k, workspace, workspace_bytes, st);
   if (rc != GCAPS_OK) return rc;
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess && direct) {
     constexpr int smem = (int)sizeof(u32) * bin_warp_words<32, 8>();
     static_assert(sizeof(GpSmem<256>) <= (size_t)smem && smem <= 48 * 1024, "no attribute to set");
-    if (busy) gpu_priority_direct_kernel<true><<<(unsigned int)n_tasksets, 32, smem, st>>>(g);
+    if (!assign) gpu_priority_given_direct_kernel<<<(unsigned int)n_tasksets, 32, sizeof(GpSmem<256>), st>>>(g);
+    else if (busy) gpu_priority_direct_kernel<true><<<(unsigned int)n_tasksets, 32, smem, st>>>(g);
     else gpu_priority_direct_kernel<false><<<(unsigned int)n_tasksets, 32, smem, st>>>(g);
     e = cudaGetLastError();
+  } else if (e == cudaSuccess && !assign) {
+    e = launch_given_bins(g, di.sm_count, st);
   } else if (e == cudaSuccess) {
     e = busy ? launch_gp_bins<true>(g, di.sm_count, st) : launch_gp_bins<false>(g, di.sm_count, st);
   }

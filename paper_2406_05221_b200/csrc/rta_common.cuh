@@ -29,6 +29,7 @@ constexpr int kPlanSmall = 8192;  // batches up to this size are planned by one 
 constexpr int kDirectMost = 12288;  // batches up to this size run without a plan (see gcaps_rta_direct.cu)
 constexpr int kDirectSweepMost = 4096;  // the same for several analyses per taskset, and for the search of GPU
                                         // priorities
+constexpr int kDirectGivenMost = 2048;  // ... for given GPU priorities (see gcaps_gpu_priority.cu)
 constexpr u64 kClamp = 1ull << 50;  // any quantity >= 2^50 exceeds every deadline (<= 2^40)
 
 struct PlanHeader {

@@ -398,7 +398,8 @@ struct TaskValues {
 // the CPU segments whose loads are issued together.  ovh_max: the largest epsilon of a GCAPS analysis.
 // PREFETCH: the caller has not prefetched the segments; the G^m and G^e slices start their way into L2 as
 // soon as their place is known, so that they do not wait for the CPU segments' sums.
-template <int LPT, int SLOTS, int BC, bool kAnyGcaps, bool PREFETCH = false, class RowsT>
+// NARROW: a taskset with a period of kNarrowLimit or more is declined before its segments are read.
+template <int LPT, int SLOTS, int BC, bool kAnyGcaps, bool PREFETCH = false, bool NARROW = false, class RowsT>
 __device__ __forceinline__ bool stage_fast(const KParams &p, bool live, i64 a, int n, u32 *buf, const RowsT rows, int lane,
                                            unsigned int gmask, bool best_effort, u32 ovh_max, TaskValues<SLOTS> &o) {
   typedef FastLayout<LPT, SLOTS> Lay;
@@ -469,7 +470,8 @@ __device__ __forceinline__ bool stage_fast(const KParams &p, bool live, i64 a, i
                    (u32)g0[s] <= (u32)Ng);
       any_wide |= v && T[s] >= kNarrowLimit;
     }
-    live = group_all<LPT>(high == 0 && ok, gmask) && live;  // (a wide priority also lands here)
+    // (a wide priority also lands here)
+    live = group_all<LPT>(high == 0 && ok && !(NARROW && any_wide), gmask) && live;
     GCAPS_LEAVE_IF_NONE_LIVE();
     if (LPT != 32 && !live) {
 #pragma unroll

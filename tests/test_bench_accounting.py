@@ -25,7 +25,8 @@ def test_launches_follow_the_dispatch():
     one, several = build.source_constant("kDirectMost"), build.source_constant("kDirectSweepMost")
     assert [bench.kernel_launches(n) for n in (1, one, one + 1, 10 ** 6)] == [1, 1, 11, 11]
     small = build.source_constant("kPlanSmall")
-    assert [bench.kernel_launches(n, several=True) for n in (several, several + 1, small, small + 1)] == [1, 7, 7, 9]
+    assert [bench.kernel_launches(n, "several") for n in (several, several + 1, small, small + 1)] == [1, 7, 7, 9]
+    assert [bench.kernel_launches(n, "search") for n in (several, several + 1, small, small + 1)] == [1, 8, 8, 10]
     text = open(build.CUDA_SRC).read()
     body = text[text.index("cudaError_t launch_all_bins("):]
     body = body[:body.index("\n}\n")]
