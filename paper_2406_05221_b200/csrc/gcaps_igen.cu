@@ -2,8 +2,8 @@
 // GCAPS, ECRTS 2024, arXiv 2406.05221, Sec. 7.1 / Table 3) for NVIDIA B200 (sm_100a).
 //
 // The generator itself is igen.h (integer-only; the host generator compiles the same
-// definition).  gcaps_gen_count: one warp per taskset does what igen_begin defines (lane = task; the
-// random source is counter-based, so every draw's position is known without the ones before it),
+// definition).  gcaps_gen_count: one warp per taskset (for many small ones a thread) does what igen_begin
+// defines (lane = task; the random source is counter-based, so every draw's position is known without the ones before it),
 // writes the three sizes of the taskset and leaves what it drew per task (period, execution demand,
 // priority, core, GPU segments: 12 bytes per task) and the position of the
 // random stream in the workspace; three exclusive scans turn the sizes into offsets (block sums,
@@ -106,6 +106,35 @@ __device__ __forceinline__ uint64_t exp2_from(const uint64_t *table, uint64_t y)
   for (int i = kExpBits + 1; i <= IGEN_FRAC_BITS; ++i)
     if ((f >> (IGEN_FRAC_BITS - i)) & 1u) r = times_root(r, i);
   return ((r >> (61 - k)) + 1) >> 1;
+}
+
+// A thread per taskset, step by step as igen.h says.  For many small tasksets, where most lanes of a warp per
+// taskset would have no task (see thread_per_taskset).
+__global__ void __launch_bounds__(kGenThreads) gen_count_thread_kernel(igen_params_t p, i64 first, i64 count, GenSpace w) {
+  const i64 t = (i64)blockIdx.x * kGenThreads + threadIdx.x;
+  if (t >= count) return;
+  igen_state_t s;
+  igen_begin(&p, (uint64_t)(first + t), &s);
+  w.off[0][t] = s.n, w.off[1][t] = s.n_csegs, w.off[2][t] = s.n_gsegs;
+  u32 *st = w.state + t * w.state_stride;
+  st[0] = (u32)s.rng.key, st[1] = (u32)(s.rng.key >> 32);
+  st[2] = (u32)s.rng.ctr, st[3] = (u32)(s.rng.ctr >> 32);
+  for (int i = 0; i < s.n; ++i) {
+    st[4 + 3 * i] = s.T[i];
+    st[5 + 3 * i] = s.E[i];
+    st[6 + 3 * i] = (u32)s.prio[i] | ((u32)s.core[i] << 16) | ((u32)s.eta[i] << 24);
+  }
+}
+
+// A thread's chain through a taskset grows with the square of its n tasks; the throughput of a thread per
+// taskset is 1.5 (32 tasks) to 8 (4 tasks) times that of a warp per taskset.  The two take the same time
+// at about 80 n^2 tasksets: 1,000 of 4 tasks 30 / 26 us (threads / warps), 10,000 of 12 tasks 50 / 46, 30,000
+// of 20 tasks 133 / 136, 100,000 of 32 tasks 236 / 239, 250,000 of 64 tasks 993 / 877; a million of 4 / 16 /
+// 24 / 40 / 64 tasks 0.19 / 0.64 / 1.03 / 1.81 / 3.25 ms by threads, 1.57 / 1.89 / 1.98 / 3.02 / 3.42 ms by
+// warps.  Tasksets of 80 tasks are faster by warps at every count (250,000: 1.40 / 1.20 ms).
+inline bool thread_per_taskset(const igen_params_t &p, i64 count) {
+  const i64 n = max_tasks_of(p);
+  return n <= 64 && count >= 80 * n * n;
 }
 
 // Bound by instruction issue (3,790 warp instructions per `large` taskset, 70 % of the slots; the ranks are
@@ -639,15 +668,22 @@ int gcaps_gen_count(const gcaps_gen_params_t *params, int64_t first, int64_t cou
   igen_params_t p;
   memcpy(&p, params, sizeof(p));
   constexpr int kWarps = kGenThreads / 32;
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  // (once per device, before the number of resident blocks is looked up: as much shared memory as there is,
-  // 24 instead of 16 warps per SM)
-  if (e == cudaSuccess && __atomic_load_n(&g_count_blocks[dev & 63], __ATOMIC_ACQUIRE) == 0)
-    e = cudaFuncSetAttribute(gen_count_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-  if (e == cudaSuccess)
-    e = launch_persistent(gen_count_kernel, g_count_blocks, 0, (long long)((count + kWarps - 1) / kWarps), di.sm_count, st,
-                          p, (i64)first, (i64)count, w);
+  cudaError_t e = cudaSuccess;
+  if (thread_per_taskset(p, count)) {
+    gen_count_thread_kernel<<<(unsigned int)((count + kGenThreads - 1) / kGenThreads), kGenThreads, 0, st>>>(
+        p, (i64)first, (i64)count, w);
+    e = cudaGetLastError();
+  } else {
+    int dev = 0;
+    e = cudaGetDevice(&dev);
+    // (once per device, before the number of resident blocks is looked up: as much shared memory as there is,
+    // 24 instead of 16 warps per SM)
+    if (e == cudaSuccess && __atomic_load_n(&g_count_blocks[dev & 63], __ATOMIC_ACQUIRE) == 0)
+      e = cudaFuncSetAttribute(gen_count_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    if (e == cudaSuccess)
+      e = launch_persistent(gen_count_kernel, g_count_blocks, 0, (long long)((count + kWarps - 1) / kWarps), di.sm_count, st,
+                            p, (i64)first, (i64)count, w);
+  }
   if (e != cudaSuccess) {
     g_last_cuda_error = (int)e;
     return GCAPS_ERR_CUDA;
