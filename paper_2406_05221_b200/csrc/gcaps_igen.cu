@@ -493,6 +493,14 @@ __device__ __forceinline__ void split_tasks(FillWarp &w, uint64_t key, uint64_t 
                                             i64 *out, i64 *fifth, int lane) {
   u32 n_parts;
   const u32 first = warp_exclusive(parts, lane, &n_parts);
+  if (!__any_sync(kFull, parts > 1)) {  // a task's only segment takes all of it, whatever its weight
+    if (parts > 0) {
+      const u32 small = FIFTH ? total / 5u : 0u;
+      out[first] = (i64)(total - small);
+      if (FIFTH) fifth[first] = (i64)small;
+    }
+    return;
+  }
   w.spare[lane] = total - parts;
   w.draw[lane] = draw;
   w.first[lane] = (unsigned short)first;
