@@ -514,16 +514,40 @@ __device__ __forceinline__ bool stage_fast(const KParams &p, bool live, i64 a, i
     }
     dense = group_all<LPT>(dense && uniq, gmask);
     if (!dense) {  // any priorities: count the tasks that come before
+      if constexpr (PREFETCH) {
+        // out of shared memory, four at a time: 12,288 tasksets of 80 tasks under GCAPS / RR 149 / 144 -> 64 / 68 us
+        // against one after the other out of global memory, which the few warps of a small batch do not hide
+        int *const P = reinterpret_cast<int *>(Q0);
+        int r[SLOTS];
 #pragma unroll
-      for (int s = 0; s < SLOTS; ++s) {
-        const int i = lane + LPT * s;
-        int r = 0;
+        for (int s = 0; s < SLOTS; ++s) r[s] = 0, P[lane + LPT * s] = prio[s];  // (behind the end: the lowest value)
+        __syncwarp();
 #pragma unroll 1
-        for (int q = 0; q < n; ++q) {
-          const int pq = (int)p.priority[a + q];
-          r += (pq > prio[s] || (pq == prio[s] && q < i)) ? 1 : 0;
+        for (int q = 0; q < n; q += 4) {
+          const int4 y = *reinterpret_cast<const int4 *>(P + q);
+#pragma unroll
+          for (int s = 0; s < SLOTS; ++s) {
+            const int i = lane + LPT * s;
+            r[s] += (y.x > prio[s] || (y.x == prio[s] && q < i)) ? 1 : 0;
+            r[s] += (y.y > prio[s] || (y.y == prio[s] && q + 1 < i)) ? 1 : 0;
+            r[s] += (y.z > prio[s] || (y.z == prio[s] && q + 2 < i)) ? 1 : 0;
+            r[s] += (y.w > prio[s] || (y.w == prio[s] && q + 3 < i)) ? 1 : 0;
+          }
         }
-        rank[s] = i < n ? r : MAXN;
+#pragma unroll
+        for (int s = 0; s < SLOTS; ++s) rank[s] = lane + LPT * s < n ? r[s] : MAXN;
+      } else {
+#pragma unroll
+        for (int s = 0; s < SLOTS; ++s) {
+          const int i = lane + LPT * s;
+          int r = 0;
+#pragma unroll 1
+          for (int q = 0; q < n; ++q) {
+            const int pq = (int)p.priority[a + q];
+            r += (pq > prio[s] || (pq == prio[s] && q < i)) ? 1 : 0;
+          }
+          rank[s] = i < n ? r : MAXN;
+        }
       }
     }
     __syncwarp();

@@ -53,3 +53,25 @@ def test_one_analysis_without_a_plan(count):
         wr, sr, _ = rta.analyse(batch, policy, 512, 25)
         assert np.array_equal(w.cpu().numpy(), wr), hex(policy)
         assert np.array_equal(s.cpu().numpy(), sr), hex(policy)
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 4, 5, 31, 32, 33, 63, 65, 94, 97, 127, 130, 191, 194, 255, 256])
+def test_ranks_of_any_priorities(n):
+    """Priorities that are no dense numbering: ties, gaps, the ends of 32 bits."""
+    torch = pytest.importorskip("torch")
+    rng = np.random.default_rng(n)
+    kinds = ([7], [1, 2], [-(1 << 31), (1 << 31) - 1, 0], list(range(-3, 40)), [int(x) for x in rng.integers(-(1 << 31), 1 << 31, 500)])
+    sets = [[dict(T=10_000 + i, prio=int(rng.choice(kind)), core=i % 3, cseg=[int(rng.integers(0, 30000 // n + 1))], gseg=[(1, 2)] * (i % 2))
+             for i in range(n)] for kind in kinds for _ in range(2)]
+    batch = batch_of(sets)
+    ts = binding.DeviceTasksets.from_host(batch)
+    for policy in (0, 1 | binding.BUSY):
+        w, s = binding.rta_batch(ts, policy, 512, 2)
+        torch.cuda.synchronize()
+        wr, sr, _ = rta.analyse(batch, policy, 512, 2)
+        assert np.array_equal(w.cpu().numpy(), wr), hex(policy)
+        assert np.array_equal(s.cpu().numpy(), sr), hex(policy)
+    w, s, g = binding.rta_gpu_priority(ts, binding.ASSIGN, 2)
+    torch.cuda.synchronize()
+    for got, want in zip((w, s, g), rta.analyse_gpu_priority(batch, binding.ASSIGN, 2)):
+        assert np.array_equal(got.cpu().numpy(), want)
