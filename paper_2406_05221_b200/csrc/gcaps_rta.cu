@@ -339,13 +339,16 @@ int enqueue_plan(KParams &p, void *workspace, size_t workspace_bytes, cudaStream
 namespace {
 
 // The stage of a bin: room for a taskset of the bin's largest size with a tenth more segments per task
-// than the batch has on average, as long as an SM then still holds kMinStages of them.  Where the
+// than the batch has on average, as long as an SM then still holds kMinStages of them.  Four hold whatever
+// the 32-bit path takes.  (With eight, most tasksets of 256 tasks and of 192 with many segments did not fit
+// and went to the second launch: 100,000 of 256 tasks with 1 to 5 GPU segments 1,089 -> 521 us under RR and
+// 935 -> 520 us under GCAPS, 12,289 of them 385 -> 119 us.)  Where the
 // batch's mean size lies in the bin its tasksets are probably alike, and 5 % above the mean (but no
 // less than the middle of the bin) has to do: more stages, i.e. more warps, per SM count for more
 // than the few tasksets left over (80-task tasksets: 18 instead of 16 warps, 1.53 instead of 1.64 ms
 // per 1,000,000).
 constexpr size_t kSmemPerSm = 228 * 1024, kSmemPerBlockReserved = 1024 + 256;
-constexpr int kMinStages = 8;
+constexpr int kMinStages = 4;
 
 template <int SLOTS, int MODE>
 cudaError_t launch_big(const KParams &p, int bin, int sm_count, cudaStream_t st) {
