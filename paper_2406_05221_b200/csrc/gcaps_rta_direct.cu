@@ -12,8 +12,12 @@ namespace {
 // one taskset's chain of dependent loads: without the plan (a launch, and two loads in front of every
 // taskset) 1,184 tasksets of 8 / 20 / 80 tasks take 9 / 12 / 10 us of a stream's time under GCAPS, with
 // plan and one kernel over all size bins 17 / 29 / 19 us.  It stays ahead of the binned kernels while
-// these cannot fill the device: 12,000 tasksets 35 / 67 / 47 us against 45 / 68 / 77 us, 24,000
-// tasksets 66 / 127 / 90 against 49 / 85 / 90 us.
+// these cannot fill the device.  12,288 tasksets of 8 / 20 / 80 / 128 / 192 tasks take 35 / 68 / 52 / 64 / 589 us
+// under GCAPS and 39 / 31 / 55 / 68 / 70 us under RR against 44 / 66 / 79 / 92 / 876 and 45 / 50 / 76 / 91 / 102 us
+// with a plan (busy-waiting modes within 10 % of these); 24,000 of 8 / 20 / 80 tasks 66 / 127 / 90 against
+// 49 / 85 / 90 us.  A mixture of 4 to 192 tasks: 95 against 120 us under GCAPS, but 114 against 91 us under RR,
+// whose line would lie at 9,000 tasksets; no argument of a call tells a mixture.  (Shared memory is set aside
+// for 256 tasks, which leaves 13 warps per SM.)
 constexpr int kDirectWords = bin_warp_words<32, 8>();
 template <int SLOTS, int MODE>
 __device__ __forceinline__ int direct_pass(const KParams &p, i64 t, i64 a, int n, u32 *buf, int lane) {

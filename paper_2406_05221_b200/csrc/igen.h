@@ -1,7 +1,7 @@
 /*
  * igen.h -- the integer-only taskset generator: the definition, as the host generator runs it
  * (gcc), and the draws and arithmetic that the on-device generator (nvcc) shares with it.  The
- * device takes the same steps with a warp per taskset (gcaps_igen.cu).
+ * device takes the same steps with a warp per taskset, or igen_begin() in a thread (gcaps_igen.cu).
  *
  * It follows the generation procedure of the paper's Sec. 7.1 / Table 3 like the floating-point
  * host generator (taskgen.c) does -- tasks per CPU, utilisation per CPU split over its tasks,
@@ -31,6 +31,7 @@
 #else
 #define IGEN_FN static inline
 #endif
+#define IGEN_HOST_FN static inline /* the device splits with a lane per segment (gcaps_igen.cu) */
 
 #define IGEN_MAX_TASKS 256
 #define IGEN_MAX_CORES 64
@@ -163,7 +164,7 @@ IGEN_FN uint64_t igen_exp2(uint64_t y) {
  * weights in [1,2); the last part takes the rounding remainder.  With `fifth` given, a fifth of
  * every part (rounded down) goes there and the rest to `out`.  The weights are drawn twice (once
  * for their sum, once to use them: the random source is counter-based) instead of being kept. */
-IGEN_FN void igen_split(igen_rng_t *r, int64_t total, int parts, int64_t *out, int64_t *fifth) {
+IGEN_HOST_FN void igen_split(igen_rng_t *r, int64_t total, int parts, int64_t *out, int64_t *fifth) {
   const uint64_t first_draw = r->ctr;
   uint64_t ws = 0;
   for (int j = 0; j < parts; ++j) ws += (1ULL << 32) + igen_unit(r);
@@ -321,7 +322,7 @@ IGEN_FN int64_t igen_task_gpu(igen_rng_t *rng, int64_t E, int eta, uint64_t rati
 
 /* The segments of a task with execution demand E and eta GPU segments, drawn from `rng`:
  * cseg[0 .. eta], gm / ge[0 .. eta-1]. */
-IGEN_FN void igen_task_segments(igen_rng_t *rng, int64_t E, int eta, uint64_t ratio_lo,
+IGEN_HOST_FN void igen_task_segments(igen_rng_t *rng, int64_t E, int eta, uint64_t ratio_lo,
                                 uint64_t ratio_hi, int64_t *cseg, int64_t *gm, int64_t *ge) {
   const int64_t G = igen_task_gpu(rng, E, eta, ratio_lo, ratio_hi);
   if (eta > 0) igen_split(rng, G, eta, ge, gm); /* 20 % miscellaneous CPU work, 80 % pure GPU work */
@@ -329,7 +330,7 @@ IGEN_FN void igen_task_segments(igen_rng_t *rng, int64_t E, int eta, uint64_t ra
 }
 
 /* The segments of task i of the state (call for i = 0, 1, ... in order). */
-IGEN_FN void igen_segments(igen_state_t *s, int i, int64_t *cseg, int64_t *gm, int64_t *ge) {
+IGEN_HOST_FN void igen_segments(igen_state_t *s, int i, int64_t *cseg, int64_t *gm, int64_t *ge) {
   igen_task_segments(&s->rng, s->E[i], s->eta[i], s->ratio_lo, s->ratio_hi, cseg, gm, ge);
 }
 

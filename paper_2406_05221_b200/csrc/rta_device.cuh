@@ -673,7 +673,7 @@ __device__ __forceinline__ int analyse_fast(const KParams &p, bool live, i64 t, 
                                             unsigned int gmask, const SweepArgs *sw = nullptr, int q_first = 0,
                                             int q_end = GCAPS_RTA_MAX_SWEEP) {
   typedef FastLayout<LPT, SLOTS> Lay;
-  constexpr int MAXN = Lay::MAXN, CAP = Lay::CAP;
+  constexpr int MAXN = Lay::MAXN;
   // prefix blocks of the CPU segments whose loads are issued together.  Tasksets of 65..96 tasks
   // with a few GPU segments per task have 200..400 CPU segments: three blocks of 128 cover them
   // in one step where two need a second, mostly empty one (80-task tasksets: -4 % for a GCAPS

@@ -7,7 +7,7 @@ from paper_2406_05221_b200 import binding, taskgen
 
 pytestmark = pytest.mark.gpu
 
-CHUNK_TASKS = 1 << 18   # kChunkTasks of csrc/gcaps_rta.cu
+CHUNK_TASKS = 1 << 18   # the least chunk_tasks of gcaps_rta_batch_host_multi (csrc/gcaps_rta.cu)
 
 
 @pytest.mark.parametrize("workload,tasks", [("large", CHUNK_TASKS - 64), ("large", CHUNK_TASKS + 80), ("pr1", 5 * CHUNK_TASKS),
