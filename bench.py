@@ -55,10 +55,10 @@ def kernel_launches(tasksets, kind="one"):
 # ncu capture of a 131,072-taskset launch (traffic grows in proportion to the tasksets of a
 # launch).  Only reported while the kernel source is the one the counters were taken from.
 CAPTURED_TRAFFIC = {
-    "source_sha256": "d72161a2f977194ed98022d5ce4278143fd1418fff695841a09c0b0cc3b32e18",
+    "source_sha256": "972e6e00e9c56f786fcdcbe6c7a11e4093439c810413a8bbd9d999be90830c89",
     "workload": "large",
-    "bytes_per_taskset": {"gcaps": (1236099000 + 80368384) / 131072.0,
-                          "rr": (1236100000 + 80585984) / 131072.0},
+    "bytes_per_taskset": {"gcaps": (1236432000 + 80774144) / 131072.0,
+                          "rr": (1236322000 + 80674560) / 131072.0},
 }
 
 

@@ -473,8 +473,8 @@ __device__ __noinline__ void search_wide(const GpParams &g, i64 t, i64 a, const 
 // bound side by side and sweep until the last of them has settled.  Returns, per group, whether its
 // taskset is done (outputs written).
 //
-// Bound by instruction issue (4,420 warp instructions per 80-task taskset of `large`, 60 % of the issue
-// slots; about 15 bounds and 43 sweeps each).  100,000 of them 1.19 -> 0.77 ms: what went are per-lane
+// Bound by instruction issue (4,204 warp instructions per 80-task taskset of `large`, 61 % of the issue
+// slots; about 15 bounds and 43 sweeps each).  100,000 of them 1.19 -> 0.72 ms: what went are per-lane
 // loops over global memory for the sums, a quadratic loop for every core's lowest task, 64-bit state
 // and the integer form of the terms (7,230 instructions).
 //

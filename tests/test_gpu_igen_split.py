@@ -10,7 +10,7 @@ from paper_2406_05221_b200 import binding, taskgen
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("segs", [(0, 0), (0, 16), (16, 16)])
+@pytest.mark.parametrize("segs", [(0, 0), (0, 1), (1, 1), (0, 16), (16, 16)])
 @pytest.mark.parametrize("tasks", [1, 31, 32, 33, 64, 65, 256])
 def test_split_matches_the_oracle(tasks, segs):
     torch = pytest.importorskip("torch")

@@ -7,7 +7,7 @@ import numpy as np
 import pytest
 
 from oracle import rta
-from paper_2406_05221_b200 import binding
+from paper_2406_05221_b200 import binding, taskgen
 from paper_2406_05221_b200.taskgen import ARRAY_FIELDS, TasksetBatch
 from tests.helpers import ALL_MODES, BEST_EFFORT, batch_of, direct_most
 
@@ -126,3 +126,23 @@ def test_constant_offsets_out_of_range(kind, where):
             a, b = batch.task_off[t], batch.task_off[t + 1]
             off[a:b + 1] = -3 if where == "below" else total + 5
     check(tasksets, [0, binding.BUSY, 1, 1 | binding.BUSY], spoil=spoil)
+
+
+@pytest.mark.parametrize("tasks_per_core,segs,overhead", [(16, (1, 5), 50), (16, (3, 8), 50), (16, (3, 8), 2), (12, (3, 8), 5), (8, (3, 8), 5)])
+def test_stages_of_large_tasksets(tasks_per_core, segs, overhead):
+    """A batch of tasksets of one size with many segments, so that a stage takes up to a quarter of an SM's
+    shared memory; some miss among the first ranks, some later."""
+    torch = pytest.importorskip("torch")
+    params = taskgen.GenParams(seed=15, cores=(16, 16), tasks_per_core=(tasks_per_core, tasks_per_core), util_per_core=(0.02, 0.8),
+                               period_us=(1e3, 1e6), gpu_frac=0.8, gpu_segments=segs, gpu_ratio=(0.2, 0.6))
+    count = direct_most() + 37
+    ts = binding.generate_device(params, 0, count)
+    batch = TasksetBatch(**{f: ts.t[f].cpu().numpy() for f in ARRAY_FIELDS})
+    sample = np.sort(np.random.default_rng(2).choice(count, 500, replace=False))
+    part, n = batch.select(sample), 16 * tasks_per_core
+    for policy in (0, binding.BUSY, 1, 1 | binding.BUSY):
+        wcrt, sched = binding.rta_batch(ts, policy, 1024, overhead)
+        torch.cuda.synchronize()
+        ref, ref_s, _ = rta.analyse(part, policy, 1024, overhead)
+        assert np.array_equal(wcrt.cpu().numpy().reshape(count, n)[sample].reshape(-1), ref), hex(policy)
+        assert np.array_equal(sched.cpu().numpy()[sample], ref_s), hex(policy)
