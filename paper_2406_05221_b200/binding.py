@@ -59,6 +59,7 @@ class GcapsError(RuntimeError):
 
 
 _lib = None
+_cuda_devices = {}   # torch.device by index
 _raw_stream = None   # torch's accessor of the current stream's handle, where it has one
 
 
@@ -154,12 +155,16 @@ class _device_and_stream:
 
     def __enter__(self) -> int:
         import torch
+        here = torch.cuda.current_device()
+        current = _cuda_devices.get(here)
+        if current is None:
+            current = _cuda_devices[here] = torch.device("cuda", here)
+        if self.stream is None and self.dev == current:   # (asking for the type takes 0.2 us, this 0.05)
+            return torch.cuda.current_stream(here).cuda_stream if _raw_stream is None else _raw_stream(here)
         if self.dev.type != "cuda":
             raise ValueError("Expected a cuda device, but got: %s" % self.dev)
-        index = self.dev.index
-        here = torch.cuda.current_device()
-        if self.stream is None and (index is None or index == here):
-            return torch.cuda.current_stream(here).cuda_stream if _raw_stream is None else _raw_stream(here)
+        if self.stream is None and self.dev.index is None:
+            return torch.cuda.current_stream(here).cuda_stream
         self.inside = contextlib.ExitStack()
         self.inside.enter_context(torch.cuda.device(self.dev))
         st = self.stream if self.stream is not None else torch.cuda.current_stream(self.dev)
