@@ -9,7 +9,8 @@ import sys
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 CUDA_SRC = os.path.join(_HERE, "csrc", "gcaps_rta.cu")
-CUDA_SRCS = [CUDA_SRC, os.path.join(_HERE, "csrc", "gcaps_rta_direct.cu"),
+CUDA_SRCS = [CUDA_SRC, os.path.join(_HERE, "csrc", "gcaps_rta_small.cu"),
+             os.path.join(_HERE, "csrc", "gcaps_rta_direct.cu"),
              os.path.join(_HERE, "csrc", "gcaps_rta_sweep.cu"),
              os.path.join(_HERE, "csrc", "gcaps_rta_direct_sweep.cu"),
              os.path.join(_HERE, "csrc", "gcaps_gpu_priority.cu"),
@@ -19,7 +20,7 @@ CUDA_LIB = os.path.join(_HERE, "libgcaps_rta.so")
 HEADER = os.path.join(os.path.dirname(_HERE), "include", "gcaps_rta.h")
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
-              "-shared", "-Xcompiler", "-fPIC", "--threads", "7"]
+              "-shared", "-Xcompiler", "-fPIC", "--threads", "8"]
 
 
 def source_constant(name: str) -> int:

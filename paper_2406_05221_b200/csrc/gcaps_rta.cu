@@ -116,23 +116,6 @@ __global__ void __launch_bounds__(1024) plan_small_kernel(KParams p) {
   }
 }
 
-// The bins of up to 32 tasks in one persistent launch, largest tasksets first: (lanes per
-// taskset, tasks per lane) = (16,2) (8,3) (8,2) (8,1) for at most 32, 24, 16, 8 tasks, i.e. two or
-// four tasksets per warp.  (A look at the first ranks out of a stage, a warp per taskset, was slower
-// here in every form tried: 100,000 24-task tasksets under round robin 163 us against 128.)
-template <int MODE>
-__global__ void __launch_bounds__(kBlockThreads, min_blocks(3)) rta_small_kernel(KParams p) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  let_dependents_start();  // the kernel of the next size bin shares no data with this one
-  u32 *warp_buf = reinterpret_cast<u32 *>(smem_raw) + (threadIdx.x >> 5) * kSmallWarpWords;
-  Ahead *ahead = reinterpret_cast<Ahead *>(warp_buf + kSmallWarpWords - kAheadWords);
-  run_bin<16, 2, 1 << MODE>(p, 3, warp_buf, ahead);
-  run_bin<8, 3, 1 << MODE>(p, 2, warp_buf, ahead);
-  run_bin<8, 2, 1 << MODE>(p, 1, warp_buf, ahead);
-  run_bin<8, 1, 1 << MODE>(p, 0, warp_buf, ahead);
-  wait_for_previous_grid();
-}
-
 // First launch of a bin of larger tasksets: a warp per taskset, SLOTS tasks per lane.
 template <int SLOTS, int MODE>
 __global__ void __launch_bounds__(kStagedThreads, staged_min_blocks(SLOTS))
@@ -351,7 +334,6 @@ namespace {
 // less than the middle of the bin) has to do: more stages, i.e. more warps, per SM count for more
 // than the few tasksets left over (80-task tasksets: 18 instead of 16 warps, 1.53 instead of 1.64 ms
 // per 1,000,000).
-constexpr size_t kSmemPerSm = 228 * 1024, kSmemPerBlockReserved = 1024 + 256;
 constexpr int kMinStages = 4;
 
 template <int SLOTS, int MODE>
@@ -371,7 +353,7 @@ cudaError_t launch_big(const KParams &p, int bin, int sm_count, cudaStream_t st)
   size_t stage = want > (double)kMost ? kMost : ((size_t)want + 15) / 16 * 16;
   if (stage < kLeast) stage = (kLeast + 15) / 16 * 16;
   const size_t smem = kWarps * (kFixed + stage);
-  return launch_staged(rta_big_kernel<SLOTS, MODE>, blocks_by_registers, kWarps * (kFixed + kMost), smem,
+  return launch_staged<kStagedThreads>(true, rta_big_kernel<SLOTS, MODE>, blocks_by_registers, kWarps * (kFixed + kMost), smem,
                        kSmemPerSm / (smem + kSmemPerBlockReserved), (p.n_tasksets + kWarps - 1) / kWarps, sm_count, st, p,
                        bin, (u32)stage);
 }
@@ -387,11 +369,7 @@ cudaError_t launch_deferred(const KParams &p, int sm_count, cudaStream_t st) {
 
 template <int MODE>
 cudaError_t launch_all_bins(const KParams &p, int sm_count, cudaStream_t st) {
-  constexpr int kWarps = kBlockThreads / 32;
-  static int blocks_per_sm[64] = {0};
-  const size_t smem = sizeof(u32) * kSmallWarpWords * kWarps;
-  cudaError_t e = launch_persistent(rta_small_kernel<MODE>, blocks_per_sm, smem,
-                                    (p.n_tasksets + kWarps - 1) / kWarps, sm_count, st, p);
+  cudaError_t e = launch_small(MODE, p, 0, sm_count, st);
   if (e == cudaSuccess) e = launch_big<2, MODE>(p, 4, sm_count, st);
   if (e == cudaSuccess) e = launch_big<3, MODE>(p, 5, sm_count, st);
   if (e == cudaSuccess) e = launch_big<4, MODE>(p, 6, sm_count, st);
@@ -414,9 +392,14 @@ int enqueue_batch(KParams p, void *workspace, size_t workspace_bytes, int sm_cou
   const bool direct = p.n_tasksets <= (sw ? kDirectSweepMost : kDirectMost);
   const int rc = place_plan(p, workspace, workspace_bytes);
   if (rc != GCAPS_OK) return rc;
-  if (!direct) enqueue_plan_kernels(p, st);
+  const int rows = direct || sw ? 0 : tile_rows(1 << mode, 1, p.ovh, p);
+  if (!direct && rows == 0) enqueue_plan_kernels(p, st);
   cudaError_t e = cudaGetLastError();
-  if (e == cudaSuccess && sw) {
+  if (e == cudaSuccess && rows > 0) {
+    e = cudaMemsetAsync(p.hdr, 0, sizeof(PlanHeader), st);
+    if (e == cudaSuccess) e = launch_small(mode, p, rows, sm_count, st);
+    if (e == cudaSuccess) e = launch_listed_tasksets(mode, p, sm_count, st);
+  } else if (e == cudaSuccess && sw) {
     SweepArgs set = *sw;
     set.block_stride = __builtin_popcount(analyses);
     for (int m = 0, k = 0; m < 4; ++m) {

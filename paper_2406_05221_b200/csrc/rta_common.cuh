@@ -42,6 +42,8 @@ struct PlanHeader {
   // the first ranks did not decide (high half)
   unsigned int first_tries[kNumBins];
 };
+// bins that list what tiles leave over (rta_tile.cuh)
+constexpr int kRestSmall = 2, kRestLarge = 8;
 constexpr unsigned int kDeferred = 0x80000000u;  // in a permutation entry: left to the second launch
 static_assert(sizeof(PlanHeader) <= 256, "header layout");
 
@@ -183,6 +185,8 @@ __device__ __forceinline__ void wait_for_previous_grid() {
 // programmatic stream serialisation and fills the SMs as that one's blocks leave instead of
 // waiting for its last block.  It needs nothing that kernel writes, and it must end with
 // wait_for_previous_grid().
+constexpr size_t kSmemPerSm = 228 * 1024, kSmemPerBlockReserved = 1024 + 256;
+
 extern std::mutex g_init_mutex;  // guards the once-per-device set-up steps of the library
 
 template <typename... Args>
@@ -222,8 +226,8 @@ cudaError_t launch_persistent_ex(bool overlap_previous, void (*kernel)(Args...),
 
 // The same for a kernel whose shared memory varies from call to call (at most `most_smem`):
 // `by_smem` blocks fit an SM by shared memory, the limit by registers is looked up once.
-template <typename... Args>
-cudaError_t launch_staged(void (*kernel)(Args...), int *by_registers, size_t most_smem, size_t smem, size_t by_smem,
+template <int THREADS, typename... Args>
+cudaError_t launch_staged(bool overlap_previous, void (*kernel)(Args...), int *by_registers, size_t most_smem, size_t smem, size_t by_smem,
                           long long want, int sm_count, cudaStream_t st, Args... args) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -237,7 +241,7 @@ cudaError_t launch_staged(void (*kernel)(Args...), int *by_registers, size_t mos
     e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
     if (e != cudaSuccess) return e;
     int per_sm = 1;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kStagedBlockThreads, 0);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, THREADS, 0);
     if (e != cudaSuccess) return e;
     resident = per_sm < 1 ? 1 : per_sm;
     __atomic_store_n(&by_registers[dev], resident, __ATOMIC_RELEASE);
@@ -247,11 +251,11 @@ cudaError_t launch_staged(void (*kernel)(Args...), int *by_registers, size_t mos
   if (grid > want) grid = want;
   if (grid < 1) grid = 1;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned int)grid), cfg.blockDim = dim3(kStagedBlockThreads);
+  cfg.gridDim = dim3((unsigned int)grid), cfg.blockDim = dim3(THREADS);
   cfg.dynamicSmemBytes = smem, cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[0].val.programmaticStreamSerializationAllowed = overlap_previous ? 1 : 0;
   cfg.attrs = attr, cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
@@ -278,6 +282,14 @@ void fill_params(KParams *p, const gcaps_tasksets_t *ts, int64_t n_tasksets, int
 // permutation of the taskset indices, zeroed work counters).  GCAPS_OK or GCAPS_ERR_WORKSPACE.
 int place_plan(KParams &p, void *workspace, size_t workspace_bytes);  // only the first part
 int enqueue_plan(KParams &p, void *workspace, size_t workspace_bytes, cudaStream_t st);
+// The rows that tiles of this batch need, or 0: no tiles (`analyses`: those of the call, `walks` of them per taskset).
+int tile_rows(int analyses, int walks, i64 max_ovh, const KParams &p);
+// rows 0: the first launch of a call with a plan, over the bins of up to 32 tasks.  Else tiles over the whole batch,
+// without a plan (the header is zero), and the first of the two launches that take what tiles leave over.  Defined in
+// gcaps_rta_small.cu.
+cudaError_t launch_small(int mode, const KParams &p, int rows, int sm_count, cudaStream_t st);
+// The second of them; defined in gcaps_rta_direct.cu.
+cudaError_t launch_listed_tasksets(int mode, const KParams &p, int sm_count, cudaStream_t st);
 // One launch for analysis `mode` (0 GCAPS self-suspension, 1 GCAPS busy-waiting, 2 RR self-suspension, 3 RR
 // busy-waiting) without a plan, a block of one warp per taskset, for batches of at most kDirectMost
 // tasksets; defined in gcaps_rta_direct.cu.
