@@ -387,17 +387,26 @@ cudaError_t launch_all_bins(const KParams &p, int sm_count, cudaStream_t st) {
 int enqueue_batch(KParams p, void *workspace, size_t workspace_bytes, int sm_count, cudaStream_t st,
                   const SweepArgs *sw = nullptr, int analyses = 0) {
   if (p.n_tasksets == 0) return GCAPS_OK;
+  if (sw && sw->n == 1 && (analyses & (analyses - 1)) == 0 && p.out_wcrt && p.n_tasksets > kDirectSweepMost) {
+    // one analysis once is what the kernels of a single analysis do
+    p.policy = (p.policy & ~(0xff | GCAPS_RTA_BUSY)) | (analyses >= 4 ? GCAPS_POLICY_RR : GCAPS_POLICY_GCAPS) |
+               ((analyses & 10) ? GCAPS_RTA_BUSY : 0);
+    sw = nullptr;
+  }
   const bool rr = (p.policy & 0xff) == GCAPS_POLICY_RR, busy = (p.policy & GCAPS_RTA_BUSY) != 0;
   const int mode = (rr ? 2 : 0) + (busy ? 1 : 0);
   const bool direct = p.n_tasksets <= (sw ? kDirectSweepMost : kDirectMost);
   const int rc = place_plan(p, workspace, workspace_bytes);
   if (rc != GCAPS_OK) return rc;
-  const int rows = direct || sw ? 0 : tile_rows(1 << mode, 1, p.ovh, p);
+  // walks of a taskset through the recurrence that a tile's lanes share.  (A single one of GCAPS and of RR each is better
+  // left to the groups of lanes, which stage once for both: 288 us for 100,001 tasksets of 20 tasks, 323 in tiles.)
+  const int walks = sw ? sw->n * (((analyses & 3) == 3 || (analyses & 12) == 12) ? 2 : 1) : 1;
+  const int rows = direct || (sw && walks == 1) ? 0 : tile_rows(sw ? analyses : 1 << mode, walks, sw ? sw->max_ovh : p.ovh, p);
   if (!direct && rows == 0) enqueue_plan_kernels(p, st);
   cudaError_t e = cudaGetLastError();
-  if (e == cudaSuccess && rows > 0) {
-    e = cudaMemsetAsync(p.hdr, 0, sizeof(PlanHeader), st);
-    if (e == cudaSuccess) e = launch_small(mode, p, rows, sm_count, st);
+  if (e == cudaSuccess && rows > 0) e = cudaMemsetAsync(p.hdr, 0, sizeof(PlanHeader), st);
+  if (e == cudaSuccess && rows > 0 && !sw) {
+    e = launch_small(mode, p, rows, sm_count, st);
     if (e == cudaSuccess) e = launch_listed_tasksets(mode, p, sm_count, st);
   } else if (e == cudaSuccess && sw) {
     SweepArgs set = *sw;
@@ -407,13 +416,20 @@ int enqueue_batch(KParams p, void *workspace, size_t workspace_bytes, int sm_cou
       k += (analyses >> m) & 1;
     }
     bool first = true;
+    if (rows > 0) {
+      set.enabled = analyses;
+      e = walks > 2 ? launch_tile_q4(p, set, rows, sm_count, st) : launch_tile_q2(p, set, rows, sm_count, st);
+    }
     for (int half = 0; half < 2 && e == cudaSuccess; ++half) {
       set.enabled = analyses & (half == 0 ? 5 : 10);
       if (set.enabled == 0) continue;
       if (!first && !direct) e = cudaMemsetAsync(p.hdr->next, 0, sizeof(p.hdr->next), st);
       first = false;
       if (e == cudaSuccess)
-        e = direct ? launch_sweep_one_warp_each(p, set, sm_count, st) : launch_sweep_set(p, set, sm_count, st);
+        e = direct     ? launch_sweep_one_warp_each(p, set, sm_count, st)
+            : rows > 0 ? launch_sweep_rest(p, set, sm_count, st)
+                       : launch_sweep_set(p, set, sm_count, st);
+      if (e == cudaSuccess && rows > 0) e = launch_sweep_listed(p, set, sm_count, st);
     }
   } else if (e == cudaSuccess) {
     if (direct) e = launch_one_warp_each(mode, p, st);

@@ -35,7 +35,8 @@ __global__ void __launch_bounds__(kTileThreads, MODE < 2 ? 9 : 12) rta_tile_kern
   const bool literal = (p.policy & GCAPS_RTA_LITERAL) != 0;
   auto walk = [&](const TileLane &me) -> bool {
     int n_rt, n_gpu;
-    const bool fits = tile_order(rows, me.n, (p.policy & GCAPS_RTA_BEST_EFFORT) != 0, n_rt, n_gpu);
+    const bool few = tile_order(rows, me.n, (p.policy & GCAPS_RTA_BEST_EFFORT) != 0, n_rt, n_gpu);
+    const bool fits = tile_worth(me.n > 0, few);
     const int n = fits ? me.n : 0;
     rows.clear();
     if (MODE >= 2) {
@@ -81,12 +82,15 @@ namespace gcaps_detail {
 // us in bins).  Under GCAPS a tile's walk is long, so there have to be enough tiles to go round: 12 tasks 43 / 54 us (tiles /
 // bins) at 12,500 tasksets and 63 / 84 at 50,000, 16 tasks 71 / 69 at 25,000 and 79 / 83 at 35,000, 20 tasks 91 / 84
 // and 97 / 105, 24 tasks 127 / 123 at 35,000 and 128 / 157 at 50,000.  Under RR tiles are the faster way from the start
-// (24 tasks 40 / 51 us at 12,500).  32 tasks: 575 / 521 us per 100,000, as a tile then takes 40 KB.
+// (24 tasks 40 / 51 us at 12,500).  Several analyses under GCAPS, 20 tasks: 170 / 138 us for five pairs of 10,000
+// tasksets, 243 / 240 of 20,000, 212 / 280 for three pairs of 50,000; 24 tasks: 203 / 182 for two pairs of 30,000, 578 / 654 for
+// 25 pairs of 5,000.  32 tasks: 575 / 521 us per 100,000, as a tile then takes 40 KB.
 int tile_rows(int analyses, int walks, i64 max_ovh, const KParams &p) {
   if (max_ovh >= (1 << 20) || ((analyses & 2) && (p.policy & GCAPS_RTA_LITERAL))) return 0;
   if (p.n_tasks % p.n_tasksets != 0 || p.n_tasks > 24 * p.n_tasksets) return 0;
   const int n = (int)(p.n_tasks / p.n_tasksets);
   if (walks == 1 && (analyses & 3) && n > 12 && p.n_tasksets < 1750 * n) return 0;
+  if (walks > 1 && (analyses & 12) == 0 && n > 12 && p.n_tasksets * walks < 100000) return 0;
   return n < 4 ? 4 : n;
 }
 

@@ -1,0 +1,13 @@
+// gcaps_rta_tile_q4.cu -- tiles whose tasksets have 4 lanes each, one per analysis and (timeslice, overhead) pair.
+#include "rta_device.cuh"
+#include "rta_tile_kept.cuh"
+
+namespace gcaps_detail {
+
+cudaError_t launch_tile_q4(const KParams &p, const SweepArgs &sw, int rows, int sm_count, cudaStream_t st) {
+  if ((sw.enabled & 12) == 0) return launch_kept<kKindGcaps, 4>(p, sw, rows, sm_count, st);
+  if ((sw.enabled & 3) == 0) return launch_kept<kKindRr, 4>(p, sw, rows, sm_count, st);
+  return launch_kept<kKindGcaps | kKindRr, 4>(p, sw, rows, sm_count, st);
+}
+
+}  // namespace gcaps_detail

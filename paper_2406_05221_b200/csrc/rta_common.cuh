@@ -297,6 +297,13 @@ cudaError_t launch_one_warp_each(int mode, const KParams &p, cudaStream_t st);
 // Launches over all size bins for the analyses sw.enabled names (bit m = mode m; one of 1, 2, 4, 8,
 // 5, 10) under every pair of `sw`; defined in gcaps_rta_sweep.cu.
 cudaError_t launch_sweep_set(const KParams &p, const SweepArgs &sw, int sm_count, cudaStream_t st);
+// The tasksets of up to 32 tasks under all analyses of sw.enabled in tiles with room for `rows` ranks, two or four lanes
+// per taskset; defined in gcaps_rta_tile_q2.cu and gcaps_rta_tile_q4.cu.  The two launches that take what they leave over, for the
+// analyses sw.enabled names there.
+cudaError_t launch_tile_q2(const KParams &p, const SweepArgs &sw, int rows, int sm_count, cudaStream_t st);
+cudaError_t launch_tile_q4(const KParams &p, const SweepArgs &sw, int rows, int sm_count, cudaStream_t st);
+cudaError_t launch_sweep_rest(const KParams &p, const SweepArgs &sw, int sm_count, cudaStream_t st);
+cudaError_t launch_sweep_listed(const KParams &p, const SweepArgs &sw, int sm_count, cudaStream_t st);
 // The same for at most kDirectSweepMost tasksets in one launch without a plan; defined in
 // gcaps_rta_direct_sweep.cu.
 cudaError_t launch_sweep_one_warp_each(const KParams &p, const SweepArgs &sw, int sm_count, cudaStream_t st);

@@ -31,7 +31,7 @@ namespace {
 constexpr int kTileThreads = 32;
 constexpr int kTileSweeps = 4096;  // sweeps of a rank after which a taskset is left over
 constexpr int kTileCores = 16;     // cores are 0 .. kTileCores-1
-constexpr int kTileOnCore = 8;     // tasks of a core, at most: a walk holds six of them in registers
+constexpr int kTileOnCore = 10;    // a walk is good for that many tasks of a core: it holds six of them in registers
 constexpr int kTileGroup = 8;      // lanes per taskset in the stage
 
 constexpr int kTileStride = 33;  // columns of a row: one more than tasksets, as the stage writes them with lanes at
@@ -252,7 +252,7 @@ __device__ __forceinline__ void tile_stage(const KParams &p, const Rows &rows, T
   }
 }
 
-// The order of this lane's taskset: by priority desc, position asc.  False if a core has more tasks than a walk is good for.
+// The order of this lane's taskset: by priority desc, position asc.  False if a core has more than kTileOnCore tasks.
 template <class Rows>
 __device__ __forceinline__ bool tile_order(const Rows &rows, int n, bool best_effort, int &n_rt, int &n_gpu) {
   int pmax = (int)0x80000000;
@@ -450,6 +450,14 @@ __device__ __forceinline__ int tile_walk(const Rows &rows, float ovh, bool liter
   if (kGcaps && out)
     for (int r = ended; r < n; ++r) out[rows.order(r)] = r < n_rt ? GCAPS_WCRT_SKIPPED : GCAPS_WCRT_BEST_EFFORT;
   return how;
+}
+
+// Whether the walks of a tile are worth while: not if three quarters of its tasksets have more tasks on a core than
+// a walk is good for (60,000 tasksets of 16 tasks on one core 162 us, 110 in groups of lanes; 20 on two cores 134 and 144,
+// 24 on two 171 and 162).  A few such tasksets in a tile (worst fit
+// leaves one core with ten small tasks now and then) are no reason to start the launches behind, 25 us for any.
+__device__ __forceinline__ bool tile_worth(bool taken, bool fits) {
+  return 4 * __popc(__ballot_sync(kFull, taken && !fits)) < 3 * __popc(__ballot_sync(kFull, taken));
 }
 
 // Under round robin most tasks lie behind a miss: the results of the whole tile start as sentinels, which takes few
