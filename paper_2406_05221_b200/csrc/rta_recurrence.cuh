@@ -163,10 +163,13 @@ __device__ __forceinline__ Outcome recurrence_narrow(const RowsT rows, int n_f, 
   out.n_done = n_f, out.verdict = 0;
   // by slot: 1/T, the two dividends' constants, the weights, the core
   float inv[SLOTS], Ja[SLOTS], Jb[SLOTS], Wa[SLOTS], Wb[SLOTS], Wc[SLOTS];
+  f32x2 inv2[SLOTS], J2s[SLOTS];  // MODE 0: (1/T, 1/T) and (J^c, J^g), as the sweeps take them
   u32 core[SLOTS];
 #pragma unroll
-  for (int s = 0; s < SLOTS; ++s)
+  for (int s = 0; s < SLOTS; ++s) {
     inv[s] = Ja[s] = Jb[s] = Wa[s] = Wb[s] = Wc[s] = 0.0f, core[s] = 0xffffffffu;
+    inv2[s] = J2s[s] = pack2(0.0f, 0.0f);
+  }
   const f32x2 two23 = pack2(kTwo23, kTwo23), minus23 = pack2(-kTwo23, -kTwo23);
   const float ovh_f = (float)pc.ovh;
   const float slot_f = pc.slot_cost >= kFastClamp ? (float)kFastClamp : (float)(u32)pc.slot_cost;
@@ -237,10 +240,11 @@ __device__ __forceinline__ Outcome recurrence_narrow(const RowsT rows, int n_f, 
       if (MODE == 0) {
 #pragma unroll
         for (int s = 0; s <= blk; ++s) {
+          // Lemma 15, jitter J^c; Lemma 13 (same core | other cores), jitter J^g.  Only the weights depend on the task
+          // under analysis
           const bool same = core[s] == core_i;
-          // Lemma 15 | Lemma 13 (other cores); Lemma 13 (same core), jitter J^g
-          const float w1 = same ? Wa[s] : (gi ? Wb[s] : 0.0f), w2 = (same && gi) ? Wc[s] : 0.0f;
-          I2[s] = pack2(inv[s], inv[s]), J2[s] = pack2(same ? Ja[s] : Jb[s], Jb[s]), W2[s] = pack2(w1, w2);
+          const float wg = same ? Wc[s] : Wb[s];
+          I2[s] = inv2[s], J2[s] = J2s[s], W2[s] = pack2(same ? Wa[s] : 0.0f, gi ? wg : 0.0f);
         }
       } else {
         float j[SLOTS + 1], w[SLOTS + 1], d[SLOTS + 1];
@@ -346,7 +350,7 @@ __device__ __forceinline__ Outcome recurrence_narrow(const RowsT rows, int n_f, 
           const float t = (T - 0.5f) - kTwo23, Rp = R - kTwo23;
           inv[blk] = __uint_as_float(fa.z), core[blk] = core_i;
           if (MODE == 0) {
-            Ja[blk] = gi ? (Rp - A) + t : t, Jb[blk] = (Rp - Ge) + t;
+            inv2[blk] = pack2(inv[blk], inv[blk]), J2s[blk] = pack2(gi ? (Rp - A) + t : t, (Rp - Ge) + t);
             Wa[blk] = A + S;      // Lemma 15: C_h, or C_h + G^{m*}_h (S = 0 for a CPU-only task)
             Wb[blk] = Ge + S;     // Lemma 13, other cores: G^{e*}_h
             Wc[blk] = Ge;
