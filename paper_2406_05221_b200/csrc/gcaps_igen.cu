@@ -48,7 +48,10 @@ __host__ __device__ inline i64 max_tasks_of(const igen_params_t &p) {
 __host__ __device__ inline i64 scan_blocks(i64 count) { return (count + kScanItems - 1) / kScanItems; }
 
 // ---- the per-task part of the generator, a warp per taskset -----------------------------------------
-constexpr int kExpBits = 10;  // leading bits of the fraction that 2^y looks up
+struct CountTables {
+  igen_exp2_tables_t exp2;
+  uint64_t inverse[IGEN_MAX_TASKS + 1];  // floor((2^64 - 1) / d)
+};
 
 // Shared memory of one warp of the count kernel.
 struct CountWarp {
@@ -79,33 +82,38 @@ __device__ __forceinline__ uint64_t draw_at(uint64_t key, u32 position) {  // th
   return igen_u64(&r);
 }
 
-// x mod d for 0 < d < 2^16, in 32-bit steps
-__device__ __forceinline__ u32 mod_small(uint64_t x, u32 d) {
-  u32 r = (u32)(x >> 32) % d;
-  r = ((r << 16) | (u32)(x >> 16 & 0xffffu)) % d;
-  return ((r << 16) | (u32)(x & 0xffffu)) % d;
+// x mod d with inverse = floor((2^64 - 1) / d): the quotient umulhi(x, inverse) is at most one too small
+__device__ __forceinline__ u32 mod_by(uint64_t x, u32 d, uint64_t inverse) {
+  const u32 r = (u32)x - (u32)__umul64hi(x, inverse) * d;  // below 2 d
+  return r >= d ? r - d : r;
 }
-__device__ __forceinline__ int int_from(uint64_t x, int lo, int hi) {  // igen_int of the draw x
-  return hi <= lo ? lo : lo + (int)mod_small(x, (u32)(hi - lo) + 1u);
+// igen_int of the draw x; `inverse`: that of hi - lo + 1 (0 for hi <= lo)
+__device__ __forceinline__ int int_from(uint64_t x, int lo, int hi, uint64_t inverse) {
+  return hi <= lo ? lo : lo + (int)mod_by(x, (u32)(hi - lo) + 1u, inverse);
+}
+// What the count kernel needs of the parameters beside them.
+struct CountConsts {
+  uint64_t inv_cores, inv_tpc, inv_seg;  // of the three ranges of integers
+  u32 bucket_shift, bucket_first;        // periods (below 2^24) lie in up to 256 buckets by the leading bits of their floating-point form
+};
+inline CountConsts count_consts(const igen_params_t &p) {
+  auto inverse = [](int lo, int hi) -> uint64_t { return hi <= lo ? 0 : ~0ULL / ((uint64_t)(hi - lo) + 1); };
+  auto bits = [](i64 period) -> u32 {
+    const float f = (float)period;
+    u32 b;
+    memcpy(&b, &f, sizeof(b));
+    return b;
+  };
+  CountConsts c;
+  c.inv_cores = inverse(p.cores_lo, p.cores_hi), c.inv_tpc = inverse(p.tpc_lo, p.tpc_hi);
+  c.inv_seg = inverse(p.gpu_mode == 0 && p.seg_lo < 1 ? 1 : p.seg_lo, p.seg_hi);
+  c.bucket_shift = 16;
+  while ((bits(p.period_hi) >> c.bucket_shift) - (bits(p.period_lo) >> c.bucket_shift) > 255u) c.bucket_shift += 1;
+  c.bucket_first = bits(p.period_lo) >> c.bucket_shift;
+  return c;
 }
 __device__ __forceinline__ uint64_t range_from(uint64_t x, uint64_t lo, uint64_t hi) {  // igen_range of the draw x
   return hi <= lo ? lo : lo + igen_mul_shr32(hi - lo, x >> 32);
-}
-
-// 2^(2^-i) = 1 + e_i as 4 * e_i in Q62: r * (1 + e_i) in Q62, rounded down, is r + umulhi(r, 4 e_i), the same
-// integer as igen_mul_q62(r, igen_root(i)).
-__device__ __forceinline__ uint64_t times_root(uint64_t r, int i) {
-  return r + __umul64hi(r, (igen_root(i) - (1ULL << 62)) << 2);
-}
-// igen_exp2 with the product of the first kExpBits roots looked up
-__device__ __forceinline__ uint64_t exp2_from(const uint64_t *table, uint64_t y) {
-  const int k = (int)(y >> 32);
-  const u32 f = (u32)y >> (32 - IGEN_FRAC_BITS);
-  uint64_t r = table[f >> (IGEN_FRAC_BITS - kExpBits)];
-#pragma unroll
-  for (int i = kExpBits + 1; i <= IGEN_FRAC_BITS; ++i)
-    if ((f >> (IGEN_FRAC_BITS - i)) & 1u) r = times_root(r, i);
-  return ((r >> (61 - k)) + 1) >> 1;
 }
 
 // A thread per taskset, step by step as igen.h says.  For many small tasksets, where most lanes of a warp per
@@ -127,40 +135,37 @@ __global__ void __launch_bounds__(kGenThreads) gen_count_thread_kernel(igen_para
 }
 
 // A thread's chain through a taskset grows with the square of its n tasks; the throughput of a thread per
-// taskset is 1.5 (32 tasks) to 8 (4 tasks) times that of a warp per taskset.  The two take the same time
-// at about 80 n^2 tasksets: 1,000 of 4 tasks 30 / 26 us (threads / warps), 10,000 of 12 tasks 50 / 46, 30,000
-// of 20 tasks 133 / 136, 100,000 of 32 tasks 236 / 239, 250,000 of 64 tasks 993 / 877; a million of 4 / 16 /
-// 24 / 40 / 64 tasks 0.19 / 0.64 / 1.03 / 1.81 / 3.25 ms by threads, 1.57 / 1.89 / 1.98 / 3.02 / 3.42 ms by
-// warps.  Tasksets of 80 tasks are faster by warps at every count (250,000: 1.40 / 1.20 ms).
+// taskset is up to 1.6 times (8 tasks) that of a warp per taskset, and beyond 48 tasks it is less.  The two take the
+// same time at 100 n^2 to 300 n^2 tasksets: with the fill pass 160 n^2 tasksets of 8 / 16 / 24 / 32 / 40 / 48 tasks 106 / 167 /
+// 301 / 569 / 1,110 / 1,771 us (threads / warps: 111 / 179 / 325 / 530 / 1,139 / 1,760), 40 n^2 of them 104 / 124 / 165 / 246 /
+// 397 / 571 by threads and 103 / 113 / 139 / 192 / 340 / 498 by warps; 64 tasks are faster by warps at every count
+// (1,500,000: 8.39 / 7.45 ms).
 inline bool thread_per_taskset(const igen_params_t &p, i64 count) {
   const i64 n = max_tasks_of(p);
-  return n <= 64 && count >= 80 * n * n;
+  return n <= 48 && count >= 160 * n * n;
 }
 
-// Bound by instruction issue (3,790 warp instructions per `large` taskset, 70 % of the slots; the ranks are
-// 16 % of the time, 2^y 12 %): 250,000 of them 1.20 ms.  A thread per taskset took 1.40 ms (2.3 KB of state
-// per thread in local memory).
-__global__ void __launch_bounds__(kGenThreads) gen_count_kernel(igen_params_t p, i64 first, i64 count,
-                                                                 GenSpace w) {
+// Bound by instruction issue.  2^y by two looked-up factors instead of fourteen conditional ones, remainders by
+// reciprocals and ranks by buckets instead of comparing all pairs: 250,000 `large` tasksets 1.20 -> 0.90 ms.  A thread
+// per taskset took 1.40 ms (2.3 KB of state per thread in local memory).
+__global__ void __launch_bounds__(kGenThreads) gen_count_kernel(igen_params_t p, CountConsts consts, int most_tasks, i64 first,
+                                                                 i64 count, GenSpace w) {
   __shared__ CountWarp warps[kGenThreads / 32];
-  __shared__ uint64_t table[1 << kExpBits];
+  __shared__ CountTables table;
   CountWarp &s = warps[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31;
+  constexpr int kEntries = (1 << IGEN_LEAD_BITS) + 2 * (1 << IGEN_TAIL_BITS);
 #pragma unroll 1
-  for (int f = threadIdx.x; f < (1 << kExpBits); f += kGenThreads) {
-    uint64_t r = 1ULL << 62;
-#pragma unroll
-    for (int i = 1; i <= kExpBits; ++i)
-      if ((f >> (kExpBits - i)) & 1) r = times_root(r, i);
-    table[f] = r;
-  }
+  for (int e = threadIdx.x; e < kEntries; e += kGenThreads) igen_exp2_entry(&table.exp2, e);
+  for (int d = threadIdx.x + 1; d <= most_tasks; d += kGenThreads) table.inverse[d] = ~0ULL / (uint64_t)d;
+  const int seg_lo = p.gpu_mode == 0 && p.seg_lo < 1 ? 1 : p.seg_lo;
   __syncthreads();
 #pragma unroll 1
   for (i64 t = (i64)blockIdx.x * (kGenThreads / 32) + (threadIdx.x >> 5); t < count; t += (i64)gridDim.x * (kGenThreads / 32)) {
     igen_rng_t rng;
     igen_rng_init(&rng, p.seed, p.stream, (uint64_t)(first + t));
     const uint64_t key = rng.key;
-    int cores = int_from(draw_at(key, 1), p.cores_lo, p.cores_hi);
+    int cores = int_from(draw_at(key, 1), p.cores_lo, p.cores_hi, consts.inv_cores);
     if (cores > IGEN_MAX_CORES) cores = IGEN_MAX_CORES;
     const bool harmonic = (draw_at(key, 2) >> 32) < p.harmonic;
     u32 ctr = 2;  // draws so far
@@ -168,7 +173,7 @@ __global__ void __launch_bounds__(kGenThreads) gen_count_kernel(igen_params_t p,
     // tasks per core: a core takes a draw for its tasks, one for its utilisation, one per cut point
 #pragma unroll 1
     for (int c = 0; c < cores; ++c) {
-      int m = p.tpc_hi <= p.tpc_lo ? p.tpc_lo : int_from(draw_at(key, ctr + 1), p.tpc_lo, p.tpc_hi);
+      int m = p.tpc_hi <= p.tpc_lo ? p.tpc_lo : int_from(draw_at(key, ctr + 1), p.tpc_lo, p.tpc_hi, consts.inv_tpc);
       if (n + m > IGEN_MAX_TASKS) m = IGEN_MAX_TASKS - n;
       if (lane == 0) s.start[c] = (u32)n, s.ctr[c] = ctr;
       for (int k = lane; k < m; k += 32) s.core[n + k] = (unsigned char)c;
@@ -221,10 +226,10 @@ __global__ void __launch_bounds__(kGenThreads) gen_count_kernel(igen_params_t p,
     for (int i = lane; i < n; i += 32) {
       i64 T;
       if (harmonic) {
-        const i64 T0 = (i64)exp2_from(table, range_from(draw_at(key, ctr + 1 + 2 * i), p.log2_lo, p.log2_hi0));
-        T = T0 << int_from(draw_at(key, ctr + 2 + 2 * i), 0, 10);
+        const i64 T0 = (i64)igen_exp2_by(&table.exp2, range_from(draw_at(key, ctr + 1 + 2 * i), p.log2_lo, p.log2_hi0));
+        T = T0 << int_from(draw_at(key, ctr + 2 + 2 * i), 0, 10, ~0ULL / 11);
       } else {
-        T = (i64)exp2_from(table, range_from(draw_at(key, ctr + 1 + i), p.log2_lo, p.log2_hi));
+        T = (i64)igen_exp2_by(&table.exp2, range_from(draw_at(key, ctr + 1 + i), p.log2_lo, p.log2_hi));
       }
       if (T < p.period_lo) T = p.period_lo;
       if (T > p.period_hi) T = p.period_hi;
@@ -245,7 +250,7 @@ __global__ void __launch_bounds__(kGenThreads) gen_count_kernel(igen_params_t p,
 #pragma unroll 1
       for (int k0 = 0; k0 < ng; k0 += 32) {
         const int k = k0 + lane;
-        const int j = k < ng ? k + (int)mod_small(draw_at(key, ctr + 1 + 2 * k), (u32)(n - k)) : -1 - lane;
+        const int j = k < ng ? k + (int)mod_by(draw_at(key, ctr + 1 + 2 * k), (u32)(n - k), table.inverse[n - k]) : -1 - lane;
         const u32 same = __match_any_sync(kFull, j);
         const u32 below = same & ((1u << lane) - 1u);
         int before = -1;
@@ -268,12 +273,12 @@ __global__ void __launch_bounds__(kGenThreads) gen_count_kernel(igen_params_t p,
         } else {
           task = ~task;
         }
-        s.eta[task] = (unsigned char)int_from(draw_at(key, ctr + 2 + 2 * k), p.seg_lo < 1 ? 1 : p.seg_lo, p.seg_hi);
+        s.eta[task] = (unsigned char)int_from(draw_at(key, ctr + 2 + 2 * k), seg_lo, p.seg_hi, consts.inv_seg);
       }
       ctr += 2 * ng;
     } else {
 #pragma unroll 1
-      for (int i = lane; i < n; i += 32) s.eta[i] = (unsigned char)int_from(draw_at(key, ctr + 1 + i), p.seg_lo, p.seg_hi);
+      for (int i = lane; i < n; i += 32) s.eta[i] = (unsigned char)int_from(draw_at(key, ctr + 1 + i), p.seg_lo, p.seg_hi, consts.inv_seg);
       ctr += n;
     }
     __syncwarp();
@@ -331,28 +336,41 @@ __global__ void __launch_bounds__(kGenThreads) gen_count_kernel(igen_params_t p,
       __syncwarp();
     }
     // rate-monotonic priorities: shorter period = higher, ties by position.  Periods below 2^24 with the
-    // position behind them are distinct 32-bit keys; 96 tasks are compared with four at a time.
+    // position behind them are distinct 32-bit keys.  Log-uniform as they are, the leading bits of their
+    // floating-point form spread them evenly over 256 buckets; a key's rank is its bucket's start and the smaller
+    // keys in the bucket.
     if (p.period_hi < (1LL << 24)) {
-      for (int i = lane; i < ((n + 3) & ~3); i += 32) s.key[i] = i < n ? (s.T[i] << 8) | (u32)i : 0xffffffffu;
+      for (int c = lane; c < 64; c += 32) reinterpret_cast<uint4 *>(s.cut)[c] = make_uint4(0, 0, 0, 0);
+      __syncwarp();
+      auto bucket = [&](u32 T) -> u32 { return (__float_as_uint((float)T) >> consts.bucket_shift) - consts.bucket_first; };
+#pragma unroll 1
+      for (int i = lane; i < n; i += 32) s.from[i] = (short)atomicAdd(&s.cut[bucket(s.T[i])], 1u);
+      __syncwarp();
+      {  // starts of the buckets, eight per lane
+        uint4 x = reinterpret_cast<uint4 *>(s.cut)[2 * lane], y = reinterpret_cast<uint4 *>(s.cut)[2 * lane + 1];
+        x.y += x.x, x.z += x.y, x.w += x.z, y.x += x.w, y.y += y.x, y.z += y.y, y.w += y.z;
+        u32 before = y.w;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+          const u32 o = __shfl_up_sync(kFull, before, d);
+          if (lane >= d) before += o;
+        }
+        before -= y.w;
+        reinterpret_cast<uint4 *>(s.cut)[2 * lane] = make_uint4(before, before + x.x, before + x.y, before + x.z);
+        reinterpret_cast<uint4 *>(s.cut)[2 * lane + 1] = make_uint4(before + x.w, before + y.x, before + y.y, before + y.z);
+      }
       __syncwarp();
 #pragma unroll 1
-      for (int i0 = lane; i0 - lane < n; i0 += 96) {
-        u32 mine[3];
-        int higher[3] = {0, 0, 0};
-#pragma unroll
-        for (int e = 0; e < 3; ++e) mine[e] = i0 + 32 * e < n ? s.key[i0 + 32 * e] : 0u;
+      for (int i = lane; i < n; i += 32) s.key[s.cut[bucket(s.T[i])] + (u32)s.from[i]] = (s.T[i] << 8) | (u32)i;
+      __syncwarp();
 #pragma unroll 1
-        for (int q = 0; q < n; q += 4) {
-          const uint4 y = *reinterpret_cast<const uint4 *>(&s.key[q]);
-#pragma unroll
-          for (int e = 0; e < 3; ++e)
-            higher[e] += (y.x < mine[e] ? 1 : 0) + (y.y < mine[e] ? 1 : 0) + (y.z < mine[e] ? 1 : 0) + (y.w < mine[e] ? 1 : 0);
-        }
-#pragma unroll
-        for (int e = 0; e < 3; ++e) {
-          const int i = i0 + 32 * e;
-          if (i < n) st[6 + 3 * i] = (u32)(n - higher[e]) | ((u32)s.core[i] << 16) | ((u32)s.eta[i] << 24);
-        }
+      for (int i = lane; i < n; i += 32) {
+        const u32 T = s.T[i], c = bucket(T), mine = (T << 8) | (u32)i;
+        const u32 from = s.cut[c], to = c < 255 ? s.cut[c + 1] : (u32)n;
+        u32 higher = from;
+#pragma unroll 1
+        for (u32 q = from; q < to; ++q) higher += s.key[q] < mine ? 1u : 0u;
+        st[6 + 3 * i] = ((u32)n - higher) | ((u32)s.core[i] << 16) | ((u32)s.eta[i] << 24);
       }
     } else {
 #pragma unroll 1
@@ -484,15 +502,13 @@ struct FillWarp {
 
 // Splits `total` us of this lane's task into `parts` segments (0: none) like igen_split does, the tasks
 // of all lanes at once.  `draw`: position of the task's first weight.  The segments of the lanes lie one
-// behind the other from out[0] on; FIFTH: a fifth of each goes to `fifth`.
+// behind the other from out[0] on (this lane's from out[first] on, n_parts in all); FIFTH: a fifth of each goes to `fifth`.
 //
 // igen_split's quotient floor(spare * w / sum of weights) is taken in double precision with the task's
 // reciprocal (wrong by at most 1, as all values stay below 2^31) and settled by its remainder.
 template <bool FIFTH>
 __device__ __forceinline__ void split_tasks(FillWarp &w, uint64_t key, uint64_t ctr, u32 draw, u32 total, u32 parts,
-                                            i64 *out, i64 *fifth, int lane) {
-  u32 n_parts;
-  const u32 first = warp_exclusive(parts, lane, &n_parts);
+                                            u32 first, u32 n_parts, i64 *out, i64 *fifth, int lane) {
   if (!__any_sync(kFull, parts > 1)) {  // a task's only segment takes all of it, whatever its weight
     if (parts > 0) {
       const u32 small = FIFTH ? total / 5u : 0u;
@@ -519,7 +535,10 @@ __device__ __forceinline__ void split_tasks(FillWarp &w, uint64_t key, uint64_t 
 #pragma unroll 1
   for (u32 j = 0; j < parts; ++j) sum += w.share[first + j];
   w.weights[lane] = sum;
-  w.inverse[lane] = 1.0 / (double)(sum + (parts == 0 ? 1 : 0));
+  {  // the reciprocal to 46 bits: one step of Newton's iteration from single precision
+    const double d = (double)(sum + (parts == 0 ? 1 : 0)), r = (double)__frcp_rn((float)d);
+    w.inverse[lane] = r * (2.0 - d * r);
+  }
   __syncwarp();
 #pragma unroll 1
   for (u32 q = lane; q < n_parts; q += 32) {
@@ -549,9 +568,10 @@ __device__ __forceinline__ void split_tasks(FillWarp &w, uint64_t key, uint64_t 
   __syncwarp();
 }
 
-// Bound by instruction issue and by the stores: 250,000 `large` tasksets (2.3 GB) 0.97 ms; a lane per
+// Bound by instruction issue and by the stores: 250,000 `large` tasksets (2.3 GB) 0.95 ms; a lane per
 // task for everything took 1.43 ms (lanes wait for the task with the most segments, weights drawn
-// twice, 8-byte stores far apart).
+// twice, 8-byte stores far apart).  The GPU and the CPU parts of a round split side by side: no gain there, and 1,000,000
+// tasksets of 8 tasks, whose GPU parts need no split, 1.03 -> 1.09 ms.
 __global__ void __launch_bounds__(kGenThreads) gen_fill_kernel(igen_params_t p, i64 first, i64 count,
                                                                 GenSpace w, GenOut o) {
   __shared__ FillWarp warps[kGenThreads / 32];
@@ -591,10 +611,10 @@ __global__ void __launch_bounds__(kGenThreads) gen_fill_kernel(igen_params_t p, 
         o.cseg_off[k0 + i] = c_start + c_run + c_before;
         o.gseg_off[k0 + i] = g_start + g_run + g_before;
       }
-      split_tasks<true>(mine_w, key, ctr, draws_before + 1, G, eta, o.gseg_exec + g_start + g_run,
+      split_tasks<true>(mine_w, key, ctr, draws_before + 1, G, eta, g_before, g_total, o.gseg_exec + g_start + g_run,
                         o.gseg_misc + g_start + g_run, lane);
-      split_tasks<false>(mine_w, key, ctr, draws_before + 1 + eta, E - G, c_parts, o.cseg_wcet + c_start + c_run, nullptr,
-                         lane);
+      split_tasks<false>(mine_w, key, ctr, draws_before + 1 + eta, E - G, c_parts, c_before, c_total,
+                         o.cseg_wcet + c_start + c_run, nullptr, lane);
       ctr += draws_total, c_run += c_total, g_run += g_total;
     }
   }
@@ -690,7 +710,7 @@ int gcaps_gen_count(const gcaps_gen_params_t *params, int64_t first, int64_t cou
       e = cudaFuncSetAttribute(gen_count_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
     if (e == cudaSuccess)
       e = launch_persistent(gen_count_kernel, g_count_blocks, 0, (long long)((count + kWarps - 1) / kWarps), di.sm_count, st,
-                            p, (i64)first, (i64)count, w);
+                            p, count_consts(p), (int)max_tasks_of(p), (i64)first, (i64)count, w);
   }
   if (e != cudaSuccess) {
     g_last_cuda_error = (int)e;

@@ -160,6 +160,47 @@ IGEN_FN uint64_t igen_exp2(uint64_t y) {
   return ((r >> (61 - k)) + 1) >> 1;
 }
 
+/* igen_exp2 from looked-up factors: the product of the leading ten roots, formed step by step as igen_exp2 does,
+ * and two products of seven roots each.  Two roundings down stand for fourteen, so the product differs by up to 12
+ * units of 2^-62; the result does not, for any fraction and 2^0 .. 2^30 (tests/test_igen_exp2.py tries them all). */
+#define IGEN_LEAD_BITS 10
+#define IGEN_TAIL_BITS 7
+typedef struct {
+  uint64_t lead[1 << IGEN_LEAD_BITS];    /* Q62 */
+  uint64_t tail[2][1 << IGEN_TAIL_BITS]; /* product - 1, in units of 2^-64 */
+} igen_exp2_tables_t;
+IGEN_FN uint64_t igen_mulhi(uint64_t a, uint64_t b) {
+#ifdef __CUDA_ARCH__
+  return __umul64hi(a, b);
+#else
+  return (uint64_t)(((unsigned __int128)a * b) >> 64);
+#endif
+}
+/* r times root i: r + r * (root - 1), rounded down, is what igen_mul_q62 gives */
+IGEN_FN uint64_t igen_times_root(uint64_t r, int i) {
+  return r + igen_mulhi(r, (igen_root(i) - (1ULL << 62)) << 2);
+}
+/* the product of the roots first + 1 .. first + bits that f names (the highest of its bits the first) */
+IGEN_FN uint64_t igen_roots(uint32_t f, int first, int bits) {
+  uint64_t r = 1ULL << 62;
+  for (int i = 1; i <= bits; ++i)
+    if ((f >> (bits - i)) & 1u) r = igen_times_root(r, first + i);
+  return r;
+}
+IGEN_FN void igen_exp2_entry(igen_exp2_tables_t *t, int e) { /* e = 0 .. 2^10 + 2 * 2^7 - 1 */
+  const int tail = e - (1 << IGEN_LEAD_BITS), which = tail >> IGEN_TAIL_BITS, f = tail & ((1 << IGEN_TAIL_BITS) - 1);
+  if (tail < 0) t->lead[e] = igen_roots((uint32_t)e, 0, IGEN_LEAD_BITS);
+  else t->tail[which][f] = (igen_roots((uint32_t)f, IGEN_LEAD_BITS + which * IGEN_TAIL_BITS, IGEN_TAIL_BITS) - (1ULL << 62)) << 2;
+}
+IGEN_FN uint64_t igen_exp2_by(const igen_exp2_tables_t *t, uint64_t y) {
+  const int k = (int)(y >> 32);
+  const uint32_t f = (uint32_t)y >> (32 - IGEN_FRAC_BITS), mask = (1u << IGEN_TAIL_BITS) - 1u;
+  uint64_t r = t->lead[f >> (2 * IGEN_TAIL_BITS)];
+  r += igen_mulhi(r, t->tail[0][(f >> IGEN_TAIL_BITS) & mask]);
+  r += igen_mulhi(r, t->tail[1][f & mask]);
+  return ((r >> (61 - k)) + 1) >> 1;
+}
+
 /* Splits `total` into `parts` integers >= 1 (needs total >= parts) in proportion to random
  * weights in [1,2); the last part takes the rounding remainder.  With `fifth` given, a fifth of
  * every part (rounded down) goes there and the rest to `out`.  The weights are drawn twice (once
