@@ -40,14 +40,27 @@ ALU_PEAK_DERIVED = 148 * 128 * 1.965e9
 MAX_TASKSETS_PER_GPU = 1_000_000
 K_TERM, K_SETUP = 6, 16   # algorithmic integer lane-operations per interference term / per task
 
-def kernel_launches(tasksets, kind="one"):
+
+def in_tiles(tasksets, tasks, gcaps, walks):
+    """Whether a batch too large for one launch without a plan goes through tiles (tile_rows of gcaps_rta.cu):
+    small tasksets of one size, and under GCAPS enough of them.  `walks`: analyses of a policy per taskset."""
+    if not tasks or tasks % tasksets or tasks > 24 * tasksets:
+        return False
+    n = tasks // tasksets
+    return not (gcaps and n > 12 and (tasksets < 1750 * n if walks == 1 else tasksets * walks < 100000))
+
+
+def kernel_launches(tasksets, kind="one", tasks=None, gcaps=True, walks=1):
     """Kernels of one call on a batch: "one" analysis, "several" (a sweep, or analyses of one waiting
-    mode) or a "search" of GPU priorities.  Small batches are one launch without a plan.  Otherwise the
+    mode) or a "search" of GPU priorities.  Small batches are one launch without a plan.  Tiles take one
+    launch, and two more what these left over.  Otherwise the
     plan takes one kernel or three; then one kernel serves the bins of up to 32 tasks, one each those of
     up to 64, 96, 128, 192 and 256, and for a single analysis two more, for a search one more, what
     these left over."""
     if tasksets <= build.source_constant("kDirectMost" if kind == "one" else "kDirectSweepMost"):
         return 1
+    if kind != "search" and (kind == "one" or walks > 1) and in_tiles(tasksets, tasks, gcaps, walks):
+        return 3
     return (1 if tasksets <= build.source_constant("kPlanSmall") else 3) + {"one": 8, "several": 6, "search": 7}[kind]
 
 
@@ -616,9 +629,10 @@ def main():
                        "input_checksum": batch.checksum() if count <= 200_000 else None},
             "clocks": clocks, "e2e": e2e,
             "gpu_launches": args.steps * sum(
-                len(pairs) * kernel_launches(count) if name == "one_call_per_pair" else
+                len(pairs) * kernel_launches(count, "one", ts.n_tasks, False) if name == "one_call_per_pair" else
                 kernel_launches(count, {"gcaps+rr": "several", "fused_sweep": "several",
-                                        "gpu_priority_search": "search"}.get(name, "one"))
+                                        "gpu_priority_search": "search"}.get(name, "one"), ts.n_tasks,
+                                name not in ("rr", "fused_sweep"), len(pairs) if name == "fused_sweep" else 1)
                 for name in names),
             "roofline": roof, "cpu_baseline": cpu, "wall_s_timed_region": t_wall,
         }

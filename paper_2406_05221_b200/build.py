@@ -9,7 +9,7 @@ import sys
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 CUDA_SRC = os.path.join(_HERE, "csrc", "gcaps_rta.cu")
-CUDA_SRCS = [CUDA_SRC, os.path.join(_HERE, "csrc", "gcaps_rta_small.cu"),
+CUDA_SRCS = [CUDA_SRC, os.path.join(_HERE, "csrc", "gcaps_rta_tile.cu"),
              os.path.join(_HERE, "csrc", "gcaps_rta_direct.cu"),
              os.path.join(_HERE, "csrc", "gcaps_rta_sweep.cu"),
              os.path.join(_HERE, "csrc", "gcaps_rta_tile_q2.cu"), os.path.join(_HERE, "csrc", "gcaps_rta_tile_q4.cu"),

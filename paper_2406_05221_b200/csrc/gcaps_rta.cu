@@ -15,6 +15,7 @@
 
 #include "rta_device.cuh"
 #include "rta_staged.cuh"
+#include "rta_tile_kept.cuh"
 
 using namespace gcaps_detail;
 
@@ -114,6 +115,24 @@ __global__ void __launch_bounds__(1024) plan_small_kernel(KParams p) {
     const int b = size_bin(p.task_off[t + 1] - p.task_off[t]);
     p.perm[start[b] + atomicAdd(&cnt[b], 1u)] = (unsigned int)t;
   }
+}
+
+// The bins of up to 32 tasks in one persistent launch, largest tasksets first: (lanes per
+// taskset, tasks per lane) = (16,2) (8,3) (8,2) (8,1) for at most 32, 24, 16, 8 tasks, i.e. two or
+// four tasksets per warp.  (A look at the first ranks out of a stage, a warp per taskset, was slower
+// here in every form tried: 100,000 24-task tasksets under round robin 163 us against 128.)
+template <int MODE>
+__global__ void __launch_bounds__(kBlockThreads, min_blocks(3)) rta_small_kernel(KParams p, bool rest) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  if (rest) wait_for_previous_grid();  // what the tiles left over is listed from here on
+  let_dependents_start();  // the kernel of the next size bin shares no data with this one
+  u32 *warp_buf = reinterpret_cast<u32 *>(smem_raw) + (threadIdx.x >> 5) * kSmallWarpWords;
+  Ahead *ahead = reinterpret_cast<Ahead *>(warp_buf + kSmallWarpWords - kAheadWords);
+  run_bin<16, 2, 1 << MODE>(p, 3, warp_buf, ahead);
+  run_bin<8, 3, 1 << MODE>(p, 2, warp_buf, ahead);
+  run_bin<8, 2, 1 << MODE>(p, 1, warp_buf, ahead);
+  run_bin<8, 1, 1 << MODE>(p, 0, warp_buf, ahead);
+  wait_for_previous_grid();
 }
 
 // First launch of a bin of larger tasksets: a warp per taskset, SLOTS tasks per lane.
@@ -368,8 +387,28 @@ cudaError_t launch_deferred(const KParams &p, int sm_count, cudaStream_t st) {
 }
 
 template <int MODE>
+int small_blocks[64] = {0};  // resident blocks of rta_small_kernel per SM
+
+// Behind tiles: what they listed of up to 24 tasks.
+cudaError_t launch_rest(int mode, const KParams &p, int sm_count, cudaStream_t st) {
+  auto rest = [&](auto kernel, int *blocks) {
+    constexpr int kWarps = kBlockThreads / 32;
+    return launch_persistent_ex(true, kernel, blocks, sizeof(u32) * kSmallWarpWords * kWarps, (p.n_tasksets + kWarps - 1) / kWarps,
+                                sm_count, st, p, true);
+  };
+  switch (mode) {
+    case 0: return rest(rta_small_kernel<0>, small_blocks<0>);
+    case 1: return rest(rta_small_kernel<1>, small_blocks<1>);
+    case 2: return rest(rta_small_kernel<2>, small_blocks<2>);
+    default: return rest(rta_small_kernel<3>, small_blocks<3>);
+  }
+}
+
+template <int MODE>
 cudaError_t launch_all_bins(const KParams &p, int sm_count, cudaStream_t st) {
-  cudaError_t e = launch_small(MODE, p, 0, sm_count, st);
+  constexpr int kWarps = kBlockThreads / 32;
+  cudaError_t e = launch_persistent(rta_small_kernel<MODE>, small_blocks<MODE>, sizeof(u32) * kSmallWarpWords * kWarps,
+                                    (p.n_tasksets + kWarps - 1) / kWarps, sm_count, st, p, false);
   if (e == cudaSuccess) e = launch_big<2, MODE>(p, 4, sm_count, st);
   if (e == cudaSuccess) e = launch_big<3, MODE>(p, 5, sm_count, st);
   if (e == cudaSuccess) e = launch_big<4, MODE>(p, 6, sm_count, st);
@@ -378,6 +417,25 @@ cudaError_t launch_all_bins(const KParams &p, int sm_count, cudaStream_t st) {
   if (e == cudaSuccess) e = launch_deferred<false, MODE>(p, sm_count, st);
   if (e == cudaSuccess) e = launch_deferred<true, MODE>(p, sm_count, st);
   return e;
+}
+
+// Tiles are for batches of tasksets of one size (a mean that is a whole number): a tile's rows are taken by the largest
+// taskset, and in a mixture the plan's bins are the better way (4 to 24 tasks, 100,000 tasksets 212 us in tiles, 162
+// us in bins).  Under GCAPS a tile's walk is long, so there have to be enough tiles to go round: 12 tasks 43 / 54 us (tiles /
+// bins) at 12,500 tasksets and 63 / 84 at 50,000, 16 tasks 71 / 69 at 25,000 and 79 / 83 at 35,000, 20 tasks 91 / 84
+// and 97 / 105, 24 tasks 127 / 123 at 35,000 and 128 / 157 at 50,000.  Under RR tiles are the faster way from the start
+// (24 tasks 40 / 51 us at 12,500).  Several analyses under GCAPS, 20 tasks: 170 / 138 us for five pairs of 10,000
+// tasksets, 243 / 240 of 20,000, 212 / 280 for three pairs of 50,000; 24 tasks: 203 / 182 for two pairs of 30,000, 578 / 654 for
+// 25 pairs of 5,000.  32 tasks: 575 / 521 us per 100,000, as a tile then takes 40 KB.
+// Returns the rows that tiles of this batch need, or 0: no tiles.  `analyses`: those of the call; `walks`: how many of a policy
+// every taskset goes through.
+int tile_rows(int analyses, int walks, i64 max_ovh, const KParams &p) {
+  if (max_ovh >= (1 << 20) || ((analyses & 2) && (p.policy & GCAPS_RTA_LITERAL))) return 0;
+  if (p.n_tasks % p.n_tasksets != 0 || p.n_tasks > kTileMost * p.n_tasksets) return 0;
+  const int n = (int)(p.n_tasks / p.n_tasksets);
+  if (walks == 1 && (analyses & 3) && n > 12 && p.n_tasksets < 1750 * n) return 0;
+  if (walks > 1 && (analyses & 12) == 0 && n > 12 && p.n_tasksets * walks < 100000) return 0;
+  return n < 4 ? 4 : n;
 }
 
 // Plan + analysis launches of one call.  `sw` null: one analysis (p.policy).  Otherwise the
@@ -406,7 +464,8 @@ int enqueue_batch(KParams p, void *workspace, size_t workspace_bytes, int sm_cou
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess && rows > 0) e = cudaMemsetAsync(p.hdr, 0, sizeof(PlanHeader), st);
   if (e == cudaSuccess && rows > 0 && !sw) {
-    e = launch_small(mode, p, rows, sm_count, st);
+    e = launch_tiles(mode, p, rows, sm_count, st);
+    if (e == cudaSuccess) e = launch_rest(mode, p, sm_count, st);
     if (e == cudaSuccess) e = launch_listed_tasksets(mode, p, sm_count, st);
   } else if (e == cudaSuccess && sw) {
     SweepArgs set = *sw;
@@ -418,7 +477,7 @@ int enqueue_batch(KParams p, void *workspace, size_t workspace_bytes, int sm_cou
     bool first = true;
     if (rows > 0) {
       set.enabled = analyses;
-      e = walks > 2 ? launch_tile_q4(p, set, rows, sm_count, st) : launch_tile_q2(p, set, rows, sm_count, st);
+      e = walks > kKeptFew ? launch_tile_q4(p, set, rows, sm_count, st) : launch_tile_q2(p, set, rows, sm_count, st);
     }
     for (int half = 0; half < 2 && e == cudaSuccess; ++half) {
       set.enabled = analyses & (half == 0 ? 5 : 10);

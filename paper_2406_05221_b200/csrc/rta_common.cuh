@@ -282,13 +282,9 @@ void fill_params(KParams *p, const gcaps_tasksets_t *ts, int64_t n_tasksets, int
 // permutation of the taskset indices, zeroed work counters).  GCAPS_OK or GCAPS_ERR_WORKSPACE.
 int place_plan(KParams &p, void *workspace, size_t workspace_bytes);  // only the first part
 int enqueue_plan(KParams &p, void *workspace, size_t workspace_bytes, cudaStream_t st);
-// The rows that tiles of this batch need, or 0: no tiles (`analyses`: those of the call, `walks` of them per taskset).
-int tile_rows(int analyses, int walks, i64 max_ovh, const KParams &p);
-// rows 0: the first launch of a call with a plan, over the bins of up to 32 tasks.  Else tiles over the whole batch,
-// without a plan (the header is zero), and the first of the two launches that take what tiles leave over.  Defined in
-// gcaps_rta_small.cu.
-cudaError_t launch_small(int mode, const KParams &p, int rows, int sm_count, cudaStream_t st);
-// The second of them; defined in gcaps_rta_direct.cu.
+// Tiles over the whole batch, without a plan (the header is zero); defined in gcaps_rta_tile.cu.
+cudaError_t launch_tiles(int mode, const KParams &p, int rows, int sm_count, cudaStream_t st);
+// The second of the two launches that take what tiles leave over; defined in gcaps_rta_direct.cu.
 cudaError_t launch_listed_tasksets(int mode, const KParams &p, int sm_count, cudaStream_t st);
 // One launch for analysis `mode` (0 GCAPS self-suspension, 1 GCAPS busy-waiting, 2 RR self-suspension, 3 RR
 // busy-waiting) without a plan, a block of one warp per taskset, for batches of at most kDirectMost

@@ -29,6 +29,7 @@
 namespace {
 
 constexpr int kTileThreads = 32;
+constexpr int kTileMost = 24;      // tasks
 constexpr int kTileSweeps = 4096;  // sweeps of a rank after which a taskset is left over
 constexpr int kTileCores = 16;     // cores are 0 .. kTileCores-1
 constexpr int kTileOnCore = 10;    // a walk is good for that many tasks of a core: it holds six of them in registers

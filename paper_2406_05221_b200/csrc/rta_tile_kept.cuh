@@ -9,6 +9,7 @@
 namespace {
 
 constexpr int kKindGcaps = 1, kKindRr = 2;
+constexpr int kKeptFew = 2;  // walks of a policy up to which a taskset has two lanes; with more it has four
 
 // Shared memory of one warp's tile of 32/Q tasksets.  A row holds what belongs to the task of a position, for every column,
 //   own  T and more, D, A = C+G^m, G^e with the sign bit = uses the GPU
