@@ -92,8 +92,9 @@ extern "C" {
 #define GCAPS_ERR_WORKSPACE (-2)     /* workspace null or smaller than gcaps_rta_workspace_bytes */
 #define GCAPS_ERR_CUDA (-3)          /* a CUDA runtime call failed; see gcaps_rta_last_cuda_error */
 #define GCAPS_ERR_NO_DEVICE (-4)     /* no CUDA device / not an sm_100 device                    */
-#define GCAPS_ERR_TOO_LARGE (-5)     /* batch larger than GCAPS_RTA_STATIC_MAX_TASKSETS (only
-                                        returned by gcaps_rta_batch_static)                     */
+#define GCAPS_ERR_TOO_LARGE (-5)     /* batch larger than GCAPS_RTA_STATIC_MAX_TASKSETS
+                                        (gcaps_rta_batch_static) or GCAPS_RTA_FEW_MAX_TASKSETS
+                                        (gcaps_rta_batch_few)                                   */
 
 /*
  * A batch of tasksets in CSR structure-of-arrays form (task model: Sec. 4).
@@ -315,6 +316,15 @@ int gcaps_rta_multi_batch(const gcaps_tasksets_t *ts, int64_t n_tasksets, int an
 int gcaps_rta_batch_static(const gcaps_tasksets_t *ts, int64_t n_tasksets, int policy,
                            int64_t timeslice_us, int64_t ctx_switch_overhead_us,
                            int64_t *out_wcrt, uint8_t *out_sched, void *stream);
+
+/*
+ * gcaps_rta_batch_few -- gcaps_rta_batch for a batch of at most GCAPS_RTA_FEW_MAX_TASKSETS tasksets, which runs as one
+ * launch and so needs no workspace: a caller that makes the buffers of every call anew (an interactive query, an
+ * admission test) saves one of its three allocations.  GCAPS_ERR_TOO_LARGE beyond; otherwise as gcaps_rta_batch.
+ */
+#define GCAPS_RTA_FEW_MAX_TASKSETS 12288
+int gcaps_rta_batch_few(const gcaps_tasksets_t *ts, int64_t n_tasksets, int policy, int64_t timeslice_us,
+                        int64_t ctx_switch_overhead_us, int64_t *out_wcrt, uint8_t *out_sched, void *stream);
 
 /*
  * On-device taskset generation.  The paper's experiments analyse randomly generated tasksets

@@ -30,6 +30,7 @@ MAX_TIME = 1 << 40
 
 OK, ERR_INVALID_ARG, ERR_WORKSPACE, ERR_CUDA, ERR_NO_DEVICE, ERR_TOO_LARGE = 0, -1, -2, -3, -4, -5
 STATIC_MAX_TASKSETS = 65536
+FEW_MAX_TASKSETS = 12288  # batches that run as one launch (gcaps_rta_batch_few)
 MAX_SWEEP = 32
 # analyses of rta_multi, in result order
 GCAPS_SUSPEND, GCAPS_BUSY, RR_SUSPEND, RR_BUSY = 1, 2, 4, 8
@@ -38,7 +39,7 @@ ANALYSIS_POLICY = {GCAPS_SUSPEND: POLICY_GCAPS, GCAPS_BUSY: POLICY_GCAPS | BUSY,
 
 EXPORTS = ("gcaps_rta_batch", "gcaps_rta_workspace_bytes", "gcaps_rta_batch_host",
            "gcaps_rta_release_host", "gcaps_rta_validate", "gcaps_rta_strerror",
-           "gcaps_rta_last_cuda_error", "gcaps_rta_version", "gcaps_rta_batch_static",
+           "gcaps_rta_last_cuda_error", "gcaps_rta_version", "gcaps_rta_batch_static", "gcaps_rta_batch_few",
            "gcaps_rta_batch_host_multi", "gcaps_rta_gpu_priority_batch", "gcaps_rta_sweep_batch", "gcaps_rta_multi_batch",
            "gcaps_gen_workspace_bytes", "gcaps_gen_count", "gcaps_gen_fill",
            "gcaps_rta_plan_batch", "gcaps_rta_int_issue_probe")
@@ -86,6 +87,8 @@ def load_library(path: Optional[str] = None):
             ctypes.POINTER(CTasksets), ctypes.c_int64, ctypes.c_int, ctypes.c_int64, ctypes.c_int64,
             ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p]
         lib.gcaps_rta_batch_static.restype = ctypes.c_int
+        lib.gcaps_rta_batch_few.argtypes = lib.gcaps_rta_batch_static.argtypes
+        lib.gcaps_rta_batch_few.restype = ctypes.c_int
         lib.gcaps_rta_workspace_bytes.argtypes = [ctypes.c_int64]
         lib.gcaps_rta_workspace_bytes.restype = ctypes.c_size_t
         lib.gcaps_rta_batch_host.argtypes = [
@@ -224,11 +227,16 @@ def rta_batch(ts: DeviceTasksets, policy: int, timeslice_us: int = 1024, overhea
             out_wcrt = torch.empty(ts.n_tasks, dtype=torch.int64, device=dev)
         if out_sched is None:
             out_sched = torch.empty(max(ts.n_tasksets, 0), dtype=torch.uint8, device=dev)
-        if workspace is None:
-            workspace = torch.empty(max(workspace_bytes(ts.n_tasksets), 256), dtype=torch.uint8, device=dev)
-        rc = lib.gcaps_rta_batch(ctypes.byref(ts.c), ts.n_tasksets, policy, timeslice_us, overhead_us,
-                                 out_wcrt.data_ptr(), out_sched.data_ptr(), workspace.data_ptr(),
-                                 workspace.numel(), st)
+        if workspace is None and ts.n_tasksets <= FEW_MAX_TASKSETS:
+            # one launch, nothing to keep in a workspace (making one took 2 us of a call's 12)
+            rc = lib.gcaps_rta_batch_few(ctypes.byref(ts.c), ts.n_tasksets, policy, timeslice_us, overhead_us,
+                                         out_wcrt.data_ptr(), out_sched.data_ptr(), st)
+        else:
+            if workspace is None:
+                workspace = torch.empty(max(workspace_bytes(ts.n_tasksets), 256), dtype=torch.uint8, device=dev)
+            rc = lib.gcaps_rta_batch(ctypes.byref(ts.c), ts.n_tasksets, policy, timeslice_us, overhead_us,
+                                     out_wcrt.data_ptr(), out_sched.data_ptr(), workspace.data_ptr(),
+                                     workspace.numel(), st)
     _check(rc)
     return out_wcrt, out_sched
 

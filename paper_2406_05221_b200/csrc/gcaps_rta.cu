@@ -650,6 +650,28 @@ int gcaps_rta_batch_static(const gcaps_tasksets_t *ts, int64_t n_tasksets, int p
                        (cudaStream_t)stream);
 }
 
+int gcaps_rta_batch_few(const gcaps_tasksets_t *ts, int64_t n_tasksets, int policy, int64_t timeslice_us,
+                        int64_t ctx_switch_overhead_us, int64_t *out_wcrt, uint8_t *out_sched, void *stream) {
+  static_assert(GCAPS_RTA_FEW_MAX_TASKSETS == kDirectMost, "what runs as one launch");
+  int rc = check_args(ts, n_tasksets, policy, timeslice_us, ctx_switch_overhead_us);
+  if (rc != GCAPS_OK) return rc;
+  if (n_tasksets > GCAPS_RTA_FEW_MAX_TASKSETS) return GCAPS_ERR_TOO_LARGE;
+  if (n_tasksets == 0) return GCAPS_OK;
+  if (!out_sched || (ts->n_tasks > 0 && !out_wcrt)) return GCAPS_ERR_INVALID_ARG;
+  DeviceInfo di;
+  rc = device_info(&di);
+  if (rc != GCAPS_OK) return rc;
+  KParams p;
+  fill_params(&p, ts, n_tasksets, policy, timeslice_us, ctx_switch_overhead_us, out_wcrt, out_sched);
+  const bool rr = (policy & 0xff) == GCAPS_POLICY_RR, busy = (policy & GCAPS_RTA_BUSY) != 0;
+  const cudaError_t e = launch_one_warp_each((rr ? 2 : 0) + (busy ? 1 : 0), p, (cudaStream_t)stream);
+  if (e != cudaSuccess) {
+    g_last_cuda_error = (int)e;
+    return GCAPS_ERR_CUDA;
+  }
+  return GCAPS_OK;
+}
+
 int gcaps_rta_validate(const gcaps_tasksets_t *ts, int64_t n_tasksets, int32_t *out_err,
                        void *stream) {
   int rc = check_args(ts, n_tasksets, GCAPS_POLICY_GCAPS, 1, 0);
