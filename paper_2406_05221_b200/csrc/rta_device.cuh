@@ -1,12 +1,14 @@
 // rta_device.cuh -- device code of the analysis kernels, shared by the translation units that
 // instantiate them: gcaps_rta.cu (one analysis per launch), gcaps_rta_direct.cu (small batches, a
-// warp per taskset), gcaps_rta_sweep.cu (several analyses per launch).  Internal.
+// warp per taskset), gcaps_rta_sweep.cu and gcaps_rta_direct_sweep.cu (several analyses per launch).
+// Batches of small tasksets of one size go through tiles (rta_tile.cuh, rta_tile_kept.cuh) and come
+// here with what those leave over.  Internal.
 //
 // One warp analyses one taskset at a time:
 //   stage      coalesced loads of the taskset's per-task slices into registers (lane = task)
-//   aggregate  coalesced loads of the segment arrays, warp prefix sums into shared memory; the
-//              per-task sums C_i, G^m_i, G^e_i and the RR slice count of Eq. 3 are differences of
-//              two prefix values
+//   aggregate  the per-task sums C_i, G^m_i, G^e_i: added up by the lane of the task, or (groups of
+//              8 or 16 lanes) as differences of two running sums in shared memory, as the RR slice
+//              count of Eq. 3 is
 //   order      rank of every task by (priority desc, position asc); the per-task values move
 //              through shared memory to the lane that owns the task's rank
 //   iterate    for each task in rank order the recurrence of Eq. 1 with the lemma set of the
@@ -596,43 +598,85 @@ __device__ __forceinline__ bool stage_fast(const KParams &p, bool live, i64 a, i
     GCAPS_LEAVE_IF_NONE_LIVE();
   }
 
-  // ---- aggregate: running sums of the segment arrays; per-task sums are differences --------
+  // ---- aggregate ---------------------------------------------------------------------------------
   u32 bad = 0;
   const i64 *__restrict__ Xc = p.cseg_wcet + cfirst;
   const i64 *__restrict__ Xm = p.gseg_misc + gfirst, *__restrict__ Xe = p.gseg_exec + gfirst;
-  const int parc = (int)(((uintptr_t)Xc >> 3) & 1), parm = (int)(((uintptr_t)Xm >> 3) & 1);
-  const int pare = (int)(((uintptr_t)Xe >> 3) & 1);
-  if (lane == 0) Q0[-1] = 0, Q1[-1] = 0;
-  {  // CPU segments -> Q0
-    const bool inside = slice_is_inside(cfirst, Nc, parc, p.n_csegs);
-    u32 carry = 0, unused = 0;
-#pragma unroll 1
-    for (int e0 = 0; more_steps<LPT>(e0, Nc + parc); e0 += Lay::kStep * BC)
-      prefix_step<LPT, BC, false>(Xc, Xc, e0, Nc, parc, parc, inside, p.cseg_wcet, p.cseg_wcet + p.n_csegs,
-                             p.cseg_wcet, p.cseg_wcet, Q0, Q0, carry, unused, bad, lane);
-  }
-  __syncwarp();
+  const int parm = (int)(((uintptr_t)Xm >> 3) & 1), pare = (int)(((uintptr_t)Xe >> 3) & 1);
+  if constexpr (LPT == 32 && (SLOTS <= 4 || !PREFETCH)) {
+    // A lane adds up the segments of its own tasks, kAtOnce of a kind at a time: independent loads in place of the
+    // chain of shuffles of running sums, which a warp per taskset waits for (redundant lines come out of L1).  From
+    // the running sums, GCAPS / RR: 1,000 tasksets of 8 tasks 8.2 / 8.4 -> 6.4 / 7.3 us, 12,288 of them 35 / 39 -> 31 /
+    // 33, of 80 tasks 51 / 55 -> 47 / 49, of 4 to 192 tasks 97 / 115 -> 73 / 88; GPU priorities of 100,000 tasksets of
+    // 80 tasks 720 -> 689; with a plan 100,000 of these 202 / 198 -> 201 / 195.  Four at once from three slots on: 4 to
+    // 192 tasks 73 -> 82.  The running sums stay for the one launch over more than 128 tasks, whose registers go from
+    // 128 to 168 otherwise (250 tasks under RR 113 -> 130), and for groups of 8 or 16 lanes, whose scans are short (32
+    // tasks under RR 146 -> 149, 30 on one core 96 -> 102).
+    constexpr int kAtOnce = SLOTS <= 2 ? 4 : 2;
 #pragma unroll
-  for (int s = 0; s < SLOTS; ++s) A[s] = Q0[c1[s] - 1 + parc] - Q0[c0[s] - 1 + parc];
-  __syncwarp();
-  {  // G^m -> Q0, G^e -> Q1
-    const bool inside = slice_is_inside(gfirst, Ng, parm, p.n_gsegs) &&
-                        slice_is_inside(gfirst, Ng, pare, p.n_gsegs);
-    u32 cm = 0, ce = 0;
+    for (int s = 0; s < SLOTS; ++s) A[s] = Ge[s] = 0;
 #pragma unroll 1
-    for (int e0 = 0; more_steps<LPT>(e0, Ng + 1); e0 += Lay::kStep * BG)
-      prefix_step<LPT, BG, true>(Xm, Xe, e0, Ng, parm, pare, inside, p.gseg_misc, p.gseg_misc + p.n_gsegs,
-                            p.gseg_exec, p.gseg_exec + p.n_gsegs, Q0, Q1, cm, ce, bad, lane);
-  }
-  __syncwarp();
+    for (int j0 = 0;; j0 += kAtOnce) {
+      bool more = false;
 #pragma unroll
-  for (int s = 0; s < SLOTS; ++s) {
-    const u32 Gm = Q0[g1[s] - 1 + parm] - Q0[g0[s] - 1 + parm];
-    Ge[s] = Q1[g1[s] - 1 + pare] - Q1[g0[s] - 1 + pare];
-    eta[s] = (u32)(g1[s] - g0[s]);
-    bad |= (A[s] | Gm | Ge[s]) >> 26;
-    A[s] += Gm;
-    bad |= A[s] >> 26;
+      for (int s = 0; s < SLOTS; ++s) more |= c0[s] + j0 < c1[s] || g0[s] + j0 < g1[s];
+      if (!__any_sync(kFull, more)) break;
+#pragma unroll
+      for (int s = 0; s < SLOTS; ++s) {
+        i64 w[kAtOnce], m[kAtOnce], e[kAtOnce];
+#pragma unroll
+        for (int j = 0; j < kAtOnce; ++j) {
+          w[j] = m[j] = e[j] = 0;
+          if (c0[s] + j0 + j < c1[s]) w[j] = __ldg(Xc + c0[s] + j0 + j);
+          if (g0[s] + j0 + j < g1[s]) m[j] = __ldg(Xm + g0[s] + j0 + j), e[j] = __ldg(Xe + g0[s] + j0 + j);
+        }
+        u32 lo = 0;
+#pragma unroll
+        for (int j = 0; j < kAtOnce; ++j) {
+          bad |= (u32)((u64)w[j] >> 32) | (u32)((u64)m[j] >> 32) | (u32)((u64)e[j] >> 32);
+          lo |= (u32)w[j] | (u32)m[j] | (u32)e[j];
+          A[s] += (u32)w[j] + (u32)m[j], Ge[s] += (u32)e[j];
+        }
+        bad |= (lo | A[s] | Ge[s]) >> 26;  // (sums below 2^26 grow by at most eight such values at a time)
+      }
+    }
+#pragma unroll
+    for (int s = 0; s < SLOTS; ++s) eta[s] = (u32)(g1[s] - g0[s]);
+  } else {
+    // running sums of the segment arrays; per-task sums are differences
+    const int parc = (int)(((uintptr_t)Xc >> 3) & 1);
+    if (lane == 0) Q0[-1] = 0, Q1[-1] = 0;
+    {  // CPU segments -> Q0
+      const bool inside = slice_is_inside(cfirst, Nc, parc, p.n_csegs);
+      u32 carry = 0, unused = 0;
+#pragma unroll 1
+      for (int e0 = 0; more_steps<LPT>(e0, Nc + parc); e0 += Lay::kStep * BC)
+        prefix_step<LPT, BC, false>(Xc, Xc, e0, Nc, parc, parc, inside, p.cseg_wcet, p.cseg_wcet + p.n_csegs,
+                               p.cseg_wcet, p.cseg_wcet, Q0, Q0, carry, unused, bad, lane);
+    }
+    __syncwarp();
+#pragma unroll
+    for (int s = 0; s < SLOTS; ++s) A[s] = Q0[c1[s] - 1 + parc] - Q0[c0[s] - 1 + parc];
+    __syncwarp();
+    {  // G^m -> Q0, G^e -> Q1
+      const bool inside = slice_is_inside(gfirst, Ng, parm, p.n_gsegs) &&
+                          slice_is_inside(gfirst, Ng, pare, p.n_gsegs);
+      u32 cm = 0, ce = 0;
+#pragma unroll 1
+      for (int e0 = 0; more_steps<LPT>(e0, Ng + 1); e0 += Lay::kStep * BG)
+        prefix_step<LPT, BG, true>(Xm, Xe, e0, Ng, parm, pare, inside, p.gseg_misc, p.gseg_misc + p.n_gsegs,
+                              p.gseg_exec, p.gseg_exec + p.n_gsegs, Q0, Q1, cm, ce, bad, lane);
+    }
+    __syncwarp();
+#pragma unroll
+    for (int s = 0; s < SLOTS; ++s) {
+      const u32 Gm = Q0[g1[s] - 1 + parm] - Q0[g0[s] - 1 + parm];
+      Ge[s] = Q1[g1[s] - 1 + pare] - Q1[g0[s] - 1 + pare];
+      eta[s] = (u32)(g1[s] - g0[s]);
+      bad |= (A[s] | Gm | Ge[s]) >> 26;
+      A[s] += Gm;
+      bad |= A[s] >> 26;
+    }
   }
   __syncwarp();
   // ---- what does not depend on the timeslice or the overhead ---------------------------------

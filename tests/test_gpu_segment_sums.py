@@ -1,0 +1,61 @@
+"""Tasksets of more than 32 tasks: the sums of a task's segments, from none to as many as the 32-bit path takes and
+beyond, below and above its 2^26 and where 32-bit sums would wrap, against the oracle."""
+import dataclasses
+
+import numpy as np
+import pytest
+
+from oracle import rta
+from paper_2406_05221_b200 import binding
+from tests.helpers import batch_of, direct_most
+
+pytestmark = pytest.mark.gpu
+
+BIG = 1 << 26
+
+
+def _taskset(rng, n, odd):
+    """Light tasks with 0 .. 5 segments of a kind, and one (odd: its segments) in their middle."""
+    ts = []
+    for i in range(n):
+        T = int(rng.integers(100_000, 2_000_000))
+        w = T // (8 * n)
+        c, g = int(rng.integers(0, 6)), int(rng.integers(0, 6))
+        ts.append(dict(T=T, D=T, core=i % 16, cseg=[int(rng.integers(0, w + 1)) for _ in range(c)],
+                       gseg=[(int(rng.integers(0, w + 1)), int(rng.integers(0, w + 1))) for _ in range(g)]))
+    ts[n // 2].update(odd)
+    for r, i in enumerate(sorted(range(n), key=lambda i: ts[i]["T"])):
+        ts[i]["prio"] = n - r
+    return ts
+
+
+ODD = [dict(), dict(cseg=[3] * 63, gseg=[(1, 2)] * 63), dict(cseg=[3] * 64), dict(gseg=[(1, 2)] * 64),
+       dict(cseg=[BIG - 1]), dict(cseg=[BIG]), dict(cseg=[1 << 32]), dict(gseg=[(0, 1 << 33)]), dict(gseg=[(1 << 34, 0)]),
+       dict(cseg=[BIG // 32] * 33), dict(gseg=[(0, BIG // 32)] * 33), dict(cseg=[BIG // 2], gseg=[(BIG // 2, 1)]),
+       dict(T=BIG - 1, D=BIG - 1, cseg=[BIG // 8] * 2, gseg=[(BIG // 8, 1)]),
+       # sums modulo 2^32 that are small again
+       dict(cseg=[BIG - 1] * 60, gseg=[(BIG - 1, 0)] * 4 + [(63, 0)]), dict(gseg=[(0, BIG - 1)] * 62 + [(0, 1)])]
+
+
+def _times(batch, k):
+    """The batch k times over."""
+    offs = {f: np.concatenate([[0], (np.diff(getattr(batch, f))[None].repeat(k, 0)).ravel().cumsum()])
+            for f in ("task_off", "cseg_off", "gseg_off")}
+    rest = [f.name for f in dataclasses.fields(batch) if f.name not in offs]
+    return dataclasses.replace(batch, **offs, **{f: np.tile(getattr(batch, f), k) for f in rest})
+
+
+@pytest.mark.parametrize("n", [33, 64, 65, 96, 97, 128, 129, 160, 161, 250])
+def test_segment_sums(n):
+    torch = pytest.importorskip("torch")
+    rng = np.random.default_rng(n)
+    few = batch_of([_taskset(rng, n, odd) for odd in ODD])
+    k = direct_most() // len(ODD) + 1
+    for batch, times in ((few, 1), (_times(few, k), k)):  # one launch, and the kernels behind a plan
+        dev = binding.DeviceTasksets.from_host(batch)
+        for policy in (0, 1, binding.BUSY, 1 | binding.BUSY):
+            wcrt, sched = binding.rta_batch(dev, policy, 256, 2)
+            torch.cuda.synchronize()
+            ref, ref_s, _ = rta.analyse(few, policy, 256, 2)
+            assert np.array_equal(wcrt.cpu().numpy(), np.tile(ref, times)), (times, policy)
+            assert np.array_equal(sched.cpu().numpy(), np.tile(ref_s, times)), (times, policy)
