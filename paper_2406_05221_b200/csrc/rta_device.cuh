@@ -7,8 +7,8 @@
 // One warp analyses one taskset at a time:
 //   stage      coalesced loads of the taskset's per-task slices into registers (lane = task)
 //   aggregate  the per-task sums C_i, G^m_i, G^e_i: added up by the lane of the task, or (groups of
-//              8 or 16 lanes) as differences of two running sums in shared memory, as the RR slice
-//              count of Eq. 3 is
+//              8 or 16 lanes with several tasks per lane) as differences of two running sums in
+//              shared memory, as the RR slice count of Eq. 3 is
 //   order      rank of every task by (priority desc, position asc); the per-task values move
 //              through shared memory to the lane that owns the task's rank
 //   iterate    for each task in rank order the recurrence of Eq. 1 with the lemma set of the
@@ -603,15 +603,17 @@ __device__ __forceinline__ bool stage_fast(const KParams &p, bool live, i64 a, i
   const i64 *__restrict__ Xc = p.cseg_wcet + cfirst;
   const i64 *__restrict__ Xm = p.gseg_misc + gfirst, *__restrict__ Xe = p.gseg_exec + gfirst;
   const int parm = (int)(((uintptr_t)Xm >> 3) & 1), pare = (int)(((uintptr_t)Xe >> 3) & 1);
-  if constexpr (LPT == 32 && (SLOTS <= 4 || !PREFETCH)) {
+  if (LPT != 32 && SLOTS == 1 && !live) c0[0] = c1[0] = g0[0] = g1[0] = 0;  // (a group that reads nothing)
+  if constexpr ((LPT == 32 && (SLOTS <= 4 || !PREFETCH)) || SLOTS == 1) {
     // A lane adds up the segments of its own tasks, kAtOnce of a kind at a time: independent loads in place of the
     // chain of shuffles of running sums, which a warp per taskset waits for (redundant lines come out of L1).  From
     // the running sums, GCAPS / RR: 1,000 tasksets of 8 tasks 8.2 / 8.4 -> 6.4 / 7.3 us, 12,288 of them 35 / 39 -> 31 /
     // 33, of 80 tasks 51 / 55 -> 47 / 49, of 4 to 192 tasks 97 / 115 -> 73 / 88; GPU priorities of 100,000 tasksets of
     // 80 tasks 720 -> 689; with a plan 100,000 of these 202 / 198 -> 201 / 195.  Four at once from three slots on: 4 to
     // 192 tasks 73 -> 82.  The running sums stay for the one launch over more than 128 tasks, whose registers go from
-    // 128 to 168 otherwise (250 tasks under RR 113 -> 130), and for groups of 8 or 16 lanes, whose scans are short (32
-    // tasks under RR 146 -> 149, 30 on one core 96 -> 102).
+    // 128 to 168 otherwise (250 tasks under RR 113 -> 130), and for groups of 8 or 16 lanes with two or three slots,
+    // whose scans are short (32 tasks under RR 146 -> 149, 30 on one core 96 -> 102).  With one slot, 300,000 tasksets
+    // of 2 to 8 tasks: 210 / 217 -> 192 / 198.
     constexpr int kAtOnce = SLOTS <= 2 ? 4 : 2;
 #pragma unroll
     for (int s = 0; s < SLOTS; ++s) A[s] = Ge[s] = 0;
