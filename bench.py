@@ -68,10 +68,10 @@ def kernel_launches(tasksets, kind="one", tasks=None, gcaps=True, walks=1):
 # ncu capture of a 131,072-taskset launch (traffic grows in proportion to the tasksets of a
 # launch).  Only reported while the kernel source is the one the counters were taken from.
 CAPTURED_TRAFFIC = {
-    "source_sha256": "972e6e00e9c56f786fcdcbe6c7a11e4093439c810413a8bbd9d999be90830c89",
+    "source_sha256": "11a88d485d7e1369e0e4bf41aa4a221e4f6fb2ed5c1cc613075113639210b093",
     "workload": "large",
-    "bytes_per_taskset": {"gcaps": (1236432000 + 80774144) / 131072.0,
-                          "rr": (1236322000 + 80674560) / 131072.0},
+    "bytes_per_taskset": {"gcaps": (1236501000 + 80218112) / 131072.0,
+                          "rr": (1236523000 + 80107520) / 131072.0},
 }
 
 
