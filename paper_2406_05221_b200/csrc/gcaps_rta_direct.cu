@@ -15,9 +15,10 @@ namespace {
 // these cannot fill the device.  12,288 tasksets of 8 / 20 / 80 / 128 / 192 tasks take 35 / 68 / 52 / 64 / 589 us
 // under GCAPS and 39 / 31 / 55 / 68 / 70 us under RR against 44 / 66 / 79 / 92 / 876 and 45 / 50 / 76 / 91 / 102 us
 // with a plan (busy-waiting modes within 10 % of these); 24,000 of 8 / 20 / 80 tasks 66 / 127 / 90 against
-// 49 / 85 / 90 us.  A mixture of 4 to 192 tasks: 95 against 120 us under GCAPS, but 114 against 91 us under RR,
-// whose line would lie at 9,000 tasksets; no argument of a call tells a mixture.  (Shared memory is set aside
-// for 256 tasks, which leaves 13 warps per SM.)
+// 49 / 85 / 90 us.  A mixture of 4 to 192 tasks: 95 against 120 us under GCAPS, but 114 against 91 us under RR.
+// (Shared memory is set aside for 256 tasks, which leaves 13 warps per SM.)  Since lanes add up their own tasks'
+// segments 12,288 of 8 / 20 / 80 tasks take 31 / 63 / 47 us under GCAPS and 33 / 27 / 49 us under RR, a mixture 73 and
+// 88 us; with a plan 13,000 of the mixture 119 and 92 us.
 constexpr int kDirectWords = bin_warp_words<32, 8>();
 template <int SLOTS, int MODE>
 __device__ __forceinline__ int direct_pass(const KParams &p, i64 t, i64 a, int n, u32 *buf, int lane) {
