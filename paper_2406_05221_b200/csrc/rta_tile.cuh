@@ -218,6 +218,7 @@ __device__ __forceinline__ void tile_stage(const KParams &p, const Rows &rows, T
         bad |= (u32)(all >> 32) | ((u32)all >> 26);
         A[u] = ((u32)w[u][0] + (u32)w[u][1]) + ((u32)w[u][2] + (u32)w[u][3]) + ((u32)m[u][0] + (u32)m[u][1]) + (u32)m[u][2];
         Ge[u] = (u32)e[u][0] + (u32)e[u][1] + (u32)e[u][2];
+        bad |= (A[u] | Ge[u]) >> 26;  // seven values below 2^26 do not wrap, nor does a sum below 2^26 with one or two more
 #pragma unroll
         for (u32 j = 0; j < 3; ++j)
           if (j < gn[u]) rows.keep_segment(c, rg[u] + j, (u32)e[u][j]);
@@ -229,12 +230,14 @@ __device__ __forceinline__ void tile_stage(const KParams &p, const Rows &rows, T
 #pragma unroll 1
       for (u32 j = 4; j < cn[u]; ++j) {
         const u64 w = (u64)__ldg(xc + rc[u] + j);
-        bad |= (u32)(w >> 32) | ((u32)w >> 26), A[u] += (u32)w;
+        A[u] += (u32)w;
+        bad |= (u32)(w >> 32) | (((u32)w | A[u]) >> 26);
       }
 #pragma unroll 1
       for (u32 j = 3; j < gn[u]; ++j) {
         const u64 m = (u64)__ldg(xm + rg[u] + j), e = (u64)__ldg(xe + rg[u] + j);
-        bad |= (u32)((m | e) >> 32) | ((u32)(m | e) >> 26), A[u] += (u32)m, Ge[u] += (u32)e;
+        A[u] += (u32)m, Ge[u] += (u32)e;
+        bad |= (u32)((m | e) >> 32) | (((u32)(m | e) | A[u] | Ge[u]) >> 26);
         rows.keep_segment(c, rg[u] + j, (u32)e);
         if (SLICES) slices[u] += slices_of((u32)e);
       }

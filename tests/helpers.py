@@ -6,7 +6,7 @@ import os
 import numpy as np
 
 from paper_2406_05221_b200 import build
-from paper_2406_05221_b200.taskgen import TasksetBatch
+from paper_2406_05221_b200.taskgen import ARRAY_FIELDS, TasksetBatch
 
 GOLDEN = os.path.join(os.path.dirname(os.path.abspath(__file__)), "golden")
 
@@ -93,6 +93,19 @@ def with_fillers(batch, several=False, middle=False):
     fillers = [few] * (max(0, direct_most(several) - batch.n_tasksets) // 64 + 1)
     half = batch.n_tasksets // 2 if middle else batch.n_tasksets
     return TasksetBatch.concat([batch.slice(0, half)] + fillers + [batch.slice(half, batch.n_tasksets)])
+
+
+def repeated(batch, k):
+    """The batch k times over."""
+    offs = {f: np.concatenate([[0], np.tile(np.diff(getattr(batch, f)), k).cumsum()]) for f in ("task_off", "cseg_off", "gseg_off")}
+    return TasksetBatch(**{f: offs[f] if f in offs else np.tile(getattr(batch, f), k) for f in ARRAY_FIELDS})
+
+
+def left_by_tiles(workspace):
+    """Tasksets that a call through tiles left to the launches behind it, from the header in its workspace.  (After
+    a call with a plan these counters hold the tasksets of all size bins.)"""
+    import torch
+    return int(workspace[:256].view(torch.int32)[12:21].sum())
 
 
 def both_ways(batch, several=False):
