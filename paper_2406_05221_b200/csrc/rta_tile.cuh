@@ -25,6 +25,7 @@
 #include <stdint.h>
 
 #include "rta_device.cuh"
+#include "tile_patience.h"
 
 namespace {
 
@@ -538,29 +539,29 @@ __device__ __forceinline__ void run_tiles(const KParams &p, int n_rows, const Ro
   i64 b;
   look_up(first, me, b);
   settle(me, b);
-  int passed_by = 0;  // tiles that are left over unseen: three quarters of the one in front of them were left over
+  TilePatience patience = {0};
 #pragma unroll 1
   while (first < count) {
-    if (passed_by > 0 && me.n > 0) me.declined = true, me.n = 0;
+    const bool looks = patience.looks();
+    if (!looks && me.n > 0) me.declined = true, me.n = 0;
     const unsigned int asked = pull();
     const int columns = count - first < chunk ? (int)(count - first) : (int)chunk;
     look_up(second, coming, b);
 #pragma unroll 1
-    for (int c0 = 0; c0 < columns; c0 += 32 / kTileGroup) {
+    for (int c0 = 0; looks && c0 < columns; c0 += 32 / kTileGroup) {
       if (n_rows <= 8) tile_stage<1, SLICES>(p, rows, me, c0, lane);
       else if (n_rows <= 16) tile_stage<2, SLICES>(p, rows, me, c0, lane);
       else tile_stage<3, SLICES>(p, rows, me, c0, lane);
       // (none of the first ones: the others are passed by as well)
       if (c0 == 0 && columns >= 4 && (__ballot_sync(kFull, me.declined) & 0xfu) == 0xfu) {
         if (me.n > 0) me.declined = true, me.n = 0;
-        passed_by = 8;
         break;
       }
     }
     __syncwarp();
     const unsigned int third = __shfl_sync(kFull, asked, 0);
     settle(coming, b);
-    if (coming.n > 0 && passed_by <= 1) {
+    if (coming.n > 0 && patience.unseen <= 1) {
       const i64 to = coming.a + coming.n;
       ask_for(p.cseg_off, coming.a, to), ask_for(p.gseg_off, coming.a, to);
       ask_for(p.period, coming.a, to), ask_for(p.deadline, coming.a, to), ask_for(p.priority, coming.a, to), ask_for(p.core, coming.a, to);
@@ -571,8 +572,7 @@ __device__ __forceinline__ void run_tiles(const KParams &p, int n_rows, const Ro
     if (!walk(me) && me.n > 0) me.declined = true;
     list(me.declined && me.size >= 1 && me.size <= 24, me.t, kRestSmall);
     list(me.declined && !(me.size >= 1 && me.size <= 24), me.t, kRestLarge);
-    const int left = __popc(__ballot_sync(kFull, me.declined));
-    passed_by = passed_by > 0 ? passed_by - 1 : (4 * left >= 3 * columns ? 7 : 0);
+    patience.done(__popc(__ballot_sync(kFull, me.declined)), columns);
     __syncwarp();
     me = coming;
     first = second, second = third;
