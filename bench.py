@@ -42,7 +42,7 @@ K_TERM, K_SETUP = 6, 16   # algorithmic integer lane-operations per interference
 
 
 def in_tiles(tasksets, tasks, gcaps, walks):
-    """Whether a batch too large for one launch without a plan goes through tiles (tile_rows of gcaps_rta.cu):
+    """Whether a batch too large for one launch without a plan goes through tiles (tile_tasks of gcaps_rta.cu):
     small tasksets of one size, and under GCAPS enough of them.  `walks`: analyses of a policy per taskset."""
     if not tasks or tasks % tasksets or tasks > 24 * tasksets:
         return False
@@ -53,14 +53,14 @@ def in_tiles(tasksets, tasks, gcaps, walks):
 def kernel_launches(tasksets, kind="one", tasks=None, gcaps=True, walks=1):
     """Kernels of one call on a batch: "one" analysis, "several" (a sweep, or analyses of one waiting
     mode) or a "search" of GPU priorities.  Small batches are one launch without a plan.  Tiles take one
-    launch, and two more what these left over.  Otherwise the
+    launch, and three more what these left over (the rest of a plan among them, for mixtures).  Otherwise the
     plan takes one kernel or three; then one kernel serves the bins of up to 32 tasks, one each those of
     up to 64, 96, 128, 192 and 256, and for a single analysis two more, for a search one more, what
     these left over."""
     if tasksets <= build.source_constant("kDirectMost" if kind == "one" else "kDirectSweepMost"):
         return 1
     if kind != "search" and (kind == "one" or walks > 1) and in_tiles(tasksets, tasks, gcaps, walks):
-        return 3
+        return 4
     return (1 if tasksets <= build.source_constant("kPlanSmall") else 3) + {"one": 8, "several": 6, "search": 7}[kind]
 
 

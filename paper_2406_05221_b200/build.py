@@ -12,6 +12,7 @@ CUDA_SRC = os.path.join(_HERE, "csrc", "gcaps_rta.cu")
 CUDA_SRCS = [CUDA_SRC, os.path.join(_HERE, "csrc", "gcaps_rta_tile.cu"),
              os.path.join(_HERE, "csrc", "gcaps_rta_direct.cu"),
              os.path.join(_HERE, "csrc", "gcaps_rta_sweep.cu"),
+             os.path.join(_HERE, "csrc", "gcaps_rta_rest.cu"), os.path.join(_HERE, "csrc", "gcaps_rta_rest_sweep.cu"),
              os.path.join(_HERE, "csrc", "gcaps_rta_tile_q2.cu"), os.path.join(_HERE, "csrc", "gcaps_rta_tile_q4.cu"),
              os.path.join(_HERE, "csrc", "gcaps_rta_direct_sweep.cu"),
              os.path.join(_HERE, "csrc", "gcaps_gpu_priority.cu"),

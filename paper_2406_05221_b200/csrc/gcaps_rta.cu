@@ -117,14 +117,47 @@ __global__ void __launch_bounds__(1024) plan_small_kernel(KParams p) {
   }
 }
 
+// Behind tiles: where the batch was none for them they have counted its size bins, and this is the rest of the plan.  Blocks of
+// tasksets get their places in the permutation from a counter per bin.
+__global__ void __launch_bounds__(256) plan_behind_tiles_kernel(KParams p) {
+  __shared__ unsigned int cnt[kBinStride], cursor[kBinStride];
+  wait_for_previous_grid();
+  let_dependents_start();
+  if (p.hdr->in_tiles) return;
+  const int bin = threadIdx.x;
+  unsigned int start = 0;
+  if (bin < kNumBins) {
+    for (int k = 0; k < bin; ++k) start += p.hdr->bin_count[k];
+    if (blockIdx.x == 0) p.hdr->bin_start[bin] = start;
+  }
+#pragma unroll 1
+  for (i64 t0 = (i64)blockIdx.x * kPlanItems; t0 < p.n_tasksets; t0 += (i64)gridDim.x * kPlanItems) {
+    if (bin < kNumBins) cnt[bin] = 0;
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kPlanItems; k += 256) {
+      const i64 t = t0 + k + threadIdx.x;
+      if (t < p.n_tasksets) atomicAdd(&cnt[size_bin(p.task_off[t + 1] - p.task_off[t])], 1u);
+    }
+    __syncthreads();
+    if (bin < kNumBins) cursor[bin] = start + atomicAdd(&p.hdr->next2[bin], cnt[bin]);
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kPlanItems; k += 256) {
+      const i64 t = t0 + k + threadIdx.x;
+      if (t < p.n_tasksets) p.perm[atomicAdd(&cursor[size_bin(p.task_off[t + 1] - p.task_off[t])], 1u)] = (unsigned int)t;
+    }
+    __syncthreads();
+  }
+}
+
 // The bins of up to 32 tasks in one persistent launch, largest tasksets first: (lanes per
 // taskset, tasks per lane) = (16,2) (8,3) (8,2) (8,1) for at most 32, 24, 16, 8 tasks, i.e. two or
 // four tasksets per warp.  (A look at the first ranks out of a stage, a warp per taskset, was slower
 // here in every form tried: 100,000 24-task tasksets under round robin 163 us against 128.)
 template <int MODE>
-__global__ void __launch_bounds__(kBlockThreads, min_blocks(3)) rta_small_kernel(KParams p, bool rest) {
+__global__ void __launch_bounds__(kBlockThreads, min_blocks(3)) rta_small_kernel(KParams p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  if (rest) wait_for_previous_grid();  // what the tiles left over is listed from here on
   let_dependents_start();  // the kernel of the next size bin shares no data with this one
   u32 *warp_buf = reinterpret_cast<u32 *>(smem_raw) + (threadIdx.x >> 5) * kSmallWarpWords;
   Ahead *ahead = reinterpret_cast<Ahead *>(warp_buf + kSmallWarpWords - kAheadWords);
@@ -386,29 +419,25 @@ cudaError_t launch_deferred(const KParams &p, int sm_count, cudaStream_t st) {
                               (p.n_tasksets + kWarps - 1) / kWarps, sm_count, st, p);
 }
 
-template <int MODE>
-int small_blocks[64] = {0};  // resident blocks of rta_small_kernel per SM
-
-// Behind tiles: what they listed of up to 24 tasks.
-cudaError_t launch_rest(int mode, const KParams &p, int sm_count, cudaStream_t st) {
-  auto rest = [&](auto kernel, int *blocks) {
-    constexpr int kWarps = kBlockThreads / 32;
-    return launch_persistent_ex(true, kernel, blocks, sizeof(u32) * kSmallWarpWords * kWarps, (p.n_tasksets + kWarps - 1) / kWarps,
-                                sm_count, st, p, true);
-  };
-  switch (mode) {
-    case 0: return rest(rta_small_kernel<0>, small_blocks<0>);
-    case 1: return rest(rta_small_kernel<1>, small_blocks<1>);
-    case 2: return rest(rta_small_kernel<2>, small_blocks<2>);
-    default: return rest(rta_small_kernel<3>, small_blocks<3>);
-  }
+cudaError_t launch_plan_behind_tiles(const KParams &p, int sm_count, cudaStream_t st) {
+  const i64 blocks = (p.n_tasksets + kPlanItems - 1) / kPlanItems, most = (i64)sm_count * 8;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned int)(blocks < most ? blocks : most)), cfg.blockDim = dim3(256);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr, cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, plan_behind_tiles_kernel, p);
 }
 
 template <int MODE>
 cudaError_t launch_all_bins(const KParams &p, int sm_count, cudaStream_t st) {
   constexpr int kWarps = kBlockThreads / 32;
-  cudaError_t e = launch_persistent(rta_small_kernel<MODE>, small_blocks<MODE>, sizeof(u32) * kSmallWarpWords * kWarps,
-                                    (p.n_tasksets + kWarps - 1) / kWarps, sm_count, st, p, false);
+  static int blocks_per_sm[64] = {0};
+  const size_t smem = sizeof(u32) * kSmallWarpWords * kWarps;
+  cudaError_t e = launch_persistent(rta_small_kernel<MODE>, blocks_per_sm, smem,
+                                    (p.n_tasksets + kWarps - 1) / kWarps, sm_count, st, p);
   if (e == cudaSuccess) e = launch_big<2, MODE>(p, 4, sm_count, st);
   if (e == cudaSuccess) e = launch_big<3, MODE>(p, 5, sm_count, st);
   if (e == cudaSuccess) e = launch_big<4, MODE>(p, 6, sm_count, st);
@@ -427,15 +456,15 @@ cudaError_t launch_all_bins(const KParams &p, int sm_count, cudaStream_t st) {
 // (24 tasks 40 / 51 us at 12,500).  Several analyses under GCAPS, 20 tasks: 170 / 138 us for five pairs of 10,000
 // tasksets, 243 / 240 of 20,000, 212 / 280 for three pairs of 50,000; 24 tasks: 203 / 182 for two pairs of 30,000, 578 / 654 for
 // 25 pairs of 5,000.  32 tasks: 575 / 521 us per 100,000, as a tile then takes 40 KB.
-// Returns the rows that tiles of this batch need, or 0: no tiles.  `analyses`: those of the call; `walks`: how many of a policy
+// Returns how many tasks the tasksets have, or 0: no tiles.  `analyses`: those of the call; `walks`: how many of a policy
 // every taskset goes through.
-int tile_rows(int analyses, int walks, i64 max_ovh, const KParams &p) {
+int tile_tasks(int analyses, int walks, i64 max_ovh, const KParams &p) {
   if (max_ovh >= (1 << 20) || ((analyses & 2) && (p.policy & GCAPS_RTA_LITERAL))) return 0;
   if (p.n_tasks % p.n_tasksets != 0 || p.n_tasks > kTileMost * p.n_tasksets) return 0;
   const int n = (int)(p.n_tasks / p.n_tasksets);
   if (walks == 1 && (analyses & 3) && n > 12 && p.n_tasksets < 1750 * n) return 0;
   if (walks > 1 && (analyses & 12) == 0 && n > 12 && p.n_tasksets * walks < 100000) return 0;
-  return n < 4 ? 4 : n;
+  return n;
 }
 
 // Plan + analysis launches of one call.  `sw` null: one analysis (p.policy).  Otherwise the
@@ -459,14 +488,14 @@ int enqueue_batch(KParams p, void *workspace, size_t workspace_bytes, int sm_cou
   // walks of a taskset through the recurrence that a tile's lanes share.  (A single one of GCAPS and of RR each is better
   // left to the groups of lanes, which stage once for both: 288 us for 100,001 tasksets of 20 tasks, 323 in tiles.)
   const int walks = sw ? sw->n * (((analyses & 3) == 3 || (analyses & 12) == 12) ? 2 : 1) : 1;
-  const int rows = direct || (sw && walks == 1) ? 0 : tile_rows(sw ? analyses : 1 << mode, walks, sw ? sw->max_ovh : p.ovh, p);
-  if (!direct && rows == 0) enqueue_plan_kernels(p, st);
+  const int tile_n = direct || (sw && walks == 1) ? 0 : tile_tasks(sw ? analyses : 1 << mode, walks, sw ? sw->max_ovh : p.ovh, p);
+  if (!direct && tile_n == 0) enqueue_plan_kernels(p, st);
   cudaError_t e = cudaGetLastError();
-  if (e == cudaSuccess && rows > 0) e = cudaMemsetAsync(p.hdr, 0, sizeof(PlanHeader), st);
-  if (e == cudaSuccess && rows > 0 && !sw) {
-    e = launch_tiles(mode, p, rows, sm_count, st);
+  if (e == cudaSuccess && tile_n > 0) e = cudaMemsetAsync(p.hdr, 0, sizeof(PlanHeader), st);
+  if (e == cudaSuccess && tile_n > 0 && !sw) {
+    e = launch_tiles(mode, p, tile_n, sm_count, st);
+    if (e == cudaSuccess) e = launch_plan_behind_tiles(p, sm_count, st);
     if (e == cudaSuccess) e = launch_rest(mode, p, sm_count, st);
-    if (e == cudaSuccess) e = launch_listed_tasksets(mode, p, sm_count, st);
   } else if (e == cudaSuccess && sw) {
     SweepArgs set = *sw;
     set.block_stride = __builtin_popcount(analyses);
@@ -475,9 +504,10 @@ int enqueue_batch(KParams p, void *workspace, size_t workspace_bytes, int sm_cou
       k += (analyses >> m) & 1;
     }
     bool first = true;
-    if (rows > 0) {
+    if (tile_n > 0) {
       set.enabled = analyses;
-      e = walks > kKeptFew ? launch_tile_q4(p, set, rows, sm_count, st) : launch_tile_q2(p, set, rows, sm_count, st);
+      e = walks > kKeptFew ? launch_tile_q4(p, set, tile_n, sm_count, st) : launch_tile_q2(p, set, tile_n, sm_count, st);
+      if (e == cudaSuccess) e = launch_plan_behind_tiles(p, sm_count, st);
     }
     for (int half = 0; half < 2 && e == cudaSuccess; ++half) {
       set.enabled = analyses & (half == 0 ? 5 : 10);
@@ -486,9 +516,8 @@ int enqueue_batch(KParams p, void *workspace, size_t workspace_bytes, int sm_cou
       first = false;
       if (e == cudaSuccess)
         e = direct     ? launch_sweep_one_warp_each(p, set, sm_count, st)
-            : rows > 0 ? launch_sweep_rest(p, set, sm_count, st)
+            : tile_n > 0 ? launch_sweep_rest(p, set, sm_count, st)
                        : launch_sweep_set(p, set, sm_count, st);
-      if (e == cudaSuccess && rows > 0) e = launch_sweep_listed(p, set, sm_count, st);
     }
   } else if (e == cudaSuccess) {
     if (direct) e = launch_one_warp_each(mode, p, st);

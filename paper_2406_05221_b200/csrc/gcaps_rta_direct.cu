@@ -25,7 +25,11 @@ __device__ __forceinline__ int direct_pass(const KParams &p, i64 t, i64 a, int n
   return analyse_fast<32, SLOTS, 1 << MODE, false, true>(p, true, t, a, n, buf, lane, kFull);
 }
 template <int MODE>
-__device__ __forceinline__ void direct_taskset(const KParams &p, i64 t, u32 *buf, int lane) {
+__global__ void __launch_bounds__(32) rta_direct_kernel(KParams p) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  u32 *const buf = reinterpret_cast<u32 *>(smem_raw);
+  const int lane = threadIdx.x;
+  const i64 t = blockIdx.x;
   const i64 a = p.task_off[t] - p.task_base, b = p.task_off[t + 1] - p.task_base;
   int how = kFastDeclined;
   if (a >= 0 && b > a && b <= p.n_tasks && b - a <= GCAPS_RTA_MAX_TASKS && p.ovh < (1 << 20)) {
@@ -40,39 +44,14 @@ __device__ __forceinline__ void direct_taskset(const KParams &p, i64 t, u32 *buf
   __syncwarp();
   if (how != kFastDone)  // the exact path reads task_off again and validates everything itself
     analyse_taskset<32, 256>(p, t, *reinterpret_cast<GroupSmem<256> *>(buf), lane, kFull);
-  __syncwarp();
-}
-
-// LISTED: the tasksets that tiles left over and that the kernel in front of this one did not take (kRestLarge).
-template <int MODE, bool LISTED>
-__global__ void __launch_bounds__(32) rta_direct_kernel(KParams p) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  u32 *const buf = reinterpret_cast<u32 *>(smem_raw);
-  if constexpr (LISTED) {
-    wait_for_previous_grid();
-    const unsigned int count = __ldcg(&p.hdr->bin_count[kRestLarge]);
-#pragma unroll 1
-    for (unsigned int k = blockIdx.x; k < count; k += gridDim.x)
-      direct_taskset<MODE>(p, (i64)__ldcg(&p.perm[(unsigned int)p.n_tasksets - 1u - k]), buf, threadIdx.x);
-  } else {
-    direct_taskset<MODE>(p, blockIdx.x, buf, threadIdx.x);
-  }
 }
 
 template <int MODE>
 cudaError_t launch_direct(const KParams &p, cudaStream_t st) {
   constexpr int smem = (int)(sizeof(u32) * kDirectWords);
   static_assert(sizeof(GroupSmem<256>) <= (size_t)smem && smem <= 48 * 1024, "no attribute to set");
-  rta_direct_kernel<MODE, false><<<(unsigned int)p.n_tasksets, 32, smem, st>>>(p);
+  rta_direct_kernel<MODE><<<(unsigned int)p.n_tasksets, 32, smem, st>>>(p);
   return cudaGetLastError();
-}
-
-template <int MODE>
-cudaError_t launch_listed(const KParams &p, int sm_count, cudaStream_t st) {
-  static int by_registers[64] = {0};
-  constexpr size_t smem = sizeof(u32) * kDirectWords;
-  return launch_staged<32>(true, rta_direct_kernel<MODE, true>, by_registers, smem, smem, kSmemPerSm / (smem + 1024),
-                           p.n_tasksets, sm_count, st, p);
 }
 
 }  // namespace
@@ -85,16 +64,6 @@ cudaError_t launch_one_warp_each(int mode, const KParams &p, cudaStream_t st) {
     case 1: return launch_direct<1>(p, st);
     case 2: return launch_direct<2>(p, st);
     case 3: return launch_direct<3>(p, st);
-    default: return cudaErrorInvalidValue;
-  }
-}
-
-cudaError_t launch_listed_tasksets(int mode, const KParams &p, int sm_count, cudaStream_t st) {
-  switch (mode) {
-    case 0: return launch_listed<0>(p, sm_count, st);
-    case 1: return launch_listed<1>(p, sm_count, st);
-    case 2: return launch_listed<2>(p, sm_count, st);
-    case 3: return launch_listed<3>(p, sm_count, st);
     default: return cudaErrorInvalidValue;
   }
 }

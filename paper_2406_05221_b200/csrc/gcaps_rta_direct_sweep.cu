@@ -14,7 +14,12 @@ constexpr int kDirectWords = bin_warp_words<32, 8>();
 // kernels).  4,000 tasksets take 79 to 202 us here and 80 to 278 us there; 8,192 tasksets up to 346
 // against 258 us.
 template <int MASK>
-__device__ __forceinline__ void direct_taskset(const KParams &p, const SweepArgs &sw, i64 t, int q0, int q1, u32 *buf, int lane) {
+__global__ void __launch_bounds__(32) rta_direct_sweep_kernel(KParams p, const __grid_constant__ SweepArgs sw) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  u32 *const buf = reinterpret_cast<u32 *>(smem_raw);
+  const int lane = threadIdx.x;
+  const i64 t = blockIdx.x;
+  const int q0 = (int)(blockIdx.y * sw.n / gridDim.y), q1 = (int)((blockIdx.y + 1) * sw.n / gridDim.y);
   const i64 a = p.task_off[t] - p.task_base, b = p.task_off[t + 1] - p.task_base;
   int how = kFastDeclined;
   if (a >= 0 && b > a && b <= p.n_tasks && b - a <= GCAPS_RTA_MAX_TASKS && sw.max_ovh < (1 << 20)) {
@@ -29,32 +34,6 @@ __device__ __forceinline__ void direct_taskset(const KParams &p, const SweepArgs
   __syncwarp();
   if (how != kFastDone)
     exact_by_pair<32, 256, MASK>(p, sw, t, *reinterpret_cast<GroupSmem<256> *>(buf), lane, kFull, q0, q1);
-  __syncwarp();
-}
-
-// LISTED: the tasksets that tiles left over and that the kernel in front of this one did not take (kRestLarge).
-template <int MASK, bool LISTED>
-__global__ void __launch_bounds__(32) rta_direct_sweep_kernel(KParams p, const __grid_constant__ SweepArgs sw) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  u32 *const buf = reinterpret_cast<u32 *>(smem_raw);
-  if constexpr (LISTED) {
-    wait_for_previous_grid();
-    const unsigned int count = __ldcg(&p.hdr->bin_count[kRestLarge]);
-#pragma unroll 1
-    for (unsigned int k = blockIdx.x; k < count; k += gridDim.x)
-      direct_taskset<MASK>(p, sw, (i64)__ldcg(&p.perm[(unsigned int)p.n_tasksets - 1u - k]), 0, sw.n, buf, threadIdx.x);
-  } else {
-    direct_taskset<MASK>(p, sw, blockIdx.x, (int)(blockIdx.y * sw.n / gridDim.y), (int)((blockIdx.y + 1) * sw.n / gridDim.y), buf,
-                         threadIdx.x);
-  }
-}
-
-template <int MASK>
-cudaError_t launch_listed(const KParams &p, const SweepArgs &sw, int sm_count, cudaStream_t st) {
-  static int by_registers[64] = {0};
-  constexpr size_t smem = sizeof(u32) * kDirectWords;
-  return launch_staged<32>(true, rta_direct_sweep_kernel<MASK, true>, by_registers, smem, smem, kSmemPerSm / (smem + 1024),
-                           p.n_tasksets, sm_count, st, p, sw);
 }
 
 template <int MASK>
@@ -63,7 +42,7 @@ cudaError_t launch_direct_sweep(const KParams &p, const SweepArgs &sw, int sm_co
   static_assert(sizeof(GroupSmem<256>) <= (size_t)smem && smem <= 48 * 1024, "no attribute to set");
   long long shares = 16LL * sm_count / p.n_tasksets;
   shares = shares < 1 ? 1 : shares > sw.n ? sw.n : shares;
-  rta_direct_sweep_kernel<MASK, false><<<dim3((unsigned int)p.n_tasksets, (unsigned int)shares), 32, smem, st>>>(p, sw);
+  rta_direct_sweep_kernel<MASK><<<dim3((unsigned int)p.n_tasksets, (unsigned int)shares), 32, smem, st>>>(p, sw);
   return cudaGetLastError();
 }
 
@@ -79,18 +58,6 @@ cudaError_t launch_sweep_one_warp_each(const KParams &p, const SweepArgs &sw, in
     case 8: return launch_direct_sweep<8>(p, sw, sm_count, st);
     case 5: return launch_direct_sweep<5>(p, sw, sm_count, st);
     case 10: return launch_direct_sweep<10>(p, sw, sm_count, st);
-    default: return cudaErrorInvalidValue;
-  }
-}
-
-cudaError_t launch_sweep_listed(const KParams &p, const SweepArgs &sw, int sm_count, cudaStream_t st) {
-  switch (sw.enabled) {
-    case 1: return launch_listed<1>(p, sw, sm_count, st);
-    case 2: return launch_listed<2>(p, sw, sm_count, st);
-    case 4: return launch_listed<4>(p, sw, sm_count, st);
-    case 8: return launch_listed<8>(p, sw, sm_count, st);
-    case 5: return launch_listed<5>(p, sw, sm_count, st);
-    case 10: return launch_listed<10>(p, sw, sm_count, st);
     default: return cudaErrorInvalidValue;
   }
 }

@@ -10,9 +10,8 @@ namespace {
 // (timeslice, overhead) pairs of `sw`.
 template <int MASK>
 __global__ void __launch_bounds__(kBlockThreads, min_blocks(3))
-rta_small_sweep_kernel(KParams p, const __grid_constant__ SweepArgs sw, bool rest) {
+rta_small_sweep_kernel(KParams p, const __grid_constant__ SweepArgs sw) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  if (rest) wait_for_previous_grid();  // what the tiles left over is listed from here on
   let_dependents_start();  // the kernel of the next size bin shares no data with this one
   u32 *warp_buf = reinterpret_cast<u32 *>(smem_raw) + (threadIdx.x >> 5) * kSmallWarpWords;
   Ahead *ahead = reinterpret_cast<Ahead *>(warp_buf + kSmallWarpWords - kAheadWords);
@@ -45,17 +44,12 @@ cudaError_t launch_big_sweep(const KParams &p, const SweepArgs &sw, int bin, int
 }
 
 template <int MASK>
-cudaError_t launch_small_sweep(const KParams &p, const SweepArgs &sw, bool rest, int sm_count, cudaStream_t st) {
+cudaError_t launch_all_bins_sweep(const KParams &p, const SweepArgs &sw, int sm_count, cudaStream_t st) {
   constexpr int kWarps = kBlockThreads / 32;
   static int blocks_per_sm[64] = {0};
   const size_t smem = sizeof(u32) * kSmallWarpWords * kWarps;
-  return launch_persistent_ex(rest, rta_small_sweep_kernel<MASK>, blocks_per_sm, smem, (p.n_tasksets + kWarps - 1) / kWarps,
-                              sm_count, st, p, sw, rest);
-}
-
-template <int MASK>
-cudaError_t launch_all_bins_sweep(const KParams &p, const SweepArgs &sw, int sm_count, cudaStream_t st) {
-  cudaError_t e = launch_small_sweep<MASK>(p, sw, false, sm_count, st);
+  cudaError_t e = launch_persistent(rta_small_sweep_kernel<MASK>, blocks_per_sm, smem,
+                                    (p.n_tasksets + kWarps - 1) / kWarps, sm_count, st, p, sw);
   if (e == cudaSuccess) e = launch_big_sweep<2, MASK>(p, sw, 4, sm_count, st);
   if (e == cudaSuccess) e = launch_big_sweep<3, MASK>(p, sw, 5, sm_count, st);
   if (e == cudaSuccess) e = launch_big_sweep<4, MASK>(p, sw, 6, sm_count, st);
@@ -76,18 +70,6 @@ cudaError_t launch_sweep_set(const KParams &p, const SweepArgs &sw, int sm_count
     case 8: return launch_all_bins_sweep<8>(p, sw, sm_count, st);
     case 5: return launch_all_bins_sweep<5>(p, sw, sm_count, st);   // GCAPS + RR, self-suspension
     case 10: return launch_all_bins_sweep<10>(p, sw, sm_count, st);  // GCAPS + RR, busy-waiting
-    default: return cudaErrorInvalidValue;
-  }
-}
-
-cudaError_t launch_sweep_rest(const KParams &p, const SweepArgs &sw, int sm_count, cudaStream_t st) {
-  switch (sw.enabled) {
-    case 1: return launch_small_sweep<1>(p, sw, true, sm_count, st);
-    case 2: return launch_small_sweep<2>(p, sw, true, sm_count, st);
-    case 4: return launch_small_sweep<4>(p, sw, true, sm_count, st);
-    case 8: return launch_small_sweep<8>(p, sw, true, sm_count, st);
-    case 5: return launch_small_sweep<5>(p, sw, true, sm_count, st);
-    case 10: return launch_small_sweep<10>(p, sw, true, sm_count, st);
     default: return cudaErrorInvalidValue;
   }
 }

@@ -4,10 +4,10 @@
 
 namespace gcaps_detail {
 
-cudaError_t launch_tile_q4(const KParams &p, const SweepArgs &sw, int rows, int sm_count, cudaStream_t st) {
-  if ((sw.enabled & 12) == 0) return launch_kept<kKindGcaps, 4>(p, sw, rows, sm_count, st);
-  if ((sw.enabled & 3) == 0) return launch_kept<kKindRr, 4>(p, sw, rows, sm_count, st);
-  return launch_kept<kKindGcaps | kKindRr, 4>(p, sw, rows, sm_count, st);
+cudaError_t launch_tile_q4(const KParams &p, const SweepArgs &sw, int n, int sm_count, cudaStream_t st) {
+  if ((sw.enabled & 12) == 0) return launch_kept<kKindGcaps, 4>(p, sw, n, sm_count, st);
+  if ((sw.enabled & 3) == 0) return launch_kept<kKindRr, 4>(p, sw, n, sm_count, st);
+  return launch_kept<kKindGcaps | kKindRr, 4>(p, sw, n, sm_count, st);
 }
 
 }  // namespace gcaps_detail

@@ -36,14 +36,17 @@ struct PlanHeader {
   unsigned int bin_start[kBinStride];
   unsigned int bin_count[kBinStride];
   unsigned int next[kBinStride];      // work counters of the analysis launches
-  unsigned int next2[kNumBins];     // ... of the second launches over the deferred tasksets
+  unsigned int next2[kNumBins];     // ... of the second launches over the deferred tasksets; behind tiles, tasksets scattered
   unsigned int deferred[kNumBins];  // tasksets the first launch left to the second
   // of each warp's first taskset in the first launch: how many there were (low half) and how many
   // the first ranks did not decide (high half)
   unsigned int first_tries[kNumBins];
+  unsigned int in_tiles;  // the batch goes through tiles (tile_batch)
 };
-// bins that list what tiles leave over (rta_tile.cuh)
-constexpr int kRestSmall = 2, kRestLarge = 8;
+// the bin that lists what tiles leave over (rta_tile.cuh) beside the one of the batch's size
+constexpr int kRestLarge = kNumBins - 1;
+constexpr int kNextTile = kNumBins;  // the work counter of tiles, which is no bin's
+static_assert(kNextTile < kBinStride, "a word of the header");
 constexpr unsigned int kDeferred = 0x80000000u;  // in a permutation entry: left to the second launch
 static_assert(sizeof(PlanHeader) <= 256, "header layout");
 
@@ -282,10 +285,10 @@ void fill_params(KParams *p, const gcaps_tasksets_t *ts, int64_t n_tasksets, int
 // permutation of the taskset indices, zeroed work counters).  GCAPS_OK or GCAPS_ERR_WORKSPACE.
 int place_plan(KParams &p, void *workspace, size_t workspace_bytes);  // only the first part
 int enqueue_plan(KParams &p, void *workspace, size_t workspace_bytes, cudaStream_t st);
-// Tiles over the whole batch, without a plan (the header is zero); defined in gcaps_rta_tile.cu.
-cudaError_t launch_tiles(int mode, const KParams &p, int rows, int sm_count, cudaStream_t st);
-// The second of the two launches that take what tiles leave over; defined in gcaps_rta_direct.cu.
-cudaError_t launch_listed_tasksets(int mode, const KParams &p, int sm_count, cudaStream_t st);
+// Tiles of tasksets of n tasks over the whole batch, without a plan (the header is zero); defined in gcaps_rta_tile.cu.
+cudaError_t launch_tiles(int mode, const KParams &p, int n, int sm_count, cudaStream_t st);
+// The two launches that take what tiles leave over; defined in gcaps_rta_rest.cu.
+cudaError_t launch_rest(int mode, const KParams &p, int sm_count, cudaStream_t st);
 // One launch for analysis `mode` (0 GCAPS self-suspension, 1 GCAPS busy-waiting, 2 RR self-suspension, 3 RR
 // busy-waiting) without a plan, a block of one warp per taskset, for batches of at most kDirectMost
 // tasksets; defined in gcaps_rta_direct.cu.
@@ -293,13 +296,12 @@ cudaError_t launch_one_warp_each(int mode, const KParams &p, cudaStream_t st);
 // Launches over all size bins for the analyses sw.enabled names (bit m = mode m; one of 1, 2, 4, 8,
 // 5, 10) under every pair of `sw`; defined in gcaps_rta_sweep.cu.
 cudaError_t launch_sweep_set(const KParams &p, const SweepArgs &sw, int sm_count, cudaStream_t st);
-// The tasksets of up to 32 tasks under all analyses of sw.enabled in tiles with room for `rows` ranks, two or four lanes
-// per taskset; defined in gcaps_rta_tile_q2.cu and gcaps_rta_tile_q4.cu.  The two launches that take what they leave over, for the
-// analyses sw.enabled names there.
-cudaError_t launch_tile_q2(const KParams &p, const SweepArgs &sw, int rows, int sm_count, cudaStream_t st);
-cudaError_t launch_tile_q4(const KParams &p, const SweepArgs &sw, int rows, int sm_count, cudaStream_t st);
+// Tasksets of n tasks under all analyses of sw.enabled in tiles, two or four lanes per taskset; defined in
+// gcaps_rta_tile_q2.cu and gcaps_rta_tile_q4.cu.  The two launches that take what they leave over, for the
+// analyses sw.enabled names there (one of 1, 2, 4, 8, 5, 10); defined in gcaps_rta_rest_sweep.cu.
+cudaError_t launch_tile_q2(const KParams &p, const SweepArgs &sw, int n, int sm_count, cudaStream_t st);
+cudaError_t launch_tile_q4(const KParams &p, const SweepArgs &sw, int n, int sm_count, cudaStream_t st);
 cudaError_t launch_sweep_rest(const KParams &p, const SweepArgs &sw, int sm_count, cudaStream_t st);
-cudaError_t launch_sweep_listed(const KParams &p, const SweepArgs &sw, int sm_count, cudaStream_t st);
 // The same for at most kDirectSweepMost tasksets in one launch without a plan; defined in
 // gcaps_rta_direct_sweep.cu.
 cudaError_t launch_sweep_one_warp_each(const KParams &p, const SweepArgs &sw, int sm_count, cudaStream_t st);

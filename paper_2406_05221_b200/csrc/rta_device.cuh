@@ -997,7 +997,8 @@ __device__ __forceinline__ void run_bin(const KParams &p, int bin, u32 *warp_buf
   const int lane32 = threadIdx.x & 31, group = lane32 / LPT, lane = lane32 % LPT;
   const unsigned int gmask = LPT == 32 ? kFull : (((1u << LPT) - 1u) << (group * LPT));
   u32 *buf = warp_buf + group * Lay::kWords;
-  const unsigned int start = p.hdr->bin_start[bin], count = p.hdr->bin_count[bin];
+  // (the last bin ends with the permutation, also where tiles list their left-over tasksets in it from the end on)
+  const unsigned int count = p.hdr->bin_count[bin], start = bin == kRestLarge ? (unsigned int)p.n_tasksets - count : p.hdr->bin_start[bin];
   if (count == 0) return;
   // keeps 2*eps*eta and (eta+1)*eps in 32 bits
   const bool fast_call = (SWEEP ? sw->max_ovh : p.ovh) < (1 << 20);

@@ -349,25 +349,24 @@ __device__ __forceinline__ bool kept_walks(const KParams &p, const SweepArgs &sw
 // sw.enabled: the analyses that run, all of KINDS.
 template <int KINDS, int Q>
 __global__ void __launch_bounds__(kTileThreads, Q == 2 ? 12 : 16)
-rta_tile_kept_kernel(KParams p, int n_rows, int segments, const __grid_constant__ SweepArgs sw) {
+rta_tile_kept_kernel(KParams p, int n, int segments, const __grid_constant__ SweepArgs sw) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  let_dependents_start();  // the kernel of the next size bin shares no data with this one
-  const KeptRows<KINDS, Q> rows(smem_raw, n_rows, segments);
+  let_dependents_start();  // (the launches behind this one wait for what it leaves over)
+  const KeptRows<KINDS, Q> rows(smem_raw, tile_rows(n), segments);
   auto walk = [&](const TileLane &me) -> bool { return kept_walks<KINDS, Q>(p, sw, rows, me); };
-  run_tiles<false>(p, n_rows, rows, walk);
-  wait_for_previous_grid();
+  run_tiles<false>(p, n, rows, walk);
 }
 
 template <int KINDS, int Q>
-cudaError_t launch_kept(const KParams &p, const SweepArgs &sw, int rows, int sm_count, cudaStream_t st) {
+cudaError_t launch_kept(const KParams &p, const SweepArgs &sw, int n, int sm_count, cudaStream_t st) {
   static int blocks_by_registers[64] = {0};
   // room for half as many GPU segments again as the batch has on average
   const double mean = (double)p.n_gsegs / (double)p.n_tasksets;
   const int segments = (KINDS & kKindRr) ? (mean > 160.0 ? 255 : (int)(1.5 * mean) + 8) : 0;
-  const size_t smem = KeptRows<KINDS, Q>::bytes(rows, segments);
+  const size_t smem = KeptRows<KINDS, Q>::bytes(tile_rows(n), segments);
   return launch_staged<kTileThreads>(false, rta_tile_kept_kernel<KINDS, Q>, blocks_by_registers,
                                      KeptRows<KINDS, Q>::bytes(32, 255), smem, kSmemPerSm / (smem + 1024), p.n_tasksets,
-                                     sm_count, st, p, rows, segments, sw);
+                                     sm_count, st, p, n, segments, sw);
 }
 
 }  // namespace

@@ -1,11 +1,13 @@
 """Tasksets of up to 24 tasks in tiles, a lane or a few per taskset: sizes around the edges of the stage, what a walk
 keeps in registers and what it loops over, and what tiles leave to the kernels behind them, against the oracle.  The
-header in the workspace tells that a call took tiles, and how many tasksets these left."""
+header in the workspace tells that a call took tiles, and how many tasksets these left; all of them where it took the size bins
+because the batch was a mixture."""
 import numpy as np
 import pytest
 
 from oracle import rta
 from paper_2406_05221_b200 import binding
+from paper_2406_05221_b200.taskgen import TasksetBatch
 from tests.helpers import BEST_EFFORT, BUSY, LITERAL, batch_of, direct_most, left_by_tiles, repeated
 
 torch = pytest.importorskip("torch")
@@ -165,3 +167,68 @@ def test_malformed_offsets(n):
         s, w = s.cpu().numpy(), w.cpu().numpy()
         assert np.array_equal(s, want_s) and (want_s[broken] == binding.SCHED_INVALID).all(), hex(policy)
         assert np.array_equal(w[inside], want_w[inside]), hex(policy)
+
+
+def a_mixture():
+    rng = np.random.default_rng(77)
+    sizes = [25, 32, 33, 64, 65, 96, 97, 128, 129, 192, 193, 256] + [1 + k % 24 for k in range(130)]
+    sizes += [1 + (-sum(sizes) - 1) % (len(sizes) + 1)]
+    assert sum(sizes) % len(sizes) == 0 and sum(sizes) // len(sizes) <= 24
+    ts = [taskset(rng, s, 1 + k % 6, 1 + k % 4, step=1 + k % 2) for k, s in enumerate(sizes)]
+    for k in range(5, len(ts), 9):
+        ts[k] = left_ones(rng, len(ts[k]))[k % 6]
+    order = rng.permutation(len(ts))
+    return batch_of([ts[k] for k in order])
+
+
+@pytest.mark.parametrize("count", [13_000, 42_000])
+def test_mixtures_take_the_size_bins(count):
+    few = a_mixture()
+    k = times(few, count)
+    batch = repeated(few, k)
+    for policy in (0, BUSY, 1, 1 | BUSY, 1 | BEST_EFFORT):
+        w, s = through_tiles(batch, batch.n_tasksets, lambda dev, ws: binding.rta_batch(dev, policy, L, OVH, workspace=ws))
+        want_w, want_s, _ = rta.analyse(few, policy, L, OVH)
+        assert np.array_equal(s, np.tile(want_s, k)) and np.array_equal(w, np.tile(want_w, k)), hex(policy)
+    for analyses, pairs in ((15, 1), (4, 3), (15, 2)):
+        policies = [p for bit, p in binding.ANALYSIS_POLICY.items() if analyses & bit]
+        want_w, want_s = rta.analyse_multi(few, policies, [L, 1][:pairs] + [77] * (pairs - 2), [OVH, 0, 4][:pairs])
+        w, s = through_tiles(batch, batch.n_tasksets, lambda dev, ws: binding.rta_multi(
+            dev, analyses, [L, 1][:pairs] + [77] * (pairs - 2), [OVH, 0, 4][:pairs], workspace=ws))
+        assert np.array_equal(s, np.tile(want_s, k)) and np.array_equal(w, np.tile(want_w, k)), (analyses, pairs)
+
+
+@pytest.mark.parametrize("n", [8, 20])
+def test_a_stretch_that_tiles_leave(n):
+    rng = np.random.default_rng(5)
+    light, wide = [taskset(rng, n, 4, 2) for _ in range(10)], [left_ones(rng, n)[0] for _ in range(10)]
+    few, k, stretch = batch_of(light + wide), 2 * 1750 * 20 // 10, 200
+    front = repeated(few.slice(10, 20), stretch)
+    batch = TasksetBatch.concat([front, repeated(few.slice(0, 10), k)])
+    dev = binding.DeviceTasksets.from_host(batch)
+    for policy in (0, 1):
+        ws = torch.zeros(binding.workspace_bytes(batch.n_tasksets), dtype=torch.uint8, device="cuda")
+        w, s = binding.rta_batch(dev, policy, L, OVH, workspace=ws)
+        assert front.n_tasksets <= left_by_tiles(ws) < front.n_tasksets + 32   # (the tile on the border)
+        want_w, want_s, _ = rta.analyse(batch.slice(0, front.n_tasksets + 10), policy, L, OVH)
+        want_w = np.concatenate([want_w, np.tile(want_w[-10 * n:], k - 1)])
+        want_s = np.concatenate([want_s, np.tile(want_s[-10:], k - 1)])
+        assert np.array_equal(s.cpu().numpy(), want_s) and np.array_equal(w.cpu().numpy(), want_w), policy
+
+
+@pytest.mark.parametrize("n,what", [(8, "long"), (20, "long"), (24, "cores"), (12, "crowded"), (16, "crowded")])
+def test_batches_that_are_none_for_tiles(n, what):
+    rng = np.random.default_rng(6)
+    ts = [taskset(rng, n, 1 if what == "crowded" else 4, 2) for _ in range(60)]
+    for t in ts[:40]:
+        if what == "long":
+            t[n - 1].update(T=1 << 40, D=1 << 40)
+        if what == "cores":
+            t[0]["core"] = 16
+    few = batch_of([ts[k] for k in rng.permutation(60)])
+    k = times(few, max(direct_most(), 1750 * n))
+    batch = repeated(few, k)
+    for policy in (0, BUSY, 1, 1 | BUSY):
+        w, s = through_tiles(batch, batch.n_tasksets, lambda dev, ws: binding.rta_batch(dev, policy, L, OVH, workspace=ws))
+        want_w, want_s, _ = rta.analyse(few, policy, L, OVH)
+        assert np.array_equal(s, np.tile(want_s, k)) and np.array_equal(w, np.tile(want_w, k)), hex(policy)
