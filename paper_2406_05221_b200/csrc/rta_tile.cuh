@@ -496,46 +496,15 @@ __host__ __device__ constexpr int tile_rows(int n) { return n < kTileLeast ? kTi
 // the tasksets are counted by size bins here, for the plan and the launches behind (plan_behind_tiles_kernel): in a mixture bins are
 // the better way, whatever its mean.  100,000 tasksets, GCAPS / RR / all four analyses in tiles and in bins: 8 and 16 tasks
 // alternating 170 / 139 / 428 and 129 / 109 / 355 us, 12 to 24 tasks 262 / 161 / 657 and 204 / 143 / 580, 8 and 40 tasks
-// 1,089 / 316 / 1,941 and 404 / 149 / 991.
-// Of every other one of them two lanes look at the tasks: tasksets that a tile does not take (three eighths of them are enough, as tiles
-// save a fifth to a half) or that it is not worth while for (three quarters, as in tile_worth).  100,000 tasksets of 8 tasks with long
-// periods 181 / 130 / 529 in tiles first, TIMES_LONG8 straight from the bins, 60,000 of 16 tasks on one core 123 / 108 / 330 and TIMES_CORE16.
-// What it costs the others is in the noise (100,000 of 20 tasks TIMES_UNI).
-struct TileSample {
-  i64 size;      // of this lane's taskset
-  bool unfit;    // this lane's tasks of a taskset that is looked into: beyond what tiles take
-  u64 cores[2];  // how many are on a core, a byte per core
-};
-__device__ __forceinline__ TileSample tile_sample(const KParams &p, int n) {
+// 1,089 / 316 / 1,941 and 404 / 149 / 991.  What it costs the others is in the noise (100,000 of 20 tasks 176.5 and 175.5 us).
+__device__ __forceinline__ i64 tile_sample(const KParams &p) {  // the size of this lane's one
   const int lane = threadIdx.x & 31;
   const i64 stride = p.n_tasksets / 32, t = lane * stride + (lane * 37) % stride;  // (at odd distances: sizes may alternate)
-  const i64 first = p.task_off[t] - p.task_base, end = p.task_off[t + 1] - p.task_base;
-  TileSample s = {end - first, false, {0, 0}};
-  const i64 a = __shfl_sync(kFull, first, lane & ~1), b = __shfl_sync(kFull, end, lane & ~1);
-  const bool there = a >= 0 && b > a && b <= p.n_tasks && b - a <= n;
-#pragma unroll
-  for (int u = 0; u < kTileMost / 2; ++u) {
-    const i64 k = a + (lane & 1) + 2 * u;
-    if (there && k < b) {
-      const u64 T = (u64)p.period[k], core = (u64)p.core[k];
-      s.unfit |= T >= kNarrowLimit || core >= kTileCores;
-      s.cores[(core >> 3) & 1] += 1ull << ((core & 7) * 8);
-    }
-  }
-  return s;
+  return p.task_off[t + 1] - p.task_off[t];
 }
-__device__ __forceinline__ bool tile_batch(const KParams &p, const TileSample &s, int n) {
+__device__ __forceinline__ bool tile_batch(const KParams &p, i64 sample, int n) {
   const int lane = threadIdx.x & 31;
-  bool crowded = false;
-#pragma unroll
-  for (int w = 0; w < 2; ++w) {
-    const u64 all = s.cores[w] + __shfl_xor_sync(kFull, s.cores[w], 1);
-    crowded |= ((all + 0x0101010101010101ull * (127 - kTileOnCore)) & 0x8080808080808080ull) != 0;
-  }
-  const u32 unfit = __ballot_sync(kFull, s.unfit);
-  const bool other_sizes = __popc(__ballot_sync(kFull, s.size > n || 4 * s.size < 3 * n)) > 4;
-  const bool others_too = __popc((unfit | unfit >> 1) & 0x55555555u) >= 6 || __popc(__ballot_sync(kFull, crowded)) >= 24;
-  if (!other_sizes && !others_too) {
+  if (__popc(__ballot_sync(kFull, sample > n || 4 * sample < 3 * n)) <= 4) {
     if (blockIdx.x == 0 && lane == 0) p.hdr->in_tiles = 1;
     return true;
   }
@@ -556,13 +525,13 @@ __device__ __forceinline__ bool tile_batch(const KParams &p, const TileSample &s
 
 // The tasksets of a batch of n tasks each in its order, a tile per warp at a time.  `rows`: where the tasks are kept, room for
 // tile_rows(n) positions of Rows::kSets tasksets.  walk(tile lane) analyses the tile; false in the lane of a taskset that is left over.
-// What tiles do not take is listed in the workspace, for two launches behind this one: tasksets that fit the size bin of
-// n tasks as that bin, from the front on, all others as bin kRestLarge from the end on.
+// What tiles do not take is listed in the workspace, for two launches behind this one: tasksets of up to 24 tasks
+// as bin kRestSmall from the front on, all others as bin kRestLarge from the end on.
 template <bool SLICES, class Rows, class Walk>
 __device__ __forceinline__ void run_tiles(const KParams &p, int n, const Rows &rows, Walk walk) {
   const unsigned int count = (unsigned int)p.n_tasksets;
-  const int lane = threadIdx.x & 31, n_rows = tile_rows(n), small_bin = (n - 1) / 8;
-  const TileSample sample = tile_sample(p, n);
+  const int lane = threadIdx.x & 31, n_rows = tile_rows(n);
+  const i64 sample = tile_sample(p);
   // columns per tile: as many as give every warp the same number of tiles
   const unsigned int rounds = (count + Rows::kSets * gridDim.x - 1) / (Rows::kSets * gridDim.x);
   unsigned int chunk = (count + rounds * gridDim.x - 1) / (rounds * gridDim.x);
@@ -599,7 +568,7 @@ __device__ __forceinline__ void run_tiles(const KParams &p, int n, const Rows &r
     unsigned int at = 0;
     if (lane == 0) at = atomicAdd(&p.hdr->bin_count[bin], (unsigned int)__popc(bits));
     at = __shfl_sync(kFull, at, 0) + __popc(bits & ((1u << lane) - 1u));
-    if (wanted) p.perm[bin == kRestLarge ? count - 1u - at : at] = t;
+    if (wanted) p.perm[bin == kRestSmall ? at : count - 1u - at] = t;
   };
   unsigned int first = __shfl_sync(kFull, pull(), 0), second = __shfl_sync(kFull, pull(), 0);
   TileLane me, coming;
@@ -611,7 +580,6 @@ __device__ __forceinline__ void run_tiles(const KParams &p, int n, const Rows &r
 #pragma unroll 1
   while (first < count) {
     const bool looks = patience.looks();
-    bool in_vain = false;
     if (!looks && me.n > 0) me.declined = true, me.n = 0;
     const unsigned int asked = pull();
     const int columns = count - first < chunk ? (int)(count - first) : (int)chunk;
@@ -621,17 +589,16 @@ __device__ __forceinline__ void run_tiles(const KParams &p, int n, const Rows &r
       if (n_rows <= 8) tile_stage<1, SLICES>(p, rows, me, c0, lane);
       else if (n_rows <= 16) tile_stage<2, SLICES>(p, rows, me, c0, lane);
       else tile_stage<3, SLICES>(p, rows, me, c0, lane);
-      // (none of the first ones: nor the others of this tile, for an eighth of its stage)
+      // (none of the first ones: the others are passed by as well)
       if (c0 == 0 && columns >= 4 && (__ballot_sync(kFull, me.declined) & 0xfu) == 0xfu) {
         if (me.n > 0) me.declined = true, me.n = 0;
-        in_vain = true;
         break;
       }
     }
     __syncwarp();
     const unsigned int third = __shfl_sync(kFull, asked, 0);
     settle(coming, b);
-    if (coming.n > 0 && patience.unseen <= 1 && !in_vain) {
+    if (coming.n > 0 && patience.unseen <= 1) {
       const i64 to = coming.a + coming.n;
       ask_for(p.cseg_off, coming.a, to), ask_for(p.gseg_off, coming.a, to);
       ask_for(p.period, coming.a, to), ask_for(p.deadline, coming.a, to), ask_for(p.priority, coming.a, to), ask_for(p.core, coming.a, to);
@@ -640,10 +607,9 @@ __device__ __forceinline__ void run_tiles(const KParams &p, int n, const Rows &r
     }
     __syncwarp();
     if (!walk(me) && me.n > 0) me.declined = true;
-    const bool small = me.size >= 1 && me.size <= 8 * (small_bin + 1);
-    list(me.declined && small, me.t, small_bin);
-    list(me.declined && !small, me.t, kRestLarge);
-    if (!in_vain) patience.done(__popc(__ballot_sync(kFull, me.declined)), columns);
+    list(me.declined && me.size >= 1 && me.size <= 24, me.t, kRestSmall);
+    list(me.declined && !(me.size >= 1 && me.size <= 24), me.t, kRestLarge);
+    patience.done(__popc(__ballot_sync(kFull, me.declined)), columns);
     __syncwarp();
     me = coming;
     first = second, second = third;
