@@ -43,8 +43,8 @@ struct PlanHeader {
   unsigned int first_tries[kNumBins];
   unsigned int in_tiles;  // the batch goes through tiles (tile_batch)
 };
-// bins that list what tiles leave over (rta_tile.cuh)
-constexpr int kRestSmall = 2, kRestLarge = kNumBins - 1;
+// the bin that lists what tiles leave over (rta_tile.cuh) beside the one of the batch's size
+constexpr int kRestLarge = kNumBins - 1;
 constexpr int kNextTile = kNumBins;  // the work counter of tiles, which is no bin's
 static_assert(kNextTile < kBinStride, "a word of the header");
 constexpr unsigned int kDeferred = 0x80000000u;  // in a permutation entry: left to the second launch

@@ -496,42 +496,59 @@ __host__ __device__ constexpr int tile_rows(int n) { return n < kTileLeast ? kTi
 // the tasksets are counted by size bins here, for the plan and the launches behind (plan_behind_tiles_kernel): in a mixture bins are
 // the better way, whatever its mean.  100,000 tasksets, GCAPS / RR / all four analyses in tiles and in bins: 8 and 16 tasks
 // alternating 170 / 139 / 428 and 129 / 109 / 355 us, 12 to 24 tasks 262 / 161 / 657 and 204 / 143 / 580, 8 and 40 tasks
-// 1,089 / 316 / 1,941 and 404 / 149 / 991.  What it costs the others is in the noise (100,000 of 20 tasks 176.5 and 175.5 us).
-__device__ __forceinline__ i64 tile_sample(const KParams &p) {  // the size of this lane's one
+// 1,089 / 316 / 1,941 and 404 / 149 / 991.
+// look_into (where a warp has more than one tile): at the tasks of four of them too, a lane each.  If three are beyond what tiles take, or
+// too crowded to be worth while (tile_worth), so is the batch.  100,000 tasksets of 8 tasks with long periods 181 / 130 / 529 us
+// in tiles first and 111 / 94 / 327 straight in bins, 60,000 of 16 tasks on one core 123 / 108 / 330 and 98 / 93 / 289.
+// A function of its own: inlined, the registers that it holds for a moment made the walks spill (25 pairs 561 -> 587 us with eight
+// tasksets looked into, 574 with four).
+constexpr int kLookedInto = 4;
+__device__ __noinline__ bool tile_batch(const i64 *task_off, const i64 *period, const i64 *core, i64 n_tasksets, i64 n_tasks, i64 task_base,
+                                        PlanHeader *hdr, int n, bool look_into) {
   const int lane = threadIdx.x & 31;
-  const i64 stride = p.n_tasksets / 32, t = lane * stride + (lane * 37) % stride;  // (at odd distances: sizes may alternate)
-  return p.task_off[t + 1] - p.task_off[t];
-}
-__device__ __forceinline__ bool tile_batch(const KParams &p, i64 sample, int n) {
-  const int lane = threadIdx.x & 31;
-  if (__popc(__ballot_sync(kFull, sample > n || 4 * sample < 3 * n)) <= 4) {
-    if (blockIdx.x == 0 && lane == 0) p.hdr->in_tiles = 1;
+  const i64 stride = n_tasksets / 32, t = lane * stride + (i64)((lane * 2654435761u) >> 8) % stride;  // (at odd distances: kinds may alternate)
+  const i64 first = task_off[t] - task_base, end = task_off[t + 1] - task_base;
+  const int other_sizes = __popc(__ballot_sync(kFull, end - first > n || 4 * (end - first) < 3 * n));
+  u64 T[kLookedInto], c[kLookedInto];
+#pragma unroll
+  for (int k = 0; k < kLookedInto; ++k) {
+    const i64 a = __shfl_sync(kFull, first, 32 / kLookedInto * k), b = __shfl_sync(kFull, end, 32 / kLookedInto * k);
+    T[k] = 0, c[k] = 0x100 + lane;  // (no task: a core of its own)
+    if (look_into && a >= 0 && b <= n_tasks && b - a <= n && lane < b - a) T[k] = (u64)period[a + lane], c[k] = (u64)core[a + lane];
+  }
+  int in_vain = 0;
+#pragma unroll
+  for (int k = 0; k < kLookedInto; ++k) {
+    const bool crowded = __popc(__match_any_sync(kFull, (u32)c[k])) > kTileOnCore;
+    in_vain += __any_sync(kFull, T[k] >= kNarrowLimit || (T[k] > 0 && c[k] >= kTileCores) || crowded) ? 1 : 0;
+  }
+  if (other_sizes <= 4 && 4 * in_vain < 3 * kLookedInto) {
+    if (blockIdx.x == 0 && lane == 0) hdr->in_tiles = 1;
     return true;
   }
   u32 counts[kNumBins];
 #pragma unroll
   for (int k = 0; k < kNumBins; ++k) counts[k] = 0;
 #pragma unroll 4
-  for (i64 t0 = (i64)blockIdx.x * 32; t0 < p.n_tasksets; t0 += (i64)gridDim.x * 32) {
-    const int bin = t0 + lane < p.n_tasksets ? size_bin(p.task_off[t0 + lane + 1] - p.task_off[t0 + lane]) : kNumBins;
+  for (i64 t0 = (i64)blockIdx.x * 32; t0 < n_tasksets; t0 += (i64)gridDim.x * 32) {
+    const int bin = t0 + lane < n_tasksets ? size_bin(task_off[t0 + lane + 1] - task_off[t0 + lane]) : kNumBins;
 #pragma unroll
     for (int k = 0; k < kNumBins; ++k) counts[k] += __popc(__ballot_sync(kFull, bin == k));
   }
 #pragma unroll
   for (int k = 0; k < kNumBins; ++k)
-    if (lane == k && counts[k] > 0) atomicAdd(&p.hdr->bin_count[k], counts[k]);
+    if (lane == k && counts[k] > 0) atomicAdd(&hdr->bin_count[k], counts[k]);
   return false;
 }
 
 // The tasksets of a batch of n tasks each in its order, a tile per warp at a time.  `rows`: where the tasks are kept, room for
 // tile_rows(n) positions of Rows::kSets tasksets.  walk(tile lane) analyses the tile; false in the lane of a taskset that is left over.
-// What tiles do not take is listed in the workspace, for two launches behind this one: tasksets of up to 24 tasks
-// as bin kRestSmall from the front on, all others as bin kRestLarge from the end on.
+// What tiles do not take is listed in the workspace, for two launches behind this one: tasksets that fit the size bin of
+// n tasks as that bin, from the front on, all others as bin kRestLarge from the end on.
 template <bool SLICES, class Rows, class Walk>
 __device__ __forceinline__ void run_tiles(const KParams &p, int n, const Rows &rows, Walk walk) {
   const unsigned int count = (unsigned int)p.n_tasksets;
-  const int lane = threadIdx.x & 31, n_rows = tile_rows(n);
-  const i64 sample = tile_sample(p);
+  const int lane = threadIdx.x & 31, n_rows = tile_rows(n), small_bin = (n - 1) / 8;
   // columns per tile: as many as give every warp the same number of tiles
   const unsigned int rounds = (count + Rows::kSets * gridDim.x - 1) / (Rows::kSets * gridDim.x);
   unsigned int chunk = (count + rounds * gridDim.x - 1) / (rounds * gridDim.x);
@@ -568,13 +585,13 @@ __device__ __forceinline__ void run_tiles(const KParams &p, int n, const Rows &r
     unsigned int at = 0;
     if (lane == 0) at = atomicAdd(&p.hdr->bin_count[bin], (unsigned int)__popc(bits));
     at = __shfl_sync(kFull, at, 0) + __popc(bits & ((1u << lane) - 1u));
-    if (wanted) p.perm[bin == kRestSmall ? at : count - 1u - at] = t;
+    if (wanted) p.perm[bin == kRestLarge ? count - 1u - at : at] = t;
   };
   unsigned int first = __shfl_sync(kFull, pull(), 0), second = __shfl_sync(kFull, pull(), 0);
   TileLane me, coming;
   i64 b;
   look_up(first, me, b);
-  if (!tile_batch(p, sample, n)) return;
+  if (!tile_batch(p.task_off, p.period, p.core, p.n_tasksets, p.n_tasks, p.task_base, p.hdr, n, rounds > 1)) return;
   settle(me, b);
   TilePatience patience = {0};
 #pragma unroll 1
@@ -589,7 +606,7 @@ __device__ __forceinline__ void run_tiles(const KParams &p, int n, const Rows &r
       if (n_rows <= 8) tile_stage<1, SLICES>(p, rows, me, c0, lane);
       else if (n_rows <= 16) tile_stage<2, SLICES>(p, rows, me, c0, lane);
       else tile_stage<3, SLICES>(p, rows, me, c0, lane);
-      // (none of the first ones: the others are passed by as well)
+      // (none of the first ones: nor the others of this tile, for an eighth of its stage)
       if (c0 == 0 && columns >= 4 && (__ballot_sync(kFull, me.declined) & 0xfu) == 0xfu) {
         if (me.n > 0) me.declined = true, me.n = 0;
         break;
@@ -607,9 +624,10 @@ __device__ __forceinline__ void run_tiles(const KParams &p, int n, const Rows &r
     }
     __syncwarp();
     if (!walk(me) && me.n > 0) me.declined = true;
-    list(me.declined && me.size >= 1 && me.size <= 24, me.t, kRestSmall);
-    list(me.declined && !(me.size >= 1 && me.size <= 24), me.t, kRestLarge);
-    patience.done(__popc(__ballot_sync(kFull, me.declined)), columns);
+    const bool small = me.size >= 1 && me.size <= 8 * (small_bin + 1);
+    list(me.declined && small, me.t, small_bin);
+    list(me.declined && !small, me.t, kRestLarge);
+    patience.done(__popc(__ballot_sync(kFull, me.declined && me.n > 0)), columns);
     __syncwarp();
     me = coming;
     first = second, second = third;

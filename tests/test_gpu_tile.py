@@ -7,6 +7,7 @@ import pytest
 
 from oracle import rta
 from paper_2406_05221_b200 import binding
+from paper_2406_05221_b200.taskgen import TasksetBatch
 from tests.helpers import BEST_EFFORT, BUSY, LITERAL, batch_of, direct_most, left_by_tiles, repeated
 
 torch = pytest.importorskip("torch")
@@ -195,3 +196,39 @@ def test_mixtures_take_the_size_bins(count):
         w, s = through_tiles(batch, batch.n_tasksets, lambda dev, ws: binding.rta_multi(
             dev, analyses, [L, 1][:pairs] + [77] * (pairs - 2), [OVH, 0, 4][:pairs], workspace=ws))
         assert np.array_equal(s, np.tile(want_s, k)) and np.array_equal(w, np.tile(want_w, k)), (analyses, pairs)
+
+
+@pytest.mark.parametrize("n", [8, 20])
+def test_a_stretch_that_tiles_leave(n):
+    rng = np.random.default_rng(5)
+    light, wide = [taskset(rng, n, 4, 2) for _ in range(10)], [left_ones(rng, n)[0] for _ in range(10)]
+    few, k, stretch = batch_of(light + wide), 2 * 1750 * 20 // 10, 200
+    front = repeated(few.slice(10, 20), stretch)
+    batch = TasksetBatch.concat([front, repeated(few.slice(0, 10), k)])
+    dev = binding.DeviceTasksets.from_host(batch)
+    for policy in (0, 1):
+        ws = torch.zeros(binding.workspace_bytes(batch.n_tasksets), dtype=torch.uint8, device="cuda")
+        w, s = binding.rta_batch(dev, policy, L, OVH, workspace=ws)
+        assert front.n_tasksets <= left_by_tiles(ws) < front.n_tasksets + 32   # (the tile on the border)
+        want_w, want_s, _ = rta.analyse(batch.slice(0, front.n_tasksets + 10), policy, L, OVH)
+        want_w = np.concatenate([want_w, np.tile(want_w[-10 * n:], k - 1)])
+        want_s = np.concatenate([want_s, np.tile(want_s[-10:], k - 1)])
+        assert np.array_equal(s.cpu().numpy(), want_s) and np.array_equal(w.cpu().numpy(), want_w), policy
+
+
+@pytest.mark.parametrize("n,what", [(8, "long"), (20, "long"), (24, "cores"), (12, "crowded"), (16, "crowded")])
+def test_batches_that_are_none_for_tiles(n, what):
+    rng = np.random.default_rng(6)
+    ts = [taskset(rng, n, 1 if what == "crowded" and k < 55 else 4, 2) for k in range(60)]
+    for t in ts[:55]:
+        if what == "long":
+            t[n - 1].update(T=1 << 40, D=1 << 40)
+        if what == "cores":
+            t[0]["core"] = 16
+    few = batch_of([ts[k] for k in rng.permutation(60)])
+    k = times(few, 60_000)   # (more than one tile per warp)
+    batch = repeated(few, k)
+    for policy in (0, BUSY, 1, 1 | BUSY):
+        w, s = through_tiles(batch, batch.n_tasksets, lambda dev, ws: binding.rta_batch(dev, policy, L, OVH, workspace=ws))
+        want_w, want_s, _ = rta.analyse(few, policy, L, OVH)
+        assert np.array_equal(s, np.tile(want_s, k)) and np.array_equal(w, np.tile(want_w, k)), hex(policy)
