@@ -467,6 +467,16 @@ int tile_tasks(int analyses, int walks, i64 max_ovh, const KParams &p) {
   return n;
 }
 
+// Whether the analyses of GCAPS and of RR go through tiles one after the other.  A kernel of both stages a tile once for all, but the more its
+// walks have to do the more it loses to instruction fetch (it holds the walks twice) and to its shared memory.  Together / apart (by bins
+// for the groups of lanes), 100,000 tasksets at U/core 0.5, 60 % GPU tasks: all four analyses of 16 tasks 330 / 355 us, 20 tasks 493 / 475,
+// 22 tasks 589 / 537 (611), 24 tasks 842 / 656 (652); three pairs of two analyses, four lanes per taskset, of 12 tasks 330 / 344,
+// 16 tasks 513 / 462 (553), 20 tasks 810 / 666 (755), 24 tasks 1,366 / 931 (862).  Small batches stay together, as GCAPS alone does
+// not take tiles there (20 tasks, 15,000 tasksets, three pairs of four analyses: 350 / 365; 24 tasks, 30,000, of two: 369 / 330).
+bool tiles_apart(int n, int walks, i64 n_tasksets) {
+  return n > (walks > kKeptFew ? 12 : 22) && n_tasksets * walks >= (n > 22 ? 80000 : 100000);
+}
+
 // Plan + analysis launches of one call.  `sw` null: one analysis (p.policy).  Otherwise the
 // analyses named in `analyses` (bit m = mode m) for every pair of `sw`: the self-suspension
 // modes in one set of launches, the busy-waiting modes in another (the plan is shared, the work
@@ -487,44 +497,66 @@ int enqueue_batch(KParams p, void *workspace, size_t workspace_bytes, int sm_cou
   if (rc != GCAPS_OK) return rc;
   // walks of a taskset through the recurrence that a tile's lanes share.  (A single one of GCAPS and of RR each is better
   // left to the groups of lanes, which stage once for both: 288 us for 100,001 tasksets of 20 tasks, 323 in tiles.)
-  const int walks = sw ? sw->n * (((analyses & 3) == 3 || (analyses & 12) == 12) ? 2 : 1) : 1;
-  const int tile_n = direct || (sw && walks == 1) ? 0 : tile_tasks(sw ? analyses : 1 << mode, walks, sw ? sw->max_ovh : p.ovh, p);
-  if (!direct && tile_n == 0) enqueue_plan_kernels(p, st);
+  auto walks_of = [&](int which) -> int { return sw ? sw->n * (((which & 3) == 3 || (which & 12) == 12) ? 2 : 1) : 1; };
+  auto tiles_of = [&](int which, int walks) -> int {
+    return direct || (sw && walks == 1) ? 0 : tile_tasks(which, walks, sw ? sw->max_ovh : p.ovh, p);
+  };
+  const int all = sw ? analyses : 1 << mode;
+  const int tile_n = tiles_of(all, walks_of(all));
   cudaError_t e = cudaGetLastError();
-  if (e == cudaSuccess && tile_n > 0) e = cudaMemsetAsync(p.hdr, 0, sizeof(PlanHeader), st);
-  if (e == cudaSuccess && tile_n > 0 && !sw) {
-    e = launch_tiles(mode, p, tile_n, sm_count, st);
-    if (e == cudaSuccess) e = launch_plan_behind_tiles(p, sm_count, st);
-    if (e == cudaSuccess) e = launch_rest(mode, p, sm_count, st);
-  } else if (e == cudaSuccess && sw) {
+  // the plan, or the header that tiles start from
+  auto begin = [&](int n) -> cudaError_t {
+    if (n > 0) return cudaMemsetAsync(p.hdr, 0, sizeof(PlanHeader), st);
+    if (!direct) enqueue_plan_kernels(p, st);
+    return cudaGetLastError();
+  };
+  if (e == cudaSuccess && sw) {
     SweepArgs set = *sw;
     set.block_stride = __builtin_popcount(analyses);
     for (int m = 0, k = 0; m < 4; ++m) {
       set.block_of_mode[m] = k;
       k += (analyses >> m) & 1;
     }
-    bool first = true;
-    if (tile_n > 0) {
-      set.enabled = analyses;
-      e = walks > kKeptFew ? launch_tile_q4(p, set, tile_n, sm_count, st) : launch_tile_q2(p, set, tile_n, sm_count, st);
-      if (e == cudaSuccess) e = launch_plan_behind_tiles(p, sm_count, st);
+    auto analyse = [&](int which, int walks, int n) -> cudaError_t {
+      cudaError_t err = begin(n);
+      if (n > 0) {
+        set.enabled = which;
+        if (err == cudaSuccess) err = walks > kKeptFew ? launch_tile_q4(p, set, n, sm_count, st) : launch_tile_q2(p, set, n, sm_count, st);
+        if (err == cudaSuccess) err = launch_plan_behind_tiles(p, sm_count, st);
+      }
+      bool first = true;
+      for (int half = 0; half < 2 && err == cudaSuccess; ++half) {
+        set.enabled = which & (half == 0 ? 5 : 10);
+        if (set.enabled == 0) continue;
+        if (!first && !direct) err = cudaMemsetAsync(p.hdr->next, 0, sizeof(p.hdr->next), st);
+        first = false;
+        if (err == cudaSuccess)
+          err = direct  ? launch_sweep_one_warp_each(p, set, sm_count, st)
+                : n > 0 ? launch_sweep_rest(p, set, sm_count, st)
+                        : launch_sweep_set(p, set, sm_count, st);
+      }
+      return err;
+    };
+    const int gcaps = analyses & 3, rr_ones = analyses & 12, gcaps_walks = walks_of(gcaps), rr_walks = walks_of(rr_ones);
+    if (tile_n > 0 && gcaps && rr_ones && gcaps_walks > 1 && rr_walks > 1 && tiles_apart(tile_n, walks_of(all), p.n_tasksets)) {
+      e = analyse(gcaps, gcaps_walks, tiles_of(gcaps, gcaps_walks));
+      if (e == cudaSuccess) e = analyse(rr_ones, rr_walks, tiles_of(rr_ones, rr_walks));
+    } else {
+      e = analyse(analyses, walks_of(all), tile_n);
     }
-    for (int half = 0; half < 2 && e == cudaSuccess; ++half) {
-      set.enabled = analyses & (half == 0 ? 5 : 10);
-      if (set.enabled == 0) continue;
-      if (!first && !direct) e = cudaMemsetAsync(p.hdr->next, 0, sizeof(p.hdr->next), st);
-      first = false;
-      if (e == cudaSuccess)
-        e = direct     ? launch_sweep_one_warp_each(p, set, sm_count, st)
-            : tile_n > 0 ? launch_sweep_rest(p, set, sm_count, st)
-                       : launch_sweep_set(p, set, sm_count, st);
-    }
+  } else if (e == cudaSuccess && tile_n > 0) {
+    e = begin(tile_n);
+    if (e == cudaSuccess) e = launch_tiles(mode, p, tile_n, sm_count, st);
+    if (e == cudaSuccess) e = launch_plan_behind_tiles(p, sm_count, st);
+    if (e == cudaSuccess) e = launch_rest(mode, p, sm_count, st);
   } else if (e == cudaSuccess) {
-    if (direct) e = launch_one_warp_each(mode, p, st);
-    else if (mode == 0) e = launch_all_bins<0>(p, sm_count, st);
-    else if (mode == 1) e = launch_all_bins<1>(p, sm_count, st);
-    else if (mode == 2) e = launch_all_bins<2>(p, sm_count, st);
-    else e = launch_all_bins<3>(p, sm_count, st);
+    e = begin(0);
+    if (e == cudaSuccess)
+      e = direct      ? launch_one_warp_each(mode, p, st)
+          : mode == 0 ? launch_all_bins<0>(p, sm_count, st)
+          : mode == 1 ? launch_all_bins<1>(p, sm_count, st)
+          : mode == 2 ? launch_all_bins<2>(p, sm_count, st)
+                      : launch_all_bins<3>(p, sm_count, st);
   }
   if (e != cudaSuccess) {
     g_last_cuda_error = (int)e;

@@ -84,11 +84,12 @@ def times(few, at_least):
 
 
 def through_tiles(batch, left, call):
-    """The results of call(tasksets, workspace), which leaves `left` tasksets behind its tiles."""
+    """The results of call(tasksets, workspace), which leaves `left` tasksets behind its tiles (and more if the few tasksets
+    of the last tile have crowded cores)."""
     dev = binding.DeviceTasksets.from_host(batch)
     ws = torch.zeros(binding.workspace_bytes(batch.n_tasksets), dtype=torch.uint8, device="cuda")
     w, s = call(dev, ws)
-    assert left_by_tiles(ws) == left
+    assert left <= left_by_tiles(ws) < left + 32
     return None if w is None else w.cpu().numpy(), s.cpu().numpy()
 
 
@@ -105,9 +106,9 @@ def check_one(few, left, policies):
         assert np.array_equal(w, np.tile(want_w, k)), (n, hex(policy))
 
 
-def check_several(few, left, analyses, pairs):
+def check_several(few, left, analyses, pairs, at_least=0):
     n = few.n_tasks // few.n_tasksets
-    k = times(few, 25_000 if n > 12 and analyses < 4 else direct_most(several=True))
+    k = times(few, max(at_least, 25_000 if n > 12 and analyses < 4 else direct_most(several=True)))
     batch = repeated(few, k)
     if analyses & 12:  # a tile of several analyses has room for half as many GPU segments again as there are on average
         segments = few.gseg_off[few.task_off[1:]] - few.gseg_off[few.task_off[:-1]]
@@ -134,6 +135,12 @@ def test_one_analysis(n):
 @pytest.mark.parametrize("analyses,pairs", [(15, 1), (3, 2), (4, 5), (10, 3), (1, 4), (12, 1), (15, 5)])
 def test_several_analyses(n, analyses, pairs):
     check_several(*some(n), analyses, pairs)
+
+
+# (GCAPS by bins and RR in tiles; both in tiles, one after the other, with four lanes per taskset and with two)
+@pytest.mark.parametrize("n,pairs,count", [(24, 3, 14_000), (16, 3, 17_000), (24, 3, 17_000), (24, 1, 50_000)])
+def test_analyses_of_both_policies_apart(n, pairs, count):
+    check_several(*some(n), 15, pairs, count)
 
 
 @pytest.mark.parametrize("n", [4, 8, 20])
