@@ -967,7 +967,7 @@ const char *gcaps_rta_strerror(int code) {
     case GCAPS_ERR_CUDA: return "CUDA runtime error (see gcaps_rta_last_cuda_error)";
     case GCAPS_ERR_NO_DEVICE: return "no usable sm_100 CUDA device";
     case GCAPS_ERR_TOO_LARGE:
-      return "batch exceeds GCAPS_RTA_STATIC_MAX_TASKSETS: split it or use gcaps_rta_batch";
+      return "batch exceeds the limit of this entry point (GCAPS_RTA_STATIC_MAX_TASKSETS, GCAPS_RTA_FEW_MAX_TASKSETS): split it or use gcaps_rta_batch";
     default: return "unknown error code";
   }
 }

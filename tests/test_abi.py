@@ -41,6 +41,8 @@ def test_host_only_entry_points(lib):
     assert big % 256 == 0 and big >= 1000 * (4 + 3 * 80) * 4
     for code in (0, -1, -2, -3, -4, -99):
         assert lib.gcaps_rta_strerror(code)
+    for limit in (b"GCAPS_RTA_STATIC_MAX_TASKSETS", b"GCAPS_RTA_FEW_MAX_TASKSETS"):   # (of the entry points that return it)
+        assert limit in lib.gcaps_rta_strerror(binding.ERR_TOO_LARGE)
 
 
 def test_header_constants_match_binding():
