@@ -43,7 +43,7 @@ K_TERM, K_SETUP = 6, 16   # algorithmic integer lane-operations per interference
 
 def in_tiles(tasksets, tasks, gcaps, walks):
     """Whether a batch too large for one launch without a plan goes through tiles (tile_tasks of gcaps_rta.cu):
-    small tasksets of one size, and under GCAPS enough of them.  `walks`: analyses of a policy per taskset."""
+    small tasksets of one size (a mixture with a whole mean takes the same launches), and under GCAPS enough of them.  `walks`: analyses of a policy per taskset."""
     if not tasks or tasks % tasksets or tasks > 24 * tasksets:
         return False
     n = tasks // tasksets
@@ -68,10 +68,10 @@ def kernel_launches(tasksets, kind="one", tasks=None, gcaps=True, walks=1):
 # ncu capture of a 131,072-taskset launch (traffic grows in proportion to the tasksets of a
 # launch).  Only reported while the kernel source is the one the counters were taken from.
 CAPTURED_TRAFFIC = {
-    "source_sha256": "11a88d485d7e1369e0e4bf41aa4a221e4f6fb2ed5c1cc613075113639210b093",
+    "source_sha256": "95199ab072a77c001c572b9ce361812d22630ff803addeb67f538e2413190d4b",
     "workload": "large",
-    "bytes_per_taskset": {"gcaps": (1236501000 + 80218112) / 131072.0,
-                          "rr": (1236523000 + 80107520) / 131072.0},
+    "bytes_per_taskset": {"gcaps": (1236487936 + 76159232) / 131072.0,
+                          "rr": (1236483328 + 76390144) / 131072.0},
 }
 
 

@@ -265,7 +265,7 @@ int gcaps_rta_sweep_batch(const gcaps_tasksets_t *ts, int64_t n_tasksets, int po
  * and aggregated once and then goes through the recurrence of gcaps_rta_batch once per requested
  * analysis and per (timeslice, overhead) pair; the two self-suspension analyses run in one
  * launch, the two busy-waiting ones in another (tasksets of up to 24 tasks and one size: all of
- * them in one).  Results are those of separate gcaps_rta_batch calls.
+ * them in one, or those of GCAPS in one and those of RR in another).  Results are those of separate gcaps_rta_batch calls.
  *
  *   analyses   OR of GCAPS_ANALYSIS_*; `flags`: GCAPS_RTA_LITERAL, GCAPS_RTA_BEST_EFFORT
  *   n_points, timeslice_us, ctx_switch_overhead_us: as for gcaps_rta_sweep_batch (the overhead of

@@ -448,9 +448,8 @@ cudaError_t launch_all_bins(const KParams &p, int sm_count, cudaStream_t st) {
   return e;
 }
 
-// Tiles are for batches of tasksets of one size (a mean that is a whole number): a tile's rows are taken by the largest
-// taskset, and in a mixture the plan's bins are the better way (4 to 24 tasks, 100,000 tasksets 212 us in tiles, 162
-// us in bins).  Under GCAPS a tile's walk is long, so there have to be enough tiles to go round: 12 tasks 43 / 54 us (tiles /
+// Tiles are for batches of tasksets of one size, whose mean is a whole number; where that is a mixture's all the same, the tile
+// kernel finds out (tile_batch).  Under GCAPS a tile's walk is long, so there have to be enough tiles to go round: 12 tasks 43 / 54 us (tiles /
 // bins) at 12,500 tasksets and 63 / 84 at 50,000, 16 tasks 71 / 69 at 25,000 and 79 / 83 at 35,000, 20 tasks 91 / 84
 // and 97 / 105, 24 tasks 127 / 123 at 35,000 and 128 / 157 at 50,000.  Under RR tiles are the faster way from the start
 // (24 tasks 40 / 51 us at 12,500).  Several analyses under GCAPS, 20 tasks: 170 / 138 us for five pairs of 10,000
@@ -704,9 +703,9 @@ int gcaps_rta_batch_static(const gcaps_tasksets_t *ts, int64_t n_tasksets, int p
   }
   KParams p;
   fill_params(&p, ts, n_tasksets, policy, timeslice_us, ctx_switch_overhead_us, out_wcrt, out_sched);
-  // Nothing in the array has to be cleared first: the plan kernels write the header (counts,
-  // starts, zeroed work counters), every per-block count and every permutation entry that the
-  // analysis kernels of this call read.
+  // Nothing in the array has to be cleared first: the header (counts, starts, work counters) is written by the plan kernels or,
+  // in front of tiles, cleared in the stream, and every per-block count and permutation entry that a kernel of
+  // this call reads is written by one before it.
   return enqueue_batch(p, scratch, (size_t)GCAPS_RTA_STATIC_SCRATCH_BYTES, di.sm_count,
                        (cudaStream_t)stream);
 }

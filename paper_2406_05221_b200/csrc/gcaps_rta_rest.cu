@@ -1,5 +1,5 @@
-// gcaps_rta_rest.cu -- one analysis of what lies behind tiles in the stream (rta_rest.cuh).
-#include "rta_rest.cuh"
+// gcaps_rta_rest.cu -- one analysis of what lies behind tiles in the stream (run_rest of rta_device.cuh).
+#include "rta_device.cuh"
 
 using namespace gcaps_detail;
 

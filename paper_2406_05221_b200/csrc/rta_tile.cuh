@@ -1,4 +1,4 @@
-// rta_tile.cuh -- tasksets of up to 32 tasks, a tile of up to 32 of them per warp.  Internal.
+// rta_tile.cuh -- tasksets of up to 24 tasks, a tile of up to 32 of them per warp.  Internal.
 //
 //   stage   four tasksets at a time, eight lanes each: values are checked, the segments added up, and every
 //           task's values go to the row of its position
@@ -6,16 +6,17 @@
 //   walk    every lane takes its own taskset through the recurrence, rank by rank, out of its column of
 //           the tile, and writes its results.  Nothing is exchanged between lanes
 //
-// What bounds it.  With a group of lanes per taskset (run_bin) a 20-task taskset took 1,544 warp instructions: a
+// What bounds it.  With a group of lanes per taskset (run_bin) a 20-task taskset took 1,345 warp instructions: a
 // sweep over its 10 interferers is one or two terms per lane and then a reduction, a vote and a branch, and setting
-// a rank up is done by every group for itself.  A lane per taskset needs none of that: 629 instructions, though
+// a rank up is done by every group for itself.  A lane per taskset needs none of that: 669 instructions, though
 // the lanes wait for the one with the most sweeps (123 in 20 ranks against 81 with four tasksets per warp, 53 for
-// one alone).  What is left is latency: a tile of 20 ranks takes 24 KB, so an SM holds nine warps.  Everything follows from
+// one alone).  What is left is latency: a tile of 20 ranks takes 24 KB, so an SM holds nine warps (eight on average).  Everything follows from
 // that: interferers lie in registers, and a sweep is straight-line code for a bound on their number that the warp
 // shares (2, 4 or 6 on the same core and twice as many in the list; with a branch per pair of entries the walk took
 // 76,000 instead of 50,000 cycles per tile); a lane's stage has all loads of a task under way at once, out of L2.
 // Two or four lanes per taskset, or copying the tasksets into shared memory first, were slower.  And as tiles take the
-// batch in its order, there is no plan and there are no bins: four operations in the stream instead of eleven.  100,000
+// batch in its order, there is no plan and there are no bins: five operations in the stream (the header is cleared; the tiles; the rest
+// of a plan, for a batch that turns out to be none for tiles; two launches over what is left) instead of eleven.  100,000
 // tasksets of 20 tasks at U/core 0.5 under GCAPS 226 -> 175 us (U/core 0.3 196 -> 146), under RR 133 -> 92; 1,000,000 of
 // 8 tasks 634 -> 338 us; 200,000 of 24 tasks under RR 208 -> 157 us.
 #ifndef GCAPS_RTA_TILE_CUH_
@@ -543,7 +544,7 @@ __device__ __noinline__ bool tile_batch(const i64 *task_off, const i64 *period, 
 
 // The tasksets of a batch of n tasks each in its order, a tile per warp at a time.  `rows`: where the tasks are kept, room for
 // tile_rows(n) positions of Rows::kSets tasksets.  walk(tile lane) analyses the tile; false in the lane of a taskset that is left over.
-// What tiles do not take is listed in the workspace, for two launches behind this one: tasksets that fit the size bin of
+// What tiles do not take is listed in the workspace, for the launches behind this one: tasksets that fit the size bin of
 // n tasks as that bin, from the front on, all others as bin kRestLarge from the end on.
 template <bool SLICES, class Rows, class Walk>
 __device__ __forceinline__ void run_tiles(const KParams &p, int n, const Rows &rows, Walk walk) {

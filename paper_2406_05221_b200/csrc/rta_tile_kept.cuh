@@ -1,4 +1,4 @@
-// rta_tile_kept.cuh -- several analyses per taskset of tasksets of up to 32 tasks: a tile is staged and ordered once,
+// rta_tile_kept.cuh -- several analyses per taskset of tasksets of up to 24 tasks: a tile is staged and ordered once,
 // then every taskset has Q lanes, each of which takes it through the recurrence under another analysis or (timeslice,
 // overhead) pair.  Internal.
 #ifndef GCAPS_RTA_TILE_KEPT_CUH_
